@@ -1,0 +1,237 @@
+// FP64 pair policies of the Newton's-third-law stages with the pair arithmetic on the
+// integer pipe (fx64.cuh).  A unit (i-rows x one j-tile) keeps its sums as 96-bit
+// integers whose unit 2^lsb follows from the softening: |d| / (d^2 + eps) <= 1 / (2 sqrt
+// eps), so no sum can overflow and every sum is exact, whatever the order.  Row sums are
+// moved into doubles (shared memory) every kFxFlush units; column sums are added over the
+// warp with redux.sync on 27-bit limbs, over the warps as integers, and stored as doubles.
+//
+// A unit that touches a coordinate beyond 2^26 sqrt(eps) (terms so small against the
+// largest possible one that 96 bits would hold less than a double) or a non-finite one
+// runs the FP64 policy's tile instead: the CTA decides per unit with one vote, which
+// replaces the barrier after the tile's load.
+#pragma once
+#include "fx64.cuh"
+#include "pairs_impl.cuh"
+
+namespace {
+
+constexpr int kFxFlush = 16;        // units between moves of the row sums into doubles
+constexpr double kFxEpsMin = 0x1p-28;  // below: the FP64 policies (the unit 2^lsb would grow)
+
+// Row sums of a thread in shared memory: [value][thread]
+template <int V>
+struct FxRowSums {
+  double *p;  // this thread's column
+  __device__ double &at(int v) const { return p[v * NT]; }
+};
+
+// Warp total of a 96-bit sum (|sum| < 2^85 per lane), low 11 bits dropped: limbs of 27, 27
+// and 31 bits, each added over the 32 lanes without overflow.
+__device__ __forceinline__ uint4 fx_warp_sum(const fx64::Acc96 &a) {
+  const unsigned l0 = fx64::shf_r(a.w0, a.w1, 11) & 0x07ffffffu;
+  const unsigned l1 = fx64::shf_r(a.w1, a.w2, 6) & 0x07ffffffu;
+  const int l2 = (int)a.w2 >> 1;
+  uint4 r;
+  r.x = __reduce_add_sync(0xffffffffu, l0);
+  r.y = __reduce_add_sync(0xffffffffu, l1);
+  r.z = (unsigned)__reduce_add_sync(0xffffffffu, l2);
+  r.w = 0u;
+  return r;
+}
+// Sum of n limb triples `stride` apart, as a double in units of 2^(lsb + 11)
+template <int n>
+__device__ __forceinline__ double fx_limb_total(const uint4 *s, int stride) {
+  unsigned long long t0 = 0, t1 = 0;
+  long long t2 = 0;
+#pragma unroll
+  for (int w = 0; w < n; w++) {
+    const uint4 v = s[w * stride];
+    t0 += v.x;
+    t1 += v.y;
+    t2 += (int)v.z;
+  }
+  return ((double)t2 * 134217728.0 + (double)t1) * 134217728.0 + (double)t0;
+}
+
+// ------------------------------------------------------------ forward 2D
+// Per pair dx and dy in FP64 (2 operations instead of 14); the squared distance, its
+// reciprocal, the products with dx and dy and the four sums are integers: about 147
+// instructions per pair, 57% of the integer pipe and of the FP64 pipe (4 warps per scheduler;
+// dependent instructions are what is left).  One force at N = 49,152: 28.1 ms with GravF64,
+// 9.74 with s on the FP64 pipe, 7.25 as it stands.
+template <int R_, int TJ_, int MODE>
+struct GravFx {
+  static constexpr bool FX = true;
+  static constexpr int THREADS = NT, MINB = 4;
+  using ColT = double;
+  using Wild = GravF64<R_, TJ_, MODE>;  // units out of the fixed-point range
+  static constexpr int R = R_, TJ = TJ_, NACC = 2, JB = RecordBytes<MD_GRAV2D, false, false>::value;
+  static constexpr bool MASK = false;
+  static constexpr int NR = R;
+  static constexpr int FMT = 0;
+  static constexpr int COL_BYTES = (NT / 32) * TJ * NACC * (int)sizeof(uint4);
+  __device__ static int row_of(int r) { return r * NT + (int)threadIdx.x; }
+  struct State {
+    double x[R], y[R];
+    fx64::Acc96 acc[R][NACC];
+    FxRowSums<R * NACC> rows;
+    int units;     // since the last flush
+    bool wild;     // a row of this thread lies out of the fixed-point range
+  };
+  // floor(log2(eps) / 2); the sums' unit is 2^lsb: a term (below 2^92) is shifted down by
+  // k = es - ex - half + 9 >= 9, and 2^12 terms fit
+  __device__ static int half_exp(const PairArgs &a) { return ((int)(fx64::hi_word(a.epsd) >> 20) - 1023) >> 1; }
+  __device__ static int lsb(const PairArgs &a) { return -82 - half_exp(a); }
+  __device__ static bool out_of_range(double v, int half) {
+    const unsigned h = fx64::hi_word(v) & 0x7fffffffu;
+    return h >= ((unsigned)(1023 + 26 + half) << 20) && h != (fx64::hi_word(1.0e150));  // padding: its terms vanish
+  }
+  __device__ static void load(State &st, const void *mirror, int64_t i0, const PairArgs &a, double *rowsm) {
+    const int half = half_exp(a);
+    st.wild = false;
+    st.units = 0;
+    st.rows.p = rowsm + threadIdx.x;
+#pragma unroll
+    for (int r = 0; r < R; r++) {
+      const double2 m = *(const double2 *)((const double *)mirror + (i0 + row_of(r)) * 2);
+      st.x[r] = m.x;
+      st.y[r] = m.y;
+      st.wild = st.wild || out_of_range(m.x, half) || out_of_range(m.y, half);
+#pragma unroll
+      for (int d = 0; d < NACC; d++) {
+        st.acc[r][d] = fx64::Acc96{0u, 0u, 0u};
+        st.rows.at(r * NACC + d) = 0.0;
+      }
+    }
+  }
+  __device__ static void flush(State &st, const PairArgs &a) {
+    const int ls = lsb(a);
+#pragma unroll
+    for (int r = 0; r < R; r++)
+#pragma unroll
+      for (int d = 0; d < NACC; d++) {
+        st.rows.at(r * NACC + d) += fx64::total96(st.acc[r][d], ls);
+        st.acc[r][d] = fx64::Acc96{0u, 0u, 0u};
+      }
+    st.units = 0;
+  }
+  __device__ static void total(const State &st, int r, double *out) {
+#pragma unroll
+    for (int d = 0; d < NACC; d++) out[d] = st.rows.at(r * NACC + d);
+  }
+  // whether a 16-byte chunk of the staged tile (one particle) is out of range
+  __device__ static bool chunk_wild(const unsigned char *chunk, const PairArgs &a) {
+    const double2 v = *(const double2 *)chunk;
+    const int half = half_exp(a);
+    return out_of_range(v.x, half) || out_of_range(v.y, half);
+  }
+  // the term |x| / s with its sign into the row and column sums
+  template <bool COL>
+  __device__ static void add(unsigned h, unsigned w2, unsigned w1, unsigned w0, fx64::Acc96 &row, fx64::Acc96 &col) {
+    const unsigned sg = (unsigned)((int)h >> 31);  // -v as ~v: one unit of the 96 bits below
+    w2 ^= sg;
+    w1 ^= sg;
+    w0 ^= sg;
+    fx64::add96(row, w2, w1, w0);
+    if (COL) fx64::add96(col, w2, w1, w0);
+  }
+  template <bool COL>
+  __device__ static void unit(State &st, const unsigned char *smb, const PairArgs &a, unsigned char *colraw) {
+    const double2 *sm = (const double2 *)smb;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int kc = 9 - half_exp(a);
+    const fx64::Soft eps = fx64::soft_of(a.epsd);
+    uint4 *colsm = (uint4 *)colraw + w * TJ * NACC;
+#pragma unroll 1
+    for (int j = 0; j < TJ; j++) {
+      const double2 o = sm[j];
+      fx64::Acc96 col[2] = {{0u, 0u, 0u}, {0u, 0u, 0u}};
+      unsigned h[R][2], yh[R][2], yl[R][2];
+      unsigned long long inv[R];
+      int k[R][2];
+      unsigned kor = 0u;
+#pragma unroll
+      for (int r = 0; r < R; r++) {
+        const double d[2] = {st.x[r] - o.x, st.y[r] - o.y};
+        int ex[2], es;
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+          h[r][c] = fx64::hi_word(d[c]);
+          ex[c] = (int)((h[r][c] >> 20) & 0x7ffu);
+          fx64::mantissa62(h[r][c], fx64::lo_word(d[c]), yh[r][c], yl[r][c]);
+        }
+        unsigned Mh, Ml;
+        fx64::square_sum<2>(yh[r], yl[r], ex, eps, Mh, Ml, es);
+        inv[r] = fx64::rcp_mantissa(Mh, Ml);
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+          k[r][c] = es + kc - ex[c];
+          kor |= (unsigned)k[r][c];
+        }
+      }
+      // one branch for the four rows: a component 2^-14 and less of the distance is rare
+      if (__builtin_expect(kor < 32u, 1)) {
+#pragma unroll
+        for (int r = 0; r < R; r++)
+#pragma unroll
+          for (int c = 0; c < 2; c++) {
+            unsigned w2, w1, w0;
+            fx64::mul_mantissa(yh[r][c], yl[r][c], inv[r], w2, w1, w0);
+            w0 = fx64::shf_r(w0, w1, k[r][c]);
+            w1 = fx64::shf_r(w1, w2, k[r][c]);
+            w2 >>= k[r][c];
+            add<COL>(h[r][c], w2, w1, w0, st.acc[r][c], col[c]);
+          }
+      } else {
+#pragma unroll
+        for (int r = 0; r < R; r++)
+#pragma unroll
+          for (int c = 0; c < 2; c++) {
+            unsigned w2, w1, w0;
+            fx64::mul_mantissa(yh[r][c], yl[r][c], inv[r], w2, w1, w0);
+            fx64::shift96_any(w2, w1, w0, k[r][c]);
+            // a zero term adds exactly zero (~0 would be -1 unit)
+            add<COL>((w2 | w1 | w0) == 0u ? 0u : h[r][c], w2, w1, w0, st.acc[r][c], col[c]);
+          }
+      }
+      if (COL) {
+        const uint4 sx = fx_warp_sum(col[0]), sy = fx_warp_sum(col[1]);
+        if (lane == 0) {
+          colsm[2 * j] = sx;
+          colsm[2 * j + 1] = sy;
+        }
+      }
+    }
+    if (++st.units == kFxFlush) flush(st, a);
+  }
+  // the unit in FP64: sums of its rows straight into the doubles, columns as doubles
+  template <bool COL>
+  __device__ static void unit_wild(State &st, const unsigned char *smb, const PairArgs &a, unsigned char *colraw,
+                                   int64_t i0, int64_t j0) {
+    typename Wild::State ws;
+#pragma unroll
+    for (int r = 0; r < R; r++) {
+      ws.x[r] = st.x[r];
+      ws.y[r] = st.y[r];
+#pragma unroll
+      for (int d = 0; d < NACC; d++) ws.accd[r][d] = st.rows.at(r * NACC + d);
+    }
+    if (COL) Wild::tile_sym(ws, smb, a, (double *)colraw);
+    else Wild::template tile<true>(ws, smb, a, i0, j0);
+#pragma unroll
+    for (int r = 0; r < R; r++)
+#pragma unroll
+      for (int d = 0; d < NACC; d++) st.rows.at(r * NACC + d) = ws.accd[r][d];
+  }
+  __device__ static double column(const unsigned char *colraw, int idx, bool wild, const PairArgs &a) {
+    if (!wild)
+      return fx_limb_total<NT / 32>((const uint4 *)colraw + idx, TJ * NACC) * fx64::pow2(lsb(a) + 11);
+    const double *c = (const double *)colraw;
+    double v = c[idx];
+#pragma unroll
+    for (int w = 1; w < NT / 32; w++) v += c[w * TJ * NACC + idx];
+    return v;
+  }
+};
+
+}  // namespace

@@ -45,6 +45,7 @@
 // kernel runs instead.
 #include <mutex>
 
+#include "pairs_fx.cuh"
 #include "pairs_impl.cuh"
 
 namespace {
@@ -60,11 +61,25 @@ struct SymArgs {
   double *chunks;    // [n_it][nc][TI][NACC] chunk sums of the column partials
 };
 
+// Policies with integer pair arithmetic (pairs_fx.cuh): their row sums partly in shared
+// memory, a unit's columns as integer limbs, and an FP64 form for units out of range.
+template <class P, class = void>
+struct IsFx : std::false_type {};
+template <class P>
+struct IsFx<P, std::void_t<decltype(P::FX)>> : std::true_type {};
+
 // CTAs of the pair kernel that cover part of row T: [cf, cl].
 __device__ __forceinline__ void sym_row_ctas(const PairArgs &a, const SymArgs &s, int64_t T, int64_t &cf,
                                              int64_t &cl) {
   cf = cta_of_unit(a.U, a.P, sym_rowstart(T, a.n_jt, s.m));
   cl = cta_of_unit(a.U, a.P, sym_rowstart(T + 1, a.n_jt, s.m) - 1);
+}
+
+// Shared-memory bytes of a unit's column sums.
+template <class Pol>
+constexpr int sym_col_bytes() {
+  if constexpr (IsFx<Pol>::value) return Pol::COL_BYTES;
+  else return Pol::THREADS / 32 * Pol::TJ * Pol::NACC * (int)sizeof(typename Pol::ColT);
 }
 
 // Pair phase: every unit's block, row partials per CTA segment, column partials per unit.
@@ -80,7 +95,9 @@ __global__ void __launch_bounds__(Pol::THREADS, Pol::MINB) sym_pairs_kernel(Pair
   using ColT = typename Pol::ColT;
   constexpr bool DIAG_SYM = HasDiagSym<Pol>::value;
   __shared__ __align__(16) unsigned char sbuf[2][TILE_BYTES];
-  __shared__ __align__(16) unsigned char colraw[NW * TJ * NACC * sizeof(ColT)];
+  constexpr bool FX = IsFx<Pol>::value;
+  __shared__ __align__(16) unsigned char colraw[sym_col_bytes<Pol>()];
+  __shared__ double rowsm[FX ? THR * Pol::R * NACC : 1];
   ColT *colsm = (ColT *)colraw;
   __shared__ unsigned s_vc;
   const int m = s.m;
@@ -89,6 +106,10 @@ __global__ void __launch_bounds__(Pol::THREADS, Pol::MINB) sym_pairs_kernel(Pair
     const unsigned char *src = mir + jt * (int64_t)TILE_BYTES;
     for (int ch = threadIdx.x; ch < CHUNKS; ch += THR) cp_async16(&sbuf[buf][ch * 16], src + ch * 16);
     cp_async_commit();
+  };
+  auto load_rows = [&](typename Pol::State &st, int64_t i0) {
+    if constexpr (FX) Pol::load(st, a.mirror_in, i0, a, rowsm);
+    else Pol::load(st, a.mirror_in, i0);
   };
 
   for (;;) {
@@ -103,7 +124,7 @@ __global__ void __launch_bounds__(Pol::THREADS, Pol::MINB) sym_pairs_kernel(Pair
     int64_t jt = (int64_t)m * it + (u0 - sym_rowstart(it, a.n_jt, m));
     bool row_from_start = (jt == (int64_t)m * it);
     int64_t i0 = it * TI;
-    Pol::load(st, a.mirror_in, i0);
+    load_rows(st, i0);
     prefetch(0, jt);
 
     for (int64_t u = u0; u < u1; u++) {
@@ -116,9 +137,20 @@ __global__ void __launch_bounds__(Pol::THREADS, Pol::MINB) sym_pairs_kernel(Pair
       } else {
         cp_async_wait<0>();
       }
-      __syncthreads();
+      bool wild = false;  // FX: a coordinate of the unit lies out of the fixed-point range
+      if constexpr (FX) {
+        wild = st.wild;
+        for (int ch = threadIdx.x; ch < CHUNKS; ch += THR) wild = wild || Pol::chunk_wild(&sbuf[buf][ch * 16], a);
+        wild = __syncthreads_or(wild);
+      } else {
+        __syncthreads();
+      }
       const bool diag = jt < (int64_t)m * (it + 1);
-      if (!diag) Pol::tile_sym(st, sbuf[buf], a, colsm);
+      if constexpr (FX) {
+        if (!wild) diag ? Pol::template unit<false>(st, sbuf[buf], a, colraw) : Pol::template unit<true>(st, sbuf[buf], a, colraw);
+        else if (diag) Pol::template unit_wild<false>(st, sbuf[buf], a, colraw, i0, jt * TJ);
+        else Pol::template unit_wild<true>(st, sbuf[buf], a, colraw, i0, jt * TJ);
+      } else if (!diag) Pol::tile_sym(st, sbuf[buf], a, colsm);
       else if constexpr (DIAG_SYM) Pol::tile_diag(st, sbuf[buf], a, colsm, (int)(jt - (int64_t)m * it));
       else Pol::template tile<true>(st, sbuf[buf], a, i0, jt * TJ);
       __syncthreads();
@@ -127,14 +159,19 @@ __global__ void __launch_bounds__(Pol::THREADS, Pol::MINB) sym_pairs_kernel(Pair
         // rewritten only after the next unit's first barrier)
         ColT *dst = (ColT *)s.colslot + u * (int64_t)(TJ * NACC);
         for (int idx = threadIdx.x; idx < TJ * NACC; idx += THR) {
-          ColT v = colsm[idx];
+          if constexpr (FX) {
+            dst[idx] = Pol::column(colraw, idx, wild, a);
+          } else {
+            ColT v = colsm[idx];
   #pragma unroll
-          for (int w = 1; w < NW; w++) v += colsm[w * TJ * NACC + idx];
-          dst[idx] = v;
+            for (int w = 1; w < NW; w++) v += colsm[w * TJ * NACC + idx];
+            dst[idx] = v;
+          }
         }
       }
       if (row_end || u + 1 == u1) {
         // this CTA's part of row it
+        if constexpr (FX) Pol::flush(st, a);
         double *sp = (row_end && row_from_start)
                          ? s.rowfull + it * NACC * TI
                          : a.slots + ((cta * 2 + (it == first_row ? 0 : 1)) * NACC) * TI;
@@ -151,7 +188,7 @@ __global__ void __launch_bounds__(Pol::THREADS, Pol::MINB) sym_pairs_kernel(Pair
           it++;
           row_from_start = true;
           i0 = it * TI;
-          Pol::load(st, a.mirror_in, i0);
+          load_rows(st, i0);
         }
       }
       jt = next_jt;
@@ -330,6 +367,7 @@ int sym_dispatch(md_ctx *c, PairArgs a) {
   } else if constexpr (!MIXED) {
     // 4 rows per thread: the column butterflies' FP64 adds are shared by twice the pairs
     if constexpr (MODEL == MD_RING) return launch_sym<RingF64<4, 128, MODE>, MODEL, false, MODE>(c, a);
+    else if (c->eps >= kFxEpsMin) return launch_sym<GravFx<4, 128, MODE>, MODEL, false, MODE>(c, a);
     else return launch_sym<GravF64<4, 128, MODE>, MODEL, false, MODE>(c, a);
   } else if constexpr (MODEL == MD_RING) {
     return launch_sym<RingTC<4, 256, MODE>, MODEL, true, MODE>(c, a);
