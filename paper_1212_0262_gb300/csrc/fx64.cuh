@@ -220,6 +220,140 @@ FX_FN void add96(Acc96 &a, u32 w2, u32 w1, u32 w0) {
   a.w2 = a.w2 + w2 + (u32)(t >> 32);
 #endif
 }
+
+// ---- sines and cosines (|x| <= 1) as fixed-point numbers ----
+
+typedef int64_t i64;
+FX_FN i64 mul_wide_s(int a, int b, i64 c) { return (i64)a * b + c; }
+
+// x 2^62 rounded to an integer, |x| <= 1, as h 2^32 + l with signed l
+struct Limbs {
+  int h, l;
+};
+FX_FN Limbs limbs_of(double x) {
+  const double y = x * 0x1p62;
+#ifdef __CUDA_ARCH__
+  const i64 v = __double2ll_rn(y);
+#else
+  const i64 v = (i64)y;  // exact from 2^53 on; below, truncation by less than one unit
+#endif
+  return Limbs{(int)((u64)(v + 0x80000000ll) >> 32), (int)(u32)v};
+}
+
+// (a c + b d) 2^60, the low x low products left out (error below 1.5 units)
+FX_FN i64 dot2(const Limbs &a, const Limbs &b, const Limbs &c, const Limbs &d) {
+  const i64 mid = mul_wide_s(a.h, c.l, mul_wide_s(a.l, c.h, mul_wide_s(b.h, d.l, mul_wide_s(b.l, d.h, 0))));
+  return mul_wide_s(a.h, c.h, mul_wide_s(b.h, d.h, mid >> 32));
+}
+
+// A number as a 96-bit integer w 2^-92
+struct Fix92 {
+  u32 w2, w1, w0;
+};
+FX_FN Fix92 fix92_of(double x) {  // 2^-27 <= x < 8
+  const int e = (int)(hi_word(x) >> 20) - 1023, sh = e + 40;  // x 2^92 = mant 2^(e + 40)
+  const u64 m = ((u64)((hi_word(x) & 0x000fffffu) | 0x00100000u) << 32) | lo_word(x);
+  const u64 lo = sh < 32 ? (m << sh) : (m << (sh - 32));
+  const u32 top = (u32)(sh == 0 ? 0 : m >> (64 - (sh < 32 ? sh : sh - 32)));
+  if (sh < 32) return Fix92{top, (u32)(lo >> 32), (u32)lo};
+  return Fix92{(u32)(lo >> 32), (u32)lo, 0u};
+}
+
+// x^2 + he for x 2^60 (|x| <= 1): ms 2^(3 - z) with ms = Mh:Ml 2^-63 in [1/4, 1) and z odd.
+// he in [2^-27, 4].  |x| as ~x where negative: one unit of 2^-60.
+FX_FN void square_plus(i64 x, const Fix92 &he, u32 &Mh, u32 &Ml, int &z) {
+  const u32 sg = (u32)((int)(u32)((u64)x >> 32) >> 31);
+  const u32 a1 = (u32)((u64)x >> 32) ^ sg, a0 = (u32)x ^ sg;
+  const u32 xh = shf_l(a0, a1, 2), xl = a0 << 2;
+  const u64 mid = mul_wide(xh, xl, (u64)(u32)(mul_wide(xl, xl, 0) >> 33));  // half of the cross terms
+  const u64 H = mul_wide(xh, xh, mid >> 31);
+  Acc96 d{he.w0, he.w1, he.w2};
+  add96(d, (u32)(H >> 32), (u32)H, (u32)mid << 1);
+  z = 156 - (int)(as_uint(to_float_rz(d.w2)) >> 23);  // leading zeros - 2
+  z |= 1;
+  Mh = shf_l(d.w1, d.w2, z);
+  Ml = shf_l(d.w0, d.w1, z);
+}
+
+// Seed of ms^(-1/2) 2^30 in [2^30, 2^31) for ms = m 2^-31, 2^29 <= m < 2^31, within 2^-21.
+FX_FN u32 seed_rsqrt(u32 m, float bias) {
+  const float f = to_float_rz(2u * m);  // ms 2^32
+#ifdef __CUDA_ARCH__
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(f));
+  (void)bias;
+#else
+  float r = (float)(1.0 / __builtin_sqrt((double)f)) * bias;
+#endif
+  r = r > 0x1p-16f ? r : 0x1p-16f;
+  r = r < 0x1.fffffep-16f ? r : 0x1.fffffep-16f;
+  return as_uint(r) * 128u + 0x80000000u;
+}
+
+// 2^60 ms^(-1/2), an integer in (2^60, 2^61]: y the seed, n = ms y^2 - 1 to 2^-58, then
+// y (1 - n/2 + 3/8 n^2): relative error below 2^-57.
+FX_FN u64 rsqrt_mantissa(u32 Mh, u32 Ml, float bias = 1.0f) {
+  const u32 Q = seed_rsqrt(Mh, bias);
+  const u64 q2 = mul_wide(Q, Q, 0);  // y^2 2^60
+  const u32 qh = (u32)(q2 >> 32), ql = (u32)q2;
+  const u64 nm = mul_wide(Ml, qh, mul_wide(Mh, ql, 0));
+  const u64 n = mul_wide(Mh, qh, (nm >> 32) | 0xF800000000000000ull);  // n 2^59
+  const int nh = (int)(u32)(n >> 8);
+  const u32 nn = (u32)((u64)mul_wide_s(nh, nh, 0) >> 32);              // n^2 2^70
+  const u64 c = (u64)((nn * 3u) >> 14) - (u64)((i64)n >> 1);           // 2^59 (3/8 n^2 - n/2)
+  const u64 C = (c << 3) + 0x4000000000000000ull;
+  return mul_wide(Q, (u32)(C >> 32), mul_wide(Q, (u32)C, 0) >> 32);
+}
+
+// Mh:Ml 2^-63 in [1, 2) times 2^e as ms 2^(2 g), ms = Mh:Ml 2^-63 in [1/4, 1)
+FX_FN int even_exponent(u32 &Mh, u32 &Ml, int e) {
+  const int sh = 2 - (e & 1);
+  Ml = shf_r(Ml, Mh, sh);
+  Mh >>= sh;
+  return (e + sh) >> 1;
+}
+
+// a b 2^-63 for a, b in [2^62, 2^63), renormalised into that range; the power of two goes
+// to e.  Relative error below 2^-60.
+FX_FN u64 mul_renorm63(u64 a, u64 b, int &e) {
+  const u32 ah = (u32)(a >> 32), al = (u32)a, bh = (u32)(b >> 32), bl = (u32)b;
+  const u64 mid = mul_wide(al, bh, mul_wide(ah, bl, 0));
+  u64 P = mul_wide(ah, bh, mid >> 32);  // [2^60, 2^62)
+  const int up = (P >> 61) ? 1 : 2;
+  e -= up;
+  P = (P << up) | ((u32)mid >> (32 - up));
+  return P;
+}
+
+// 2^58 ms^(-3/2), an integer in [2^58, 2^61): y the seed, n = ms y^2 - 1 to 2^-58, then
+// y^3 (1 - 3/2 n + 15/8 n^2): relative error below 2^-56.
+FX_FN u64 rsqrt3_mantissa(u32 Mh, u32 Ml, float bias = 1.0f) {
+  const u32 Q = seed_rsqrt(Mh, bias);
+  const u64 q2 = mul_wide(Q, Q, 0);  // y^2 2^60
+  const u32 qh = (u32)(q2 >> 32), ql = (u32)q2;
+  const u64 nm = mul_wide(Ml, qh, mul_wide(Mh, ql, 0));
+  const u64 n = mul_wide(Mh, qh, (nm >> 32) | 0xF800000000000000ull);  // n 2^59
+  const u64 q4 = q2 << 2;
+  const u64 Y = mul_wide((u32)(q4 >> 32), Q, mul_wide((u32)q4, Q, 0) >> 32);  // y^3 2^60
+  const int nh = (int)(u32)(n >> 8);
+  const u32 nn = (u32)((u64)mul_wide_s(nh, nh, 0) >> 32);                     // n^2 2^70
+  const u64 c = (u64)(((nn >> 4) * 15u) >> 10) - n - (u64)((i64)n >> 1);             // 2^59 (15/8 n^2 - 3/2 n)
+  const u64 C = (c << 3) + 0x4000000000000000ull;                             // 2^62 (1 + ...)
+  const u32 Yh = (u32)(Y >> 32), Yl = (u32)Y, Ch = (u32)(C >> 32), Cl = (u32)C;
+  return mul_wide(Yh, Ch, mul_wide(Yl, Ch, mul_wide(Yh, Cl, 0)) >> 32);
+}
+
+// |x| W as (w2 w1 w0) 2^-86 for x 2^60 and W 2^58 < 2^61; the sign of x in sg (0 or ~0)
+FX_FN void mul_fixed(i64 x, u64 W, u32 &sg, u32 &w2, u32 &w1, u32 &w0) {
+  sg = (u32)((int)(u32)((u64)x >> 32) >> 31);
+  const u32 xh = (u32)((u64)x >> 32) ^ sg, xl = (u32)x ^ sg, Wh = (u32)(W >> 32), Wl = (u32)W;
+  const u64 mid = mul_wide(xl, Wh, mul_wide(xh, Wl, mul_wide(xl, Wl, 0) >> 32));
+  const u64 P = mul_wide(xh, Wh, mid >> 32);
+  w2 = (u32)(P >> 32);
+  w1 = (u32)P;
+  w0 = (u32)mid;
+}
+
 // (w2 w1 w0) >> k for any k >= 0 (a non-negative value)
 FX_FN void shift96_any(u32 &w2, u32 &w1, u32 &w0, int k) {
   if (k >= 64) {

@@ -16,7 +16,6 @@
 namespace {
 
 constexpr int kFxFlush = 16;        // units between moves of the row sums into doubles
-constexpr double kFxEpsMin = 0x1p-28;  // below: the FP64 policies (the unit 2^lsb would grow)
 
 // Row sums of a thread in shared memory: [value][thread]
 template <int V>
@@ -53,6 +52,51 @@ __device__ __forceinline__ double fx_limb_total(const uint4 *s, int stride) {
   return ((double)t2 * 134217728.0 + (double)t1) * 134217728.0 + (double)t0;
 }
 
+// Rows, flushes and columns shared by the policies: State has acc[R][NACC] and rows.
+template <class State, int R, int NACC>
+__device__ __forceinline__ void fx_flush(State &st, int lsb) {
+#pragma unroll
+  for (int r = 0; r < R; r++)
+#pragma unroll
+    for (int d = 0; d < NACC; d++) {
+      st.rows.at(r * NACC + d) += fx64::total96(st.acc[r][d], lsb);
+      st.acc[r][d] = fx64::Acc96{0u, 0u, 0u};
+    }
+  st.units = 0;
+}
+template <class State, int R, int NACC>
+__device__ __forceinline__ void fx_clear(State &st, double *rowsm) {
+  st.rows.p = rowsm + threadIdx.x;
+  st.units = 0;
+#pragma unroll
+  for (int r = 0; r < R; r++)
+#pragma unroll
+    for (int d = 0; d < NACC; d++) {
+      st.acc[r][d] = fx64::Acc96{0u, 0u, 0u};
+      st.rows.at(r * NACC + d) = 0.0;
+    }
+}
+// column idx of a finished unit: the warps' integer limbs, or (FP64 tile) their doubles
+template <int TJ, int NACC>
+__device__ __forceinline__ double fx_column(const unsigned char *colraw, int idx, bool wild, int lsb) {
+  if (!wild) return fx_limb_total<NT / 32>((const uint4 *)colraw + idx, TJ * NACC) * fx64::pow2(lsb + 11);
+  const double *c = (const double *)colraw;
+  double v = c[idx];
+#pragma unroll
+  for (int w = 1; w < NT / 32; w++) v += c[w * TJ * NACC + idx];
+  return v;
+}
+// -v as ~v (one unit of the 96 bits below): the term w with sign mask sg into a row and a column
+template <bool COL>
+__device__ __forceinline__ void fx_add(unsigned sg, unsigned w2, unsigned w1, unsigned w0, fx64::Acc96 &row,
+                                       fx64::Acc96 &col) {
+  w2 ^= sg;
+  w1 ^= sg;
+  w0 ^= sg;
+  fx64::add96(row, w2, w1, w0);
+  if (COL) fx64::add96(col, w2, w1, w0);
+}
+
 // ------------------------------------------------------------ forward 2D
 // Per pair dx and dy in FP64 (2 operations instead of 14); the squared distance, its
 // reciprocal, the products with dx and dy and the four sums are integers: about 147
@@ -70,6 +114,8 @@ struct GravFx {
   static constexpr int NR = R;
   static constexpr int FMT = 0;
   static constexpr int COL_BYTES = (NT / 32) * TJ * NACC * (int)sizeof(uint4);
+  // eps of the fixed-point form (below, the unit 2^lsb of the sums would grow too large)
+  static bool applies(double eps) { return eps >= 0x1p-28; }
   __device__ static int row_of(int r) { return r * NT + (int)threadIdx.x; }
   struct State {
     double x[R], y[R];
@@ -89,54 +135,30 @@ struct GravFx {
   __device__ static void load(State &st, const void *mirror, int64_t i0, const PairArgs &a, double *rowsm) {
     const int half = half_exp(a);
     st.wild = false;
-    st.units = 0;
-    st.rows.p = rowsm + threadIdx.x;
+    fx_clear<State, R, NACC>(st, rowsm);
 #pragma unroll
     for (int r = 0; r < R; r++) {
       const double2 m = *(const double2 *)((const double *)mirror + (i0 + row_of(r)) * 2);
       st.x[r] = m.x;
       st.y[r] = m.y;
       st.wild = st.wild || out_of_range(m.x, half) || out_of_range(m.y, half);
-#pragma unroll
-      for (int d = 0; d < NACC; d++) {
-        st.acc[r][d] = fx64::Acc96{0u, 0u, 0u};
-        st.rows.at(r * NACC + d) = 0.0;
-      }
     }
   }
-  __device__ static void flush(State &st, const PairArgs &a) {
-    const int ls = lsb(a);
-#pragma unroll
-    for (int r = 0; r < R; r++)
-#pragma unroll
-      for (int d = 0; d < NACC; d++) {
-        st.rows.at(r * NACC + d) += fx64::total96(st.acc[r][d], ls);
-        st.acc[r][d] = fx64::Acc96{0u, 0u, 0u};
-      }
-    st.units = 0;
-  }
+  __device__ static void flush(State &st, const PairArgs &a) { fx_flush<State, R, NACC>(st, lsb(a)); }
   __device__ static void total(const State &st, int r, double *out) {
 #pragma unroll
     for (int d = 0; d < NACC; d++) out[d] = st.rows.at(r * NACC + d);
   }
-  // whether a 16-byte chunk of the staged tile (one particle) is out of range
-  __device__ static bool chunk_wild(const unsigned char *chunk, const PairArgs &a) {
-    const double2 v = *(const double2 *)chunk;
+  // a 16-byte chunk of the tile (one particle): whether it is out of range
+  static constexpr int STAGE_BYTES = 16;  // nothing is staged
+  __device__ static bool stage(const unsigned char *tile, int ch, unsigned char *, const PairArgs &a) {
+    const double2 v = ((const double2 *)tile)[ch];
     const int half = half_exp(a);
     return out_of_range(v.x, half) || out_of_range(v.y, half);
   }
-  // the term |x| / s with its sign into the row and column sums
   template <bool COL>
-  __device__ static void add(unsigned h, unsigned w2, unsigned w1, unsigned w0, fx64::Acc96 &row, fx64::Acc96 &col) {
-    const unsigned sg = (unsigned)((int)h >> 31);  // -v as ~v: one unit of the 96 bits below
-    w2 ^= sg;
-    w1 ^= sg;
-    w0 ^= sg;
-    fx64::add96(row, w2, w1, w0);
-    if (COL) fx64::add96(col, w2, w1, w0);
-  }
-  template <bool COL>
-  __device__ static void unit(State &st, const unsigned char *smb, const PairArgs &a, unsigned char *colraw) {
+  __device__ static void unit(State &st, const unsigned char *smb, const unsigned char *, const PairArgs &a,
+                              unsigned char *colraw, int64_t, int64_t) {
     const double2 *sm = (const double2 *)smb;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int kc = 9 - half_exp(a);
@@ -180,7 +202,7 @@ struct GravFx {
             w0 = fx64::shf_r(w0, w1, k[r][c]);
             w1 = fx64::shf_r(w1, w2, k[r][c]);
             w2 >>= k[r][c];
-            add<COL>(h[r][c], w2, w1, w0, st.acc[r][c], col[c]);
+            fx_add<COL>((unsigned)((int)h[r][c] >> 31), w2, w1, w0, st.acc[r][c], col[c]);
           }
       } else {
 #pragma unroll
@@ -191,7 +213,7 @@ struct GravFx {
             fx64::mul_mantissa(yh[r][c], yl[r][c], inv[r], w2, w1, w0);
             fx64::shift96_any(w2, w1, w0, k[r][c]);
             // a zero term adds exactly zero (~0 would be -1 unit)
-            add<COL>((w2 | w1 | w0) == 0u ? 0u : h[r][c], w2, w1, w0, st.acc[r][c], col[c]);
+            fx_add<COL>((w2 | w1 | w0) == 0u ? 0u : (unsigned)((int)h[r][c] >> 31), w2, w1, w0, st.acc[r][c], col[c]);
           }
       }
       if (COL) {
@@ -224,13 +246,119 @@ struct GravFx {
       for (int d = 0; d < NACC; d++) st.rows.at(r * NACC + d) = ws.accd[r][d];
   }
   __device__ static double column(const unsigned char *colraw, int idx, bool wild, const PairArgs &a) {
-    if (!wild)
-      return fx_limb_total<NT / 32>((const uint4 *)colraw + idx, TJ * NACC) * fx64::pow2(lsb(a) + 11);
-    const double *c = (const double *)colraw;
-    double v = c[idx];
+    return fx_column<TJ, NACC>(colraw, idx, wild, lsb(a));
+  }
+};
+
+// ------------------------------------------------------------ forward Ring
+// Sines and cosines are numbers of at most 1, so the whole pair term is fixed-point: S and
+// sin(d/2) as 62-bit dot products, sin^2 + eps/2 in 96 bits, its power -3/2 from an FP32 seed
+// and one third-order step, no FP64 operation (15.5 in RingF64).  The tile's records are
+// turned into integers once per unit, by the thread that loaded them.  137 instructions per
+// pair; one force at N = 49,152: 36.3 ms with RingF64, 7.47 here (bound by the integer pipe,
+// 51%, and by dependent instructions at 4 warps per scheduler).
+template <int R_, int TJ_, int MODE>
+struct RingFx {
+  static constexpr bool FX = true;
+  static constexpr int THREADS = NT, MINB = 4;
+  using ColT = double;
+  using Wild = RingF64<R_, TJ_, MODE>;
+  static constexpr int R = R_, TJ = TJ_, NACC = 1, JB = RecordBytes<MD_RING, false, false>::value;
+  static constexpr bool MASK = true;
+  static constexpr int NR = R;
+  static constexpr int FMT = 0;
+  static constexpr int COL_BYTES = (NT / 32) * TJ * NACC * (int)sizeof(uint4);
+  static constexpr int STAGE_BYTES = TJ * JB;
+  // eps of the fixed-point form: shifts of 0 .. 31 bits, sums below 2^95
+  static bool applies(double eps) { return eps >= 0x1p-17 && eps <= 4.0; }
+  __device__ static int row_of(int r) { return r * NT + (int)threadIdx.x; }
+  struct State {
+    fx64::Limbs s[R], c[R], a[R], g[R];
+    fx64::Acc96 acc[R][NACC];
+    FxRowSums<R * NACC> rows;
+    int units;
+    bool wild;
+  };
+  // |term| <= 0.77 / he <= 2^T for he = eps/2; T also makes the shift of the closest pairs,
+  // whose power -3/2 is the largest, non-negative
+  __device__ static int top(const PairArgs &a) {
+    const int h = (int)(fx64::hi_word(a.epsd) >> 20) - 1023;
+    const int t = (-8 - 3 * h) >> 1;  // ceil(-4.5 - 1.5 h)
+    return -h > t ? -h : t;
+  }
+  __device__ static int lsb(const PairArgs &a) { return top(a) - 83; }
+  __device__ static bool out_of_range(double v) { return (fx64::hi_word(v) & 0x7fffffffu) > 0x3ff00000u; }
+  __device__ static void load(State &st, const void *mirror, int64_t i0, const PairArgs &a, double *rowsm) {
+    st.wild = false;
+    fx_clear<State, R, NACC>(st, rowsm);
 #pragma unroll
-    for (int w = 1; w < NT / 32; w++) v += c[w * TJ * NACC + idx];
-    return v;
+    for (int r = 0; r < R; r++) {
+      const double *m = (const double *)mirror + (i0 + row_of(r)) * 4;
+      st.wild = st.wild || out_of_range(m[0]) || out_of_range(m[1]) || out_of_range(m[2]) || out_of_range(m[3]);
+      st.s[r] = fx64::limbs_of(m[0]);
+      st.c[r] = fx64::limbs_of(m[1]);
+      st.a[r] = fx64::limbs_of(m[2]);
+      st.g[r] = fx64::limbs_of(m[3]);
+    }
+  }
+  __device__ static void flush(State &st, const PairArgs &a) { fx_flush<State, R, NACC>(st, lsb(a)); }
+  __device__ static void total(const State &st, int r, double *out) { out[0] = st.rows.at(r); }
+  // half a record, (s, c) or (a, g): as (-s, c) or (-a, g) limbs
+  __device__ static bool stage(const unsigned char *tile, int ch, unsigned char *out, const PairArgs &) {
+    const double2 v = ((const double2 *)tile)[ch];
+    const fx64::Limbs x = fx64::limbs_of(-v.x), y = fx64::limbs_of(v.y);
+    ((int4 *)out)[ch] = make_int4(x.h, x.l, y.h, y.l);
+    return out_of_range(v.x) || out_of_range(v.y);
+  }
+  template <bool COL>
+  __device__ static void unit(State &st, const unsigned char *, const unsigned char *staged, const PairArgs &a,
+                              unsigned char *colraw, int64_t i0, int64_t j0) {
+    const int4 *sm = (const int4 *)staged;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const fx64::Fix92 he = fx64::fix92_of(a.epsd);
+    const int kc = 3 + top(a);
+    uint4 *colsm = (uint4 *)colraw + w * TJ * NACC;
+#pragma unroll 1
+    for (int j = 0; j < TJ; j++) {
+      const int4 p = sm[2 * j], q = sm[2 * j + 1];
+      const fx64::Limbs ns{p.x, p.y}, c{p.z, p.w}, na{q.x, q.y}, g{q.z, q.w};
+      fx64::Acc96 col{0u, 0u, 0u};
+#pragma unroll
+      for (int r = 0; r < R; r++) {
+        const long long S = fx64::dot2(st.s[r], st.c[r], c, ns);     // sin(theta_i - theta_j) 2^60
+        const long long sh = fx64::dot2(st.a[r], st.g[r], g, na);    // sin((theta_i - theta_j)/2) 2^60
+        unsigned Mh, Ml, sg, w2, w1, w0;
+        int z;
+        fx64::square_plus(sh, he, Mh, Ml, z);
+        fx64::mul_fixed(S, fx64::rsqrt3_mantissa(Mh, Ml), sg, w2, w1, w0);
+        const int k = kc - 3 * ((z - 3) >> 1);
+        w0 = fx64::shf_r(w0, w1, k);
+        w1 = fx64::shf_r(w1, w2, k);
+        w2 >>= k;
+        if (!COL && i0 + row_of(r) == j0 + j) w2 = w1 = w0 = sg = 0u;
+        fx_add<COL>(sg, w2, w1, w0, st.acc[r][0], col);
+      }
+      if (COL) {
+        const uint4 sum = fx_warp_sum(col);
+        if (lane == 0) colsm[j] = sum;
+      }
+    }
+    if (++st.units == kFxFlush) flush(st, a);
+  }
+  template <bool COL>
+  __device__ static void unit_wild(State &st, const unsigned char *smb, const PairArgs &a, unsigned char *colraw,
+                                   int64_t i0, int64_t j0) {
+    typename Wild::State ws;
+    Wild::load(ws, a.mirror_in, i0);
+#pragma unroll
+    for (int r = 0; r < R; r++) ws.accd[r][0] = st.rows.at(r);
+    if (COL) Wild::tile_sym(ws, smb, a, (double *)colraw);
+    else Wild::template tile<true>(ws, smb, a, i0, j0);
+#pragma unroll
+    for (int r = 0; r < R; r++) st.rows.at(r) = ws.accd[r][0];
+  }
+  __device__ static double column(const unsigned char *colraw, int idx, bool wild, const PairArgs &a) {
+    return fx_column<TJ, NACC>(colraw, idx, wild, lsb(a));
   }
 };
 

@@ -82,6 +82,13 @@ constexpr int sym_col_bytes() {
   else return Pol::THREADS / 32 * Pol::TJ * Pol::NACC * (int)sizeof(typename Pol::ColT);
 }
 
+// Bytes of a tile turned into integers (FX).
+template <class Pol>
+constexpr int sym_stage_bytes() {
+  if constexpr (IsFx<Pol>::value) return Pol::STAGE_BYTES;
+  else return 16;
+}
+
 // Pair phase: every unit's block, row partials per CTA segment, column partials per unit.
 template <class Pol>
 __global__ void __launch_bounds__(Pol::THREADS, Pol::MINB) sym_pairs_kernel(PairArgs a, SymArgs s) {
@@ -98,6 +105,7 @@ __global__ void __launch_bounds__(Pol::THREADS, Pol::MINB) sym_pairs_kernel(Pair
   constexpr bool FX = IsFx<Pol>::value;
   __shared__ __align__(16) unsigned char colraw[sym_col_bytes<Pol>()];
   __shared__ double rowsm[FX ? THR * Pol::R * NACC : 1];
+  __shared__ __align__(16) unsigned char staged[sym_stage_bytes<Pol>()];
   ColT *colsm = (ColT *)colraw;
   __shared__ unsigned s_vc;
   const int m = s.m;
@@ -140,14 +148,15 @@ __global__ void __launch_bounds__(Pol::THREADS, Pol::MINB) sym_pairs_kernel(Pair
       bool wild = false;  // FX: a coordinate of the unit lies out of the fixed-point range
       if constexpr (FX) {
         wild = st.wild;
-        for (int ch = threadIdx.x; ch < CHUNKS; ch += THR) wild = wild || Pol::chunk_wild(&sbuf[buf][ch * 16], a);
+        for (int ch = threadIdx.x; ch < CHUNKS; ch += THR) wild |= Pol::stage(sbuf[buf], ch, staged, a);
         wild = __syncthreads_or(wild);
       } else {
         __syncthreads();
       }
       const bool diag = jt < (int64_t)m * (it + 1);
       if constexpr (FX) {
-        if (!wild) diag ? Pol::template unit<false>(st, sbuf[buf], a, colraw) : Pol::template unit<true>(st, sbuf[buf], a, colraw);
+        if (!wild && diag) Pol::template unit<false>(st, sbuf[buf], staged, a, colraw, i0, jt * TJ);
+        else if (!wild) Pol::template unit<true>(st, sbuf[buf], staged, a, colraw, i0, jt * TJ);
         else if (diag) Pol::template unit_wild<false>(st, sbuf[buf], a, colraw, i0, jt * TJ);
         else Pol::template unit_wild<true>(st, sbuf[buf], a, colraw, i0, jt * TJ);
       } else if (!diag) Pol::tile_sym(st, sbuf[buf], a, colsm);
@@ -366,9 +375,13 @@ int sym_dispatch(md_ctx *c, PairArgs a) {
     else return launch_sym<SheetF64<4, 128, MODE>, MODEL, false, MODE>(c, a);
   } else if constexpr (!MIXED) {
     // 4 rows per thread: the column butterflies' FP64 adds are shared by twice the pairs
-    if constexpr (MODEL == MD_RING) return launch_sym<RingF64<4, 128, MODE>, MODEL, false, MODE>(c, a);
-    else if (c->eps >= kFxEpsMin) return launch_sym<GravFx<4, 128, MODE>, MODEL, false, MODE>(c, a);
-    else return launch_sym<GravF64<4, 128, MODE>, MODEL, false, MODE>(c, a);
+    if constexpr (MODEL == MD_RING) {
+      if (RingFx<4, 128, MODE>::applies(c->eps)) return launch_sym<RingFx<4, 128, MODE>, MODEL, false, MODE>(c, a);
+      return launch_sym<RingF64<4, 128, MODE>, MODEL, false, MODE>(c, a);
+    } else {
+      if (GravFx<4, 128, MODE>::applies(c->eps)) return launch_sym<GravFx<4, 128, MODE>, MODEL, false, MODE>(c, a);
+      return launch_sym<GravF64<4, 128, MODE>, MODEL, false, MODE>(c, a);
+    }
   } else if constexpr (MODEL == MD_RING) {
     return launch_sym<RingTC<4, 256, MODE>, MODEL, true, MODE>(c, a);
   } else {

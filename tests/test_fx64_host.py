@@ -30,6 +30,16 @@ template <int D> static void quotient(const double *x, double eps, float bias, u
 extern "C" {
 void quotient2(const double *x, double eps, float bias, u32 *out) { quotient<2>(x, eps, bias, out); }
 void quotient3(const double *x, double eps, float bias, u32 *out) { quotient<3>(x, eps, bias, out); }
+void ring_term(double si, double ci, double sj, double cj, double he, float bias, i64 *S, u32 *out) {
+  const i64 s = dot2(limbs_of(si), limbs_of(ci), limbs_of(cj), limbs_of(-sj));
+  u32 Mh, Ml; int z;
+  square_plus(s, fix92_of(he), Mh, Ml, z);
+  const u64 W = rsqrt3_mantissa(Mh, Ml, bias), V = rsqrt_mantissa(Mh, Ml, bias);
+  *S = s; out[0] = Mh; out[1] = Ml; out[2] = (u32)z;
+  mul_fixed(s, W, out[3], out[4], out[5], out[6]);
+  out[7] = (u32)(W >> 32); out[8] = (u32)W; out[9] = (u32)(V >> 32); out[10] = (u32)V;
+}
+u64 product(u64 a, u64 b, int *e) { return mul_renorm63(a, b, *e); }
 double total(const u32 *w, int n, int lsb) { Acc96 a{0, 0, 0}; for (int i = 0; i < n; i++) add96(a, w[3 * i], w[3 * i + 1], w[3 * i + 2]); return total96(a, lsb); }
 void shift(u32 *w, int k) { shift96_any(w[0], w[1], w[2], k); }
 }
@@ -50,6 +60,9 @@ def lib(tmp_path_factory):
         f.argtypes = [ctypes.c_void_p, ctypes.c_double, ctypes.c_float, ctypes.c_void_p]
     so.total.restype = ctypes.c_double
     so.total.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_int]
+    so.ring_term.argtypes = [ctypes.c_double] * 5 + [ctypes.c_float, ctypes.c_void_p, ctypes.c_void_p]
+    so.product.restype = ctypes.c_uint64
+    so.product.argtypes = [ctypes.c_uint64, ctypes.c_uint64, ctypes.c_void_p]
     return so
 
 
@@ -80,6 +93,49 @@ def test_quotients_are_exact_to_better_than_a_double(lib, dim):
             ex = (int(x[:1].view(np.uint64)[0]) >> 52) & 0x7FF
             t = Fraction((w2 << 64) | (w1 << 32) | w0) * _pow2(-91 + ex - es)
             assert w2 < 1 << 28 and abs(t * s / abs(Fraction(float(x[0]))) - 1) < _pow2(-54)
+
+
+def test_ring_terms(lib):
+    """S and sin(d/2) within 2^-59, sin^2 + eps/2 within the rounding of its argument (one
+    unit of 2^-60) and 2^-60, the powers -1/2 and -3/2 within 2^-56."""
+    g = np.random.default_rng(7)
+    S = ctypes.c_int64()
+    out = np.zeros(11, np.uint32)
+    for i in range(4000):
+        he = float(np.ldexp(1 + g.random(), -int(g.integers(0, 18))))
+        a = (2 * g.random() - 1) * np.pi
+        b = a if i % 50 == 0 else a + (2 * g.random() - 1) * 2.0 ** -int(g.integers(0, 24))
+        v = [float(x) for x in (np.sin(a), np.cos(a), np.sin(b), np.cos(b))]
+        bias = np.float32(1 + (2 * g.random() - 1) * 2.0**-22)
+        lib.ring_term(*v, he, bias, ctypes.byref(S), out.ctypes.data)
+        Mh, Ml, z, sg, w2, w1, w0, Wh, Wl, Vh, Vl = (int(x) for x in out)
+        f = [Fraction(x) for x in v]
+        s = Fraction(S.value) * _pow2(-60)
+        assert abs(s - (f[0] * f[3] - f[1] * f[2])) < _pow2(-59)
+        if a == b:
+            assert S.value == 0
+        d = s * s + Fraction(he)
+        ms = Fraction((Mh << 32) | Ml) * _pow2(-63)
+        assert z % 2 == 1 and Fraction(1, 4) <= ms < 1
+        assert abs(ms * _pow2(3 - z) - d) < 2 * abs(s) * _pow2(-60) + _pow2(-60) * d
+        W, V = Fraction((Wh << 32) | Wl) * _pow2(-58), Fraction((Vh << 32) | Vl) * _pow2(-60)
+        assert abs(W * W * ms**3 - 1) < 2 * _pow2(-56) and abs(V * V * ms - 1) < 2 * _pow2(-56)
+        t = Fraction((w2 << 64) | (w1 << 32) | w0) * _pow2(-86)
+        assert abs((-t if sg else t) - s * W) < 8 * _pow2(-60) + 2 * _pow2(-64)
+
+
+def test_products_keep_their_exponent(lib):
+    g = np.random.default_rng(8)
+    for i in range(3000):
+        a, b = (int(g.integers(2**62, 2**63, dtype=np.uint64)) for _ in range(2))
+        if i % 10 == 0:
+            a = 2**62
+        e = ctypes.c_int(2)
+        m = lib.product(a, b, ctypes.byref(e))
+        assert 2**62 <= m < 2**63
+        exact = Fraction(a * b) * _pow2(-124)
+        # the caller adds the factor's own exponent + 2
+        assert abs(Fraction(m) * _pow2(-62) * _pow2(e.value) / exact - 1) < _pow2(-59)
 
 
 def test_shifts_and_sums(lib):
