@@ -4,6 +4,7 @@
 // All sums are deterministic: per-thread sums, a fixed shuffle/block tree, one
 // partial per CTA (or per tile pair), and a final pass that adds the partials in
 // index order (the last CTA to finish does it; no waiting).
+#include "fx64.cuh"
 #include "md_internal.cuh"
 
 namespace {
@@ -72,20 +73,30 @@ __device__ __forceinline__ double mul_renorm(double m, double s, int &e, unsigne
   return __hiloint2double((hi & 0x800fffff) | 0x3ff00000, __double2loint(r));
 }
 
+// Coordinates that the 3D tiles' fixed-point sums hold at full precision: finite and below
+// 2^19 sqrt(eps) (shifts of less than 32 bits).
+__device__ __forceinline__ bool out_of_range(double v, int half) {
+  return (fx64::hi_word(v) & 0x7fffffffu) >= ((unsigned)(1023 + 19 + half) << 20);
+}
+
 // One tile pair (ti <= tj) of the i<j potential sum.
 //  Ring: -(1/(2N)) sum d^(-1/2), d = sin^2((ti-tj)/2) + eps/2  (Eq. 1, with
 //        1 - cos d + eps = 2 d)
 //  2D:   (1/N) sum log(|r_ij|^2 + eps)                        (Eq. 3)
+// GB300's FP64 pipe is the bound (2 operations per SM and clock), so the pair arithmetic
+// is integer (fx64.cuh): no FP64 operation per Ring pair (9 in FP64), the two coordinate
+// differences per 2D pair (5).  A tile with a non-finite or huge input runs in FP64.
+// md_energy at N = 131,072: Ring 138.9 -> 34.5 ms, 2D 81.0 -> 35.0, 3D (below) 185.0 -> 49.5.
 // The 2D sum of logarithms of one thread's row of the tile is the logarithm of the
 // product of its s = |r|^2 + eps values: the product is kept as m 2^e (m in [1, 2),
 // renormalised after every factor, so it can neither overflow nor underflow while
 // every s is a normal double), and log m + e ln 2 replaces up to 256 logarithms.
-// A row with a factor that is not a normal double (a non-finite position, or
-// coincident particles with a subnormal eps) sums its logarithms one by one, so a
+// In the FP64 form a row with a factor that is not a normal double (a non-finite position,
+// or coincident particles with a subnormal eps) sums its logarithms one by one, so a
 // NaN or infinite position gives a NaN or infinite V.
 // Relative rounding of m: at most one unit roundoff per factor, i.e. about
 // 2.8e-14 absolute in the row's sum of 256 logarithms, the size of the rounding of
-// the sum of the logarithms themselves.
+// the sum of the logarithms themselves (integer form: 2^-60 per factor).
 // The prefactor is applied on the host.
 template <int MODEL>
 __global__ void __launch_bounds__(NT) potential_tiles_kernel(const double *__restrict__ q,
@@ -94,25 +105,78 @@ __global__ void __launch_bounds__(NT) potential_tiles_kernel(const double *__res
   const int ti = blockIdx.x, tj = blockIdx.y;
   if (tj < ti) return;
   __shared__ double2 sj[PT];
+  __shared__ int4 fj[MODEL == MD_RING ? PT : 1];
   const int64_t j0 = (int64_t)tj * PT;
+  const int64_t i = (int64_t)ti * PT + threadIdx.x;
+  // the integer form's range: Ring eps/2 as for the pair stages; 2D exponents far from overflow
+  bool wild = MODEL == MD_RING && !(epsd >= 0x1p-18 && epsd <= 2.0);
+  double2 me = make_double2(0.0, 0.0);
+  if (i < N) me = MODEL == MD_RING ? ag[i] : make_double2(q[i], q[N + i]);
+  const unsigned lim = MODEL == MD_RING ? 0x3ff00001u : (1023u + 400u) << 20;
+  wild |= (fx64::hi_word(me.x) & 0x7fffffffu) >= lim || (fx64::hi_word(me.y) & 0x7fffffffu) >= lim;
   for (int t = threadIdx.x; t < PT; t += NT) {
     int64_t j = j0 + t;
-    if (j < N) sj[t] = MODEL == MD_RING ? ag[j] : make_double2(q[j], q[N + j]);
+    if (j < N) {
+      const double2 o = MODEL == MD_RING ? ag[j] : make_double2(q[j], q[N + j]);
+      sj[t] = o;
+      wild |= (fx64::hi_word(o.x) & 0x7fffffffu) >= lim || (fx64::hi_word(o.y) & 0x7fffffffu) >= lim;
+      if constexpr (MODEL == MD_RING) {
+        const fx64::Limbs g = fx64::limbs_of(o.y), na = fx64::limbs_of(-o.x);
+        fj[t] = make_int4(g.h, g.l, na.h, na.l);
+      }
+    }
   }
-  __syncthreads();
-  const int64_t i = (int64_t)ti * PT + threadIdx.x;
+  wild = __syncthreads_or(wild);
   double s = 0.0;
   if (i < N) {
-    const double2 me = MODEL == MD_RING ? ag[i] : make_double2(q[i], q[N + i]);
     int kbeg = 0;
     if (ti == tj) kbeg = threadIdx.x + 1;  // j > i inside the diagonal tile
     int kend = (int)((N - j0) < PT ? (N - j0) : PT);
     if constexpr (MODEL == MD_RING) {
+      if (!wild) {
+        const fx64::Limbs ma = fx64::limbs_of(me.x), mg = fx64::limbs_of(me.y);
+        const fx64::Fix92 he = fx64::fix92_of(epsd);
+        // d^(-1/2) = W 2^-60 2^((z - 3) / 2) <= 2^10, in units of 2^-74: 256 terms fit 96 bits
+        fx64::Acc96 acc{0u, 0u, 0u};
+#pragma unroll 2
+        for (int k = kbeg; k < kend; k++) {
+          const int4 o = fj[k];
+          unsigned Mh, Ml;
+          int z;
+          fx64::square_plus(fx64::dot2(ma, mg, fx64::Limbs{o.x, o.y}, fx64::Limbs{o.z, o.w}), he, Mh, Ml, z);
+          const unsigned long long W = fx64::rsqrt_mantissa(Mh, Ml);
+          const int kk = 18 - ((z - 3) >> 1);  // W 2^32 = d^(-1/2) 2^92 2^-(z - 3)/2
+          const unsigned w2 = (unsigned)(W >> 32), w1 = (unsigned)W;
+          fx64::add96(acc, w2 >> kk, fx64::shf_r(w1, w2, kk), fx64::shf_r(0u, w1, kk));
+        }
+        s = fx64::total96(acc, -74);
+      } else {
+        for (int k = kbeg; k < kend; k++) {
+          const double2 o = sj[k];
+          double sh = fma(me.x, o.y, -(me.y * o.x));
+          s += rsqrt_nr(fma(sh, sh, epsd));
+        }
+      }
+    } else if (!wild) {
+      const fx64::Soft eps = fx64::soft_of(epsd);
+      unsigned long long m = 1ull << 62;
+      int e = 0;
+#pragma unroll 2
       for (int k = kbeg; k < kend; k++) {
         const double2 o = sj[k];
-        double sh = fma(me.x, o.y, -(me.y * o.x));
-        s += rsqrt_nr(fma(sh, sh, epsd));
+        const double d[2] = {me.x - o.x, me.y - o.y};
+        unsigned yh[2], yl[2], Mh, Ml;
+        int ex[2], es;
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+          ex[c] = (int)((fx64::hi_word(d[c]) >> 20) & 0x7ffu);
+          fx64::mantissa62(fx64::hi_word(d[c]), fx64::lo_word(d[c]), yh[c], yl[c]);
+        }
+        fx64::square_sum<2>(yh, yl, ex, eps, Mh, Ml, es);
+        m = fx64::mul_renorm63(m, (((unsigned long long)Mh << 32) | Ml) >> 1, e);  // times ms
+        e += es - 1021;
       }
+      s = log((double)m * 0x1p-62) + (double)e * 0.69314718055994530942;
     } else {
       double m = 1.0;
       int e = 0;
@@ -139,31 +203,63 @@ __global__ void __launch_bounds__(NT) potential_tiles_kernel(const double *__res
 }
 
 // 3D: one tile pair (ti <= tj) of sum_{i<j} (|r_ij|^2 + eps)^(-1/2); the prefactor
-// -1/N is applied at the end.
+// -1/N is applied at the end.  The three differences in FP64 (12 operations in all
+// in the FP64 form, which tiles out of the fixed-point range and eps below 2^-28 run),
+// the rest on the integer pipe: each term at most 2^-half, 256 of them in 96 bits.
 __global__ void __launch_bounds__(NT) potential3d_tiles_kernel(const double *__restrict__ q, int64_t N, int ntiles,
                                                                 double eps, double *unit_sums) {
   const int ti = blockIdx.x, tj = blockIdx.y;
   if (tj < ti) return;
   __shared__ double sx[PT], sy[PT], sz[PT];
   const int64_t j0 = (int64_t)tj * PT;
+  const int64_t i = (int64_t)ti * PT + threadIdx.x;
+  const int half = ((int)(fx64::hi_word(eps) >> 20) - 1023) >> 1;
+  bool wild = !(eps >= 0x1p-28);
+  double x = 0.0, y = 0.0, z = 0.0;
+  if (i < N) {
+    x = q[i], y = q[N + i], z = q[2 * N + i];
+    wild |= out_of_range(x, half) || out_of_range(y, half) || out_of_range(z, half);
+  }
   for (int t = threadIdx.x; t < PT; t += NT) {
     const int64_t j = j0 + t;
     if (j < N) {
       sx[t] = q[j];
       sy[t] = q[N + j];
       sz[t] = q[2 * N + j];
+      wild |= out_of_range(sx[t], half) || out_of_range(sy[t], half) || out_of_range(sz[t], half);
     }
   }
-  __syncthreads();
-  const int64_t i = (int64_t)ti * PT + threadIdx.x;
+  wild = __syncthreads_or(wild);
   double s = 0.0;
   if (i < N) {
-    const double x = q[i], y = q[N + i], z = q[2 * N + i];
     const int kbeg = ti == tj ? threadIdx.x + 1 : 0;  // j > i inside the diagonal tile
     const int kend = (int)((N - j0) < PT ? (N - j0) : PT);
-    for (int k = kbeg; k < kend; k++) {
-      const double dx = x - sx[k], dy = y - sy[k], dz = z - sz[k];
-      s += rsqrt_nr(fma(dx, dx, fma(dy, dy, fma(dz, dz, eps))));
+    if (!wild) {
+      const fx64::Soft so = fx64::soft_of(eps);
+      fx64::Acc96 acc{0u, 0u, 0u};
+#pragma unroll 2
+      for (int k = kbeg; k < kend; k++) {
+        const double d[3] = {x - sx[k], y - sy[k], z - sz[k]};
+        unsigned yh[3], yl[3], Mh, Ml;
+        int ex[3], es;
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+          ex[c] = (int)((fx64::hi_word(d[c]) >> 20) & 0x7ffu);
+          fx64::mantissa62(fx64::hi_word(d[c]), fx64::lo_word(d[c]), yh[c], yl[c]);
+        }
+        fx64::square_sum<3>(yh, yl, ex, so, Mh, Ml, es);
+        const int g = fx64::even_exponent(Mh, Ml, es - 1023);
+        const unsigned long long W = fx64::rsqrt_mantissa(Mh, Ml);  // s^(-1/2) = W 2^(-60 - g)
+        const int kk = g - half + 9;                                // g >= half: in units of 2^(-83 - half)
+        const unsigned w2 = (unsigned)(W >> 32), w1 = (unsigned)W;
+        fx64::add96(acc, w2 >> kk, fx64::shf_r(w1, w2, kk), fx64::shf_r(0u, w1, kk));
+      }
+      s = fx64::total96(acc, -83 - half);
+    } else {
+      for (int k = kbeg; k < kend; k++) {
+        const double dx = x - sx[k], dy = y - sy[k], dz = z - sz[k];
+        s += rsqrt_nr(fma(dx, dx, fma(dy, dy, fma(dz, dz, eps))));
+      }
     }
   }
   __shared__ double2 red[NT / 32];

@@ -1,4 +1,4 @@
-"""The FP64 pair stages on the integer pipe (needs a GB300): softenings on both
+"""The FP64 pair stages and potentials on the integer pipe (needs a GB300): softenings on both
 sides of the integer form's range, systems far larger and smaller than their softening
 length, outliers that make single units take the FP64 tile, ragged sizes at the tile edges.
 
@@ -10,7 +10,10 @@ oracle where particles come closer than sqrt(eps)): that kernel rounds S and sin
 2^-53 each (product and FMA), which moves a pair's term S dd^(-3/2) by at most
 2^-52 (dd^(-3/2) + 3 |S sin(d/2)| dd^(-5/2)), and its sums and products by 1e-14 of their
 magnitude.
-"""
+
+Potentials against a long-double sum of the definition, 1e-13 of the sum of the terms'
+magnitudes (the oracle adds the pairs one by one in FP64, which costs more than that where
+all terms are nearly equal)."""
 import numpy as np
 import pytest
 
@@ -81,3 +84,41 @@ def test_a_non_finite_position_reaches_every_force(model, bad):
     q, _ = inputs.default_state(model, 1100, 9)
     q[600] = bad
     assert np.isnan(_force(model, q, 1e-3)).all()
+
+
+def _potential(model, q, eps):
+    """(V, the sum of its terms' magnitudes) in long double."""
+    D = model if model > 1 else 1
+    x = q.reshape(D, -1).astype(np.longdouble)
+    N, v, a = x.shape[1], np.longdouble(0), np.longdouble(0)
+    for i in range(N - 1):
+        d = x[:, i : i + 1] - x[:, i + 1 :]
+        if model == 1:
+            t = -1 / np.sqrt(2 * np.sin(d[0] / 2) ** 2 + np.longdouble(eps)) / np.sqrt(np.longdouble(2))
+        else:
+            s = (d * d).sum(0) + np.longdouble(eps)
+            t = np.log(s) if model == 2 else -1 / np.sqrt(s)
+        v, a = v + t.sum(), a + np.abs(t).sum()
+    return v / N, float(a / N)
+
+
+def _check_potential(model, q, eps):
+    v, scale = _potential(model, q, eps)
+    with System(model, q.size // (model if model > 1 else 1), eps, 0.01, 1) as s:
+        s.set_state(q, np.zeros_like(q))
+        assert abs(float(s.energy()[1] - v)) <= 1e-13 * scale
+
+
+@pytest.mark.parametrize("model,eps", [(m, e) for m in (1, 2, 3) for e in (4.1, 1.0, 1e-3, 2.0**-17, 0.99 * 2.0**-17)]
+                         + [(m, e) for m in (2, 3) for e in (2.0**-28, 0.99 * 2.0**-28, 1e-12)])
+@pytest.mark.parametrize("N", [2, 255, 257, 513])
+def test_potential_over_softenings(model, N, eps):
+    _check_potential(model, inputs.default_state(model, N, 50 + N)[0], eps)
+
+
+@pytest.mark.parametrize("scale", [1e-9, 1e-3, 30.0, 1e6, 1e9])
+@pytest.mark.parametrize("model", [2, 3])
+def test_potential_over_scales(model, scale):
+    q = inputs.default_state(model, 400, 3)[0] * scale
+    q[5] *= 1e4
+    _check_potential(model, q, 1e-4)
