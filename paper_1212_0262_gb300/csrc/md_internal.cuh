@@ -215,6 +215,10 @@ int ensure_pair_buffers(md_ctx *c, int TI, int P, int nacc);       // stream-K s
 bool sym_applies(const md_ctx *c);
 int sym_pair_stage(md_ctx *c, int mode, double kick, double drift, double *fout);
 
+// sheet.cu: the symmetric form of the sheets at eps = 0, by counting ranks
+bool sheet_rank_applies(const md_ctx *c);
+int sheet_rank_stage(md_ctx *c, int mode, double kick, double drift, double *fout);
+
 // pairs.cu / hmf.cu: row shards (md_shard_*).  *_shard_prime writes this rank's segment of
 // the exchange buffer from its state; *_shard_stage runs one fused stage over the shard's
 // rows (STAGE_KICK_DRIFT, drift 0 allowed, or STAGE_FORCE_ONLY into fout); *_shard_segment

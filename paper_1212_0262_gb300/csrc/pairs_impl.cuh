@@ -1055,8 +1055,12 @@ struct SheetMixed {
     else body<false>(st, sm, e2);
     flush(st);
   }
-  template <bool SMOOTH>
-  __device__ static void body_sym(State &st, const float2 *sm, float2 e2, float *colsm) {
+  // Newton's-third-law variant (eps > 0; at eps = 0 the forces are rank counts, sheet.cu):
+  // the i-rows as in tile<>, and per j the sum over this warp's rows of the same terms into
+  // colsm[warp TJ + j]; sixteen j's at a time.
+  __device__ static void tile_sym(State &st, const unsigned char *smb, const PairArgs &a, float *colsm) {
+    const float2 *sm = (const float2 *)smb;
+    const float2 e2 = f2((float)a.epsd);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll 1
     for (int k8 = 0; k8 < TJ / 16; k8++) {
@@ -1067,7 +1071,7 @@ struct SheetMixed {
         float2 col = f2(0.f);
 #pragma unroll
         for (int r = 0; r < R; r++) {
-          const float2 t = term(st.x[r], nx, e2, SMOOTH);
+          const float2 t = term(st.x[r], nx, e2, true);
           st.acc[r] = __fadd2_rn(st.acc[r], t);
           col = __fadd2_rn(col, t);
         }
@@ -1078,14 +1082,6 @@ struct SheetMixed {
       sum += __shfl_xor_sync(0xffffffffu, sum, 1);
       if ((lane & 1) == 0) colsm[w * TJ + 16 * k8 + (lane >> 1)] = sum;
     }
-  }
-  // Newton's-third-law variant: the i-rows as in tile<>, and per j the sum over this
-  // warp's rows of the same terms into colsm[warp TJ + j]; sixteen j's at a time.
-  __device__ static void tile_sym(State &st, const unsigned char *smb, const PairArgs &a, float *colsm) {
-    const float2 *sm = (const float2 *)smb;
-    const float2 e2 = f2((float)a.epsd);
-    if (a.epsd > 0.0) body_sym<true>(st, sm, e2, colsm);
-    else body_sym<false>(st, sm, e2, colsm);
     flush(st);
   }
 };
@@ -1147,57 +1143,31 @@ struct SheetF64 {
       for (int r = 0; r < R; r++) st.accd[r][0] += (double)acc[r];
     }
   }
+  // Newton's-third-law variant, eps > 0 (at eps = 0: rank counts, sheet.cu)
   __device__ static void tile_sym(State &st, const unsigned char *smb, const PairArgs &a, double *colsm) {
     const long long *sm = (const long long *)smb;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (a.epsd > 0.0) {
-      double x[R];
+    double x[R];
 #pragma unroll
-      for (int r = 0; r < R; r++) x[r] = sheet_unkey(st.k[r]);
+    for (int r = 0; r < R; r++) x[r] = sheet_unkey(st.k[r]);
 #pragma unroll 1
-      for (int k16 = 0; k16 < TJ / 16; k16++) {
-        double v[16];
+    for (int k16 = 0; k16 < TJ / 16; k16++) {
+      double v[16];
 #pragma unroll
-        for (int kk = 0; kk < 16; kk++) {
-          const long long kj = sm[16 * k16 + kk];
-          double col = 0.0;
+      for (int kk = 0; kk < 16; kk++) {
+        const long long kj = sm[16 * k16 + kk];
+        double col = 0.0;
 #pragma unroll
-          for (int r = 0; r < R; r++) {
-            const double t = smooth_term(x[r], kj, a.epsd);
-            st.accd[r][0] += t;
-            col += t;
-          }
-          v[kk] = col;
+        for (int r = 0; r < R; r++) {
+          const double t = smooth_term(x[r], kj, a.epsd);
+          st.accd[r][0] += t;
+          col += t;
         }
-        double sum = butterfly_sum<16, 16>(v, lane);
-        sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-        if ((lane & 1) == 0) colsm[w * TJ + 16 * k16 + (lane >> 1)] = sum;
+        v[kk] = col;
       }
-    } else {
-      int acc[R];
-#pragma unroll
-      for (int r = 0; r < R; r++) acc[r] = 0;
-#pragma unroll 1
-      for (int k16 = 0; k16 < TJ / 16; k16++) {
-        int v[16];
-#pragma unroll
-        for (int kk = 0; kk < 16; kk++) {
-          const long long kj = sm[16 * k16 + kk];
-          int col = 0;
-#pragma unroll
-          for (int r = 0; r < R; r++) {
-            const int t = cmp(st.k[r], kj);
-            acc[r] += t;
-            col += t;
-          }
-          v[kk] = col;
-        }
-        int sum = butterfly_sum<16, 16>(v, lane);
-        sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-        if ((lane & 1) == 0) colsm[w * TJ + 16 * k16 + (lane >> 1)] = (double)sum;
-      }
-#pragma unroll
-      for (int r = 0; r < R; r++) st.accd[r][0] += (double)acc[r];
+      double sum = butterfly_sum<16, 16>(v, lane);
+      sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+      if ((lane & 1) == 0) colsm[w * TJ + 16 * k16 + (lane >> 1)] = sum;
     }
   }
 };

@@ -406,8 +406,9 @@ bool sym_applies(const md_ctx *c) {
   if (!c->pt.symmetric) return false;
   int64_t TI, TJ, nacc = c->dim, colbytes;
   if (c->model == MD_HMF) return false;
+  if (c->prec == MD_FP64 && c->pt.r_fp64 != 2) return false;
+  if (sheet_rank_applies(c)) return true;  // no column partials
   if (c->prec == MD_FP64) {
-    if (c->pt.r_fp64 != 2) return false;
     TI = 512, TJ = 128, colbytes = 8;
   } else if (c->model == MD_GRAV3D) {
     TI = 512, TJ = 256, colbytes = 4;
@@ -428,6 +429,7 @@ bool sym_applies(const md_ctx *c) {
 }
 
 int sym_pair_stage(md_ctx *c, int mode, double kick, double drift, double *fout) {
+  if (sheet_rank_applies(c)) return sheet_rank_stage(c, mode, kick, drift, fout);
   PairArgs a{};
   a.kick = kick;
   a.drift = drift;
