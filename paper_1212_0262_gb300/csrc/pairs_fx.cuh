@@ -5,7 +5,7 @@
 // moved into doubles (shared memory) every kFxFlush units; column sums are added over the
 // warp with redux.sync on 27-bit limbs, over the warps as integers, and stored as doubles.
 //
-// A unit that touches a coordinate beyond 2^26 sqrt(eps) (terms so small against the
+// A unit that touches a coordinate beyond 2^26 sqrt(eps) (3D: 2^15; terms so small against the
 // largest possible one that 96 bits would hold less than a double) or a non-finite one
 // runs the FP64 policy's tile instead: the CTA decides per unit with one vote, which
 // replaces the barrier after the tile's load.
@@ -97,40 +97,80 @@ __device__ __forceinline__ void fx_add(unsigned sg, unsigned w2, unsigned w1, un
   if (COL) fx64::add96(col, w2, w1, w0);
 }
 
-// ------------------------------------------------------------ forward 2D
-// Per pair dx and dy in FP64 (2 operations instead of 14); the squared distance, its
-// reciprocal, the products with dx and dy and the four sums are integers: about 147
-// instructions per pair, 57% of the integer pipe and of the FP64 pipe (4 warps per scheduler;
-// dependent instructions are what is left).  One force at N = 49,152: 28.1 ms with GravF64,
-// 9.74 with s on the FP64 pipe, 7.25 as it stands.
-template <int R_, int TJ_, int MODE>
-struct GravFx {
+// ------------------------------------------------------------ forward 2D and 3D
+// Terms d / s (2D) and d s^(-3/2) (3D), s = |d|^2 + eps.  Per pair only the coordinate
+// differences are FP64 operations (2 instead of 14, 3 instead of 23.4); the squared distance,
+// its inverse power, the products and the sums are integers: about 147 instructions per 2D
+// pair, 57% of the integer pipe and of the FP64 pipe (4 warps per scheduler; dependent
+// instructions are what is left).  One 2D force at N = 49,152: 28.1 ms with GravF64, 9.74 with
+// s on the FP64 pipe, 7.25 as it stands.
+// eps of the fixed-point form (below, the unit 2^lsb of the sums would grow too large)
+inline bool fx_grav_applies(double eps) { return eps >= 0x1p-28; }
+
+template <int D>
+struct FxGravTraits;
+template <>
+struct FxGravTraits<2> {
+  static constexpr int MODEL = MD_GRAV2D, MINB = 4;
+  static constexpr int RANGE = 26;  // coordinates below 2^RANGE sqrt(eps)
+  template <int R, int TJ>
+  using Wild = GravF64<R, TJ, STAGE_KICK_DRIFT>;
+  using Vec = double2;
+  // |d| / s <= 1 / (2 sqrt eps) <= 2^(-half - 1): unit 2^lsb of the sums
+  __device__ static int lsb(int half) { return -82 - half; }
+  // inverse power of s = ms 2^(es - 1023) as an integer and the shift of a term with exponent ex
+  __device__ static unsigned long long power(unsigned Mh, unsigned Ml, int es, int half, int &k) {
+    k = es + 9 - half;  // y R 2^-32 = |d| / s 2^(91 - ex + es); at least 9, so 2^12 terms fit
+    return fx64::rcp_mantissa(Mh, Ml);
+  }
+};
+template <>
+struct FxGravTraits<3> {
+  static constexpr int MODEL = MD_GRAV3D, MINB = 4;
+  static constexpr int RANGE = 15;  // terms fall as 1 / r^2
+  template <int R, int TJ>
+  using Wild = Grav3DF64<R, TJ, STAGE_KICK_DRIFT>;
+  using Vec = double4_16a;
+  // |d| s^(-3/2) <= 0.385 / eps <= 2^(-2 half - 1)
+  __device__ static int lsb(int half) { return -84 - 2 * half; }
+  __device__ static unsigned long long power(unsigned Mh, unsigned Ml, int es, int half, int &k) {
+    const int g = fx64::even_exponent(Mh, Ml, es - 1023);
+    k = 3 * g + 1026 - 2 * half;  // y W 2^-32 = |d| s^(-3/2) 2^(87 - (ex - 1023) + 3 g); at least 4
+    return fx64::rsqrt3_mantissa(Mh, Ml);
+  }
+};
+__device__ __forceinline__ double fx_coord(const double2 &v, int d) { return d == 0 ? v.x : v.y; }
+__device__ __forceinline__ double fx_coord(const double4_16a &v, int d) { return d == 0 ? v.x : d == 1 ? v.y : v.z; }
+
+template <int D, int R_, int TJ_>
+struct FxGrav {
+  using Tr = FxGravTraits<D>;
+  using Vec = typename Tr::Vec;
   static constexpr bool FX = true;
-  static constexpr int THREADS = NT, MINB = 4;
+  static constexpr int THREADS = NT, MINB = Tr::MINB;
   using ColT = double;
-  using Wild = GravF64<R_, TJ_, MODE>;  // units out of the fixed-point range
-  static constexpr int R = R_, TJ = TJ_, NACC = 2, JB = RecordBytes<MD_GRAV2D, false, false>::value;
+  using Wild = typename Tr::template Wild<R_, TJ_>;  // units out of the fixed-point range
+  static constexpr int R = R_, TJ = TJ_, NACC = D, JB = RecordBytes<Tr::MODEL, false, false>::value;
+  static_assert(JB == (int)sizeof(Vec), "one record per particle");
   static constexpr bool MASK = false;
   static constexpr int NR = R;
   static constexpr int FMT = 0;
   static constexpr int COL_BYTES = (NT / 32) * TJ * NACC * (int)sizeof(uint4);
-  // eps of the fixed-point form (below, the unit 2^lsb of the sums would grow too large)
-  static bool applies(double eps) { return eps >= 0x1p-28; }
+  static constexpr int STAGE_BYTES = 16;  // nothing is staged
   __device__ static int row_of(int r) { return r * NT + (int)threadIdx.x; }
   struct State {
-    double x[R], y[R];
+    double x[R][D];
     fx64::Acc96 acc[R][NACC];
     FxRowSums<R * NACC> rows;
     int units;     // since the last flush
     bool wild;     // a row of this thread lies out of the fixed-point range
   };
-  // floor(log2(eps) / 2); the sums' unit is 2^lsb: a term (below 2^92) is shifted down by
-  // k = es - ex - half + 9 >= 9, and 2^12 terms fit
+  // floor(log2(eps) / 2)
   __device__ static int half_exp(const PairArgs &a) { return ((int)(fx64::hi_word(a.epsd) >> 20) - 1023) >> 1; }
-  __device__ static int lsb(const PairArgs &a) { return -82 - half_exp(a); }
+  __device__ static int lsb(const PairArgs &a) { return Tr::lsb(half_exp(a)); }
   __device__ static bool out_of_range(double v, int half) {
     const unsigned h = fx64::hi_word(v) & 0x7fffffffu;
-    return h >= ((unsigned)(1023 + 26 + half) << 20) && h != (fx64::hi_word(1.0e150));  // padding: its terms vanish
+    return h >= ((unsigned)(1023 + Tr::RANGE + half) << 20) && h != (fx64::hi_word(1.0e150));  // padding: its terms vanish
   }
   __device__ static void load(State &st, const void *mirror, int64_t i0, const PairArgs &a, double *rowsm) {
     const int half = half_exp(a);
@@ -138,10 +178,12 @@ struct GravFx {
     fx_clear<State, R, NACC>(st, rowsm);
 #pragma unroll
     for (int r = 0; r < R; r++) {
-      const double2 m = *(const double2 *)((const double *)mirror + (i0 + row_of(r)) * 2);
-      st.x[r] = m.x;
-      st.y[r] = m.y;
-      st.wild = st.wild || out_of_range(m.x, half) || out_of_range(m.y, half);
+      const Vec m = ((const Vec *)mirror)[i0 + row_of(r)];
+#pragma unroll
+      for (int d = 0; d < D; d++) {
+        st.x[r][d] = fx_coord(m, d);
+        st.wild = st.wild || out_of_range(st.x[r][d], half);
+      }
     }
   }
   __device__ static void flush(State &st, const PairArgs &a) { fx_flush<State, R, NACC>(st, lsb(a)); }
@@ -149,8 +191,7 @@ struct GravFx {
 #pragma unroll
     for (int d = 0; d < NACC; d++) out[d] = st.rows.at(r * NACC + d);
   }
-  // a 16-byte chunk of the tile (one particle): whether it is out of range
-  static constexpr int STAGE_BYTES = 16;  // nothing is staged
+  // a 16-byte chunk of the tile: whether it is out of range (3D: (x, y) or (z, 0))
   __device__ static bool stage(const unsigned char *tile, int ch, unsigned char *, const PairArgs &a) {
     const double2 v = ((const double2 *)tile)[ch];
     const int half = half_exp(a);
@@ -159,46 +200,47 @@ struct GravFx {
   template <bool COL>
   __device__ static void unit(State &st, const unsigned char *smb, const unsigned char *, const PairArgs &a,
                               unsigned char *colraw, int64_t, int64_t) {
-    const double2 *sm = (const double2 *)smb;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int kc = 9 - half_exp(a);
+    const Vec *sm = (const Vec *)smb;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, half = half_exp(a);
     const fx64::Soft eps = fx64::soft_of(a.epsd);
     uint4 *colsm = (uint4 *)colraw + w * TJ * NACC;
-#pragma unroll 1
+#pragma unroll(4 / R)
     for (int j = 0; j < TJ; j++) {
-      const double2 o = sm[j];
-      fx64::Acc96 col[2] = {{0u, 0u, 0u}, {0u, 0u, 0u}};
-      unsigned h[R][2], yh[R][2], yl[R][2];
-      unsigned long long inv[R];
-      int k[R][2];
+      const Vec o = sm[j];
+      fx64::Acc96 col[D];
+#pragma unroll
+      for (int c = 0; c < D; c++) col[c] = fx64::Acc96{0u, 0u, 0u};
+      unsigned h[R][D], yh[R][D], yl[R][D];
+      unsigned long long pw[R];
+      int k[R][D];
       unsigned kor = 0u;
 #pragma unroll
       for (int r = 0; r < R; r++) {
-        const double d[2] = {st.x[r] - o.x, st.y[r] - o.y};
-        int ex[2], es;
+        int ex[D], es, kc;
 #pragma unroll
-        for (int c = 0; c < 2; c++) {
-          h[r][c] = fx64::hi_word(d[c]);
+        for (int c = 0; c < D; c++) {
+          const double d = st.x[r][c] - fx_coord(o, c);
+          h[r][c] = fx64::hi_word(d);
           ex[c] = (int)((h[r][c] >> 20) & 0x7ffu);
-          fx64::mantissa62(h[r][c], fx64::lo_word(d[c]), yh[r][c], yl[r][c]);
+          fx64::mantissa62(h[r][c], fx64::lo_word(d), yh[r][c], yl[r][c]);
         }
         unsigned Mh, Ml;
-        fx64::square_sum<2>(yh[r], yl[r], ex, eps, Mh, Ml, es);
-        inv[r] = fx64::rcp_mantissa(Mh, Ml);
+        fx64::square_sum<D>(yh[r], yl[r], ex, eps, Mh, Ml, es);
+        pw[r] = Tr::power(Mh, Ml, es, half, kc);
 #pragma unroll
-        for (int c = 0; c < 2; c++) {
-          k[r][c] = es + kc - ex[c];
+        for (int c = 0; c < D; c++) {
+          k[r][c] = kc - ex[c];
           kor |= (unsigned)k[r][c];
         }
       }
-      // one branch for the four rows: a component 2^-14 and less of the distance is rare
+      // one branch for the rows: a component far below the distance (2D: 2^-14) is rare
       if (__builtin_expect(kor < 32u, 1)) {
 #pragma unroll
         for (int r = 0; r < R; r++)
 #pragma unroll
-          for (int c = 0; c < 2; c++) {
+          for (int c = 0; c < D; c++) {
             unsigned w2, w1, w0;
-            fx64::mul_mantissa(yh[r][c], yl[r][c], inv[r], w2, w1, w0);
+            fx64::mul_mantissa(yh[r][c], yl[r][c], pw[r], w2, w1, w0);
             w0 = fx64::shf_r(w0, w1, k[r][c]);
             w1 = fx64::shf_r(w1, w2, k[r][c]);
             w2 >>= k[r][c];
@@ -208,19 +250,19 @@ struct GravFx {
 #pragma unroll
         for (int r = 0; r < R; r++)
 #pragma unroll
-          for (int c = 0; c < 2; c++) {
+          for (int c = 0; c < D; c++) {
             unsigned w2, w1, w0;
-            fx64::mul_mantissa(yh[r][c], yl[r][c], inv[r], w2, w1, w0);
+            fx64::mul_mantissa(yh[r][c], yl[r][c], pw[r], w2, w1, w0);
             fx64::shift96_any(w2, w1, w0, k[r][c]);
             // a zero term adds exactly zero (~0 would be -1 unit)
             fx_add<COL>((w2 | w1 | w0) == 0u ? 0u : (unsigned)((int)h[r][c] >> 31), w2, w1, w0, st.acc[r][c], col[c]);
           }
       }
       if (COL) {
-        const uint4 sx = fx_warp_sum(col[0]), sy = fx_warp_sum(col[1]);
-        if (lane == 0) {
-          colsm[2 * j] = sx;
-          colsm[2 * j + 1] = sy;
+#pragma unroll
+        for (int c = 0; c < D; c++) {
+          const uint4 s = fx_warp_sum(col[c]);
+          if (lane == 0) colsm[D * j + c] = s;
         }
       }
     }
@@ -231,13 +273,11 @@ struct GravFx {
   __device__ static void unit_wild(State &st, const unsigned char *smb, const PairArgs &a, unsigned char *colraw,
                                    int64_t i0, int64_t j0) {
     typename Wild::State ws;
+    Wild::load(ws, a.mirror_in, i0);
 #pragma unroll
-    for (int r = 0; r < R; r++) {
-      ws.x[r] = st.x[r];
-      ws.y[r] = st.y[r];
+    for (int r = 0; r < R; r++)
 #pragma unroll
       for (int d = 0; d < NACC; d++) ws.accd[r][d] = st.rows.at(r * NACC + d);
-    }
     if (COL) Wild::tile_sym(ws, smb, a, (double *)colraw);
     else Wild::template tile<true>(ws, smb, a, i0, j0);
 #pragma unroll
@@ -250,27 +290,33 @@ struct GravFx {
   }
 };
 
+template <int R, int TJ>
+using FxGrav2D = FxGrav<2, R, TJ>;
+template <int R, int TJ>
+using FxGrav3D = FxGrav<3, R, TJ>;
+
 // ------------------------------------------------------------ forward Ring
 // Sines and cosines are numbers of at most 1, so the whole pair term is fixed-point: S and
 // sin(d/2) as 62-bit dot products, sin^2 + eps/2 in 96 bits, its power -3/2 from an FP32 seed
 // and one third-order step, no FP64 operation (15.5 in RingF64).  The tile's records are
 // turned into integers once per unit, by the thread that loaded them.  137 instructions per
-// pair; one force at N = 49,152: 36.3 ms with RingF64, 7.47 here (bound by the integer pipe,
+// pair; one force at N = 49,152: 36.3 ms with RingF64, 7.11 here (bound by the integer pipe,
 // 51%, and by dependent instructions at 4 warps per scheduler).
-template <int R_, int TJ_, int MODE>
+// eps of the fixed-point form: shifts of 0 .. 31 bits, sums below 2^95
+inline bool fx_ring_applies(double eps) { return eps >= 0x1p-17 && eps <= 4.0; }
+
+template <int R_, int TJ_>
 struct RingFx {
   static constexpr bool FX = true;
   static constexpr int THREADS = NT, MINB = 4;
   using ColT = double;
-  using Wild = RingF64<R_, TJ_, MODE>;
+  using Wild = RingF64<R_, TJ_, STAGE_KICK_DRIFT>;
   static constexpr int R = R_, TJ = TJ_, NACC = 1, JB = RecordBytes<MD_RING, false, false>::value;
   static constexpr bool MASK = true;
   static constexpr int NR = R;
   static constexpr int FMT = 0;
   static constexpr int COL_BYTES = (NT / 32) * TJ * NACC * (int)sizeof(uint4);
   static constexpr int STAGE_BYTES = TJ * JB;
-  // eps of the fixed-point form: shifts of 0 .. 31 bits, sums below 2^95
-  static bool applies(double eps) { return eps >= 0x1p-17 && eps <= 4.0; }
   __device__ static int row_of(int r) { return r * NT + (int)threadIdx.x; }
   struct State {
     fx64::Limbs s[R], c[R], a[R], g[R];
@@ -318,7 +364,7 @@ struct RingFx {
     const fx64::Fix92 he = fx64::fix92_of(a.epsd);
     const int kc = 3 + top(a);
     uint4 *colsm = (uint4 *)colraw + w * TJ * NACC;
-#pragma unroll 1
+#pragma unroll(4 / R)
     for (int j = 0; j < TJ; j++) {
       const int4 p = sm[2 * j], q = sm[2 * j + 1];
       const fx64::Limbs ns{p.x, p.y}, c{p.z, p.w}, na{q.x, q.y}, g{q.z, q.w};

@@ -318,8 +318,11 @@ int launch_sym(md_ctx *c, PairArgs a) {
   // virtual CTAs per CTA, measured at the bench sizes (sweeps of 1-16 show sharp dips at
   // single values, 4 for these two among them): 8 for the Ring tensor-core kernel, 3 for
   // the FP64 3D kernel, 4 for the others
-  const int kv = c->pt.vcta > 0 ? c->pt.vcta : Pol::FMT == 1 ? 8 : (MODEL == MD_GRAV3D && !MIXED) ? 3 : 4;
-  a.P = (int)vcta_count(G, a.U, kv);
+  int kv = c->pt.vcta > 0 ? c->pt.vcta : Pol::FMT == 1 ? 8 : (MODEL == MD_GRAV3D && !MIXED) ? 3 : 4;
+  // integer policies: units are long; below 16 per CTA one range each is best (N = 16,385,
+  // Ring: 983 us, 1079 / 1031 / 994 with 2 / 3 / 4 ranges)
+  if (IsFx<Pol>::value && c->pt.vcta == 0 && a.U < 16 * G) kv = 1;
+  a.P = (int)vcta_count(G, a.U, kv, IsFx<Pol>::value ? 1 : 16);
   int rc = ensure_pair_buffers(c, (int)TI, a.P, NACC);
   if (rc) return rc;
   const int64_t max_rows = a.n_it - 1 + (HasDiagSym<Pol>::value ? 1 : 0);  // of the last tile
@@ -364,22 +367,37 @@ int launch_sym(md_ctx *c, PairArgs a) {
   return MD_OK;
 }
 
+// FP64 stages with integer pair arithmetic: Fx<rows per thread, j-tile>.  A unit is one
+// CTA's work of 128 rows x tile, 256 x tile, 512 x tile pairs, and a pair takes thousands of
+// cycles of latency, so small systems want small units (N = 1,000, microseconds per force,
+// 2D: 45 with <1, 64>, 58 with <2, 64>, 147 with <4, 128>), larger ones more rows to share
+// the column reductions (N = 16,385: 967, 915, 1020; N = 8,192: 264, 281, 343).  <4, 128> needs
+// half the column storage of <2, 64> and is 2-5% slower (N = 49,152: 7.17 against 7.07 ms).
+constexpr int64_t kFxSmall = 10000, kFxLarge = 262144;
+template <template <int, int> class Fx, int MODEL, int MODE>
+int fx_dispatch(md_ctx *c, PairArgs a) {
+  if (c->N <= kFxSmall) return launch_sym<Fx<1, 64>, MODEL, false, MODE>(c, a);
+  if (c->N <= kFxLarge) return launch_sym<Fx<2, 64>, MODEL, false, MODE>(c, a);
+  return launch_sym<Fx<4, 128>, MODEL, false, MODE>(c, a);
+}
+
 template <int MODEL, bool MIXED, int MODE>
 int sym_dispatch(md_ctx *c, PairArgs a) {
   if constexpr (MODEL == MD_GRAV3D) {
     if constexpr (MIXED) return launch_sym<Grav3DMixed<4, 256, MODE>, MODEL, true, MODE>(c, a);
+    else if (fx_grav_applies(c->eps)) return fx_dispatch<FxGrav3D, MODEL, MODE>(c, a);
     else return launch_sym<Grav3DF64<4, 128, MODE>, MODEL, false, MODE>(c, a);
   } else if constexpr (MODEL == MD_SHEET1D) {
     // registers for 5 CTAs per SM (96, no spills): 1.4% faster than for 4 at N = 262,144
     if constexpr (MIXED) return launch_sym<SheetMixed<8, 256, MODE, 5>, MODEL, true, MODE>(c, a);
     else return launch_sym<SheetF64<4, 128, MODE>, MODEL, false, MODE>(c, a);
   } else if constexpr (!MIXED) {
-    // 4 rows per thread: the column butterflies' FP64 adds are shared by twice the pairs
+    // FP64 tiles: 4 rows per thread, so that the column butterflies' FP64 adds are shared
     if constexpr (MODEL == MD_RING) {
-      if (RingFx<4, 128, MODE>::applies(c->eps)) return launch_sym<RingFx<4, 128, MODE>, MODEL, false, MODE>(c, a);
+      if (fx_ring_applies(c->eps)) return fx_dispatch<RingFx, MODEL, MODE>(c, a);
       return launch_sym<RingF64<4, 128, MODE>, MODEL, false, MODE>(c, a);
     } else {
-      if (GravFx<4, 128, MODE>::applies(c->eps)) return launch_sym<GravFx<4, 128, MODE>, MODEL, false, MODE>(c, a);
+      if (fx_grav_applies(c->eps)) return fx_dispatch<FxGrav2D, MODEL, MODE>(c, a);
       return launch_sym<GravF64<4, 128, MODE>, MODEL, false, MODE>(c, a);
     }
   } else if constexpr (MODEL == MD_RING) {

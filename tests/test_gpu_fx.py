@@ -22,7 +22,7 @@ from paper_1212_0262_gb300 import System, inputs
 
 pytestmark = pytest.mark.gpu
 
-PLANAR = [2]
+PLANAR = [2, 3]
 
 
 def _force(model, q, eps, symmetric=1):
@@ -39,7 +39,7 @@ def _bound(model, q, eps):
 
 
 @pytest.mark.parametrize("eps", [1.0, 1e-3, 2.0**-28, 0.99 * 2.0**-28, 1e-12])
-@pytest.mark.parametrize("N", [2, 127, 129, 513, 1025])
+@pytest.mark.parametrize("N", [2, 63, 65, 127, 129, 513, 1025])
 @pytest.mark.parametrize("model", PLANAR)
 def test_force_over_softenings(model, N, eps):
     q, _ = inputs.default_state(model, N, 50 + N)
@@ -57,6 +57,17 @@ def test_ring_force_over_softenings(N, eps):
     dd = sh * sh + 0.5 * eps
     tol = (2.0**-52 * (dd**-1.5 + 3 * S * sh * dd**-2.5) + 1e-14 * S * dd**-1.5).sum(1) / (8 * N)
     assert np.all(np.abs(_force(1, q, eps) - _force(1, q, eps, 0)) <= tol)
+
+
+@pytest.mark.parametrize("N", [9_999, 10_000, 10_001, 262_144, 262_145])
+@pytest.mark.parametrize("model", [1] + PLANAR)
+def test_force_at_the_kernel_shapes_edges(model, N):
+    """Sampled rows on both sides of the sizes where the tile shape changes."""
+    q, _ = inputs.default_state(model, N, 50)
+    f = _force(model, q, 1e-3).reshape(-1, N)
+    rows = np.unique(np.concatenate([[0, 63, 64, 127, 128, N - 1], np.linspace(0, N - 1, 20).astype(np.int64)]))
+    fo, scale = ora.force_rows(model, q, rows, 1e-3, True)
+    assert np.all(np.abs(f[:, rows] - fo) <= 1e-12 * scale)
 
 
 @pytest.mark.parametrize("scale", [1e-9, 1e-3, 30.0, 1e4, 1e7])
