@@ -251,6 +251,7 @@ void md_free(md_ctx *c) {
   dev_free(c->sym_rowfull);
   dev_free(c->sym_colslot);
   dev_free(c->sym_chunks);
+  dev_free(c->fx_vmax);
   destroy_step_graphs(c);
   dev_free(c->red);
   dev_free(c->gw);

@@ -171,6 +171,18 @@ FX_FN void square_sum(const u32 (&yh)[D], const u32 (&yl)[D], const int (&ex)[D]
   es = 2 * E - 1018 - z;
 }
 
+// -2 / s as a double (rounded), from R = 2^62 / ms and the biased exponent es of s
+FX_FN double minus_two_over(u64 R, int es) {
+  const u64 b = ((u64)(u32)(2046 - es) << 52) + ((R + 256) >> 9) - (1ull << 52) + (1ull << 63);
+#ifdef __CUDA_ARCH__
+  return __longlong_as_double((long long)b);
+#else
+  double d;
+  memcpy(&d, &b, 8);
+  return d;
+#endif
+}
+
 // Mantissa of 1/s for s = ms 2^(es - 1023), ms = Mh:Ml 2^-63 in [1, 2): 2^62 / ms as an
 // integer in (2^61, 2^62].  Seed r0 (24 bits), its defect n = ms r0 - 1 exact to 2^-62
 // (|n| < 2^-21), 1/ms = r0 (1 - n + n^2): relative error below 2^-58 (the n^3 term is below

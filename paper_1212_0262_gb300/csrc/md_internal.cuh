@@ -87,6 +87,8 @@ struct md_ctx {
   size_t sym_colslot_bytes = 0;
   double *sym_chunks = nullptr;   // and chunk sums of the column partials
   size_t sym_chunk_bytes = 0;
+  unsigned *fx_vmax = nullptr;    // integer reverse stages: the largest |v| of this stage and the next (ping-pong)
+  int fx_vcur = 0;
 
   // reductions (energies)
   double *red = nullptr;
@@ -214,6 +216,11 @@ int ensure_pair_buffers(md_ctx *c, int TI, int P, int nacc);       // stream-K s
 // sym.cu (Newton's-third-law variant of the FP32 forward stages)
 bool sym_applies(const md_ctx *c);
 int sym_pair_stage(md_ctx *c, int mode, double kick, double drift, double *fout);
+
+// and of the FP64 2D reverse and tangent stages (STAGE_ADJOINT, STAGE_TANGENT)
+bool sym_reverse_applies(const md_ctx *c);
+int sym_reverse_stage(md_ctx *c, int mode, double kick, double undo, double drift, double *lq, double *lp,
+                      double *epsacc);
 
 // sheet.cu: the symmetric form of the sheets at eps = 0, by counting ranks
 bool sheet_rank_applies(const md_ctx *c);

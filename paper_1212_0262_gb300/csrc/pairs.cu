@@ -552,6 +552,7 @@ int reverse_pair_launch(md_ctx *c, PairArgs a) {
 
 int pair_adjoint_stage(md_ctx *c, double b_adj, double b_undo, double drift, double *lq, double *lp,
                        double *epsacc) {
+  if (sym_reverse_applies(c)) return sym_reverse_stage(c, STAGE_ADJOINT, b_adj, b_undo, drift, lq, lp, epsacc);
   PairArgs a{};
   a.kick = b_adj;
   a.undo = b_undo;
@@ -563,6 +564,7 @@ int pair_adjoint_stage(md_ctx *c, double b_adj, double b_undo, double drift, dou
 }
 
 int pair_tangent_stage(md_ctx *c, double kick, double drift, double *dq, double *dp) {
+  if (sym_reverse_applies(c)) return sym_reverse_stage(c, STAGE_TANGENT, kick, 0.0, drift, dq, dp, nullptr);
   PairArgs a{};
   a.kick = kick;
   a.drift = drift;

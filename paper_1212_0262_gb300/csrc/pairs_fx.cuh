@@ -408,4 +408,206 @@ struct RingFx {
   }
 };
 
+// ------------------------------------------------------------ reverse 2D
+// Reverse and tangent stages of 2D (w = v_i - v_j, v = lambda_p or dq) in the
+// Newton's-third-law form: per pair
+//   f = d / s,  j = (w - 2 d (d.w) / s) / s,  e = d / s^2,
+// all antisymmetric.  d, w, d.w, and w - 2 d (d.w)/s are FP64 (9 operations; 22 per ordered
+// pair in GravF64Adj); the reciprocal, the products and the sums are integers.  The sums of j
+// have a unit that follows from the largest |v| (vmax, found before the stage).  Bound by the
+// FP64 pipe (78% at N = 16,384).  A reverse stage at N = 8,192: 2.9 ms one-sided in FP64, 0.69
+// here; a gradient of 4 steps there 41.4 -> 12.6 ms.
+template <int R_, int TJ_>
+struct FxGrav2DAdj {
+  using Fwd = FxGrav<2, R_, TJ_>;
+  static constexpr bool FX = true;
+  static constexpr int THREADS = NT, MINB = R_ == 1 ? 4 : 3;
+  using ColT = double;
+  static constexpr int R = R_, TJ = TJ_, NACC = 6, JB = RecordBytes<MD_GRAV2D, false, true>::value;
+  static constexpr bool MASK = false;
+  static constexpr int NR = R;
+  static constexpr int FMT = 0;
+  static constexpr int COL_BYTES = (NT / 32) * TJ * NACC * (int)sizeof(uint4);
+  static constexpr int STAGE_BYTES = 16;
+  __device__ static int row_of(int r) { return r * NT + (int)threadIdx.x; }
+  struct State {
+    double x[R][2], v[R][2];
+    fx64::Acc96 acc[R][NACC];
+    FxRowSums<R * NACC> rows;
+    int units;
+    bool wild;
+  };
+  // exponent bound of |v|: |v_d| < 2^ev
+  __device__ static int vexp(const PairArgs &a) { return max((int)(*a.vmax >> 20) - 1022, -800); }
+  // |v| too large (or not finite) or, not all zero, too small for the exponents used here
+  __device__ static bool v_wild(const PairArgs &a) {
+    const unsigned m = *a.vmax;
+    return m >= (1322u << 20) || (m != 0u && m < (223u << 20));
+  }
+  // units of the sums of f, j, e: |f| <= 2^(-half - 1), |j| <= 2^(ev + 2 - 2 half),
+  // |e| <= 0.325 eps^(-3/2) <= 2^(-3 half - 1), each 2^83 units at most
+  __device__ static int lsb_of(int kind, int half, int ev) {
+    return kind == 0 ? -82 - half : kind == 1 ? ev - 81 - 2 * half : -84 - 3 * half;
+  }
+  __device__ static int lsb(const PairArgs &a, int d) { return lsb_of(d >> 1, Fwd::half_exp(a), vexp(a)); }
+  __device__ static void load(State &st, const void *mirror, int64_t i0, const PairArgs &a, double *rowsm) {
+    const int half = Fwd::half_exp(a);
+    st.wild = v_wild(a);
+    fx_clear<State, R, NACC>(st, rowsm);
+#pragma unroll
+    for (int r = 0; r < R; r++) {
+      const double4_16a m = ((const double4_16a *)mirror)[i0 + row_of(r)];
+      st.x[r][0] = m.x;
+      st.x[r][1] = m.y;
+      st.v[r][0] = m.z;
+      st.v[r][1] = m.w;
+      st.wild = st.wild || Fwd::out_of_range(m.x, half) || Fwd::out_of_range(m.y, half);
+    }
+  }
+  __device__ static void flush(State &st, const PairArgs &a) {
+#pragma unroll
+    for (int r = 0; r < R; r++)
+#pragma unroll
+      for (int d = 0; d < NACC; d++) {
+        st.rows.at(r * NACC + d) += fx64::total96(st.acc[r][d], lsb(a, d));
+        st.acc[r][d] = fx64::Acc96{0u, 0u, 0u};
+      }
+    st.units = 0;
+  }
+  __device__ static void total(const State &st, int r, double *out) {
+#pragma unroll
+    for (int d = 0; d < NACC; d++) out[d] = st.rows.at(r * NACC + d);
+  }
+  // half a record, (x, y) or (vx, vy)
+  __device__ static bool stage(const unsigned char *tile, int ch, unsigned char *, const PairArgs &a) {
+    const double2 m = ((const double2 *)tile)[ch];
+    const int half = Fwd::half_exp(a);
+    return (ch & 1) == 0 && (Fwd::out_of_range(m.x, half) || Fwd::out_of_range(m.y, half));
+  }
+  template <bool COL>
+  __device__ static void unit(State &st, const unsigned char *smb, const unsigned char *, const PairArgs &a,
+                              unsigned char *colraw, int64_t, int64_t) {
+    const double4_16a *sm = (const double4_16a *)smb;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, half = Fwd::half_exp(a);
+    const fx64::Soft eps = fx64::soft_of(a.epsd);
+    // shifts: f k = es - ex + kf, j k = es - ex(g) + kj, e k = 2 es - ex + ke
+    const int kf = 9 - half, kj = vexp(a) + 10 - 2 * half, ke = -1018 - 3 * half;
+    uint4 *colsm = (uint4 *)colraw + w * TJ * NACC;
+#pragma unroll 1
+    for (int j = 0; j < TJ; j++) {
+      const double4_16a o = sm[j];
+      fx64::Acc96 col[NACC];
+#pragma unroll
+      for (int c = 0; c < NACC; c++) col[c] = fx64::Acc96{0u, 0u, 0u};
+#pragma unroll
+      for (int r = 0; r < R; r++) {
+        const double d[2] = {st.x[r][0] - o.x, st.x[r][1] - o.y}, v[2] = {st.v[r][0] - o.z, st.v[r][1] - o.w};
+        unsigned yh[2], yl[2], Mh, Ml;
+        int ex[2], es;
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+          ex[c] = (int)((fx64::hi_word(d[c]) >> 20) & 0x7ffu);
+          fx64::mantissa62(fx64::hi_word(d[c]), fx64::lo_word(d[c]), yh[c], yl[c]);
+        }
+        fx64::square_sum<2>(yh, yl, ex, eps, Mh, Ml, es);
+        const unsigned long long inv = fx64::rcp_mantissa(Mh, Ml);
+        const double m2q = fma(d[1], v[1], d[0] * v[0]) * fx64::minus_two_over(inv, es);
+        unsigned gh[2], gl[2], hg[2];
+        int k[6];
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+          const double g = fma(m2q, d[c], v[c]);
+          hg[c] = fx64::hi_word(g);
+          fx64::mantissa62(hg[c], fx64::lo_word(g), gh[c], gl[c]);
+          k[c] = es + kf - ex[c];
+          k[2 + c] = es + kj - (int)((hg[c] >> 20) & 0x7ffu);
+          k[4 + c] = 2 * es + ke - ex[c];
+        }
+        const bool small = ((unsigned)(k[0] | k[1] | k[2] | k[3] | k[4] | k[5])) < 32u;
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+          unsigned w2[3], w1[3], w0[3];
+          fx64::mul_mantissa(yh[c], yl[c], inv, w2[0], w1[0], w0[0]);
+          fx64::mul_mantissa(gh[c], gl[c], inv, w2[1], w1[1], w0[1]);
+          fx64::mul_mantissa(w2[0], w1[0], inv, w2[2], w1[2], w0[2]);  // the product of f again
+          const unsigned sd = (unsigned)((int)fx64::hi_word(d[c]) >> 31), sg = (unsigned)((int)hg[c] >> 31);
+#pragma unroll
+          for (int t = 0; t < 3; t++) {
+            const int kk = k[2 * t + c];
+            unsigned sgn = t == 1 ? sg : sd;
+            if (__builtin_expect(small, 1)) {
+              w0[t] = fx64::shf_r(w0[t], w1[t], kk);
+              w1[t] = fx64::shf_r(w1[t], w2[t], kk);
+              w2[t] >>= kk;
+            } else {
+              fx64::shift96_any(w2[t], w1[t], w0[t], kk);
+              if ((w2[t] | w1[t] | w0[t]) == 0u) sgn = 0u;
+            }
+            fx_add<COL>(sgn, w2[t], w1[t], w0[t], st.acc[r][2 * t + c], col[2 * t + c]);
+          }
+        }
+      }
+      if (COL) {
+#pragma unroll
+        for (int c = 0; c < NACC; c++) {
+          const uint4 s = fx_warp_sum(col[c]);
+          if (lane == 0) colsm[NACC * j + c] = s;
+        }
+      }
+    }
+    if (++st.units == kFxFlush) flush(st, a);
+  }
+  // the unit in FP64 (GravF64Adj's terms), columns reduced over the warp as doubles
+  template <bool COL>
+  __device__ static void unit_wild(State &st, const unsigned char *smb, const PairArgs &a, unsigned char *colraw,
+                                   int64_t, int64_t) {
+    const double4_16a *sm = (const double4_16a *)smb;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    double *colsm = (double *)colraw + w * TJ * NACC;
+#pragma unroll 1
+    for (int j = 0; j < TJ; j++) {
+      const double4_16a o = sm[j];
+      double col[NACC];
+#pragma unroll
+      for (int c = 0; c < NACC; c++) col[c] = 0.0;
+#pragma unroll
+      for (int r = 0; r < R; r++) {
+        const double dx = st.x[r][0] - o.x, dy = st.x[r][1] - o.y, wx = st.v[r][0] - o.z, wy = st.v[r][1] - o.w;
+        const double inv = rcp_nr(fma(dx, dx, fma(dy, dy, a.epsd))), inv2 = inv * inv;
+        const double m2u = -2.0 * fma(dy, wy, dx * wx) * inv2;
+        const double t[NACC] = {dx * inv, dy * inv, fma(m2u, dx, wx * inv), fma(m2u, dy, wy * inv), dx * inv2, dy * inv2};
+#pragma unroll
+        for (int c = 0; c < NACC; c++) {
+          st.rows.at(r * NACC + c) += t[c];
+          col[c] += t[c];
+        }
+      }
+      if (COL) {
+#pragma unroll
+        for (int c = 0; c < NACC; c++) {
+          double s = col[c];
+#pragma unroll
+          for (int m = 16; m > 0; m >>= 1) s += __shfl_xor_sync(0xffffffffu, s, m);
+          if (lane == 0) colsm[NACC * j + c] = s;
+        }
+      }
+    }
+  }
+  __device__ static double column(const unsigned char *colraw, int idx, bool wild, const PairArgs &a) {
+    return fx_column<TJ, NACC>(colraw, idx, wild, lsb(a, idx % NACC));
+  }
+};
+
+// Largest |v_k| as the high word of a double into *cur (zero before); *next = 0 for the next
+// stage's.  A NaN has the largest high word.
+__global__ void fx_vmax_kernel(const double *__restrict__ v, int64_t n, unsigned *cur, unsigned *next) {
+  unsigned m = 0u;
+  const int64_t G = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += G)
+    m = max(m, fx64::hi_word(v[i]) & 0x7fffffffu);
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) atomicMax(cur, m);
+  if (blockIdx.x == 0 && threadIdx.x == 0) *next = 0u;
+}
+
 }  // namespace

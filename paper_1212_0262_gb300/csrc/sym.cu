@@ -359,11 +359,27 @@ int launch_sym(md_ctx *c, PairArgs a) {
   a.slots = c->sk_slots;
   a.tickets = c->sk_tickets;
   a.sched = pair_sched(c);
+  if constexpr (MODE == STAGE_ADJOINT || MODE == STAGE_TANGENT) {
+    // the largest |v| of the records (lambda_p, or dq), for the unit of the sums of j
+    if (!c->fx_vmax) {
+      c->fx_vmax = (unsigned *)dev_alloc(2 * sizeof(unsigned));
+      if (!c->fx_vmax) return set_err(c, MD_ENOMEM, "reverse stage scratch");
+      MD_CUDA(c, cudaMemsetAsync(c->fx_vmax, 0, 2 * sizeof(unsigned), c->stream));
+    }
+    const int64_t n = (int64_t)c->dim * c->N;
+    const int64_t g = std::min<int64_t>((n + 255) / 256, c->nsm);
+    a.vmax = c->fx_vmax + c->fx_vcur;
+    fx_vmax_kernel<<<(int)g, 256, 0, c->stream>>>(MODE == STAGE_ADJOINT ? a.lp : a.lq, n, c->fx_vmax + c->fx_vcur,
+                                                 c->fx_vmax + (1 - c->fx_vcur));
+    MD_LAUNCHED(c);
+    c->fx_vcur = 1 - c->fx_vcur;
+  }
   kern<<<(int)G, THR, 0, c->stream>>>(a, s);
   MD_LAUNCHED(c);
   sym_finish_kernel<Pol, MODEL, MIXED, MODE><<<a.n_it * s.nc, kFinishThreads, 0, c->stream>>>(a, s);
   MD_LAUNCHED(c);
-  if (MODE == STAGE_KICK_DRIFT) c->mirror_cur = 1 - c->mirror_cur;
+  if (MODE == STAGE_KICK_DRIFT || ((MODE == STAGE_ADJOINT || MODE == STAGE_TANGENT) && a.drift != 0.0))
+    c->mirror_cur = 1 - c->mirror_cur;
   return MD_OK;
 }
 
@@ -459,4 +475,31 @@ int sym_pair_stage(md_ctx *c, int mode, double kick, double drift, double *fout)
   if (c->model == MD_SHEET1D)
     return mixed ? sym_mode<MD_SHEET1D, true>(c, mode, a) : sym_mode<MD_SHEET1D, false>(c, mode, a);
   return mixed ? sym_mode<MD_GRAV2D, true>(c, mode, a) : sym_mode<MD_GRAV2D, false>(c, mode, a);
+}
+
+// Reverse and tangent stages in the symmetric form: FP64 2D with the integer pair arithmetic,
+// while its six column partials fit.
+bool sym_reverse_applies(const md_ctx *c) {
+  if (!c->pt.symmetric || c->prec != MD_FP64 || c->pt.r_fp64 != 2) return false;
+  if (c->model != MD_GRAV2D || !fx_grav_applies(c->eps)) return false;
+  const int64_t TI = c->N <= kFxSmall ? 128 : 256, TJ = 64, m = TI / TJ, n_it = (c->N + TI - 1) / TI;
+  return (size_t)sym_rowstart(n_it, m * n_it, (int)m) * TJ * 6 * sizeof(double) <= kSymMaxColBytes;
+}
+
+template <int MODE>
+int sym_reverse(md_ctx *c, const PairArgs &a) {
+  if (c->N <= kFxSmall) return launch_sym<FxGrav2DAdj<1, 64>, MD_GRAV2D, false, MODE>(c, a);
+  return launch_sym<FxGrav2DAdj<2, 64>, MD_GRAV2D, false, MODE>(c, a);
+}
+
+int sym_reverse_stage(md_ctx *c, int mode, double kick, double undo, double drift, double *lq, double *lp,
+                      double *epsacc) {
+  PairArgs a{};
+  a.kick = kick;
+  a.undo = undo;
+  a.drift = drift;
+  a.lq = lq;
+  a.lp = lp;
+  a.epsacc = epsacc;
+  return mode == STAGE_ADJOINT ? sym_reverse<STAGE_ADJOINT>(c, a) : sym_reverse<STAGE_TANGENT>(c, a);
 }

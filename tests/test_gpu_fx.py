@@ -133,3 +133,53 @@ def test_potential_over_scales(model, scale):
     q = inputs.default_state(model, 400, 3)[0] * scale
     q[5] *= 1e4
     _check_potential(model, q, 1e-4)
+
+
+def _tangent(q, v, eps, symmetric, dt=0.01):
+    with System(2, q.size // 2, eps, dt, 1, precision="fp64") as s:
+        s.set_tuning("symmetric", symmetric)
+        s.set_state(q, np.zeros_like(q))
+        return s.tangent_step(1, v, np.zeros_like(v))
+
+
+TANGENTS = {
+    "random": lambda g, n: g.standard_normal(n),
+    "one particle": lambda g, n: np.eye(1, n, 5)[0],
+    "wide range": lambda g, n: np.exp(30 * g.standard_normal(n)),
+    "zero": lambda g, n: np.zeros(n),
+    "tiny": lambda g, n: 1e-290 * g.standard_normal(n),
+    "huge": lambda g, n: 1e150 * g.standard_normal(n),
+}
+
+
+@pytest.mark.parametrize("kind", TANGENTS)
+@pytest.mark.parametrize("N,eps", [(1, 1e-3), (2, 1e-3), (65, 1.0), (129, 1e-4), (700, 2.0**-28), (10_001, 1e-3)])
+def test_tangent_stages_equal_the_one_sided_kernel(N, eps, kind):
+    """One step of the tangent dynamics against the one-sided FP64 kernel: per kick each
+    side's J v is within 1e-13 of sum_j |J_ij| (|v_i| + |v_j|), |J_ij| <= 3 / s_ij <= 3 / eps,
+    of which the largest row bounds the difference of dp (and, drifted, of dq); the state's own
+    difference (1e-13 of the forces) enters the next kicks' J the same way.  Four kicks,
+    |b| summing to 2.4, and a factor 4 for the growth within the step."""
+    g = np.random.default_rng(N)
+    q, _ = inputs.default_state(2, N, 3)
+    if N > 600:
+        q[7], q[N + 9] = 1e9, -3e4  # outliers: units in FP64
+    v = TANGENTS[kind](g, 2 * N)
+    x, a = q.reshape(2, N), np.abs(v).reshape(2, N).sum(0)
+    S = 0.0
+    for i in range(0, N, 500):
+        d = x[:, i : i + 500, None] - x[:, None, :]
+        s = (d * d).sum(0) + eps
+        S = max(S, ((a[i : i + 500, None] + a) / s).sum(1).max() * 6.0 / N)
+    tol = 1e-13 * 4 * 2.4 * 0.01 * S + 1e-15 * np.abs(v).max()
+    for got, want in zip(_tangent(q, v, eps, 1), _tangent(q, v, eps, 0)):
+        assert np.abs(got - want).max() <= tol
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_a_non_finite_tangent_reaches_every_particle(bad):
+    q, _ = inputs.default_state(2, 300, 3)
+    v = np.ones(600)
+    v[40] = bad
+    dq, dp = _tangent(q, v, 1e-3, 1)
+    assert not np.isfinite(dp[:300]).any()
