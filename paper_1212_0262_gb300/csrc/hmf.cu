@@ -9,10 +9,8 @@
 // so the state is read once and written once per stage (32 B per particle).
 // The paper stores sin and cos in global memory and reloads them.  The mixed
 // path recomputes them instead (FP32 polynomials are cheaper than 32 B more
-// traffic); the FP64 path is bound by the FP64 pipe (an FP64 sincos is tens of
-// DFMA at 2.3 per SM per clock), so it keeps (cos, sin) of the current angles in
-// a buffer, as the paper does, and computes one FP64 sincos per particle-stage
-// instead of two.
+// traffic); the FP64 path keeps (cos, sin) of the current angles in a buffer, as the
+// paper does, and computes one sine and cosine per particle-stage instead of two.
 //
 // Consecutive stages sweep the particles in opposite directions: the last part of
 // a stage's writes is still in L2 when the next stage starts on it.
@@ -26,6 +24,7 @@
 
 #include "md_internal.cuh"
 #include "sincos_fp64.cuh"
+#include "sincos_fx.cuh"
 
 namespace {
 
@@ -58,17 +57,49 @@ __device__ __forceinline__ void load_sincos_tab(double2 *sm) {
   __syncthreads();
 }
 
-// c 2^52 rounded to the nearest integer (halves up in magnitude), for |c| <= 1, from
-// the bits of c with integer instructions only; 0 for zero, subnormal or non-finite c.
-// The FP64 stages add their cosines and sines in this fixed point (exactly, on the
-// integer pipe) and move the per-thread sums into FP64 every kFlush angles.
-__device__ __forceinline__ long long fix52(double c) {
-  const long long b = __double_as_longlong(c);
-  const int e = (int)(b >> 52) & 0x7ff;
-  const int sh = 1023 - e;  // c 2^52 = significand >> sh
-  const long long m = (b & 0x000fffffffffffffLL) | 0x0010000000000000LL;
-  const long long v = (sh < 0 || sh > 53) ? 0LL : (m + ((1LL << sh) >> 1)) >> sh;
-  return b < 0 ? -v : v;
+// The FP64 stages hold (cos, sin) of the current angles as 62-bit fixed-point numbers
+// (sincos_fx.cuh), 16 bytes per particle, so that the stage's force, its sine and cosine and
+// the magnetization sums are integer arithmetic; the kick and the drift are its FP64
+// operations (12 with the sine and cosine of sincos_fp64.cuh and an FP64 force, which bound
+// the stage).  Per stage at N = 5e7: 1149 -> 582 us, 3.2 GB at 81% of the copy rate; the
+// integer pipe is half busy, the next pair's loads run ahead of the arithmetic (604 us without).
+// A non-finite angle is marked by kNoAngle: its force is NaN, and the sums of the stages leave
+// it out.
+__device__ scfx::Entry g_sincos_fx[kTabN];
+constexpr int kNoAngle = (int)0x80000000;
+
+__device__ __forceinline__ void load_sincos_fx(scfx::Entry *sm) {
+  for (int k = threadIdx.x; k < kTabN; k += blockDim.x) sm[k] = g_sincos_fx[k];
+  __syncthreads();
+}
+
+// (cos, sin) of th as stored (cos.h, cos.l, sin.h, sin.l), and their sums in units of 2^-54
+__device__ __forceinline__ int4 angle_fx(double th, const scfx::Entry *tab, long long &aci, long long &asi) {
+  fx64::i64 s62, c62;
+  if (!scfx::sincos_fx(th, tab, s62, c62)) {
+    if (!(fabs(th) <= 1.7976931348623157e308)) return make_int4(kNoAngle, 0, 0, 0);
+    double s, c;
+    sincos(th, &s, &c);
+    s62 = __double2ll_rn(s * 0x1p62);
+    c62 = __double2ll_rn(c * 0x1p62);
+  }
+  aci += (c62 + 128) >> 8;
+  asi += (s62 + 128) >> 8;
+  const fx64::Limbs c = scfx::split(c62), s = scfx::split(s62);
+  return make_int4(c.h, c.l, s.h, s.l);
+}
+
+// The FP64 stages' magnetization: as limbs (My, -Mx) for the integer force
+struct HmfM {
+  fx64::Limbs my, nmx;
+  bool fx;  // finite and of ordinary size
+};
+__device__ __forceinline__ HmfM hmf_m_of(double mx, double my) {
+  HmfM m;
+  m.fx = fabs(mx) < 1.5 && fabs(my) < 1.5;
+  m.my = fx64::limbs_of(m.fx ? my : 0.0);
+  m.nmx = fx64::limbs_of(m.fx ? -mx : 0.0);
+  return m;
 }
 
 struct HmfArgs {
@@ -81,7 +112,7 @@ struct HmfArgs {
   double *m_out;     // (sum cos, sum sin) of the new angles
   unsigned *ticket;
   double *fout;  // STAGE_FORCE_ONLY output
-  double2 *cs;   // FP64 path: (cos, sin) of the current angles, rewritten by drifts
+  int4 *cs;      // FP64 path: (cos, sin) of the current angles, rewritten by drifts
   int rev;       // sweep the particles from the top end down
   int nsum;      // row shard: m_in holds nsum (sum cos, sum sin) pairs, one per rank
 };
@@ -93,49 +124,50 @@ __device__ __forceinline__ double hmf_force_fp64(double c, double s, double mx, 
   return invN == 1.0 ? 0.0 : fma(c, my, -(s * mx));
 }
 
-// One particle of a stage.  MIXED: FP64 state update, FP32 sine/cosine of the
+// One particle of a mixed stage: FP64 state update, FP32 sine/cosine of the
 // FP64-range-reduced angle; the new angle's reduced value is carried in FP32.
-template <bool MIXED, int MODE>
-__device__ __forceinline__ void hmf_particle(double &th, double &pp, const HmfArgs &a, float mxf,
-                                             float myf, double mx, double my, float dtf, float &acf,
-                                             float &asf, long long &aci, long long &asi, int64_t i,
-                                             const double2 *tab) {
-  if (MIXED) {
-    // Only the kick and the drift use the FP64 pipe (two DFMA per particle):
-    // range reduction and float<->double conversions move bits on the integer
-    // pipe, and the sines and cosines are FP32 polynomials.
-    float r = reduce_2pi_f(th);
-    float s, c;
-    sincos_small(r, &s, &c);
-    float f = __fsub_rn(__fmul_rn(c, myf), __fmul_rn(s, mxf));
-    if (MODE == STAGE_FORCE_ONLY) {
-      a.fout[i] = f2d_bits(f);
-      return;
-    }
-    pp = fma(a.kick, f2d_bits(f), pp);
-    if (MODE == STAGE_KICK_DRIFT) {
-      th = fma(a.drift, pp, th);
-      float r2 = fmaf(dtf, d2f_trunc_bits(pp), r);
-      sincos_small(r2, &s, &c);
-      acf += c;
-      asf += s;
-    }
-  } else {
-    const double2 cs = a.cs[i];
-    const double f = hmf_force_fp64(cs.x, cs.y, mx, my, a.invN);
-    if (MODE == STAGE_FORCE_ONLY) {
-      a.fout[i] = f;
-      return;
-    }
-    pp = fma(a.kick, f, pp);
-    if (MODE == STAGE_KICK_DRIFT) {
-      th = fma(a.drift, pp, th);
-      double s, c;
-      sincos_tab(th, tab, &s, &c);
-      a.cs[i] = make_double2(c, s);
-      aci += fix52(c);
-      asi += fix52(s);
-    }
+// Only the kick and the drift use the FP64 pipe (two DFMA per particle): range
+// reduction and float<->double conversions move bits on the integer pipe, and the
+// sines and cosines are FP32 polynomials.
+template <int MODE>
+__device__ __forceinline__ void hmf_particle_mixed(double &th, double &pp, const HmfArgs &a, float mxf, float myf,
+                                                   float dtf, float &acf, float &asf, int64_t i) {
+  float r = reduce_2pi_f(th);
+  float s, c;
+  sincos_small(r, &s, &c);
+  float f = __fsub_rn(__fmul_rn(c, myf), __fmul_rn(s, mxf));
+  if (MODE == STAGE_FORCE_ONLY) {
+    a.fout[i] = f2d_bits(f);
+    return;
+  }
+  pp = fma(a.kick, f2d_bits(f), pp);
+  if (MODE == STAGE_KICK_DRIFT) {
+    th = fma(a.drift, pp, th);
+    float r2 = fmaf(dtf, d2f_trunc_bits(pp), r);
+    sincos_small(r2, &s, &c);
+    acf += c;
+    asf += s;
+  }
+}
+
+// One particle of an FP64 stage; cs: its (cos, sin), rewritten by a drift.
+template <int MODE>
+__device__ __forceinline__ void hmf_particle_fp64(double &th, double &pp, int4 &cs, const HmfArgs &a, const HmfM &m,
+                                                  double mx, double my, long long &aci, long long &asi, int64_t i,
+                                                  const scfx::Entry *tab) {
+  const fx64::Limbs c{cs.x, cs.y}, s{cs.z, cs.w};
+  double f = scfx::to_double60(fx64::dot2(c, s, m.my, m.nmx));  // cos My - sin Mx
+  if (a.invN == 1.0) f = 0.0;  // a lone particle's self-term
+  if (!m.fx) f = hmf_force_fp64((double)scfx::join(c.h, c.l) * 0x1p-62, (double)scfx::join(s.h, s.l) * 0x1p-62, mx, my, a.invN);
+  if (cs.x == kNoAngle) f = __longlong_as_double(0x7ff8000000000000LL);
+  if (MODE == STAGE_FORCE_ONLY) {
+    a.fout[i] = f;
+    return;
+  }
+  pp = fma(a.kick, f, pp);
+  if (MODE == STAGE_KICK_DRIFT) {
+    th = fma(a.drift, pp, th);
+    cs = angle_fx(th, tab, aci, asi);
   }
 }
 
@@ -171,8 +203,10 @@ __device__ __forceinline__ void grid_finish(double sc, double ss, double *partia
 
 // SHARD: the magnetization is the sum of every rank's pair in m_in, added in rank
 // order (the same value on every rank), over the whole system's N (invN).
+// Register budgets of the kick-drift stages: mixed 4 CTAs per SM (64 registers; 80 and 3 CTAs: 262
+// against 248 us per stage at N = 5e7), FP64 3 (80; 112 and 2 CTAs: 750 against 566 us).
 template <bool MIXED, int MODE, bool SHARD = false>
-__global__ void __launch_bounds__(NT) hmf_stage_kernel(HmfArgs a) {
+__global__ void __launch_bounds__(NT, MODE != STAGE_KICK_DRIFT ? 1 : MIXED ? 4 : 3) hmf_stage_kernel(HmfArgs a) {
   double sx = a.m_in[0], sy = a.m_in[1];
   if constexpr (SHARD)
     for (int r = 1; r < a.nsum; r++) {
@@ -180,8 +214,10 @@ __global__ void __launch_bounds__(NT) hmf_stage_kernel(HmfArgs a) {
       sy += a.m_in[2 * r + 1];
     }
   const double mx = sx * a.invN, my = sy * a.invN;
-  extern __shared__ double2 tab[];  // FP64 kick-drift stages: the sine/cosine table (kTabBytes)
-  if constexpr (!MIXED && MODE == STAGE_KICK_DRIFT) load_sincos_tab(tab);
+  extern __shared__ __align__(16) unsigned char tabraw[];  // FP64 kick-drift stages: the sine/cosine table (kTabBytes)
+  scfx::Entry *tab = (scfx::Entry *)tabraw;
+  if constexpr (!MIXED && MODE == STAGE_KICK_DRIFT) load_sincos_fx(tab);
+  const HmfM m = hmf_m_of(mx, my);
   const float mxf = (float)mx, myf = (float)my, dtf = (float)a.drift;
   float acf = 0.f, asf = 0.f;
   long long aci = 0, asi = 0;
@@ -196,27 +232,54 @@ __global__ void __launch_bounds__(NT) hmf_stage_kernel(HmfArgs a) {
   const int64_t block = (int64_t)(kFlush / (2 * UNROLL)) * UNROLL * G;
   for (int64_t kb = t0; kb < npairs; kb += block) {
   const int64_t kend = kb + block < npairs ? kb + block : npairs;
-  for (int64_t k = kb; k < kend; k += UNROLL * G) {
-    double2 qv[UNROLL], pv[UNROLL];
+  if constexpr (MIXED) {
+    for (int64_t k = kb; k < kend; k += UNROLL * G) {
+      double2 qv[UNROLL], pv[UNROLL];
 #pragma unroll
-    for (int u = 0; u < UNROLL; u++) {
-      const int64_t kk = k + u * G;
-      const int64_t ix = a.rev ? npairs - 1 - kk : kk;
-      if (kk < npairs) {
-        qv[u] = q2[ix];
-        pv[u] = p2[ix];
+      for (int u = 0; u < UNROLL; u++) {
+        const int64_t kk = k + u * G;
+        const int64_t ix = a.rev ? npairs - 1 - kk : kk;
+        if (kk < npairs) {
+          qv[u] = q2[ix];
+          pv[u] = p2[ix];
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < UNROLL; u++) {
+        const int64_t kk = k + u * G;
+        const int64_t ix = a.rev ? npairs - 1 - kk : kk;
+        if (kk < npairs) {
+          hmf_particle_mixed<MODE>(qv[u].x, pv[u].x, a, mxf, myf, dtf, acf, asf, 2 * ix);
+          hmf_particle_mixed<MODE>(qv[u].y, pv[u].y, a, mxf, myf, dtf, acf, asf, 2 * ix + 1);
+          if (MODE == STAGE_KICK_DRIFT) q2[ix] = qv[u];
+          if (MODE != STAGE_FORCE_ONLY) p2[ix] = pv[u];
+        }
       }
     }
-#pragma unroll
-    for (int u = 0; u < UNROLL; u++) {
-      const int64_t kk = k + u * G;
-      const int64_t ix = a.rev ? npairs - 1 - kk : kk;
-      if (kk < npairs) {
-        hmf_particle<MIXED, MODE>(qv[u].x, pv[u].x, a, mxf, myf, mx, my, dtf, acf, asf, aci, asi, 2 * ix, tab);
-        hmf_particle<MIXED, MODE>(qv[u].y, pv[u].y, a, mxf, myf, mx, my, dtf, acf, asf, aci, asi, 2 * ix + 1, tab);
-        if (MODE == STAGE_KICK_DRIFT) q2[ix] = qv[u];
-        if (MODE != STAGE_FORCE_ONLY) p2[ix] = pv[u];
+  } else {
+    // one pair ahead: the next pair's 64 bytes are on their way while this one is computed
+    auto at = [&](int64_t kk) { return a.rev ? npairs - 1 - kk : kk; };
+    double2 qn = q2[at(kb)], pn = p2[at(kb)];
+    int4 an = a.cs[2 * at(kb)], bn = a.cs[2 * at(kb) + 1];
+    for (int64_t k = kb; k < kend; k += G) {
+      const int64_t ix = at(k);
+      double2 qv = qn, pv = pn;
+      int4 ca = an, cb = bn;
+      if (k + G < kend) {
+        const int64_t nx = at(k + G);
+        qn = q2[nx];
+        pn = p2[nx];
+        an = a.cs[2 * nx];
+        bn = a.cs[2 * nx + 1];
       }
+      hmf_particle_fp64<MODE>(qv.x, pv.x, ca, a, m, mx, my, aci, asi, 2 * ix, tab);
+      hmf_particle_fp64<MODE>(qv.y, pv.y, cb, a, m, mx, my, aci, asi, 2 * ix + 1, tab);
+      if (MODE == STAGE_KICK_DRIFT) {
+        a.cs[2 * ix] = ca;
+        a.cs[2 * ix + 1] = cb;
+        q2[ix] = qv;
+      }
+      if (MODE != STAGE_FORCE_ONLY) p2[ix] = pv;
     }
   }
   if constexpr (MIXED && MODE == STAGE_KICK_DRIFT) {
@@ -225,15 +288,21 @@ __global__ void __launch_bounds__(NT) hmf_stage_kernel(HmfArgs a) {
     acf = asf = 0.f;
   }
   if constexpr (!MIXED && MODE == STAGE_KICK_DRIFT) {
-    acd += (double)aci * 0x1p-52;
-    asd += (double)asi * 0x1p-52;
+    acd += (double)aci * 0x1p-54;
+    asd += (double)asi * 0x1p-54;
     aci = asi = 0;
   }
   }
   if ((a.N & 1) && t0 == 0) {
     int64_t i = a.N - 1;
     double th = a.q[i], pp = a.p[i];
-    hmf_particle<MIXED, MODE>(th, pp, a, mxf, myf, mx, my, dtf, acf, asf, aci, asi, i, tab);
+    if constexpr (MIXED) {
+      hmf_particle_mixed<MODE>(th, pp, a, mxf, myf, dtf, acf, asf, i);
+    } else {
+      int4 c = a.cs[i];
+      hmf_particle_fp64<MODE>(th, pp, c, a, m, mx, my, aci, asi, i, tab);
+      if (MODE == STAGE_KICK_DRIFT) a.cs[i] = c;
+    }
     if (MODE == STAGE_KICK_DRIFT) a.q[i] = th;
     if (MODE != STAGE_FORCE_ONLY) a.p[i] = pp;
   }
@@ -242,22 +311,45 @@ __global__ void __launch_bounds__(NT) hmf_stage_kernel(HmfArgs a) {
       acd += (double)acf;
       asd += (double)asf;
     } else {
-      acd += (double)aci * 0x1p-52;
-      asd += (double)asi * 0x1p-52;
+      acd += (double)aci * 0x1p-54;
+      asd += (double)asi * 0x1p-54;
     }
     grid_finish(acd, asd, a.partials, a.m_out, a.ticket);
   }
 }
 
+// (cos, sin) of every angle as the FP64 stages read them, and their sums.  A non-finite angle
+// makes the sums NaN.
+__global__ void __launch_bounds__(NT) hmf_prime_fp64_kernel(const double *__restrict__ q, int64_t N, double *partials,
+                                                            double *m_out, unsigned *ticket, int4 *__restrict__ cs) {
+  extern __shared__ __align__(16) unsigned char tabraw[];
+  scfx::Entry *tab = (scfx::Entry *)tabraw;
+  load_sincos_fx(tab);
+  double acd = 0.0, asd = 0.0;
+  const int64_t G = (int64_t)gridDim.x * NT;
+  const int64_t block = (int64_t)kFlush * G;  // kFlush angles per thread, then the FP64 move
+  for (int64_t ib = (int64_t)blockIdx.x * NT + threadIdx.x; ib < N; ib += block) {
+    const int64_t iend = ib + block < N ? ib + block : N;
+    long long aci = 0, asi = 0;
+    for (int64_t i = ib; i < iend; i += G) {
+      const int4 v = angle_fx(q[i], tab, aci, asi);
+      cs[i] = v;
+      if (v.x == kNoAngle) acd = __longlong_as_double(0x7ff8000000000000LL);
+    }
+    acd += (double)aci * 0x1p-54;
+    asd += (double)asi * 0x1p-54;
+  }
+  grid_finish(acd, asd, partials, m_out, ticket);
+}
+
 // (sum cos, sum sin) of the given angles.  MIXED: FP32 sine/cosine after FP64
 // range reduction, FP32 per-thread sums; otherwise FP64 throughout.
 // FP64: use_tab selects the table-driven sine and cosine of the FP64 stages (the table
-// in kTabBytes of dynamic shared memory) over sincos; cs_out (may be NULL) also gets
-// (cos, sin) of every angle.
+// in kTabBytes of dynamic shared memory) over sincos.
 template <bool MIXED>
 __global__ void __launch_bounds__(NT) hmf_sums_kernel(const double *__restrict__ q, int64_t N,
                                                       double *partials, double *m_out, unsigned *ticket,
-                                                      double2 *cs_out, int use_tab) {
+                                                      int use_tab) {
   extern __shared__ double2 tab[];
   if (!MIXED && use_tab) load_sincos_tab(tab);  // use_tab is the same for the whole grid
   float acf = 0.f, asf = 0.f;
@@ -279,7 +371,6 @@ __global__ void __launch_bounds__(NT) hmf_sums_kernel(const double *__restrict__
         sincos_tab(th, tab, &s, &c);
       else
         sincos(th, &s, &c);
-      if (cs_out) cs_out[i] = make_double2(c, s);
       acd += c;
       asd += s;
     }
@@ -322,7 +413,7 @@ int launch_stage(md_ctx *c, double kick, double drift, double *fout) {
   a.m_out = c->hmf_m + 2 * (1 - c->hmf_cur);
   a.ticket = c->hmf_ticket;
   a.fout = fout;
-  a.cs = (double2 *)c->hmf_cs;
+  a.cs = (int4 *)c->hmf_cs;
   // Consecutive stages sweep the state in opposite directions, so a stage starts on
   // the lines the previous one wrote last, which are still in L2 (dirty lines that
   // are overwritten before eviction are never written back either).
@@ -365,12 +456,20 @@ int hmf_sincos_table(md_ctx *c, bool probe) {
     t[k] = make_double2((double)sinl(x), (double)cosl(x));
   }
   MD_CUDA(c, cudaMemcpyToSymbol(g_sincos_tab, t, sizeof t));
+  static scfx::Entry tf[kTabN];
+  for (int k = 0; k < kTabN; k++) {
+    const long double x = (long double)k * pi / (long double)(kTabN / 2);
+    const fx64::Limbs s = scfx::split(llrintl(sinl(x) * 0x1p62L)), co = scfx::split(llrintl(cosl(x) * 0x1p62L));
+    tf[k] = scfx::Entry{s.h, s.l, co.h, co.l};
+  }
+  MD_CUDA(c, cudaMemcpyToSymbol(g_sincos_fx, tf, sizeof tf));
   // the kernels that hold the table in dynamic shared memory (64 KB, above the 48 KB default)
   MD_CUDA(c, cudaFuncSetAttribute(hmf_stage_kernel<false, STAGE_KICK_DRIFT, false>,
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, kTabBytes));
   MD_CUDA(c, cudaFuncSetAttribute(hmf_stage_kernel<false, STAGE_KICK_DRIFT, true>,
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, kTabBytes));
   MD_CUDA(c, cudaFuncSetAttribute(hmf_sums_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTabBytes));
+  MD_CUDA(c, cudaFuncSetAttribute(hmf_prime_fp64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTabBytes));
   done[c->device] = true;
   return MD_OK;
 }
@@ -386,7 +485,7 @@ void hmf_sums_raw(cudaStream_t st, int nsm, int grid_cap, const double *q, int64
   if (g > need) g = need;
   if (g > grid_cap) g = grid_cap;
   if (g < 1) g = 1;
-  hmf_sums_kernel<false><<<(int)g, NT, 0, st>>>(q, N, partials, out2, ticket, nullptr, 0);
+  hmf_sums_kernel<false><<<(int)g, NT, 0, st>>>(q, N, partials, out2, ticket, 0);
 }
 
 int hmf_sums_fp64_of(md_ctx *c, const double *q, double *d_out2) {
@@ -394,7 +493,7 @@ int hmf_sums_fp64_of(md_ctx *c, const double *q, double *d_out2) {
   if (rc) return rc;
   auto kern = hmf_sums_kernel<false>;
   int g = grid_for(c, (const void *)kern, c->N, 0, kTabBytes);
-  kern<<<g, NT, kTabBytes, c->stream>>>(q, c->N, c->hmf_partials, d_out2, c->hmf_ticket, nullptr, 1);
+  kern<<<g, NT, kTabBytes, c->stream>>>(q, c->N, c->hmf_partials, d_out2, c->hmf_ticket, 1);
   MD_LAUNCHED(c);
   return MD_OK;
 }
@@ -407,20 +506,20 @@ int hmf_prime(md_ctx *c) {
   if (c->prec == MD_MIXED) {
     auto kern = hmf_sums_kernel<true>;
     int g = grid_for(c, (const void *)kern, c->N);
-    kern<<<g, NT, 0, c->stream>>>(c->q, c->N, c->hmf_partials, out, c->hmf_ticket, nullptr, 0);
+    kern<<<g, NT, 0, c->stream>>>(c->q, c->N, c->hmf_partials, out, c->hmf_ticket, 0);
     MD_LAUNCHED(c);
   } else {
     // FP64: the sums and the (cos, sin) buffer the FP64 stages read
-    const size_t need = sizeof(double2) * (size_t)c->N;
+    const size_t need = sizeof(int4) * (size_t)c->N;
     if (need > c->hmf_cs_bytes) {
       dev_free(c->hmf_cs);
       c->hmf_cs = (double *)dev_alloc(need);
       c->hmf_cs_bytes = c->hmf_cs ? need : 0;
       if (!c->hmf_cs) return set_err(c, MD_ENOMEM, "HMF (cos, sin) buffer: %zu bytes", need);
     }
-    auto kern = hmf_sums_kernel<false>;
-    int g = grid_for(c, (const void *)kern, c->N, 0, kTabBytes);
-    kern<<<g, NT, kTabBytes, c->stream>>>(c->q, c->N, c->hmf_partials, out, c->hmf_ticket, (double2 *)c->hmf_cs, 1);
+    int g = grid_for(c, (const void *)hmf_prime_fp64_kernel, c->N, 0, kTabBytes);
+    hmf_prime_fp64_kernel<<<g, NT, kTabBytes, c->stream>>>(c->q, c->N, c->hmf_partials, out, c->hmf_ticket,
+                                                           (int4 *)c->hmf_cs);
     MD_LAUNCHED(c);
   }
   c->hmf_m_valid = true;
@@ -448,18 +547,18 @@ int hmf_shard_prime(md_ctx *c) {
   if (c->prec == MD_MIXED) {
     auto kern = hmf_sums_kernel<true>;
     int g = grid_for(c, (const void *)kern, c->N);
-    kern<<<g, NT, 0, c->stream>>>(c->q, c->N, c->hmf_partials, out, c->hmf_ticket, nullptr, 0);
+    kern<<<g, NT, 0, c->stream>>>(c->q, c->N, c->hmf_partials, out, c->hmf_ticket, 0);
   } else {
-    const size_t need = sizeof(double2) * (size_t)c->N;
+    const size_t need = sizeof(int4) * (size_t)c->N;
     if (need > c->hmf_cs_bytes) {
       dev_free(c->hmf_cs);
       c->hmf_cs = (double *)dev_alloc(need);
       c->hmf_cs_bytes = c->hmf_cs ? need : 0;
       if (!c->hmf_cs) return set_err(c, MD_ENOMEM, "HMF (cos, sin) buffer: %zu bytes", need);
     }
-    auto kern = hmf_sums_kernel<false>;
-    int g = grid_for(c, (const void *)kern, c->N, 0, kTabBytes);
-    kern<<<g, NT, kTabBytes, c->stream>>>(c->q, c->N, c->hmf_partials, out, c->hmf_ticket, (double2 *)c->hmf_cs, 1);
+    int g = grid_for(c, (const void *)hmf_prime_fp64_kernel, c->N, 0, kTabBytes);
+    hmf_prime_fp64_kernel<<<g, NT, kTabBytes, c->stream>>>(c->q, c->N, c->hmf_partials, out, c->hmf_ticket,
+                                                           (int4 *)c->hmf_cs);
   }
   MD_LAUNCHED(c);
   c->hmf_m_valid = false;  // md_step's own sums are not kept on a shard
@@ -483,7 +582,7 @@ int launch_shard_stage(md_ctx *c, double kick, double drift, double *fout) {
   a.m_out = c->shard_sums + 2 * (P * (1 - c->shard_cur) + c->shard_rank);
   a.ticket = c->hmf_ticket;
   a.fout = fout;
-  a.cs = (double2 *)c->hmf_cs;
+  a.cs = (int4 *)c->hmf_cs;
   a.rev = c->hmf_rev;
   c->hmf_rev ^= 1;
   auto kern = hmf_stage_kernel<MIXED, MODE, true>;

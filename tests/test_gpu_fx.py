@@ -183,3 +183,13 @@ def test_a_non_finite_tangent_reaches_every_particle(bad):
     v[40] = bad
     dq, dp = _tangent(q, v, 1e-3, 1)
     assert not np.isfinite(dp[:300]).any()
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_a_non_finite_hmf_angle(bad):
+    """The magnetization of the given state, and with it every force, is NaN."""
+    q, p = inputs.default_state(0, 1001, 3)
+    q[500] = bad
+    with System(0, 1001, 0.0, 0.1, 1, precision="fp64") as s:
+        s.set_state(q, p)
+        assert np.isnan(s.force()).all()
