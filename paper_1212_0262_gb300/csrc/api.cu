@@ -466,6 +466,15 @@ int replay_steps(md_ctx *c, const double *k, double h) {
 
 }  // namespace
 
+int run_direction(md_ctx *c, int parity, double h, int now) {
+  const StepGraphKey key = step_key_of(c, h);
+  if (c->run_rev[parity] < 0 || memcmp(&key, &c->run_key[parity], sizeof key) != 0) {
+    c->run_rev[parity] = now;
+    memcpy((void *)&c->run_key[parity], &key, sizeof key);
+  }
+  return c->run_rev[parity];
+}
+
 void destroy_step_graphs(md_ctx *c) {
   for (int k = 0; k < 2; k++)
     if (c->step_graph[k]) {
@@ -483,6 +492,12 @@ int integrate(md_ctx *c, int64_t nsteps) {
   yoshida_coefficients(k);
   const double h = c->dt, B0 = k[0], B1 = k[1], D0 = k[2], D1 = k[3];
   int rc;
+  if (c->model == MD_HMF && c->use_graphs) {
+    bool done = false;
+    const int64_t blocks = graphs_usable(c) ? (nsteps - 1) / kStepGraphSteps : 0;
+    if ((rc = hmf_run(c, nsteps, blocks * kStepGraphSteps, k, h, &done))) return rc;
+    if (done) return hmf_stage(c, STAGE_KICK_ONLY, B0 * h, 0.0, nullptr);
+  }
   if (c->model == MD_HMF) {
     if ((rc = hmf_stage(c, STAGE_KICK_DRIFT, B0 * h, D0 * h, nullptr))) return rc;
     if ((rc = hmf_stage(c, STAGE_KICK_DRIFT, B1 * h, D1 * h, nullptr))) return rc;

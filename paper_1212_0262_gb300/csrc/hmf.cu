@@ -18,6 +18,7 @@
 // Reduction: per-thread sums, warp shuffles and a block tree give one FP64
 // partial per CTA; the last CTA to finish (atomic ticket, no waiting) adds the
 // partials in CTA order, so the result is deterministic.
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include <mutex>
@@ -201,27 +202,20 @@ __device__ __forceinline__ void grid_finish(double sc, double ss, double *partia
   }
 }
 
-// SHARD: the magnetization is the sum of every rank's pair in m_in, added in rank
-// order (the same value on every rank), over the whole system's N (invN).
-// Register budgets of the kick-drift stages: mixed 4 CTAs per SM (64 registers; 80 and 3 CTAs: 262
-// against 248 us per stage at N = 5e7), FP64 3 (80; 112 and 2 CTAs: 750 against 566 us).
-template <bool MIXED, int MODE, bool SHARD = false>
-__global__ void __launch_bounds__(NT, MODE != STAGE_KICK_DRIFT ? 1 : MIXED ? 4 : 3) hmf_stage_kernel(HmfArgs a) {
-  double sx = a.m_in[0], sy = a.m_in[1];
-  if constexpr (SHARD)
-    for (int r = 1; r < a.nsum; r++) {
-      sx += a.m_in[2 * r];
-      sy += a.m_in[2 * r + 1];
-    }
-  const double mx = sx * a.invN, my = sy * a.invN;
-  extern __shared__ __align__(16) unsigned char tabraw[];  // FP64 kick-drift stages: the sine/cosine table (kTabBytes)
-  scfx::Entry *tab = (scfx::Entry *)tabraw;
-  if constexpr (!MIXED && MODE == STAGE_KICK_DRIFT) load_sincos_fx(tab);
+// One sweep over the particles: the stage's work of this thread, its sums of the new angles'
+// cosines and sines into acd, asd.  CG: the loads bypass L1 (a kernel of several stages reads
+// what other CTAs wrote in its previous stage).
+template <bool MIXED, int MODE, bool CG>
+__device__ __forceinline__ void hmf_sweep(const HmfArgs &a, double mx, double my, const scfx::Entry *tab, double &acd,
+                                          double &asd) {
+  auto load = [](const auto *ptr) {
+    if constexpr (CG) return __ldcg(ptr);
+    else return *ptr;
+  };
   const HmfM m = hmf_m_of(mx, my);
   const float mxf = (float)mx, myf = (float)my, dtf = (float)a.drift;
   float acf = 0.f, asf = 0.f;
   long long aci = 0, asi = 0;
-  double acd = 0.0, asd = 0.0;
   const int64_t npairs = a.N >> 1;
   const int64_t G = (int64_t)gridDim.x * NT;
   const int64_t t0 = (int64_t)blockIdx.x * NT + threadIdx.x;
@@ -240,8 +234,8 @@ __global__ void __launch_bounds__(NT, MODE != STAGE_KICK_DRIFT ? 1 : MIXED ? 4 :
         const int64_t kk = k + u * G;
         const int64_t ix = a.rev ? npairs - 1 - kk : kk;
         if (kk < npairs) {
-          qv[u] = q2[ix];
-          pv[u] = p2[ix];
+          qv[u] = load(q2 + ix);
+          pv[u] = load(p2 + ix);
         }
       }
 #pragma unroll
@@ -259,18 +253,18 @@ __global__ void __launch_bounds__(NT, MODE != STAGE_KICK_DRIFT ? 1 : MIXED ? 4 :
   } else {
     // one pair ahead: the next pair's 64 bytes are on their way while this one is computed
     auto at = [&](int64_t kk) { return a.rev ? npairs - 1 - kk : kk; };
-    double2 qn = q2[at(kb)], pn = p2[at(kb)];
-    int4 an = a.cs[2 * at(kb)], bn = a.cs[2 * at(kb) + 1];
+    double2 qn = load(q2 + at(kb)), pn = load(p2 + at(kb));
+    int4 an = load(a.cs + 2 * at(kb)), bn = load(a.cs + 2 * at(kb) + 1);
     for (int64_t k = kb; k < kend; k += G) {
       const int64_t ix = at(k);
       double2 qv = qn, pv = pn;
       int4 ca = an, cb = bn;
       if (k + G < kend) {
         const int64_t nx = at(k + G);
-        qn = q2[nx];
-        pn = p2[nx];
-        an = a.cs[2 * nx];
-        bn = a.cs[2 * nx + 1];
+        qn = load(q2 + nx);
+        pn = load(p2 + nx);
+        an = load(a.cs + 2 * nx);
+        bn = load(a.cs + 2 * nx + 1);
       }
       hmf_particle_fp64<MODE>(qv.x, pv.x, ca, a, m, mx, my, aci, asi, 2 * ix, tab);
       hmf_particle_fp64<MODE>(qv.y, pv.y, cb, a, m, mx, my, aci, asi, 2 * ix + 1, tab);
@@ -295,11 +289,11 @@ __global__ void __launch_bounds__(NT, MODE != STAGE_KICK_DRIFT ? 1 : MIXED ? 4 :
   }
   if ((a.N & 1) && t0 == 0) {
     int64_t i = a.N - 1;
-    double th = a.q[i], pp = a.p[i];
+    double th = load(a.q + i), pp = load(a.p + i);
     if constexpr (MIXED) {
       hmf_particle_mixed<MODE>(th, pp, a, mxf, myf, dtf, acf, asf, i);
     } else {
-      int4 c = a.cs[i];
+      int4 c = load(a.cs + i);
       hmf_particle_fp64<MODE>(th, pp, c, a, m, mx, my, aci, asi, i, tab);
       if (MODE == STAGE_KICK_DRIFT) a.cs[i] = c;
     }
@@ -314,8 +308,187 @@ __global__ void __launch_bounds__(NT, MODE != STAGE_KICK_DRIFT ? 1 : MIXED ? 4 :
       acd += (double)aci * 0x1p-54;
       asd += (double)asi * 0x1p-54;
     }
-    grid_finish(acd, asd, a.partials, a.m_out, a.ticket);
   }
+}
+
+// SHARD: the magnetization is the sum of every rank's pair in m_in, added in rank
+// order (the same value on every rank), over the whole system's N (invN).
+// Register budgets of the kick-drift stages: mixed 4 CTAs per SM (64 registers; 80 and 3 CTAs: 262
+// against 248 us per stage at N = 5e7), FP64 3 (80; 112 and 2 CTAs: 750 against 566 us).
+template <bool MIXED, int MODE, bool SHARD = false>
+__global__ void __launch_bounds__(NT, MODE != STAGE_KICK_DRIFT ? 1 : MIXED ? 4 : 3) hmf_stage_kernel(HmfArgs a) {
+  double sx = a.m_in[0], sy = a.m_in[1];
+  if constexpr (SHARD)
+    for (int r = 1; r < a.nsum; r++) {
+      sx += a.m_in[2 * r];
+      sy += a.m_in[2 * r + 1];
+    }
+  const double mx = sx * a.invN, my = sy * a.invN;
+  extern __shared__ __align__(16) unsigned char tabraw[];  // FP64 kick-drift stages: the sine/cosine table (kTabBytes)
+  scfx::Entry *tab = (scfx::Entry *)tabraw;
+  if constexpr (!MIXED && MODE == STAGE_KICK_DRIFT) load_sincos_fx(tab);
+  double acd = 0.0, asd = 0.0;
+  hmf_sweep<MIXED, MODE, false>(a, mx, my, tab, acd, asd);
+  if (MODE == STAGE_KICK_DRIFT) grid_finish(acd, asd, a.partials, a.m_out, a.ticket);
+}
+
+// Small systems: the 3 n kick-drift stages of n steps in one launch of one cluster.  A stage of
+// these sizes is all latency, so the stages follow one another behind a cluster barrier instead
+// of a kernel boundary, with the grid, the sweep directions and the groupings of the launched
+// stages, and so with their results.  Microseconds per stage at N = 300, 3,000, 10,007:
+// mixed 5.9, 6.7, 7.8 launched, 1.5, 2.0, 2.1 here; FP64 7.9, 10.8, 12.3 and 4.5, 6.2, 6.9 (the
+// state through L2: 4.5 us in mixed, too).
+constexpr int kRunCtas = 16;  // CTAs of the largest cluster
+
+struct HmfRun {
+  int64_t begin, end;            // kick-drift stages: (b0, d0) (b1, d1) (b1, d0), b0 = first, then b0
+  double first, b0, b1, d0, d1;  // times dt
+  // sweep directions: stages [3, 3 + fixed) alternate from rev_fixed on (the captured blocks of
+  // steps, whose directions stay as captured), the others from HmfArgs::rev
+  int64_t fixed;
+  int rev_fixed;
+  __device__ int rev(int64_t st, int rev0) const {
+    if (st >= 3 && st < 3 + fixed) return rev_fixed ^ (int)((st - 3) & 1);
+    return rev0 ^ (int)((st < 3 ? st : st - fixed) & 1);
+  }
+};
+
+// FP64: the sweep of the launched stage; the CTAs exchange their partial sums through
+// distributed shared memory and every CTA adds them, in grid_finish's order.
+__global__ void __launch_bounds__(NT, 3) hmf_run_fp64_kernel(HmfArgs a, HmfRun r) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  extern __shared__ __align__(16) unsigned char tabraw[];
+  scfx::Entry *tab = (scfx::Entry *)tabraw;
+  __shared__ double2 part[2], msum;
+  __shared__ double2 red[NT / 32];
+  load_sincos_fx(tab);
+  const int rev0 = a.rev;
+  double2 s = make_double2(a.m_in[0], a.m_in[1]);
+  for (int64_t st = r.begin; st < r.end; st++) {
+    const int ph = (int)(st % 3);
+    a.kick = ph == 0 ? (st == 0 ? r.first : r.b0) : r.b1;
+    a.drift = ph == 1 ? r.d1 : r.d0;
+    a.rev = r.rev(st, rev0);
+    double acd = 0.0, asd = 0.0;
+    hmf_sweep<false, STAGE_KICK_DRIFT, true>(a, s.x * a.invN, s.y * a.invN, tab, acd, asd);
+    const double2 b = block_sum2<NT>(acd, asd, red);
+    if (threadIdx.x == 0) part[st & 1] = b;
+    cluster.sync();  // the partial sums and the state of every CTA are visible
+    if (threadIdx.x < 32) {
+      double2 v = make_double2(0.0, 0.0);
+      if (threadIdx.x < gridDim.x) v = *cluster.map_shared_rank(&part[st & 1], threadIdx.x);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        v.x += __shfl_down_sync(0xffffffffu, v.x, o);
+        v.y += __shfl_down_sync(0xffffffffu, v.y, o);
+      }
+      if (threadIdx.x == 0) msum = v;
+    }
+    __syncthreads();
+    s = msum;
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    a.m_out[0] = s.x;
+    a.m_out[1] = s.y;
+  }
+  cluster.sync();  // no CTA leaves while another reads its partial sums
+}
+
+// Sum of a thread's at most five cosines (or sines) in units of 2^-38: exact for an FP32 sum
+// of 2^-15 and more, within 2^-39 below.
+__device__ __forceinline__ long long fix38(float v) {
+  const float h = rintf(v * 0x1p28f);  // below 2^31
+  return ((long long)__float2int_rn(h) << 10) + __float2int_rn((v - h * 0x1p-28f) * 0x1p38f);
+}
+
+// Mixed: a thread keeps its particles (at most two pairs, UNROLL of the launched grid, and the
+// odd one) in registers through all stages.  A reverse sweep groups the same pairs, p and
+// p + G, in the other order.  The groups' FP32 sums are added as integers (the launched stages
+// add them in FP64, where they are exact too, but for sums below 2^-16 whose last bits are
+// beyond M's FP32): every warp puts its total into every CTA's shared memory, and after the
+// cluster barrier every warp adds them for itself.
+__global__ void __launch_bounds__(NT, 1) hmf_run_mixed_kernel(HmfArgs a, HmfRun r) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  constexpr int NW = NT / 32;
+  __shared__ longlong2 part[2][kRunCtas * NW];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t npairs = a.N >> 1, G = (int64_t)gridDim.x * NT;
+  const int64_t t0 = (int64_t)blockIdx.x * NT + threadIdx.x;
+  double2 *q2 = reinterpret_cast<double2 *>(a.q), *p2 = reinterpret_cast<double2 *>(a.p);
+  const bool has[2] = {t0 < npairs, t0 + G < npairs}, odd = (a.N & 1) && t0 == 0;
+  double2 q[2], p[2];
+  double qo = 0.0, po = 0.0;
+#pragma unroll
+  for (int u = 0; u < 2; u++) {
+    q[u] = has[u] ? q2[t0 + u * G] : make_double2(0.0, 0.0);
+    p[u] = has[u] ? p2[t0 + u * G] : make_double2(0.0, 0.0);
+  }
+  if (odd) {
+    qo = a.q[a.N - 1];
+    po = a.p[a.N - 1];
+  }
+  double sx = a.m_in[0], sy = a.m_in[1];
+  for (int64_t st = r.begin; st < r.end; st++) {
+    const int ph = (int)(st % 3);
+    a.kick = ph == 0 ? (st == 0 ? r.first : r.b0) : r.b1;
+    a.drift = ph == 1 ? r.d1 : r.d0;
+    const float mxf = (float)(sx * a.invN), myf = (float)(sy * a.invN), dtf = (float)a.drift;
+    float c[2][2] = {}, s[2][2] = {};
+#pragma unroll
+    for (int u = 0; u < 2; u++)
+      if (has[u]) {
+        hmf_particle_mixed<STAGE_KICK_DRIFT>(q[u].x, p[u].x, a, mxf, myf, dtf, c[u][0], s[u][0], 0);
+        hmf_particle_mixed<STAGE_KICK_DRIFT>(q[u].y, p[u].y, a, mxf, myf, dtf, c[u][1], s[u][1], 0);
+      }
+    // the group's FP32 sums in its sweep's order (a missing pair adds zeros first or last)
+    const bool f = r.rev(st, a.rev) != 0;
+    const float ac = (((f ? c[1][0] : c[0][0]) + (f ? c[1][1] : c[0][1])) + (f ? c[0][0] : c[1][0])) + (f ? c[0][1] : c[1][1]);
+    const float as = (((f ? s[1][0] : s[0][0]) + (f ? s[1][1] : s[0][1])) + (f ? s[0][0] : s[1][0])) + (f ? s[0][1] : s[1][1]);
+    longlong2 v = make_longlong2(fix38(ac), fix38(as));
+    if (odd) {
+      float co = 0.f, so = 0.f;
+      hmf_particle_mixed<STAGE_KICK_DRIFT>(qo, po, a, mxf, myf, dtf, co, so, 0);
+      v.x += fix38(co);
+      v.y += fix38(so);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+      v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+    }
+    longlong2 *slot = &part[st & 1][blockIdx.x * NW + w];
+    if (lane < (int)gridDim.x) *cluster.map_shared_rank(slot, lane) = v;
+    cluster.sync();
+    v = make_longlong2(0, 0);
+    for (int k = lane; k < (int)gridDim.x * NW; k += 32) {
+      v.x += part[st & 1][k].x;
+      v.y += part[st & 1][k].y;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+      v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+    }
+    sx = (double)v.x * 0x1p-38;
+    sy = (double)v.y * 0x1p-38;
+  }
+#pragma unroll
+  for (int u = 0; u < 2; u++)
+    if (has[u]) {
+      q2[t0 + u * G] = q[u];
+      p2[t0 + u * G] = p[u];
+    }
+  if (odd) {
+    a.q[a.N - 1] = qo;
+    a.p[a.N - 1] = po;
+  }
+  if (t0 == 0) {
+    a.m_out[0] = sx;
+    a.m_out[1] = sy;
+  }
+  cluster.sync();  // no CTA leaves while another writes into its shared memory
 }
 
 // (cos, sin) of every angle as the FP64 stages read them, and their sums.  A non-finite angle
@@ -602,6 +775,68 @@ int hmf_shard_stage(md_ctx *c, int mode, double kick, double drift, double *fout
                  : launch_shard_stage<false, STAGE_FORCE_ONLY>(c, 0.0, 0.0, fout);
   return mixed ? launch_shard_stage<true, STAGE_KICK_DRIFT>(c, kick, drift, nullptr)
                : launch_shard_stage<false, STAGE_KICK_DRIFT>(c, kick, drift, nullptr);
+}
+
+// The kick-drift stages of nsteps steps as one cluster launch, when the stages' grid is at
+// most one cluster and the device can hold it (*done = false, nothing launched, otherwise).
+// block_steps of them (after the first step) would be replayed blocks.
+int hmf_run(md_ctx *c, int64_t nsteps, int64_t block_steps, const double *k4, double h, bool *done) {
+  *done = false;
+  const bool mixed = c->prec == MD_MIXED;
+  const void *stage = mixed ? (const void *)hmf_stage_kernel<true, STAGE_KICK_DRIFT>
+                            : (const void *)hmf_stage_kernel<false, STAGE_KICK_DRIFT>;
+  const size_t dyn = mixed ? 0 : kTabBytes;
+  const int g = grid_for(c, stage, (c->N + 1) / 2 / UNROLL + 1, mixed ? 4 : 0, dyn);
+  if (g > kRunCtas) return MD_OK;
+  auto kern = mixed ? hmf_run_mixed_kernel : hmf_run_fp64_kernel;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(g);
+  cfg.blockDim = dim3(NT);
+  cfg.dynamicSmemBytes = dyn;
+  cfg.stream = c->stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = g;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if (g > 8) MD_CUDA(c, cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  if (dyn) MD_CUDA(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
+  int clusters = 0;
+  if (cudaOccupancyMaxActiveClusters(&clusters, (const void *)kern, &cfg) != cudaSuccess || clusters < 1) {
+    cudaGetLastError();
+    return MD_OK;
+  }
+  if (!c->hmf_m_valid || c->hmf_m_prec != c->prec) {
+    int rc = hmf_prime(c);
+    if (rc) return rc;
+  }
+  HmfArgs a{};
+  a.q = c->q;
+  a.p = c->p;
+  a.N = c->N;
+  a.invN = 1.0 / (double)c->N;
+  a.cs = (int4 *)c->hmf_cs;
+  a.m_in = c->hmf_m + 2 * c->hmf_cur;
+  a.rev = c->hmf_rev;
+  // launched stages alternate the direction, replayed blocks keep the one they were captured with
+  const int64_t launched = 3 * (nsteps - block_steps);
+  const int cur1 = 1 - c->hmf_cur;  // parity after the first step
+  HmfRun r{0, 0, k4[0] * h, 2.0 * k4[0] * h, k4[1] * h, k4[2] * h, k4[3] * h, 3 * block_steps, 0};
+  if (block_steps) r.rev_fixed = run_direction(c, cur1, h, 1 - c->hmf_rev);
+  if (nsteps & 1) c->hmf_cur = 1 - c->hmf_cur;
+  if (launched & 1) c->hmf_rev ^= 1;
+  a.m_out = c->hmf_m + 2 * c->hmf_cur;
+  // pieces of kRunStages, so that a launch stays in the milliseconds
+  constexpr int64_t kRunStages = 768;
+  for (; r.begin < 3 * nsteps; r.begin = r.end) {
+    r.end = r.begin + kRunStages < 3 * nsteps ? r.begin + kRunStages : 3 * nsteps;
+    MD_CUDA(c, cudaLaunchKernelEx(&cfg, kern, a, r));
+    MD_LAUNCHED(c);
+    a.m_in = a.m_out;
+  }
+  *done = true;
+  return MD_OK;
 }
 
 int hmf_stage(md_ctx *c, int mode, double kick, double drift, double *fout) {

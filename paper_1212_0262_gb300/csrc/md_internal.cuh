@@ -107,6 +107,8 @@ struct md_ctx {
   cudaGraphExec_t step_graph[2] = {nullptr, nullptr};
   StepGraphKey step_key[2];
   int64_t step_graph_launches[2] = {0, 0};
+  StepGraphKey run_key[2];            // small HMF systems, whose steps run in one launch: the key
+  int run_rev[2] = {-1, -1};          // and first sweep direction a block of each parity would have
   bool use_graphs = true;
 
   // Row shard (md_shard_*): the state holds rows [row0, row0 + N) of a system of
@@ -161,6 +163,9 @@ void dev_free(void *p);
   } while (0)
 
 void destroy_step_graphs(md_ctx *c);
+// api.cu: the sweep direction that a block of steps of this parity is captured with (`now` on its
+// first use), for runs that take the place of the replayed blocks.
+int run_direction(md_ctx *c, int parity, double h, int now);
 
 // Yoshida coefficients of Eq. 4 (B0, B1, D0, D1), from the triple-jump closed form.
 void yoshida_coefficients(double c[4]);
@@ -204,6 +209,7 @@ int hmf_magnetization_terminal(md_ctx *c, double cx, double cy, double *lq);
 int hmf_prime(md_ctx *c);                                         // sums of the current angles
 int hmf_sincos_table(md_ctx *c, bool probe);  // the FP64 stages' sine/cosine table on the context's device
 int hmf_stage(md_ctx *c, int mode, double kick, double drift, double *fout);
+int hmf_run(md_ctx *c, int64_t nsteps, int64_t block_steps, const double *k4, double h, bool *done);  // the steps' kick-drift stages in one launch
 int hmf_sums_fp64(md_ctx *c, double *d_out2);                     // FP64 (sum cos, sum sin) into device out
 int hmf_sums_fp64_of(md_ctx *c, const double *q, double *d_out2);
 
