@@ -481,8 +481,9 @@ int ensure_pair_buffers(md_ctx *c, int TI, int P, int nacc) {
     }
     c->sk_slots_bytes = need_slots;
   }
-  // a ticket per i-tile, then the dynamic stream-K counters (pair_sched)
-  size_t n_it = (size_t)((c->N + TI - 1) / TI) + 2;
+  // a ticket per 128 particles (the finish blocks of sym.cu; i-tiles are whole numbers of
+  // them), then the dynamic stream-K counters (pair_sched)
+  size_t n_it = (size_t)(padded(c->N) / 128) + 2;
   if (n_it > c->sk_tickets_count) {
     dev_free(c->sk_tickets);
     c->sk_tickets = (unsigned *)dev_alloc(n_it * sizeof(unsigned));

@@ -32,12 +32,11 @@
 //
 // Finish phase (sym_finish_kernel).  Tile T needs its row partials and the
 // column partials of the units (I', J), J in tile T, I' < T (I' <= T with
-// tile_diag).  One CTA per
-// (tile, chunk of sym_chunk rows I') sums a chunk's column partials per particle
-// and component (compensated FP32, then one double); the last chunk of a tile to
-// arrive (atomic ticket, no waiting) adds the row partials in CTA order and the
-// chunk sums in chunk order, and runs the stage epilogue (kick, drift, new mirror
-// record) for the tile's particles.  Every sum has a fixed order, so results are
+// tile_diag).  One CTA per (128 particles of a tile, chunk of rows I' or of row
+// partials) sums its chunk per particle and component (column partials in compensated
+// FP32, then one double); the last chunk to arrive (atomic ticket, no waiting) adds the
+// chunk sums in order and runs the stage epilogue (kick, drift, new mirror record) for
+// the 128 particles.  Every sum has a fixed order, so results are
 // deterministic.  The finish phase spreads the O(N^2 / TJ) column reads over the
 // whole GPU; finishing a tile inside the pair kernel instead serialised them on
 // the few CTAs that cover the many short rows at the end of the order.
@@ -54,11 +53,12 @@ constexpr size_t kSymMaxColBytes = (size_t)16 << 30;  // Ring and 2D at N = 1e6 
 
 struct SymArgs {
   int m;             // TI / TJ
-  int nc;            // chunk slots per tile in the finish phase
+  int nc;            // chunk slots per block in the finish phase
+  int ch;            // column-partial rows or row segments per chunk
   double *rowfull;   // [n_it][NACC][TI] row partials of rows covered by one CTA
   void *colslot;     // [U][TJ][NACC] column partials of the units (Pol::ColT:
                      // FP32 for the mixed policies, FP64 for the FP64 ones)
-  double *chunks;    // [n_it][nc][TI][NACC] chunk sums of the column partials
+  double *chunks;    // [blocks][nc][kFinishBlock][NACC] chunk sums
 };
 
 // Policies with integer pair arithmetic (pairs_fx.cuh): their row sums partly in shared
@@ -206,42 +206,45 @@ __global__ void __launch_bounds__(Pol::THREADS, Pol::MINB) sym_pairs_kernel(Pair
   vcta_done(a.sched);
 }
 
-// Finish phase, one CTA per (tile T, chunk c of sym_chunk rows I' < T, or I' <= T
-// with tile_diag): the chunk's column partials summed per particle and component
-// (compensated FP32) into one double; the last chunk of the tile to arrive (atomic
-// ticket, no waiting) adds the row partials (CTA order) and the chunk sums (chunk
-// order) and runs the stage epilogue.  A tile with no rows I' has one empty chunk.
-constexpr int kFinishThreads = 256;
-
-// Column-partial rows per finish CTA: about 16K loads per CTA whatever the tile's
-// output count (Ring FP32 tiles have 256 outputs, 2D 2048).
-template <class Pol>
-constexpr int sym_chunk() {
-  constexpr int out = Pol::THREADS * Pol::R * Pol::NACC;
-  return out <= 256 ? 64 : out <= 512 ? 32 : 16;
-}
+// Finish phase, one CTA per (block b of kFinishBlock particles, chunk c).  The force of a
+// particle of tile T is the sum of its row's segments (one per virtual CTA that covers part of
+// row T) minus the column partials of the rows I' < T (I' <= T with tile_diag).  A chunk CTA
+// sums s.ch column partials (compensated FP32, or FP64) or s.ch segments per particle and
+// component into one double; the last chunk of the block to arrive (atomic ticket, no
+// waiting) adds the chunk sums, segments first, and runs the stage epilogue.
+// Small tiles of few rows are all latency: with one CTA per tile, which added up to 64 segments
+// one after the other for 1024 particles, this phase took 290 us at N = 16,385 (2D, mixed)
+// beside 73 us for the pair phase; split by blocks and segments it takes 13.  Microseconds per
+// force, before and after: mixed Ring N = 4,096 31.8, 22.6; 2D N = 4,096 71.7, 33.3, N = 16,385
+// 282, 86, N = 65,536 763, 700; 3D N = 16,385 163, 110; FP64 Ring N = 4,096 107, 84.  At N = 131,072
+// (Ring) and 262,144 (2D), where it is bound by the column reads, 87 -> 41 and 180 -> 135 us.
+constexpr int kFinishBlock = 128;
 
 template <class Pol, int MODEL, bool MIXED, int MODE>
-__global__ void __launch_bounds__(kFinishThreads) sym_finish_kernel(PairArgs a, SymArgs s) {
+__global__ void __launch_bounds__(kFinishBlock * Pol::NACC) sym_finish_kernel(PairArgs a, SymArgs s) {
   constexpr int NACC = Pol::NACC, TJ = Pol::TJ;
   constexpr int64_t TI = (int64_t)Pol::THREADS * Pol::R;
-  constexpr int OUT = (int)TI * NACC;  // outputs of a tile: (particle, component)
+  constexpr int FT = kFinishBlock * NACC;          // threads: one per (particle, component)
+  constexpr int SB = (int)(TI / kFinishBlock);     // blocks per tile
+  static_assert(TI % kFinishBlock == 0, "whole blocks per tile");
   __shared__ bool s_last;
-  const int64_t T = blockIdx.x / s.nc;
-  const int c = (int)(blockIdx.x % s.nc);
-  constexpr int CH = sym_chunk<Pol>();
-  const int64_t rows = T + (HasDiagSym<Pol>::value ? 1 : 0);  // column-partial rows I of tile T
-  const int nch = rows == 0 ? 1 : (int)((rows + CH - 1) / CH);
-  if (c >= nch) return;
+  const int64_t b = blockIdx.x / s.nc, T = b / SB;
+  const int c = (int)(blockIdx.x % s.nc), sb = (int)(b % SB);
   const int m = s.m;
-  const int64_t I_lo = (int64_t)c * CH, I_hi = min(rows, I_lo + CH);
-  double *chunk = s.chunks + (T * s.nc) * OUT;
-  using ColT = typename Pol::ColT;
-  const ColT *col = (const ColT *)s.colslot;
-  for (int o = threadIdx.x; o < OUT; o += kFinishThreads) {
-    const int jsub = o / (TJ * NACC), rest = o % (TJ * NACC);
+  const int64_t rows = T + (HasDiagSym<Pol>::value ? 1 : 0);  // column-partial rows I of tile T
+  int64_t cf, cl;
+  sym_row_ctas(a, s, T, cf, cl);
+  const int nchc = (int)((rows + s.ch - 1) / s.ch), nch = nchc + (int)((cl - cf + s.ch) / s.ch);
+  if (c >= nch) return;
+  double *chunk = s.chunks + b * s.nc * FT;
+  const int lr = sb * kFinishBlock + threadIdx.x / NACC, d = threadIdx.x % NACC;
+  double v = 0.0;
+  if (c < nchc) {
+    using ColT = typename Pol::ColT;
+    const ColT *col = (const ColT *)s.colslot;
+    const int64_t I_lo = (int64_t)c * s.ch, I_hi = min(rows, I_lo + s.ch);
+    const int jsub = lr / TJ, rest = (lr % TJ) * NACC + d;
     CompSum cs{0.f, 0.f};  // FP32 column partials: compensated FP32 sum
-    double sd = 0.0;       // FP64 column partials
     // unit (I2, T m + jsub) = rowstart(I2) + T m + jsub - m I2; from I2 to I2 + 1 it
     // advances by the length of row I2 minus m, i.e. n_jt - m (I2 + 1)
     int64_t off = (sym_rowstart(I_lo, a.n_jt, m) + (T * m + jsub - (int64_t)m * I_lo)) * (TJ * NACC) + rest;
@@ -250,44 +253,44 @@ __global__ void __launch_bounds__(kFinishThreads) sym_finish_kernel(PairArgs a, 
 #pragma unroll 8
     for (int64_t I2 = I_lo; I2 < I_hi; I2++) {
       if constexpr (sizeof(ColT) == 4) csum_add(cs, __ldcg(col + off));
-      else sd += __ldcg(col + off);
+      else v += __ldcg(col + off);
       off += step;
       step -= dstep;
     }
-    chunk[(int64_t)c * OUT + o] = sizeof(ColT) == 4 ? csum_total(cs) : sd;
+    v = sizeof(ColT) == 4 ? -csum_total(cs) : -v;
+  } else if (cf == cl) {
+    v = __ldcg(s.rowfull + (T * NACC + d) * TI + lr);
+  } else {
+    // virtual CTA c2 > cf begins inside row T: its first slot; cf may begin in an earlier row
+    const int64_t lo = cf + (int64_t)(c - nchc) * s.ch, hi = min(cl + 1, lo + s.ch);
+    const bool cf_first = unit_begin(a.U, a.P, cf) >= sym_rowstart(T, a.n_jt, m);
+    const double *src = a.slots + d * TI + lr;
+#pragma unroll 8
+    for (int64_t c2 = lo; c2 < hi; c2++)
+      v += __ldcg(src + (c2 * 2 + (c2 > cf || cf_first ? 0 : 1)) * (NACC * TI));
   }
+  chunk[(int64_t)c * FT + threadIdx.x] = v;
   __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(&a.tickets[T], 1u) + 1u == (unsigned)nch;
+  if (threadIdx.x == 0) s_last = atomicAdd(&a.tickets[b], 1u) + 1u == (unsigned)nch;
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  int64_t cf, cl;
-  sym_row_ctas(a, s, T, cf, cl);
-  for (int lr = threadIdx.x; lr < TI; lr += kFinishThreads) {
-    const int64_t i = T * TI + lr;
-    if (i >= a.N) break;
+  const int64_t i = b * kFinishBlock + threadIdx.x;
+  if (threadIdx.x < kFinishBlock && i < a.N) {
     double tot[NACC];
-    if (cf == cl) {
 #pragma unroll
-      for (int d = 0; d < NACC; d++) tot[d] = __ldcg(s.rowfull + (T * NACC + d) * TI + lr);
-    } else {
+    for (int e = 0; e < NACC; e++) tot[e] = 0.0;
+    const double *mine = chunk + threadIdx.x * NACC;
+#pragma unroll 2
+    for (int k = 0; k < nch; k++) {
+      const int64_t at = (int64_t)(k < nch - nchc ? nchc + k : k - (nch - nchc)) * FT;
 #pragma unroll
-      for (int d = 0; d < NACC; d++) tot[d] = 0.0;
-      for (int64_t c2 = cf; c2 <= cl; c2++) {
-        const int64_t fr = sym_row_of_unit(unit_begin(a.U, a.P, c2), a.n_it, a.n_jt, m);
-        const double *src = a.slots + ((c2 * 2 + (T == fr ? 0 : 1)) * NACC) * TI;
-#pragma unroll
-        for (int d = 0; d < NACC; d++) tot[d] += __ldcg(src + d * TI + lr);
-      }
+      for (int e = 0; e < NACC; e++) tot[e] += __ldcg(mine + at + e);
     }
-    // output o = (lr / TJ) TJ NACC + (lr % TJ) NACC + d = lr NACC + d
-    for (int c2 = 0; c2 < nch; c2++)
-#pragma unroll
-      for (int d = 0; d < NACC; d++) tot[d] -= __ldcg(chunk + (int64_t)c2 * OUT + lr * NACC + d);
     finish<Pol, MODEL, MIXED, MODE>(a, i, tot);
   }
-  if (threadIdx.x == 0) a.tickets[T] = 0u;
+  if (threadIdx.x == 0) a.tickets[b] = 0u;
 }
 
 // ------------------------------------------------------------ host side ---
@@ -325,11 +328,20 @@ int launch_sym(md_ctx *c, PairArgs a) {
   a.P = (int)vcta_count(G, a.U, kv, IsFx<Pol>::value ? 1 : 16);
   int rc = ensure_pair_buffers(c, (int)TI, a.P, NACC);
   if (rc) return rc;
-  const int64_t max_rows = a.n_it - 1 + (HasDiagSym<Pol>::value ? 1 : 0);  // of the last tile
-  s.nc = (int)std::max<int64_t>(1, (max_rows + sym_chunk<Pol>() - 1) / sym_chunk<Pol>());
+  // Chunks: row T has n_jt - m T units in ranges of U / P, and T (+ 1) column-partial rows.
+  // The bound on their number is linear in T: the larger of its ends sizes the grid (spare
+  // CTAs leave at once).  Longer chunks where the column partials are many and narrow (Ring
+  // FP32: the chunk sums would cost an eighth of their traffic).
+  s.ch = Pol::NACC == 1 && a.n_it >= 256 ? 64 : 16;
+  auto chunks = [&](int64_t T) {
+    const int64_t seg = (a.n_jt - (int64_t)s.m * T) * a.P / a.U + 2;
+    return (T + 1 + s.ch - 1) / s.ch + (seg + s.ch - 1) / s.ch;
+  };
+  s.nc = (int)std::max(chunks(0), chunks(a.n_it - 1));
+  const int64_t blocks = a.n_it * (TI / kFinishBlock);
   const size_t need_row = (size_t)a.n_it * NACC * TI * sizeof(double);
   const size_t need_col = (size_t)a.U * TJ * NACC * sizeof(typename Pol::ColT);
-  const size_t need_chunk = (size_t)a.n_it * s.nc * NACC * TI * sizeof(double);
+  const size_t need_chunk = (size_t)blocks * s.nc * NACC * kFinishBlock * sizeof(double);
   if (need_row > c->sym_rowfull_bytes) {
     dev_free(c->sym_rowfull);
     c->sym_rowfull = (double *)dev_alloc(need_row);
@@ -376,7 +388,7 @@ int launch_sym(md_ctx *c, PairArgs a) {
   }
   kern<<<(int)G, THR, 0, c->stream>>>(a, s);
   MD_LAUNCHED(c);
-  sym_finish_kernel<Pol, MODEL, MIXED, MODE><<<a.n_it * s.nc, kFinishThreads, 0, c->stream>>>(a, s);
+  sym_finish_kernel<Pol, MODEL, MIXED, MODE><<<blocks * s.nc, kFinishBlock * NACC, 0, c->stream>>>(a, s);
   MD_LAUNCHED(c);
   if (MODE == STAGE_KICK_DRIFT || ((MODE == STAGE_ADJOINT || MODE == STAGE_TANGENT) && a.drift != 0.0))
     c->mirror_cur = 1 - c->mirror_cur;
