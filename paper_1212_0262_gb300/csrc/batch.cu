@@ -18,10 +18,8 @@
 // triangular (system, i-tile, j-tile) units of its systems stream-K style and
 // writing row and column partials (diagonal units too: their above-diagonal
 // blocks are evaluated once, with column sums), then one finish launch with a CTA
-// per (system, tile, chunk of column-partial rows: 128 for the Ring part's
-// 256-output tiles, 32 for the 2D part's 2048) that sums them in a fixed order and
-// runs the epilogue; the grid holds only the chunks each tile has (tile t sums the
-// rows 0 .. t, ceil((t + 1) / chunk) chunks).  (The one-sided form shares one launch
+// per (system, block of 256 outputs, chunk of 128 row segments or column-partial rows)
+// that sums them in a fixed order and runs the epilogue.  (The one-sided form shares one launch
 // between the parts, split by md_batch_set_tuning's `split`.)
 #include <algorithm>
 #include <vector>
@@ -43,8 +41,7 @@ struct SysDesc {
   int64_t N, n_it, n_jt;
   int64_t ubeg;  // first unit of the system in its part
   int64_t rbeg;  // first row (i-tile) of the system in its part
-  int64_t fbeg;  // symmetric form: first finish CTA of the system in its part
-  int64_t nfin;  // symmetric form: finish CTAs of the system (chunks of all its tiles)
+  int64_t bbeg;  // symmetric form: first finish block of the system in its part
   double epsd, dt;
 };
 
@@ -61,10 +58,11 @@ struct PartArgs {
   int waves;         // virtual CTAs per physical CTA: P = waves x grid
   unsigned *next;    // next virtual CTA to take (the finish kernel sets it back to 0)
   int m;             // TI / TJ of the part
-  int64_t nfin;      // finish CTAs of the part
+  int64_t nblk;      // finish blocks of the part
+  int nc;            // chunks per finish block, at most
   double *rowfull;   // [rows][NACC][TI]
   float *colslot;    // [U][TJ][NACC]
-  double *chunks;    // [nfin][TI][NACC]
+  double *chunks;    // [nblk][nc][kFinishThreadsB]
 };
 
 // index of the system whose unit range holds u (binary search on ubeg)
@@ -234,33 +232,17 @@ __global__ void __launch_bounds__(NT) batch_kernel(PartArgs ring, PartArgs grav)
 
 // ------------------------------------------------- Newton's-third-law form --
 
+// Finish phase as in sym.cu, in blocks of 256 outputs (256 Ring or 128 2D particles) and
+// chunks of kChunkB column-partial rows or row segments (ranges that cover part of the row).
+// A tile per CTA took 145 us of a stage of 4 systems (pair phase 557 us); a stage of 4, 8, 24
+// systems 770, 974, 2855 us, now 573, 896, 2825 (chunks of 32 rows: 582, 910, 2870: more CTAs
+// with nothing to sum).
 constexpr int kFinishThreadsB = 256;
+constexpr int kChunkB = 128;
 
-// Column-partial rows per finish CTA, by the tile's outputs (TI NACC): longer chunks
-// where a CTA has fewer outputs to sum, twice the single-system finish's, as the
-// ensemble's tiles have few rows above them (small systems) and the finish phase is
-// bound by its CTA count rather than by its loads.
-__host__ __device__ constexpr int chunk_rows(int64_t outputs) { return outputs <= 256 ? 128 : outputs <= 512 ? 64 : 32; }
-
-// Finish CTAs: tile t sums the column partials of its units (I, t m .. t m + m - 1)
-// for I = 0 .. t (its own diagonal units included: their above-diagonal blocks) in
-// ceil((t + 1) / ch) chunks of ch rows I.  CTAs of tiles 0 .. T-1:
-// sum_{s=1}^{T} ceil(s / ch) = ch q (q + 1) / 2 + r (q + 1) with T = q ch + r.
-__host__ __device__ __forceinline__ int64_t fin_prefix(int64_t T, int ch) {
-  const int64_t q = T / ch, r = T % ch;
-  return (int64_t)ch * q * (q + 1) / 2 + r * (q + 1);
-}
-
-// The tile whose chunks hold finish CTA f of a system of n_it tiles: the largest T
-// with fin_prefix(T) <= f.
-__device__ __forceinline__ int64_t fin_tile(int64_t f, int64_t n_it, int ch) {
-  int64_t lo = 0, hi = n_it - 1;
-  while (lo < hi) {
-    const int64_t mid = (lo + hi + 1) >> 1;
-    if (fin_prefix(mid, ch) <= f) lo = mid;
-    else hi = mid - 1;
-  }
-  return lo;
+template <class Pol>
+constexpr int finish_block() {
+  return kFinishThreadsB / Pol::NACC;
 }
 
 // (system, local row) of part-local unit u in the triangular layout
@@ -361,36 +343,40 @@ __device__ __forceinline__ void batch_sym_pairs(const PartArgs &A, int64_t cta, 
   }
 }
 
-// index of the system whose finish-CTA range holds f (binary search on fbeg)
-__device__ __forceinline__ int sys_of_fin(const PartArgs &A, int64_t f) {
+// index of the system whose finish blocks hold block b (binary search on bbeg)
+__device__ __forceinline__ int sys_of_block(const PartArgs &A, int64_t b) {
   int lo = 0, hi = A.nsys - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
-    if (A.sys[mid].fbeg <= f) lo = mid;
+    if (A.sys[mid].bbeg <= b) lo = mid;
     else hi = mid - 1;
   }
   return lo;
 }
 
-// Finish phase of one part, CTA f: chunk c of tile T of system s (as in sym.cu).
+// Finish phase of one part, CTA f: chunk c of block b (of tile T of a system).
 template <class Pol, int MODEL, int MODE>
 __device__ __noinline__ void batch_sym_finish(const PartArgs &A, int64_t f) {
-  constexpr int NACC = Pol::NACC, TJ = Pol::TJ;
+  constexpr int NACC = Pol::NACC, TJ = Pol::TJ, FB = finish_block<Pol>();
   constexpr int64_t TI = (int64_t)NT * Pol::R;
-  constexpr int OUT = (int)TI * NACC;
+  static_assert(TI % FB == 0, "whole blocks per tile");
   __shared__ bool s_last;
-  constexpr int CH = chunk_rows(OUT);
-  const int s = sys_of_fin(A, f);
-  const SysDesc &S = A.sys[s];
-  const int64_t lf = f - S.fbeg;
-  const int64_t T = fin_tile(lf, S.n_it, CH), tbeg = fin_prefix(T, CH);
-  const int c = (int)(lf - tbeg);
-  const int nch = (int)(T / CH + 1);
+  const int64_t b = f / A.nc;
+  const int c = (int)(f % A.nc);
+  const SysDesc &S = A.sys[sys_of_block(A, b)];
+  const int64_t lb = b - S.bbeg, T = lb / (TI / FB);
   const int m = A.m;
-  const int64_t I_lo = (int64_t)c * CH, I_hi = min(T + 1, I_lo + CH);
-  double *chunk = A.chunks + (S.fbeg + tbeg) * OUT;
-  for (int o = threadIdx.x; o < OUT; o += kFinishThreadsB) {
-    const int jsub = o / (TJ * NACC), rest = o % (TJ * NACC);
+  const int64_t ubeg = S.ubeg + sym_rowstart(T, S.n_jt, m);  // first unit of the row
+  const int64_t cf = cta_of_unit(A.U, A.P, ubeg);
+  const int64_t cl = cta_of_unit(A.U, A.P, S.ubeg + sym_rowstart(T + 1, S.n_jt, m) - 1);
+  const int nchc = (int)((T + kChunkB) / kChunkB), nch = nchc + (int)((cl - cf + kChunkB) / kChunkB);
+  if (c >= nch) return;
+  double *chunk = A.chunks + b * A.nc * kFinishThreadsB;
+  const int lr = (int)((lb % (TI / FB)) * FB) + threadIdx.x / NACC, d = threadIdx.x % NACC;
+  double v = 0.0;
+  if (c < nchc) {  // column partials of the rows I_lo .. (the diagonal units' included)
+    const int64_t I_lo = (int64_t)c * kChunkB, I_hi = min(T + 1, I_lo + kChunkB);
+    const int jsub = lr / TJ, rest = (lr % TJ) * NACC + d;
     CompSum cs{0.f, 0.f};
     // unit (I2, T m + jsub) advances by n_jt - m (I2 + 1) from I2 to I2 + 1
     int64_t off = (S.ubeg + sym_rowstart(I_lo, S.n_jt, m) + (T * m + jsub - (int64_t)m * I_lo)) * (TJ * NACC) + rest;
@@ -402,43 +388,40 @@ __device__ __noinline__ void batch_sym_finish(const PartArgs &A, int64_t f) {
       off += step;
       step -= dstep;
     }
-    chunk[(int64_t)c * OUT + o] = csum_total(cs);
+    v = -csum_total(cs);
+  } else if (cf == cl) {
+    v = __ldcg(A.rowfull + ((S.rbeg + T) * NACC + d) * TI + lr);
+  } else {
+    // virtual CTA c2 > cf begins inside the row: its first slot; cf may begin before it
+    const int64_t lo = cf + (int64_t)(c - nchc) * kChunkB, hi = min(cl + 1, lo + kChunkB);
+    const bool cf_first = unit_begin(A.U, A.P, cf) >= ubeg;
+    const double *src = A.slots + d * TI + lr;
+#pragma unroll 8
+    for (int64_t c2 = lo; c2 < hi; c2++)
+      v += __ldcg(src + (c2 * 2 + (c2 > cf || cf_first ? 0 : 1)) * (NACC * TI));
   }
+  chunk[c * kFinishThreadsB + threadIdx.x] = v;
   __threadfence();
   __syncthreads();
-  const int64_t row = S.rbeg + T;
-  if (threadIdx.x == 0) s_last = atomicAdd(&A.tickets[row], 1u) + 1u == (unsigned)nch;
+  if (threadIdx.x == 0) s_last = atomicAdd(&A.tickets[b], 1u) + 1u == (unsigned)nch;
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  const int64_t cf = cta_of_unit(A.U, A.P, S.ubeg + sym_rowstart(T, S.n_jt, m));
-  const int64_t cl = cta_of_unit(A.U, A.P, S.ubeg + sym_rowstart(T + 1, S.n_jt, m) - 1);
-  const PairArgs v = view(A, S);
-  for (int lr = threadIdx.x; lr < TI; lr += kFinishThreadsB) {
-    const int64_t i = T * TI + lr;
-    if (i >= S.N) break;
+  const int64_t i = lb * FB + threadIdx.x;
+  if (threadIdx.x < FB && i < S.N) {
     double tot[NACC];
-    if (cf == cl) {
 #pragma unroll
-      for (int d = 0; d < NACC; d++) tot[d] = __ldcg(A.rowfull + (row * NACC + d) * TI + lr);
-    } else {
+    for (int e = 0; e < NACC; e++) tot[e] = 0.0;
+    const double *mine = chunk + threadIdx.x * NACC;
+#pragma unroll 2
+    for (int k = 0; k < nch; k++) {  // segments, then columns
+      const int at = (k < nch - nchc ? nchc + k : k - (nch - nchc)) * kFinishThreadsB;
 #pragma unroll
-      for (int d = 0; d < NACC; d++) tot[d] = 0.0;
-      for (int64_t c2 = cf; c2 <= cl; c2++) {
-        int s2;
-        int64_t it2, jt2;
-        sym_locate(A, unit_begin(A.U, A.P, c2), s2, it2, jt2);
-        const double *src = A.slots + ((c2 * 2 + (row == A.sys[s2].rbeg + it2 ? 0 : 1)) * NACC) * TI;
-#pragma unroll
-        for (int d = 0; d < NACC; d++) tot[d] += __ldcg(src + d * TI + lr);
-      }
+      for (int e = 0; e < NACC; e++) tot[e] += __ldcg(mine + at + e);
     }
-    for (int c2 = 0; c2 < nch; c2++)
-#pragma unroll
-      for (int d = 0; d < NACC; d++) tot[d] -= __ldcg(chunk + (int64_t)c2 * OUT + lr * NACC + d);
-    finish<Pol, MODEL, true, MODE>(v, i, tot);
+    finish<Pol, MODEL, true, MODE>(view(A, S), i, tot);
   }
-  if (threadIdx.x == 0) A.tickets[row] = 0u;
+  if (threadIdx.x == 0) A.tickets[b] = 0u;
 }
 
 template <class Pol>
@@ -471,10 +454,11 @@ __global__ void __launch_bounds__(NT, Pol::MINB) batch_sym_pairs_kernel(PartArgs
 template <class PolR, class PolG, int MODE>
 __global__ void __launch_bounds__(kFinishThreadsB) batch_sym_finish_kernel(PartArgs ring, PartArgs grav) {
   if (blockIdx.x == 0 && threadIdx.x == 0) *ring.next = *grav.next = 0u;  // the pair kernels have ended
-  if ((int64_t)blockIdx.x < ring.nfin)
+  const int64_t nr = ring.nblk * ring.nc;
+  if ((int64_t)blockIdx.x < nr)
     batch_sym_finish<PolR, MD_RING, MODE>(ring, blockIdx.x);
   else
-    batch_sym_finish<PolG, MD_GRAV2D, MODE>(grav, (int64_t)blockIdx.x - ring.nfin);
+    batch_sym_finish<PolG, MD_GRAV2D, MODE>(grav, (int64_t)blockIdx.x - nr);
 }
 
 struct Config {
@@ -506,7 +490,7 @@ struct md_batch {
   int64_t graph_launches[2] = {0, 0};
   // unit / row layout uploaded for tile shapes and form (layout_key)
   int64_t layout_key[7] = {-1, -1, -1, -1, -1, -1, -1};
-  int64_t Ur = 0, Ug = 0, rows_r = 0, rows_g = 0, nfin_r = 0, nfin_g = 0;
+  int64_t Ur = 0, Ug = 0, rows_r = 0, rows_g = 0, blk_r = 0, blk_g = 0;
   int64_t rec_bytes_r = 0, rec_bytes_g = 0;  // forward-record bytes of each part's systems
   int nr = 0;
   int mirror_sym = -1;  // form the mirrors were written for (Ring records differ)
@@ -551,7 +535,7 @@ void drop_graphs(md_batch *b) {
 int build_layout(md_batch *b, const int64_t TI[2], const int64_t TJ[2], const int nacc[2], bool sym,
                  std::vector<SysDesc> &hs) {
   hs.clear();
-  b->Ur = b->Ug = b->rows_r = b->rows_g = b->nfin_r = b->nfin_g = 0;
+  b->Ur = b->Ug = b->rows_r = b->rows_g = b->blk_r = b->blk_g = 0;
   b->rec_bytes_r = b->rec_bytes_g = 0;
   b->nr = 0;
   for (int pass = 0; pass < 2; pass++) {
@@ -571,16 +555,15 @@ int build_layout(md_batch *b, const int64_t TI[2], const int64_t TJ[2], const in
       d.n_jt = sym ? m * d.n_it : (c->N + tj - 1) / tj;
       d.epsd = want == MD_RING ? 0.5 * c->eps : c->eps;
       d.dt = c->dt;
-      d.nfin = fin_prefix(d.n_it, chunk_rows(ti * nacc[pass]));
       int64_t &U = pass == 0 ? b->Ur : b->Ug;
       int64_t &rows = pass == 0 ? b->rows_r : b->rows_g;
-      int64_t &nfin = pass == 0 ? b->nfin_r : b->nfin_g;
+      int64_t &blk = pass == 0 ? b->blk_r : b->blk_g;
       d.ubeg = U;
       d.rbeg = rows;
-      d.fbeg = nfin;
+      d.bbeg = blk;
       U += sym ? sym_rowstart(d.n_it, d.n_jt, (int)m) : d.n_it * d.n_jt;
       rows += d.n_it;
-      nfin += d.nfin;
+      blk += sym ? d.n_it * (ti * nacc[pass] / kFinishThreadsB) : d.n_it;
       // forward records: Ring tensor-core fragments (symmetric form) or interleaved FP32
       (pass == 0 ? b->rec_bytes_r : b->rec_bytes_g) += c->N * (pass == 0 ? (sym ? 64 : 16) : 8);
       hs.push_back(d);
@@ -620,8 +603,9 @@ int grow(md_batch *b, T *&ptr, size_t &have, size_t need, const char *what) {
 }
 
 int ensure_tickets(md_batch *b) {
-  // a ticket per row of both parts, then the two parts' virtual-CTA counters
-  const size_t nt = (size_t)(b->rows_r + b->rows_g) + 2;
+  // a ticket per row (one-sided form) or finish block of both parts, then the two parts'
+  // virtual-CTA counters
+  const size_t nt = (size_t)(b->blk_r + b->blk_g) + 2;
   if (nt > b->tickets_count) {
     dev_free(b->tickets);
     b->tickets = (unsigned *)dev_alloc(nt * sizeof(unsigned));
@@ -691,7 +675,21 @@ int launch_batch_sym(md_batch *b, double bc, double dc) {
   const size_t slot_r = (size_t)Pr * 2 * NAr * TIr, slot_g = (size_t)Pg * 2 * NAg * TIg;
   const size_t row_r = (size_t)b->rows_r * NAr * TIr, row_g = (size_t)b->rows_g * NAg * TIg;
   const size_t col_r = (size_t)b->Ur * PolR::TJ * NAr, col_g = (size_t)b->Ug * PolG::TJ * NAg;
-  const size_t ch_r = (size_t)b->nfin_r * TIr * NAr, ch_g = (size_t)b->nfin_g * TIg * NAg;
+  // chunks per finish block: a system's row T has at most (n_jt - m T) P / U + 2 segments and
+  // T + 1 column rows; the bound is linear in T, the larger of its ends counts
+  auto chunks_of = [&](int model, int64_t ti, int64_t tj, int64_t P, int64_t U) {
+    int64_t nc = 1;
+    for (int s = 0; s < b->nsys; s++) {
+      if (b->model[s] != model) continue;
+      const int64_t m = ti / tj, n_it = (b->ctx[s]->N + ti - 1) / ti, n_jt = m * n_it;
+      for (const int64_t T : {(int64_t)0, n_it - 1})
+        nc = std::max<int64_t>(nc, (T + kChunkB) / kChunkB + ((n_jt - m * T) * P / U + 2 + kChunkB - 1) / kChunkB);
+    }
+    return (int)nc;
+  };
+  const int nc_r = b->Ur > 0 ? chunks_of(MD_RING, TIr, PolR::TJ, Pr, b->Ur) : 1;
+  const int nc_g = b->Ug > 0 ? chunks_of(MD_GRAV2D, TIg, PolG::TJ, Pg, b->Ug) : 1;
+  const size_t ch_r = (size_t)b->blk_r * nc_r * kFinishThreadsB, ch_g = (size_t)b->blk_g * nc_g * kFinishThreadsB;
   if ((rc = grow(b, b->slots, b->slots_bytes, (slot_r + slot_g) * sizeof(double), "batch slots")) ||
       (rc = grow(b, b->rowfull, b->rowfull_bytes, (row_r + row_g) * sizeof(double), "batch row partials")) ||
       (rc = grow(b, b->colslot, b->colslot_bytes, (col_r + col_g) * sizeof(float), "batch column partials")) ||
@@ -704,9 +702,10 @@ int launch_batch_sym(md_batch *b, double bc, double dc) {
   ar.U = b->Ur;
   ar.P = (int)Pr;
   ar.waves = Wr;
-  ar.next = b->tickets + b->rows_r + b->rows_g;
+  ar.next = b->tickets + b->blk_r + b->blk_g;
   ar.m = (int)(TIr / PolR::TJ);
-  ar.nfin = b->nfin_r;
+  ar.nblk = b->blk_r;
+  ar.nc = nc_r;
   ar.slots = b->slots;
   ar.rowfull = b->rowfull;
   ar.colslot = b->colslot;
@@ -719,12 +718,13 @@ int launch_batch_sym(md_batch *b, double bc, double dc) {
   ag.waves = Wg;
   ag.next = ar.next + 1;
   ag.m = (int)(TIg / PolG::TJ);
-  ag.nfin = b->nfin_g;
+  ag.nblk = b->blk_g;
+  ag.nc = nc_g;
   ag.slots = b->slots + slot_r;
   ag.rowfull = b->rowfull + row_r;
   ag.colslot = b->colslot + col_r;
   ag.chunks = b->chunks + ch_r;
-  ag.tickets = b->tickets + b->rows_r;
+  ag.tickets = b->tickets + b->blk_r;
   ar.cur = ag.cur = b->cur;
   ar.b = ag.b = bc;
   ar.d = ag.d = dc;
@@ -736,7 +736,7 @@ int launch_batch_sym(md_batch *b, double bc, double dc) {
     kern_g<<<(int)Gg, NT, 0, b->stream>>>(ag);
     b->launches++;
   }
-  batch_sym_finish_kernel<PolR, PolG, MODE><<<(unsigned)(b->nfin_r + b->nfin_g), kFinishThreadsB, 0, b->stream>>>(ar, ag);
+  batch_sym_finish_kernel<PolR, PolG, MODE><<<(unsigned)(b->blk_r * nc_r + b->blk_g * nc_g), kFinishThreadsB, 0, b->stream>>>(ar, ag);
   b->launches++;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return berr(b, MD_ECUDA, "batch launch: %s", cudaGetErrorString(e));
