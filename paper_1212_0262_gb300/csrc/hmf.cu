@@ -64,21 +64,31 @@ __device__ __forceinline__ void load_sincos_tab(double2 *sm) {
 // operations (12 with the sine and cosine of sincos_fp64.cuh and an FP64 force, which bound
 // the stage).  Per stage at N = 5e7: 1149 -> 582 us, 3.2 GB at 81% of the copy rate; the
 // integer pipe is half busy, the next pair's loads run ahead of the arithmetic (604 us without).
-// A non-finite angle is marked by kNoAngle: its force is NaN, and the sums of the stages leave
-// it out.
+// A non-finite angle is marked by kNoAngle: its force is NaN, and so are the sums.
 __device__ scfx::Entry g_sincos_fx[kTabN];
 constexpr int kNoAngle = (int)0x80000000;
 
+// Set by a thread of this CTA that met a non-finite angle.  In shared memory: as a NaN in the
+// thread's FP64 sums it would keep registers through the sweep (12 bytes of spills).
+__device__ __forceinline__ volatile int &no_angle_flag() {
+  __shared__ int flag;
+  return flag;
+}
+
 __device__ __forceinline__ void load_sincos_fx(scfx::Entry *sm) {
+  if (threadIdx.x == 0) no_angle_flag() = 0;
   for (int k = threadIdx.x; k < kTabN; k += blockDim.x) sm[k] = g_sincos_fx[k];
   __syncthreads();
 }
 
-// (cos, sin) of th as stored (cos.h, cos.l, sin.h, sin.l), and their sums in units of 2^-54
+// (cos, sin) of th as stored (cos.h, cos.l, sin.h, sin.l), and their sums in units of 2^-54.
 __device__ __forceinline__ int4 angle_fx(double th, const scfx::Entry *tab, long long &aci, long long &asi) {
   fx64::i64 s62, c62;
   if (!scfx::sincos_fx(th, tab, s62, c62)) {
-    if (!(fabs(th) <= 1.7976931348623157e308)) return make_int4(kNoAngle, 0, 0, 0);
+    if (!(fabs(th) <= 1.7976931348623157e308)) {
+      no_angle_flag() = 1;
+      return make_int4(kNoAngle, 0, 0, 0);
+    }
     double s, c;
     sincos(th, &s, &c);
     s62 = __double2ll_rn(s * 0x1p62);
@@ -158,9 +168,9 @@ __device__ __forceinline__ void hmf_particle_fp64(double &th, double &pp, int4 &
                                                   const scfx::Entry *tab) {
   const fx64::Limbs c{cs.x, cs.y}, s{cs.z, cs.w};
   double f = scfx::to_double60(fx64::dot2(c, s, m.my, m.nmx));  // cos My - sin Mx
-  if (a.invN == 1.0) f = 0.0;  // a lone particle's self-term
   if (!m.fx) f = hmf_force_fp64((double)scfx::join(c.h, c.l) * 0x1p-62, (double)scfx::join(s.h, s.l) * 0x1p-62, mx, my, a.invN);
   if (cs.x == kNoAngle) f = __longlong_as_double(0x7ff8000000000000LL);
+  if (a.invN == 1.0) f = 0.0;  // a lone particle's self-term
   if (MODE == STAGE_FORCE_ONLY) {
     a.fout[i] = f;
     return;
@@ -307,6 +317,7 @@ __device__ __forceinline__ void hmf_sweep(const HmfArgs &a, double mx, double my
     } else {
       acd += (double)aci * 0x1p-54;
       asd += (double)asi * 0x1p-54;
+      if (no_angle_flag()) acd = asd = __longlong_as_double(0x7ff8000000000000LL);
     }
   }
 }
@@ -395,8 +406,8 @@ __global__ void __launch_bounds__(NT, 3) hmf_run_fp64_kernel(HmfArgs a, HmfRun r
   cluster.sync();  // no CTA leaves while another reads its partial sums
 }
 
-// Sum of a thread's at most five cosines (or sines) in units of 2^-38: exact for an FP32 sum
-// of 2^-15 and more, within 2^-39 below.
+// Sum of a thread's at most five cosines (or sines), below 8, in units of 2^-38: exact for an
+// FP32 sum of 2^-15 and more, within 2^-39 below.
 __device__ __forceinline__ long long fix38(float v) {
   const float h = rintf(v * 0x1p28f);  // below 2^31
   return ((long long)__float2int_rn(h) << 10) + __float2int_rn((v - h * 0x1p-28f) * 0x1p38f);
@@ -407,12 +418,17 @@ __device__ __forceinline__ long long fix38(float v) {
 // p + G, in the other order.  The groups' FP32 sums are added as integers (the launched stages
 // add them in FP64, where they are exact too, but for sums below 2^-16 whose last bits are
 // beyond M's FP32): every warp puts its total into every CTA's shared memory, and after the
-// cluster barrier every warp adds them for itself.
+// cluster barrier every warp adds them for itself.  A drift of some 2^23 and more in one stage
+// leaves the FP32 reduction's range: its cosine can be of any size, infinite or NaN.  A warp
+// that holds one puts kWildSum in place of its total, every CTA sees it in the sum, and the
+// stage's sums are added in FP64, as the launched stages do.
+constexpr long long kWildSum = 1ll << 54;  // the particles' own sums stay below 2^53, 128 of these below 2^62
 __global__ void __launch_bounds__(NT, 1) hmf_run_mixed_kernel(HmfArgs a, HmfRun r) {
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   constexpr int NW = NT / 32;
   __shared__ longlong2 part[2][kRunCtas * NW];
+  __shared__ double2 wide, red[NW];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int64_t npairs = a.N >> 1, G = (int64_t)gridDim.x * NT;
   const int64_t t0 = (int64_t)blockIdx.x * NT + threadIdx.x;
@@ -446,18 +462,16 @@ __global__ void __launch_bounds__(NT, 1) hmf_run_mixed_kernel(HmfArgs a, HmfRun 
     const bool f = r.rev(st, a.rev) != 0;
     const float ac = (((f ? c[1][0] : c[0][0]) + (f ? c[1][1] : c[0][1])) + (f ? c[0][0] : c[1][0])) + (f ? c[0][1] : c[1][1]);
     const float as = (((f ? s[1][0] : s[0][0]) + (f ? s[1][1] : s[0][1])) + (f ? s[0][0] : s[1][0])) + (f ? s[0][1] : s[1][1]);
-    longlong2 v = make_longlong2(fix38(ac), fix38(as));
-    if (odd) {
-      float co = 0.f, so = 0.f;
-      hmf_particle_mixed<STAGE_KICK_DRIFT>(qo, po, a, mxf, myf, dtf, co, so, 0);
-      v.x += fix38(co);
-      v.y += fix38(so);
-    }
+    float co = 0.f, so = 0.f;
+    if (odd) hmf_particle_mixed<STAGE_KICK_DRIFT>(qo, po, a, mxf, myf, dtf, co, so, 0);
+    const bool tame = fabsf(ac) + fabsf(as) + fabsf(co) + fabsf(so) < 8.f;  // five angles: at most 5 sqrt(2)
+    longlong2 v = make_longlong2(fix38(ac) + fix38(co), fix38(as) + fix38(so));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
       v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
     }
+    if (!__all_sync(0xffffffffu, tame)) v.x = kWildSum;
     longlong2 *slot = &part[st & 1][blockIdx.x * NW + w];
     if (lane < (int)gridDim.x) *cluster.map_shared_rank(slot, lane) = v;
     cluster.sync();
@@ -473,6 +487,21 @@ __global__ void __launch_bounds__(NT, 1) hmf_run_mixed_kernel(HmfArgs a, HmfRun 
     }
     sx = (double)v.x * 0x1p-38;
     sy = (double)v.y * 0x1p-38;
+    if (v.x > kWildSum / 2) {  // the same in every thread of the cluster
+      const double2 b = block_sum2<NT>((double)ac + (double)co, (double)as + (double)so, red);
+      if (threadIdx.x == 0) wide = b;
+      cluster.sync();
+      double2 d = make_double2(0.0, 0.0);
+      if (lane < (int)gridDim.x) d = *cluster.map_shared_rank(&wide, lane);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        d.x += __shfl_down_sync(0xffffffffu, d.x, o);
+        d.y += __shfl_down_sync(0xffffffffu, d.y, o);
+      }
+      sx = __shfl_sync(0xffffffffu, d.x, 0);
+      sy = __shfl_sync(0xffffffffu, d.y, 0);
+      cluster.sync();  // every CTA has read them before the next such stage writes
+    }
   }
 #pragma unroll
   for (int u = 0; u < 2; u++)
@@ -505,13 +534,12 @@ __global__ void __launch_bounds__(NT) hmf_prime_fp64_kernel(const double *__rest
     const int64_t iend = ib + block < N ? ib + block : N;
     long long aci = 0, asi = 0;
     for (int64_t i = ib; i < iend; i += G) {
-      const int4 v = angle_fx(q[i], tab, aci, asi);
-      cs[i] = v;
-      if (v.x == kNoAngle) acd = __longlong_as_double(0x7ff8000000000000LL);
+      cs[i] = angle_fx(q[i], tab, aci, asi);
     }
     acd += (double)aci * 0x1p-54;
     asd += (double)asi * 0x1p-54;
   }
+  if (no_angle_flag()) acd = asd = __longlong_as_double(0x7ff8000000000000LL);
   grid_finish(acd, asd, partials, m_out, ticket);
 }
 

@@ -40,3 +40,24 @@ def test_more_steps_than_one_launch_holds():
             out.append(s.get_state())
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("prec", ["mixed", "fp64"])
+@pytest.mark.parametrize("N", [2, 1025, 10_007])
+@pytest.mark.parametrize("speed", [1e7, 1e12, 1e36, 1.7e308, np.inf, np.nan])
+def test_angles_beyond_any_range(N, prec, speed):
+    """One particle's speed drives its angle out of the FP32 reduction's range, or to infinity:
+    the other particles feel what they feel in the launched stages."""
+    q, p = inputs.default_state(0, N, 5)
+    p[N // 2] = speed
+    out = []
+    for graphs in (1, 0):
+        with System(0, N, 0.0, 10.0, 1, precision=prec) as s:
+            s.set_tuning("step_graphs", graphs)
+            s.set_state(q, p)
+            s.step(1)
+            out.append(s.get_state())
+    for a, b in zip(*out):
+        assert np.array_equal(a, b, equal_nan=True)
+    if prec == "fp64" and not abs(speed) < 1e308:  # a sum with a non-finite angle is NaN
+        assert np.all(np.isnan(out[0][1]))
