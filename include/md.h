@@ -143,9 +143,12 @@ int md_set_eps(md_ctx *ctx, double eps);
  *                      orders, Sec. 3.2).  Needs column-partial storage of about
  *                      N^2 / 128 bytes (Ring, FP32 or FP64), N^2 / 256 (FP32 2D),
  *                      N^2 / 64 (FP64 2D), 3 N^2 / 256 (FP32 3D) or N^2 / 512 (FP32
- *                      sheets, eps > 0; at eps = 0 the sheets' counts come from ranks
- *                      in sorted tiles, the same whole numbers); above 16 GiB of it (N beyond about 1.48e6 for Ring,
- *                      2.1e6 for FP32 2D) the one-sided kernel runs.
+ *                      sheets, eps > 0), FP64 up to N = 262,144 twice that; above 16 GiB
+ *                      of it (N beyond about 1.48e6 for Ring, 2.1e6 for FP32 2D) the
+ *                      one-sided kernel runs.  Sheets at eps = 0 count ranks in sorted
+ *                      tiles instead (the same whole numbers, no such storage).  FP64 2D
+ *                      md_grad / md_tangent_step stages take this form too (3 N^2 / 16
+ *                      bytes up to N = 10,000, 3 N^2 / 32 above).
  *   "step_graphs"      md_step replays its steps after the first from captured CUDA
  *                      graphs of 8 steps (1, default) or launches every stage (0).
  * MD_EINVAL for an unknown key or value. */

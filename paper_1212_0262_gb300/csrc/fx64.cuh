@@ -3,9 +3,8 @@
 // GB300 issues about 2 FP64 operations per SM and clock, against 64 32 x 32 -> 64 bit
 // multiply-adds and 128 integer adds (measured: mad.wide.u32 60, add 120, DFMA 1.9 per SM
 // and clock): an FP64 operation costs as much issue time as some 30 multiply-adds.  The
-// FP64 pair kernels therefore keep on the FP64 pipe only the operations that need a
-// floating-point alignment (coordinate differences, squared distance) and do the rest on
-// mantissas held as integers.  Every quantity keeps at least the 53 bits of a double
+// FP64 pair kernels therefore keep on the FP64 pipe only the coordinate differences (and
+// the FP64 sums of the 2D reverse stages) and do the rest on mantissas held as integers.  Every quantity keeps at least the 53 bits of a double
 // (errors below 2^-57 relative, noted at each function), and sums are exact.
 //
 // The header has no GPU-only constructs but the reciprocal seed and the carry chain, so
