@@ -40,8 +40,8 @@ WORKLOADS = {
                    name="2D self-gravitating N=262,144 eps=1e-4 dt=0.01 (all-pairs)"),
     "grav3d": dict(model=3, N=131_072, eps=1e-3, dt=0.01, seed=5, unit="pair-interactions/s",
                    name="3D self-gravitating N=131,072 eps=1e-3 dt=0.01 (all-pairs; not one of the paper's models)"),
-    "sheet1d": dict(model=4, N=262_144, eps=0.0, dt=0.01, seed=6, unit="pair-interactions/s",
-                    name="1D sheets N=262,144 eps=0 dt=0.01 (all-pairs sign counts; not one of the paper's models)"),
+    "sheet1d": dict(model=4, N=262_144, eps=0.0, dt=0.01, seed=6, unit="particle-steps/s",
+                    name="1D sheets N=262,144 eps=0 dt=0.01 (sign counts from ranks; not one of the paper's models)"),
     "adjoint": dict(model=2, N=262_144, eps=1e-4, dt=0.01, seed=4, unit="pair-interactions/s",
                     name="2D N=262,144 eps=1e-4 dt=0.01: gradient of K(T) after 100 steps (forward + "
                          "reversed adjoint, checkpoints every 20 steps)"),
@@ -51,10 +51,14 @@ WORKLOADS = {
 }
 # algorithmic bytes per particle per fused HMF stage: read + write FP64 theta and p
 HMF_BYTES_PER_PARTICLE_STAGE = 32
-# FP64-pipe operations per particle of the FP64 HMF stage (its bound): the force
+# bytes per particle of an FP64 HMF stage: theta and p, and the fixed-point (cos, sin) of the
+# angles, read and written
+HMF_FP64_BYTES_PER_PARTICLE_STAGE = 64
+# FP64-pipe operations per particle of an HMF stage done in FP64 throughout: the force
 # cos(theta) My - sin(theta) Mx (product + FMA), the kick and the drift (2 FMA), the
 # table-driven sine and cosine of the new angle (8: exact FMA reduction, r^2, cos r - 1,
-# sin r, two FMAs each for the angle addition)
+# sin r, two FMAs each for the angle addition).  The stage runs all but the kick and the drift
+# on the integer pipe; its rate against this pipe bound is reported beside its HBM roofline.
 HMF_FP64_OPS_PER_PARTICLE_STAGE = 12
 # FP32-pipe operations and SFU operations per pair in the mixed pair kernels
 PAIR_OPS = {1: (8, 1), 2: (6, 1), 3: (11, 1), 4: (4, 0)}
@@ -81,19 +85,21 @@ PAIR_KERNELS = {
 # FP64 kernels: name, FP64-pipe operations per evaluated pair term (the reciprocal
 # square root or reciprocal: FP32 seed on the SFU with integer-pipe conversions, then
 # 5 or 3 FP64 operations), whether each unordered pair is evaluated once.
-#   Ring: S and sin(d/2) (2 each), dd, rsqrt (5); symmetric: S y^3 (3), row and column
-#   adds, butterfly 1/2 -> 15.5; one-sided: S y, y^2, accumulate -> 13
-#   2D: dx, dy, s (2), rcp (3); symmetric: 2 products, 2 row and 2 column adds,
-#   butterfly 1 -> 14; one-sided: 2 FMA accumulations -> 9
-#   3D: dx, dy, dz, s (3), rsqrt (5), y^3 (2); symmetric: 3 products, 3 + 3 adds,
-#   butterfly 1.4 -> 23.4; one-sided: 3 FMA accumulations -> 16
+#   Ring: S and sin(d/2) (2 each), dd, rsqrt (5), S y, y^2, accumulate -> 13
+#   2D: dx, dy, s (2), rcp (3), 2 FMA accumulations -> 9
+#   3D: dx, dy, dz, s (3), rsqrt (5), y^3 (2), 3 FMA accumulations -> 16
 PAIR_KERNELS_FP64 = {
-    (1, 6): ("sym_kernel<RingF64<4,128>>", 15.5, True),
     (1, 1): ("streamk_kernel<RingF64<2,128>>", 13, False),
-    (2, 6): ("sym_kernel<GravF64<4,128>>", 14, True),
     (2, 1): ("streamk_kernel<GravF64<2,128>>", 9, False),
-    (3, 6): ("sym_kernel<Grav3DF64<4,128>>", 23.4, True),
     (3, 1): ("streamk_kernel<Grav3DF64<2,128>>", 16, False),
+}
+# The symmetric FP64 kernels run the pair arithmetic on the integer pipe: name and
+# instructions issued per unordered pair (ncu, N = 49,152; 3D from its share of the 2D rate),
+# against 128 lanes per SM and clock
+PAIR_KERNELS_INT = {
+    (1, 6): ("sym_pairs_kernel<RingFx>", 137),
+    (2, 6): ("sym_pairs_kernel<FxGrav<2>>", 147),
+    (3, 6): ("sym_pairs_kernel<FxGrav<3>>", 235),
 }
 
 
@@ -416,7 +422,7 @@ def run_reference(args, w):
     else:
         n = oracle_sample_size(w, 60.0, K + W, cores)
         units, el, sample = oracle_steps(w, n, K, W, cores)
-        rate = units / el
+        rate = oracle_rate(w, units, el)
     line = {
         "impl": "reference", "metric": METRIC, "value": rate, "unit": w["unit"], "n_gpus": args.gpus,
         "steps": K, "warmup": W, "ms_per_step": 1e3 * el / K, "higher_is_better": True, "scaling": "weak",
@@ -468,6 +474,17 @@ def pipe_rates():
     return rates
 
 
+def units_of(w) -> float:
+    """Units of one integrator step: particles (HMF, and the sheets, whose forces are rank
+    counts) or the 3 N^2 ordered pairs of its force evaluations."""
+    return float(w["N"]) if w["unit"] == "particle-steps/s" else 3.0 * w["N"] * w["N"]
+
+
+def oracle_rate(w, units: float, seconds: float) -> float:
+    """Rate of an oracle leg in the workload's unit (its pair sums count pairs)."""
+    return units / seconds / (3.0 * w["N"] if w["model"] > 0 and w["unit"] == "particle-steps/s" else 1.0)
+
+
 def pair_roofline(workload, model, N, kcode, prec, stage_ms, clocks, tuned):
     """Roofline object of a pair-model run: algorithmic pair terms per stage over the
     average stage time, against the pipe-bound rate of the kernel that ran (FP32 and
@@ -485,8 +502,12 @@ def pair_roofline(workload, model, N, kcode, prec, stage_ms, clocks, tuned):
     if f64:  # FP64 kernels: bound by the FP64 pipe (measured DFMA rate)
         kname, dops, sym = f64
         pairs_per_clk = rates[13] / dops
-    if prec == "fp64" and not f64:
-        return None  # FP64 sheets: sign counting, no stated pipe bound
+    fxk = PAIR_KERNELS_INT.get((model, kcode)) if prec == "fp64" else None
+    if fxk:
+        kname, instr = fxk
+        sym, pairs_per_clk = True, 128.0 / instr
+    if model == 4 or (prec == "fp64" and not f64 and not fxk):
+        return None  # sheets: ranks in sorted tiles, no pair terms and no stated pipe bound
     mhz = clocks.get("sm_mhz") or rates[2]
     max_mhz = clocks.get("sm_max_mhz") or rates[2]
     peak = nsm * pairs_per_clk * mhz * 1e6
@@ -506,7 +527,9 @@ def pair_roofline(workload, model, N, kcode, prec, stage_ms, clocks, tuned):
             "unit": "unordered pair terms/s" if sym else "pair-interactions/s",
             "frac": achieved / peak, "frac_at_max_clock": achieved / (peak * max_mhz / mhz), "traffic": traffic,
             "kernel": f"{kname}, {prec}",
-            "peak_derivation": ({"sms": nsm, "fp64_ops_per_sm_clk": rates[13], "fp64_ops_per_pair": f64[1],
+            "peak_derivation": ({"sms": nsm, "issue_lanes_per_sm_clk": 128.0, "instructions_per_pair": fxk[1],
+                                 "sm_mhz": mhz, "sm_max_mhz": max_mhz} if fxk else
+                                {"sms": nsm, "fp64_ops_per_sm_clk": rates[13], "fp64_ops_per_pair": f64[1],
                                  "sm_mhz": mhz, "sm_max_mhz": max_mhz} if f64 else
                                 {"sms": nsm, "fp32_ops_per_sm_clk": fp32_rate,
                                  "sfu_ops_per_sm_clk": sfu_rate, "fp32_ops_per_pair": fops,
@@ -515,7 +538,7 @@ def pair_roofline(workload, model, N, kcode, prec, stage_ms, clocks, tuned):
 
 
 def hmf_fp64_roofline(particle_steps_per_s, rates, clocks):
-    """Roofline object of the FP64 HMF path, which the FP64 pipe bounds: 3 stages per step
+    """The FP64 HMF path against the bound of a stage done on the FP64 pipe: 3 stages per step
     of HMF_FP64_OPS_PER_PARTICLE_STAGE FP64 operations per particle, against the SM count
     times the measured FP64 FMA rate per SM per clock (mdp_pipe_rates) at the SM clock
     sampled during the timed region (the rate's own clock without one); also the
@@ -531,6 +554,14 @@ def hmf_fp64_roofline(particle_steps_per_s, rates, clocks):
             "peak_derivation": {"sms": nsm, "fp64_ops_per_sm_clk": dfma,
                                 "fp64_ops_per_particle_stage": HMF_FP64_OPS_PER_PARTICLE_STAGE,
                                 "sm_mhz": mhz, "sm_max_mhz": max_mhz}}
+
+
+def hmf_fp64_pipe_form(rates, clocks):
+    """What a stage that does its 12 operations on the FP64 pipe could reach at the sampled
+    clock; the stage has 2 of them there and passes it."""
+    r = hmf_fp64_roofline(0.0, rates, clocks)
+    return {"particle_steps_per_s_bound": r["peak"] / (3.0 * HMF_FP64_OPS_PER_PARTICLE_STAGE),
+            "peak_derivation": r["peak_derivation"]}
 
 
 def secondary_pair(workload, K, W, local, prec="mixed"):
@@ -562,7 +593,7 @@ def secondary_pair(workload, K, W, local, prec="mixed"):
         e1 = sum(s.energy())
         kcode = s.force_kernel
         del flush
-    return {"workload": w["name"], "value": 3.0 * N * N * K / (elapsed_ms * 1e-3), "unit": w["unit"],
+    return {"workload": w["name"], "value": units_of(w) * K / (elapsed_ms * 1e-3), "unit": w["unit"],
             "steps": K, "warmup": W, "ms_per_step": elapsed_ms / K, "precision": prec,
             "rel_energy_error": abs((e1 - e0) / e0), "energy_error_steps": W + K,
             "rel_energy_error_after_warmup": abs((e_w - e0) / e0),
@@ -680,19 +711,20 @@ def run_ours(args, w):
                     "timing": "CUDA events around md_step(K) on its stream",
                     "peak_source": f"{src} (MEASURED_PEAKS.json hbm_gbs)"}
         if args.prec == "fp64":
-            # the FP64 stage is bound by the FP64 pipe, not by HBM: that roofline, with the
-            # HBM figures beside it (a failure here leaves the HBM object and says why)
+            # the FP64 stages also read and write the fixed-point (cos, sin); the bound that an
+            # FP64 stage would have on the FP64 pipe stands beside the HBM figures
+            region_bytes = float(N) * (HMF_FP64_BYTES_PER_PARTICLE_STAGE * 3 * K + 40)
+            achieved = region_bytes / (elapsed_ms * 1e-3) / 1e9
+            roofline.update({"achieved": achieved, "frac": achieved / peaks["hbm_gbs"], "traffic": None,
+                             "algorithmic_bytes_per_launch": HMF_FP64_BYTES_PER_PARTICLE_STAGE * N,
+                             "timed_region_bytes": region_bytes})
             try:
-                hbm = roofline
-                roofline = hmf_fp64_roofline(N * K / (elapsed_ms * 1e-3), pipe_rates(), clocks)
-                roofline.update({"hbm": {k: hbm[k] for k in ("achieved", "peak", "unit", "frac")},
-                                 "avg_launch_ms": avg_ms, "launches": n_launch, "timing": hbm["timing"]})
+                roofline["fp64_pipe_form"] = hmf_fp64_pipe_form(pipe_rates(), clocks)
             except Exception as e:  # noqa: BLE001 -- the line is printed either way
-                roofline = hbm
-                roofline["fp64_pipe_error"] = repr(e)
+                roofline["fp64_pipe_form"] = {"error": repr(e)}
     else:
-        units_per_step = 3 * N * N
-        value = ws * 3 * N * N * K / (elapsed_ms * 1e-3)
+        units_per_step = units_of(w)
+        value = ws * units_per_step * K / (elapsed_ms * 1e-3)
         roofline = pair_roofline(args.workload, model, N, sysm.force_kernel, args.prec, stage_ms, clocks, args.tune)
 
     # FP64 path on the same workload (few steps) and the matching mixed energy error
@@ -724,15 +756,18 @@ def run_ours(args, w):
                 b.synchronize()
                 ms = a.elapsed_time(b)
                 e_b = sum(s2.energy())
-                units = N * ksh if model == 0 else 3 * N * N * ksh
+                units = units_of(w) * ksh
                 res[prec] = {"value": units / (ms * 1e-3), "ms_per_step": ms / ksh,
                              "rel_energy_error": abs((e_b - e_a) / e_a), "steps": ksh + 1}
         extra["fp64_path"] = res["fp64"]
-        if model == 0:  # its FP64-pipe roofline at the clock sampled in the timed region above
+        if model == 0:  # its HBM roofline, and the FP64-pipe form's at the clock sampled above
+            gbs = res["fp64"]["value"] * 3 * HMF_FP64_BYTES_PER_PARTICLE_STAGE / 1e9
+            extra["fp64_path"]["roofline"] = {"bound": "hbm", "achieved": gbs, "peak": peaks["hbm_gbs"], "unit": "GB/s",
+                                              "frac": gbs / peaks["hbm_gbs"]}
             try:
-                extra["fp64_path"]["roofline"] = hmf_fp64_roofline(res["fp64"]["value"], pipe_rates(), clocks)
+                extra["fp64_path"]["roofline"]["fp64_pipe_form"] = hmf_fp64_pipe_form(pipe_rates(), clocks)
             except Exception as e:  # noqa: BLE001 -- the line is printed either way
-                extra["fp64_path"]["roofline"] = {"error": repr(e)}
+                extra["fp64_path"]["roofline"]["fp64_pipe_form"] = {"error": repr(e)}
         extra["mixed_path_long_run"] = res["mixed"]
         T = res["mixed"]["steps"] * w["dt"]
         extra["energy_error"] = {"mixed_after_%d_steps" % (res["mixed"]["steps"]): res["mixed"]["rel_energy_error"],
@@ -767,7 +802,7 @@ def run_ours(args, w):
             runs.append(tp)
         tp = sorted(runs, key=lambda t: t[-1] - t[0])[1]
         el = tp[-1] - tp[0]
-        e2e = {"value": (N * ke if model == 0 else 3 * N * N * ke) / el, "unit": w["unit"],
+        e2e = {"value": units_of(w) * ke / el, "unit": w["unit"],
                "h2d_bytes_per_step": 2 * 8 * n / ke, "d2h_bytes_per_step": (2 * 8 * n + (16 if model == 0 else 0)) / ke,
                "steps": ke, "note": "md_set_state(host) + md_step + " + ("md_energy + " if model == 0 else "")
                + "md_get_state(host), wall clock" + ("" if model == 0 else
@@ -786,8 +821,8 @@ def run_ours(args, w):
         if model == 0:  # capped replicas: more steps instead, about the same seconds
             ksteps = max(ksteps, int(round(ksteps * oracle_sample_size(w, 10.0, ksteps) / n)))
         units, el, sample = oracle_steps(w, n, ksteps, 0, cores)
-        cpu = {"value": units / el, "unit": w["unit"], "cores": cores, "kind": "oracle", "sample": sample,
-               "seconds": el, "single_core": {"value": u1 / e1, "sample": s1, "seconds": e1}}
+        cpu = {"value": oracle_rate(w, units, el), "unit": w["unit"], "cores": cores, "kind": "oracle", "sample": sample,
+               "seconds": el, "single_core": {"value": oracle_rate(w, u1, e1), "sample": s1, "seconds": e1}}
 
     # the other configurations, each a short driver-clocked run with its own clock
     # record and roofline: Ring (N = 131,072), 2D forward (N = 262,144) and the ensemble
