@@ -89,6 +89,8 @@ struct md_ctx {
   size_t sym_chunk_bytes = 0;
   unsigned *fx_vmax = nullptr;    // integer reverse stages: the largest |v| of this stage and the next (ping-pong)
   int fx_vcur = 0;
+  bool fx_wide_units = false;     // the small units' column partials did not fit in memory,
+  bool sym_reverse_off = false;   // nor those of the symmetric reverse stages
 
   // reductions (energies)
   double *red = nullptr;
@@ -224,7 +226,7 @@ bool sym_applies(const md_ctx *c);
 int sym_pair_stage(md_ctx *c, int mode, double kick, double drift, double *fout);
 
 // and of the FP64 2D reverse and tangent stages (STAGE_ADJOINT, STAGE_TANGENT)
-bool sym_reverse_applies(const md_ctx *c);
+bool sym_reverse_applies(md_ctx *c);
 int sym_reverse_stage(md_ctx *c, int mode, double kick, double undo, double drift, double *lq, double *lp,
                       double *epsacc);
 

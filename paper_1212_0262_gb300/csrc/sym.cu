@@ -395,6 +395,25 @@ int launch_sym(md_ctx *c, PairArgs a) {
   return MD_OK;
 }
 
+// Bytes of the column partials: one per unit, column and component.
+size_t column_bytes(int64_t N, int64_t TI, int64_t TJ, int nacc, int col) {
+  const int64_t m = TI / TJ, n_it = (N + TI - 1) / TI;
+  return (size_t)sym_rowstart(n_it, m * n_it, (int)m) * TJ * nacc * col;
+}
+
+// The context's column buffer made this large; false if the memory is not to be had.  Inside a
+// caller's capture, where nothing can be allocated, the stage itself reports what is missing.
+bool reserve_columns(md_ctx *c, size_t need) {
+  if (need <= c->sym_colslot_bytes) return true;
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c->stream, &st) != cudaSuccess) cudaGetLastError();
+  else if (st != cudaStreamCaptureStatusNone) return true;
+  dev_free(c->sym_colslot);
+  c->sym_colslot = dev_alloc(need);
+  c->sym_colslot_bytes = c->sym_colslot ? need : 0;
+  return c->sym_colslot != nullptr;
+}
+
 // FP64 stages with integer pair arithmetic: Fx<rows per thread, j-tile>.  A unit is one
 // CTA's work of 128 rows x tile, 256 x tile, 512 x tile pairs, and a pair takes thousands of
 // cycles of latency, so small systems want small units (N = 1,000, microseconds per force,
@@ -402,10 +421,19 @@ int launch_sym(md_ctx *c, PairArgs a) {
 // the column reductions (N = 16,385: 967, 915, 1020; N = 8,192: 264, 281, 343).  <4, 128> needs
 // half the column storage of <2, 64> and is 2-5% slower (N = 49,152: 7.17 against 7.07 ms).
 constexpr int64_t kFxSmall = 10000, kFxLarge = 262144;
+// Where it does not fit (the caller's allocator may be bounded), <4, 128> runs at every size.
 template <template <int, int> class Fx, int MODEL, int MODE>
 int fx_dispatch(md_ctx *c, PairArgs a) {
-  if (c->N <= kFxSmall) return launch_sym<Fx<1, 64>, MODEL, false, MODE>(c, a);
-  if (c->N <= kFxLarge) return launch_sym<Fx<2, 64>, MODEL, false, MODE>(c, a);
+  constexpr int NACC = Fx<4, 128>::NACC, COL = (int)sizeof(typename Fx<4, 128>::ColT);
+  if (c->N <= kFxLarge && !c->fx_wide_units) {
+    const int rows = c->N <= kFxSmall ? 128 : 256;
+    if (!reserve_columns(c, column_bytes(c->N, rows, 64, NACC, COL)))
+      c->fx_wide_units = true;  // kept: the choice must not change inside a capture
+    else if (rows == 128)
+      return launch_sym<Fx<1, 64>, MODEL, false, MODE>(c, a);
+    else
+      return launch_sym<Fx<2, 64>, MODEL, false, MODE>(c, a);
+  }
   return launch_sym<Fx<4, 128>, MODEL, false, MODE>(c, a);
 }
 
@@ -490,12 +518,14 @@ int sym_pair_stage(md_ctx *c, int mode, double kick, double drift, double *fout)
 }
 
 // Reverse and tangent stages in the symmetric form: FP64 2D with the integer pair arithmetic,
-// while its six column partials fit.
-bool sym_reverse_applies(const md_ctx *c) {
-  if (!c->pt.symmetric || c->prec != MD_FP64 || c->pt.r_fp64 != 2) return false;
+// while its six column partials fit, also in the memory there is (one-sided stages need none).
+bool sym_reverse_applies(md_ctx *c) {
+  if (!c->pt.symmetric || c->prec != MD_FP64 || c->pt.r_fp64 != 2 || c->sym_reverse_off) return false;
   if (c->model != MD_GRAV2D || !fx_grav_applies(c->eps)) return false;
-  const int64_t TI = c->N <= kFxSmall ? 128 : 256, TJ = 64, m = TI / TJ, n_it = (c->N + TI - 1) / TI;
-  return (size_t)sym_rowstart(n_it, m * n_it, (int)m) * TJ * 6 * sizeof(double) <= kSymMaxColBytes;
+  const size_t need = column_bytes(c->N, c->N <= kFxSmall ? 128 : 256, 64, 6, sizeof(double));
+  if (need > kSymMaxColBytes) return false;
+  c->sym_reverse_off = !reserve_columns(c, need);
+  return !c->sym_reverse_off;
 }
 
 template <int MODE>
