@@ -426,6 +426,7 @@ constexpr long long kWildSum = 1ll << 54;  // the particles' own sums stay below
 __global__ void __launch_bounds__(NT, 1) hmf_run_mixed_kernel(HmfArgs a, HmfRun r) {
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
+  cluster.barrier_arrive();  // here: waited for before the first store into another CTA's shared memory
   constexpr int NW = NT / 32;
   __shared__ longlong2 part[2][kRunCtas * NW];
   __shared__ double2 wide, red[NW];
@@ -446,6 +447,7 @@ __global__ void __launch_bounds__(NT, 1) hmf_run_mixed_kernel(HmfArgs a, HmfRun 
     po = a.p[a.N - 1];
   }
   double sx = a.m_in[0], sy = a.m_in[1];
+  cluster.barrier_wait();  // every CTA of the cluster has started
   for (int64_t st = r.begin; st < r.end; st++) {
     const int ph = (int)(st % 3);
     a.kick = ph == 0 ? (st == 0 ? r.first : r.b0) : r.b1;
