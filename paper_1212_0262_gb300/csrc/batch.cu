@@ -366,10 +366,9 @@ __device__ __noinline__ void batch_sym_finish(const PartArgs &A, int64_t f) {
   const SysDesc &S = A.sys[sys_of_block(A, b)];
   const int64_t lb = b - S.bbeg, T = lb / (TI / FB);
   const int m = A.m;
-  const int64_t ubeg = S.ubeg + sym_rowstart(T, S.n_jt, m);  // first unit of the row
-  const int64_t cf = cta_of_unit(A.U, A.P, ubeg);
-  const int64_t cl = cta_of_unit(A.U, A.P, S.ubeg + sym_rowstart(T + 1, S.n_jt, m) - 1);
-  const int nchc = (int)((T + kChunkB) / kChunkB), nch = nchc + (int)((cl - cf + kChunkB) / kChunkB);
+  const RowChunks rc = row_chunks(A.U, A.P, S.ubeg, S.n_jt, m, T, T + 1, kChunkB);
+  const int64_t cf = rc.cf, cl = rc.cl;
+  const int nchc = rc.cols, nch = nchc + rc.segs;
   if (c >= nch) return;
   double *chunk = A.chunks + b * A.nc * kFinishThreadsB;
   const int lr = (int)((lb % (TI / FB)) * FB) + threadIdx.x / NACC, d = threadIdx.x % NACC;
@@ -394,7 +393,7 @@ __device__ __noinline__ void batch_sym_finish(const PartArgs &A, int64_t f) {
   } else {
     // virtual CTA c2 > cf begins inside the row: its first slot; cf may begin before it
     const int64_t lo = cf + (int64_t)(c - nchc) * kChunkB, hi = min(cl + 1, lo + kChunkB);
-    const bool cf_first = unit_begin(A.U, A.P, cf) >= ubeg;
+    const bool cf_first = unit_begin(A.U, A.P, cf) >= rc.ubeg;
     const double *src = A.slots + d * TI + lr;
 #pragma unroll 8
     for (int64_t c2 = lo; c2 < hi; c2++)
@@ -675,17 +674,17 @@ int launch_batch_sym(md_batch *b, double bc, double dc) {
   const size_t slot_r = (size_t)Pr * 2 * NAr * TIr, slot_g = (size_t)Pg * 2 * NAg * TIg;
   const size_t row_r = (size_t)b->rows_r * NAr * TIr, row_g = (size_t)b->rows_g * NAg * TIg;
   const size_t col_r = (size_t)b->Ur * PolR::TJ * NAr, col_g = (size_t)b->Ug * PolG::TJ * NAg;
-  // chunks per finish block: a system's row T has at most (n_jt - m T) P / U + 2 segments and
-  // T + 1 column rows; the bound is linear in T, the larger of its ends counts
+  // chunks per finish block: those of the tile with the most
   auto chunks_of = [&](int model, int64_t ti, int64_t tj, int64_t P, int64_t U) {
-    int64_t nc = 1;
+    int nc = 1;
+    int64_t ubeg = 0;
     for (int s = 0; s < b->nsys; s++) {
       if (b->model[s] != model) continue;
-      const int64_t m = ti / tj, n_it = (b->ctx[s]->N + ti - 1) / ti, n_jt = m * n_it;
-      for (const int64_t T : {(int64_t)0, n_it - 1})
-        nc = std::max<int64_t>(nc, (T + kChunkB) / kChunkB + ((n_jt - m * T) * P / U + 2 + kChunkB - 1) / kChunkB);
+      const int64_t m = ti / tj, n_it = (b->ctx[s]->N + ti - 1) / ti;
+      nc = std::max(nc, most_chunks(U, (int)P, ubeg, n_it, (int)m, true, kChunkB));
+      ubeg += sym_rowstart(n_it, m * n_it, (int)m);
     }
-    return (int)nc;
+    return nc;
   };
   const int nc_r = b->Ur > 0 ? chunks_of(MD_RING, TIr, PolR::TJ, Pr, b->Ur) : 1;
   const int nc_g = b->Ug > 0 ? chunks_of(MD_GRAV2D, TIg, PolG::TJ, Pg, b->Ug) : 1;

@@ -6,6 +6,7 @@
 #include <type_traits>
 
 #include "md_internal.cuh"
+#include "streamk.cuh"
 
 namespace {
 
@@ -182,10 +183,6 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(K) : "memory");
 }
 
-__host__ __device__ __forceinline__ int64_t unit_begin(int64_t U, int P, int64_t c) { return (U * c) / P; }
-// CTA whose range holds unit u: max c with U c / P <= u.
-__device__ __forceinline__ int64_t cta_of_unit(int64_t U, int P, int64_t u) { return ((u + 1) * P - 1) / U; }
-
 // Dynamic stream-K.  The U units are split into P static ranges ("virtual CTAs",
 // several per CTA), which the CTAs of the launch take in increasing order from
 // sched[0]: the CTAs that share an SM progress unevenly under its warp schedulers,
@@ -224,12 +221,6 @@ inline int64_t vcta_count(int64_t G, int64_t U, int k, int least = 16) {
   if (P < G) P = G;
   if (P > U) P = U;
   return P < 1 ? 1 : P;
-}
-
-// Triangular unit table of the Newton's-third-law form: row I (i-tile of m
-// j-tiles) holds the j-tiles J = m I .. n_jt - 1.
-__host__ __device__ __forceinline__ int64_t sym_rowstart(int64_t I, int64_t n_jt, int m) {
-  return I * n_jt - (int64_t)m * I * (I - 1) / 2;
 }
 
 // Policies with a Newton's-third-law diagonal tile (tile_diag: the above-diagonal

@@ -68,13 +68,6 @@ struct IsFx : std::false_type {};
 template <class P>
 struct IsFx<P, std::void_t<decltype(P::FX)>> : std::true_type {};
 
-// CTAs of the pair kernel that cover part of row T: [cf, cl].
-__device__ __forceinline__ void sym_row_ctas(const PairArgs &a, const SymArgs &s, int64_t T, int64_t &cf,
-                                             int64_t &cl) {
-  cf = cta_of_unit(a.U, a.P, sym_rowstart(T, a.n_jt, s.m));
-  cl = cta_of_unit(a.U, a.P, sym_rowstart(T + 1, a.n_jt, s.m) - 1);
-}
-
 // Shared-memory bytes of a unit's column sums.
 template <class Pol>
 constexpr int sym_col_bytes() {
@@ -232,9 +225,9 @@ __global__ void __launch_bounds__(kFinishBlock * Pol::NACC) sym_finish_kernel(Pa
   const int c = (int)(blockIdx.x % s.nc), sb = (int)(b % SB);
   const int m = s.m;
   const int64_t rows = T + (HasDiagSym<Pol>::value ? 1 : 0);  // column-partial rows I of tile T
-  int64_t cf, cl;
-  sym_row_ctas(a, s, T, cf, cl);
-  const int nchc = (int)((rows + s.ch - 1) / s.ch), nch = nchc + (int)((cl - cf + s.ch) / s.ch);
+  const RowChunks rc = row_chunks(a.U, a.P, 0, a.n_jt, m, T, rows, s.ch);
+  const int64_t cf = rc.cf, cl = rc.cl;
+  const int nchc = rc.cols, nch = nchc + rc.segs;
   if (c >= nch) return;
   double *chunk = s.chunks + b * s.nc * FT;
   const int lr = sb * kFinishBlock + threadIdx.x / NACC, d = threadIdx.x % NACC;
@@ -263,7 +256,7 @@ __global__ void __launch_bounds__(kFinishBlock * Pol::NACC) sym_finish_kernel(Pa
   } else {
     // virtual CTA c2 > cf begins inside row T: its first slot; cf may begin in an earlier row
     const int64_t lo = cf + (int64_t)(c - nchc) * s.ch, hi = min(cl + 1, lo + s.ch);
-    const bool cf_first = unit_begin(a.U, a.P, cf) >= sym_rowstart(T, a.n_jt, m);
+    const bool cf_first = unit_begin(a.U, a.P, cf) >= rc.ubeg;
     const double *src = a.slots + d * TI + lr;
 #pragma unroll 8
     for (int64_t c2 = lo; c2 < hi; c2++)
@@ -328,16 +321,11 @@ int launch_sym(md_ctx *c, PairArgs a) {
   a.P = (int)vcta_count(G, a.U, kv, IsFx<Pol>::value ? 1 : 16);
   int rc = ensure_pair_buffers(c, (int)TI, a.P, NACC);
   if (rc) return rc;
-  // Chunks: row T has n_jt - m T units in ranges of U / P, and T (+ 1) column-partial rows.
-  // The bound on their number is linear in T: the larger of its ends sizes the grid (spare
-  // CTAs leave at once).  Longer chunks where the column partials are many and narrow (Ring
-  // FP32: the chunk sums would cost an eighth of their traffic).
+  // Chunks: the tile with the most sizes the grid (spare CTAs of the others leave at once).
+  // Longer chunks where the column partials are many and narrow (Ring FP32: the chunk sums
+  // would cost an eighth of their traffic).
   s.ch = Pol::NACC == 1 && a.n_it >= 256 ? 64 : 16;
-  auto chunks = [&](int64_t T) {
-    const int64_t seg = (a.n_jt - (int64_t)s.m * T) * a.P / a.U + 2;
-    return (T + 1 + s.ch - 1) / s.ch + (seg + s.ch - 1) / s.ch;
-  };
-  s.nc = (int)std::max(chunks(0), chunks(a.n_it - 1));
+  s.nc = most_chunks(a.U, a.P, 0, a.n_it, s.m, HasDiagSym<Pol>::value, s.ch);
   const int64_t blocks = a.n_it * (TI / kFinishBlock);
   const size_t need_row = (size_t)a.n_it * NACC * TI * sizeof(double);
   const size_t need_col = (size_t)a.U * TJ * NACC * sizeof(typename Pol::ColT);
