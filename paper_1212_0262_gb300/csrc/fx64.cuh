@@ -4,8 +4,9 @@
 // multiply-adds and 128 integer adds (measured: mad.wide.u32 60, add 120, DFMA 1.9 per SM
 // and clock): an FP64 operation costs as much issue time as some 30 multiply-adds.  The
 // FP64 pair kernels therefore keep on the FP64 pipe only the coordinate differences (and
-// the FP64 sums of the 2D reverse stages) and do the rest on mantissas held as integers.  Every quantity keeps at least the 53 bits of a double
-// (errors below 2^-57 relative, noted at each function), and sums are exact.
+// those of w and the dot products of the 2D reverse stages) and do the rest on mantissas held as
+// integers.  A term has a relative error below 2^-54 (noted at each function) and is truncated
+// at the unit of its sum, which the policies choose (pairs_fx.cuh); the sums themselves are exact.
 //
 // The header has no GPU-only constructs but the reciprocal seed and the carry chain, so
 // that the CPU tests compile it and check it against extended precision.
@@ -230,6 +231,21 @@ FX_FN void add96(Acc96 &a, u32 w2, u32 w1, u32 w0) {
   a.w1 = (u32)t;
   a.w2 = a.w2 + w2 + (u32)(t >> 32);
 #endif
+}
+
+// A lane's column sum (|sum| < 2^85) as limbs of 27, 27 and 27 bits and a sign, each of which
+// adds over 32 lanes without overflow (the top one below 2^31: 0.77 2^85 is the largest sum of
+// the policies).  The low 5 bits are rounded to nearest: but for half a unit (ties go up) that
+// error has no sign, so it does not grow with the number of sums like a truncation's.
+FX_FN void column_limbs(Acc96 a, u32 &l0, u32 &l1, int &l2) {
+  add96(a, 0u, 0u, 16u);
+  l0 = a.w0 >> 5;
+  l1 = a.w1 & 0x07ffffffu;
+  l2 = (int)shf_r(a.w1, a.w2, 27);
+}
+// Sums of limbs as a double in units of 2^5
+FX_FN double limbs_total(u64 t0, u64 t1, int64_t t2) {
+  return ((double)t2 * 134217728.0 + (double)t1) * 134217728.0 + (double)t0;
 }
 
 // ---- sines and cosines (|x| <= 1) as fixed-point numbers ----
