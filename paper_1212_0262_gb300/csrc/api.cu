@@ -251,7 +251,7 @@ void md_free(md_ctx *c) {
   dev_free(c->sym_rowfull);
   dev_free(c->sym_colslot);
   dev_free(c->sym_chunks);
-  dev_free(c->fx_vmax);
+  dev_free(c->fx_vrange);
   destroy_step_graphs(c);
   dev_free(c->red);
   dev_free(c->gw);

@@ -233,6 +233,19 @@ FX_FN void add96(Acc96 &a, u32 w2, u32 w1, u32 w0) {
 #endif
 }
 
+// a + w + c, c = 0 or 1
+FX_FN void add96_carry(Acc96 &a, u32 w2, u32 w1, u32 w0, u32 c) {
+#ifdef __CUDA_ARCH__
+  u32 t;
+  asm("add.cc.u32 %3, %7, 0xffffffff;\n\taddc.cc.u32 %0, %0, %4;\n\taddc.cc.u32 %1, %1, %5;\n\taddc.u32 %2, %2, %6;"
+      : "+r"(a.w0), "+r"(a.w1), "+r"(a.w2), "=&r"(t)
+      : "r"(w0), "r"(w1), "r"(w2), "r"(c));
+#else
+  add96(a, 0u, 0u, c);
+  add96(a, w2, w1, w0);
+#endif
+}
+
 // A lane's column sum (|sum| < 2^85) as limbs of 27, 27 and 27 bits and a sign, each of which
 // adds over 32 lanes without overflow (the top one below 2^31: 0.77 2^85 is the largest sum of
 // the policies).  The low 5 bits are rounded to nearest: but for half a unit (ties go up) that
@@ -395,6 +408,20 @@ FX_FN void shift96_any(u32 &w2, u32 &w1, u32 &w0, int k) {
   w0 = shf_r(w0, w1, k);
   w1 = shf_r(w1, w2, k);
   w2 >>= k;
+}
+// The term (w2 w1 w0) >> k, k >= 1, with the sign mask sg, rounded to nearest: what to add,
+// and its carry (a negative number as ~w + 1, a term rounded up as w + 1: both of the carry).
+template <bool SMALL>  // k < 32
+FX_FN u32 signed_shift96(u32 &w2, u32 &w1, u32 &w0, int k, u32 sg) {
+  if (!SMALL) {
+    shift96_any(w2, w1, w0, k - 1);
+    k = 1;
+  }
+  const u32 c = ((w0 >> (k - 1)) ^ sg) & 1u;
+  w0 = shf_r(w0, w1, k) ^ sg;
+  w1 = shf_r(w1, w2, k) ^ sg;
+  w2 = (w2 >> k) ^ sg;
+  return c;
 }
 // 2^e as a double, -1022 <= e <= 1023
 FX_FN double pow2(int e) {

@@ -87,7 +87,7 @@ struct md_ctx {
   size_t sym_colslot_bytes = 0;
   double *sym_chunks = nullptr;   // and chunk sums of the column partials
   size_t sym_chunk_bytes = 0;
-  unsigned *fx_vmax = nullptr;    // integer reverse stages: the largest |v| of this stage and the next (ping-pong)
+  unsigned *fx_vrange = nullptr;  // integer reverse stages: the largest |v_k - v_0| of this stage and the next (ping-pong)
   int fx_vcur = 0;
   bool fx_wide_units = false;     // the small units' column partials did not fit in memory,
   bool sym_reverse_off = false;   // nor those of the symmetric reverse stages

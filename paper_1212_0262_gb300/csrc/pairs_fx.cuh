@@ -21,6 +21,8 @@
 namespace {
 
 constexpr int kFxFlush = 16;        // units between moves of the row sums into doubles
+// What stage() finds in a 16-byte chunk of a tile, and load() in a thread's rows (State::flags)
+constexpr int kFxWild = 1;    // out of the fixed-point range
 
 // Row sums of a thread in shared memory: [value][thread]
 template <int V>
@@ -42,10 +44,20 @@ __device__ __forceinline__ uint4 fx_warp_sum(const fx64::Acc96 &a) {
   r.w = 0u;
   return r;
 }
-// Sum of n limb triples `stride` apart, as a double in units of 2^(lsb + 5)
+// and exactly (|sum| < 2^85 per lane): the low 5 bits as a fourth limb.
+__device__ __forceinline__ uint4 fx_warp_sum_exact(const fx64::Acc96 &a) {
+  uint4 r;
+  r.x = __reduce_add_sync(0xffffffffu, a.w0 >> 5);
+  r.y = __reduce_add_sync(0xffffffffu, a.w1 & 0x07ffffffu);
+  r.z = (unsigned)__reduce_add_sync(0xffffffffu, (int)fx64::shf_r(a.w1, a.w2, 27));
+  r.w = __reduce_add_sync(0xffffffffu, a.w0 & 31u);
+  return r;
+}
+// Sum of n warps' limbs `stride` apart, as a double in units of 2^(lsb + 5)
 template <int n>
 __device__ __forceinline__ double fx_limb_total(const uint4 *s, int stride) {
   unsigned long long t0 = 0, t1 = 0;
+  unsigned t3 = 0;
   long long t2 = 0;
 #pragma unroll
   for (int w = 0; w < n; w++) {
@@ -53,8 +65,9 @@ __device__ __forceinline__ double fx_limb_total(const uint4 *s, int stride) {
     t0 += v.x;
     t1 += v.y;
     t2 += (int)v.z;
+    t3 += v.w;
   }
-  return fx64::limbs_total(t0, t1, t2);
+  return fx64::limbs_total(t0, t1, t2) + (double)t3 * 0.03125;
 }
 
 // Rows, flushes and columns shared by the policies: State has acc[R][NACC] and rows.
@@ -168,18 +181,18 @@ struct FxGrav {
     fx64::Acc96 acc[R][NACC];
     FxRowSums<R * NACC> rows;
     int units;     // since the last flush
-    bool wild;     // a row of this thread lies out of the fixed-point range
+    int flags;     // kFxWild, of the rows of this thread
   };
   // floor(log2(eps) / 2)
   __device__ static int half_exp(const PairArgs &a) { return ((int)(fx64::hi_word(a.epsd) >> 20) - 1023) >> 1; }
   __device__ static int lsb(const PairArgs &a) { return Tr::lsb(half_exp(a)); }
-  __device__ static bool out_of_range(double v, int half) {
+  __device__ static bool out_of_range(double v, int half, int range = Tr::RANGE) {
     const unsigned h = fx64::hi_word(v) & 0x7fffffffu;
-    return h >= ((unsigned)(1023 + Tr::RANGE + half) << 20) && h != (fx64::hi_word(1.0e150));  // padding: its terms vanish
+    return h >= ((unsigned)(1023 + range + half) << 20) && h != (fx64::hi_word(1.0e150));  // padding: its terms vanish
   }
   __device__ static void load(State &st, const void *mirror, int64_t i0, const PairArgs &a, double *rowsm) {
     const int half = half_exp(a);
-    st.wild = false;
+    st.flags = 0;
     fx_clear<State, R, NACC>(st, rowsm);
 #pragma unroll
     for (int r = 0; r < R; r++) {
@@ -187,7 +200,7 @@ struct FxGrav {
 #pragma unroll
       for (int d = 0; d < D; d++) {
         st.x[r][d] = fx_coord(m, d);
-        st.wild = st.wild || out_of_range(st.x[r][d], half);
+        if (out_of_range(st.x[r][d], half)) st.flags = kFxWild;
       }
     }
   }
@@ -197,10 +210,10 @@ struct FxGrav {
     for (int d = 0; d < NACC; d++) out[d] = st.rows.at(r * NACC + d);
   }
   // a 16-byte chunk of the tile: whether it is out of range (3D: (x, y) or (z, 0))
-  __device__ static bool stage(const unsigned char *tile, int ch, unsigned char *, const PairArgs &a) {
+  __device__ static int stage(const unsigned char *tile, int ch, unsigned char *, const PairArgs &a) {
     const double2 v = ((const double2 *)tile)[ch];
     const int half = half_exp(a);
-    return out_of_range(v.x, half) || out_of_range(v.y, half);
+    return out_of_range(v.x, half) || out_of_range(v.y, half) ? kFxWild : 0;
   }
   template <bool COL>
   __device__ static void unit(State &st, const unsigned char *smb, const unsigned char *, const PairArgs &a,
@@ -328,7 +341,7 @@ struct RingFx {
     fx64::Acc96 acc[R][NACC];
     FxRowSums<R * NACC> rows;
     int units;
-    bool wild;
+    int flags;
   };
   // |term| <= 0.77 / he <= 2^T for he = eps/2; T also makes the shift of the closest pairs,
   // whose power -3/2 is the largest, non-negative
@@ -340,12 +353,12 @@ struct RingFx {
   __device__ static int lsb(const PairArgs &a) { return top(a) - 83; }
   __device__ static bool out_of_range(double v) { return (fx64::hi_word(v) & 0x7fffffffu) > 0x3ff00000u; }
   __device__ static void load(State &st, const void *mirror, int64_t i0, const PairArgs &a, double *rowsm) {
-    st.wild = false;
+    st.flags = 0;
     fx_clear<State, R, NACC>(st, rowsm);
 #pragma unroll
     for (int r = 0; r < R; r++) {
       const double *m = (const double *)mirror + (i0 + row_of(r)) * 4;
-      st.wild = st.wild || out_of_range(m[0]) || out_of_range(m[1]) || out_of_range(m[2]) || out_of_range(m[3]);
+      if (out_of_range(m[0]) || out_of_range(m[1]) || out_of_range(m[2]) || out_of_range(m[3])) st.flags |= kFxWild;
       st.s[r] = fx64::limbs_of(m[0]);
       st.c[r] = fx64::limbs_of(m[1]);
       st.a[r] = fx64::limbs_of(m[2]);
@@ -355,11 +368,11 @@ struct RingFx {
   __device__ static void flush(State &st, const PairArgs &a) { fx_flush<State, R, NACC>(st, lsb(a)); }
   __device__ static void total(const State &st, int r, double *out) { out[0] = st.rows.at(r); }
   // half a record, (s, c) or (a, g): as (-s, c) or (-a, g) limbs
-  __device__ static bool stage(const unsigned char *tile, int ch, unsigned char *out, const PairArgs &) {
+  __device__ static int stage(const unsigned char *tile, int ch, unsigned char *out, const PairArgs &) {
     const double2 v = ((const double2 *)tile)[ch];
     const fx64::Limbs x = fx64::limbs_of(-v.x), y = fx64::limbs_of(v.y);
     ((int4 *)out)[ch] = make_int4(x.h, x.l, y.h, y.l);
-    return out_of_range(v.x) || out_of_range(v.y);
+    return out_of_range(v.x) || out_of_range(v.y) ? kFxWild : 0;
   }
   template <bool COL>
   __device__ static void unit(State &st, const unsigned char *, const unsigned char *staged, const PairArgs &a,
@@ -418,10 +431,23 @@ struct RingFx {
 // Newton's-third-law form: per pair
 //   f = d / s,  j = (w - 2 d (d.w) / s) / s,  e = d / s^2,
 // all antisymmetric.  d, w, d.w, and w - 2 d (d.w)/s are FP64 (9 operations; 22 per ordered
-// pair in GravF64Adj); the reciprocal, the products and the sums are integers.  The sums of j
-// have a unit that follows from the largest |v| (vmax, found before the stage).  Bound by the
-// FP64 pipe (78% at N = 16,384).  A reverse stage at N = 8,192: 2.9 ms one-sided in FP64, 0.69
-// here; a gradient of 4 steps there 41.4 -> 12.6 ms.
+// pair in GravF64Adj); the reciprocal, the products and the sums are integers.
+//
+// f falls as 1 / r, j as 1 / r^2, e as 1 / r^3, each against a unit that its largest term,
+// at r = sqrt(eps), sets: RANGE is where a term of e is still 2^52 units long (coordinates
+// below 2^9 sqrt(eps); farther apart e at 2^26, the forward range, would be 2^5 units).  The
+// unit of j also follows from the v: from W, the largest |v_k - v_0| (found before the stage).
+// Every particle has a partner whose w is at least W / 2, however the other w are spread, so
+// the sum of its |j| is at least 2^58 units within RANGE; terms of j are rounded to
+// nearest and column sums are exact, so that N small terms beside that one add no bias.  Error
+// against 64 bits of 1,024 particles in a disk of radius R, rms of |error| / sum of |terms|,
+// one-sided in FP64 and here: R = 1, eps = 1e-3 (2^5 sqrt(eps)) j 1.1e-16, 4.7e-17, e 1.5e-16,
+// 9.5e-17; eps = 4e-6 (2^9) j 2.1e-16, 9.3e-17, e 2.9e-16, 1.5e-16; eps = 1e-8 (FP64 units here)
+// j 2.2e-16, 1.4e-16, e 2.9e-16, 2.1e-16.
+//
+// Bound by the FP64 pipe (78% at N = 16,384).  A stage of N = 1,000, 8,192 and 16,385: one-sided in
+// FP64 165, 2290, 8070 us, here 61, 526, 2160; all units out of range, as in GravF64Adj but with
+// columns, 92, 1930, 7160.
 template <int R_, int TJ_>
 struct FxGrav2DAdj {
   using Fwd = FxGrav<2, R_, TJ_>;
@@ -440,24 +466,27 @@ struct FxGrav2DAdj {
     fx64::Acc96 acc[R][NACC];
     FxRowSums<R * NACC> rows;
     int units;
-    bool wild;
+    int flags;
   };
-  // exponent bound of |v|: |v_d| < 2^ev
-  __device__ static int vexp(const PairArgs &a) { return max((int)(*a.vmax >> 20) - 1022, -800); }
-  // |v| too large (or not finite) or, not all zero, too small for the exponents used here
+  static constexpr int RANGE = 9;
+  __device__ static bool out_of_range(double v, int half) { return Fwd::out_of_range(v, half, RANGE); }
+  // |w_d| <= 2 W < 2^vexp.  All v equal: any exponent will do (the w of padding, up to 2^299,
+  // divided by its s must vanish)
+  __device__ static int vexp(const PairArgs &a) { return *a.vrange == 0u ? 299 : (int)(*a.vrange >> 20) - 1021; }
+  // the v too large (or not finite) or, not all equal, too close for the exponents used here
   __device__ static bool v_wild(const PairArgs &a) {
-    const unsigned m = *a.vmax;
+    const unsigned m = *a.vrange;
     return m >= (1322u << 20) || (m != 0u && m < (223u << 20));
   }
-  // units of the sums of f, j, e: |f| <= 2^(-half - 1), |j| <= 2^(ev + 2 - 2 half),
+  // units of the sums of f, j, e: |f| <= 2^(-half - 1), |j| <= 2^(vexp + 1/2 - 2 half),
   // |e| <= 0.325 eps^(-3/2) <= 2^(-3 half - 1), each 2^83 units at most
   __device__ static int lsb_of(int kind, int half, int ev) {
-    return kind == 0 ? -82 - half : kind == 1 ? ev - 81 - 2 * half : -84 - 3 * half;
+    return kind == 0 ? -82 - half : kind == 1 ? ev - 82 - 2 * half : -84 - 3 * half;
   }
   __device__ static int lsb(const PairArgs &a, int d) { return lsb_of(d >> 1, Fwd::half_exp(a), vexp(a)); }
   __device__ static void load(State &st, const void *mirror, int64_t i0, const PairArgs &a, double *rowsm) {
     const int half = Fwd::half_exp(a);
-    st.wild = v_wild(a);
+    st.flags = v_wild(a) ? kFxWild : 0;
     fx_clear<State, R, NACC>(st, rowsm);
 #pragma unroll
     for (int r = 0; r < R; r++) {
@@ -466,7 +495,7 @@ struct FxGrav2DAdj {
       st.x[r][1] = m.y;
       st.v[r][0] = m.z;
       st.v[r][1] = m.w;
-      st.wild = st.wild || Fwd::out_of_range(m.x, half) || Fwd::out_of_range(m.y, half);
+      if (out_of_range(m.x, half) || out_of_range(m.y, half)) st.flags = kFxWild;
     }
   }
   __device__ static void flush(State &st, const PairArgs &a) {
@@ -484,10 +513,10 @@ struct FxGrav2DAdj {
     for (int d = 0; d < NACC; d++) out[d] = st.rows.at(r * NACC + d);
   }
   // half a record, (x, y) or (vx, vy)
-  __device__ static bool stage(const unsigned char *tile, int ch, unsigned char *, const PairArgs &a) {
+  __device__ static int stage(const unsigned char *tile, int ch, unsigned char *, const PairArgs &a) {
     const double2 m = ((const double2 *)tile)[ch];
     const int half = Fwd::half_exp(a);
-    return (ch & 1) == 0 && (Fwd::out_of_range(m.x, half) || Fwd::out_of_range(m.y, half));
+    return (ch & 1) == 0 && (out_of_range(m.x, half) || out_of_range(m.y, half)) ? kFxWild : 0;
   }
   template <bool COL>
   __device__ static void unit(State &st, const unsigned char *smb, const unsigned char *, const PairArgs &a,
@@ -496,7 +525,7 @@ struct FxGrav2DAdj {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, half = Fwd::half_exp(a);
     const fx64::Soft eps = fx64::soft_of(a.epsd);
     // shifts: f k = es - ex + kf, j k = es - ex(g) + kj, e k = 2 es - ex + ke
-    const int kf = 9 - half, kj = vexp(a) + 10 - 2 * half, ke = -1018 - 3 * half;
+    const int kf = 9 - half, kj = vexp(a) + 9 - 2 * half, ke = -1018 - 3 * half;
     uint4 *colsm = (uint4 *)colraw + w * TJ * NACC;
 #pragma unroll 1
     for (int j = 0; j < TJ; j++) {
@@ -539,7 +568,15 @@ struct FxGrav2DAdj {
 #pragma unroll
           for (int t = 0; t < 3; t++) {
             const int kk = k[2 * t + c];
-            unsigned sgn = t == 1 ? sg : sd;
+            if (t == 1) {
+              const unsigned cy = __builtin_expect(small, 1)
+                                      ? fx64::signed_shift96<true>(w2[t], w1[t], w0[t], kk, sg)
+                                      : fx64::signed_shift96<false>(w2[t], w1[t], w0[t], kk, sg);
+              fx64::add96_carry(st.acc[r][2 + c], w2[t], w1[t], w0[t], cy);
+              if (COL) fx64::add96_carry(col[2 + c], w2[t], w1[t], w0[t], cy);
+              continue;
+            }
+            unsigned sgn = sd;
             if (__builtin_expect(small, 1)) {
               w0[t] = fx64::shf_r(w0[t], w1[t], kk);
               w1[t] = fx64::shf_r(w1[t], w2[t], kk);
@@ -555,26 +592,27 @@ struct FxGrav2DAdj {
       if (COL) {
 #pragma unroll
         for (int c = 0; c < NACC; c++) {
-          const uint4 s = fx_warp_sum(col[c]);
+          const uint4 s = fx_warp_sum_exact(col[c]);
           if (lane == 0) colsm[NACC * j + c] = s;
         }
       }
     }
     if (++st.units == kFxFlush) flush(st, a);
   }
-  // the unit in FP64 (GravF64Adj's terms), columns reduced over the warp as doubles
+  // the unit in FP64 (GravF64Adj's terms); a column's six sums are reduced over the warp
+  // together, by a butterfly over 8 values
   template <bool COL>
   __device__ static void unit_wild(State &st, const unsigned char *smb, const PairArgs &a, unsigned char *colraw,
                                    int64_t, int64_t) {
     const double4_16a *sm = (const double4_16a *)smb;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     double *colsm = (double *)colraw + w * TJ * NACC;
+    flush(st, a);  // frees the integer sums' registers
+    double row[R][NACC] = {};
 #pragma unroll 1
     for (int j = 0; j < TJ; j++) {
       const double4_16a o = sm[j];
-      double col[NACC];
-#pragma unroll
-      for (int c = 0; c < NACC; c++) col[c] = 0.0;
+      double col[8] = {};
 #pragma unroll
       for (int r = 0; r < R; r++) {
         const double dx = st.x[r][0] - o.x, dy = st.x[r][1] - o.y, wx = st.v[r][0] - o.z, wy = st.v[r][1] - o.w;
@@ -583,33 +621,42 @@ struct FxGrav2DAdj {
         const double t[NACC] = {dx * inv, dy * inv, fma(m2u, dx, wx * inv), fma(m2u, dy, wy * inv), dx * inv2, dy * inv2};
 #pragma unroll
         for (int c = 0; c < NACC; c++) {
-          st.rows.at(r * NACC + c) += t[c];
-          col[c] += t[c];
+          row[r][c] += t[c];
+          if (COL) col[c] += t[c];
         }
       }
       if (COL) {
-#pragma unroll
-        for (int c = 0; c < NACC; c++) {
-          double s = col[c];
-#pragma unroll
-          for (int m = 16; m > 0; m >>= 1) s += __shfl_xor_sync(0xffffffffu, s, m);
-          if (lane == 0) colsm[NACC * j + c] = s;
-        }
+        double s = butterfly_sum<8, 16>(col, lane);  // value number: bits 4, 3, 2 of the lane
+        s += __shfl_xor_sync(0xffffffffu, s, 2);
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        const int c = lane >> 2;
+        if ((lane & 3) == 0 && c < NACC) colsm[NACC * j + c] = s;
       }
     }
+#pragma unroll
+    for (int r = 0; r < R; r++)
+#pragma unroll
+      for (int c = 0; c < NACC; c++) st.rows.at(r * NACC + c) += row[r][c];
   }
   __device__ static double column(const unsigned char *colraw, int idx, bool wild, const PairArgs &a) {
     return fx_column<TJ, NACC>(colraw, idx, wild, lsb(a, idx % NACC));
   }
 };
 
-// Largest |v_k| as the high word of a double into *cur (zero before); *next = 0 for the next
-// stage's.  A NaN has the largest high word.
-__global__ void fx_vmax_kernel(const double *__restrict__ v, int64_t n, unsigned *cur, unsigned *next) {
+// The largest |v_k - v_0| over both components as the high word of a double into *cur (zero
+// before; at least 1 unless all v are equal, ~0 for |v| from 2^299 on or not finite); *next = 0
+// for the next stage's.
+__global__ void fx_vrange_kernel(const double *__restrict__ v, int64_t N, unsigned *cur, unsigned *next) {
   unsigned m = 0u;
   const int64_t G = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += G)
-    m = max(m, fx64::hi_word(v[i]) & 0x7fffffffu);
+  const double v0[2] = {v[0], v[N]};
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += G)
+#pragma unroll
+    for (int c = 0; c < 2; c++) {
+      const double x = v[c * N + i], d = x - v0[c];
+      m = max(m, max(fx64::hi_word(d) & 0x7fffffffu, d != 0.0 ? 1u : 0u));
+      if ((fx64::hi_word(x) & 0x7fffffffu) >= (1322u << 20)) m = ~0u;
+    }
   m = __reduce_max_sync(0xffffffffu, m);
   if ((threadIdx.x & 31) == 0) atomicMax(cur, m);
   if (blockIdx.x == 0 && threadIdx.x == 0) *next = 0u;

@@ -164,7 +164,7 @@ struct PairArgs {
   double *lq, *lp;   // lambda_q, lambda_p (dim*N)
   double *epsacc;    // per-particle accumulated d O / d eps terms (N)
   double undo;       // kick coefficient (times dt) removed from p
-  const unsigned *vmax;  // integer reverse stages: the largest |v_k|'s high word
+  const unsigned *vrange;  // integer reverse stages: high word of the largest |v_k - v_0|
   // row shard (md_shard_*): the i-tiles cover global rows [row0, row0 + nrow) and the
   // state arrays q, p, fout hold those rows only (leading dimension nrow); the
   // mirror and N stay global

@@ -140,9 +140,9 @@ __global__ void __launch_bounds__(Pol::THREADS, Pol::MINB) sym_pairs_kernel(Pair
       }
       bool wild = false;  // FX: a coordinate of the unit lies out of the fixed-point range
       if constexpr (FX) {
-        wild = st.wild;
-        for (int ch = threadIdx.x; ch < CHUNKS; ch += THR) wild |= Pol::stage(sbuf[buf], ch, staged, a);
-        wild = __syncthreads_or(wild);
+        int flags = st.flags;
+        for (int ch = threadIdx.x; ch < CHUNKS; ch += THR) flags |= Pol::stage(sbuf[buf], ch, staged, a);
+        wild = __syncthreads_or(flags & kFxWild);
       } else {
         __syncthreads();
       }
@@ -360,17 +360,16 @@ int launch_sym(md_ctx *c, PairArgs a) {
   a.tickets = c->sk_tickets;
   a.sched = pair_sched(c);
   if constexpr (MODE == STAGE_ADJOINT || MODE == STAGE_TANGENT) {
-    // the largest |v| of the records (lambda_p, or dq), for the unit of the sums of j
-    if (!c->fx_vmax) {
-      c->fx_vmax = (unsigned *)dev_alloc(2 * sizeof(unsigned));
-      if (!c->fx_vmax) return set_err(c, MD_ENOMEM, "reverse stage scratch");
-      MD_CUDA(c, cudaMemsetAsync(c->fx_vmax, 0, 2 * sizeof(unsigned), c->stream));
+    // the spread of the v of the records (lambda_p, or dq), for the unit of the sums of j
+    if (!c->fx_vrange) {
+      c->fx_vrange = (unsigned *)dev_alloc(2 * sizeof(unsigned));
+      if (!c->fx_vrange) return set_err(c, MD_ENOMEM, "reverse stage scratch");
+      MD_CUDA(c, cudaMemsetAsync(c->fx_vrange, 0, 2 * sizeof(unsigned), c->stream));
     }
-    const int64_t n = (int64_t)c->dim * c->N;
-    const int64_t g = std::min<int64_t>((n + 255) / 256, c->nsm);
-    a.vmax = c->fx_vmax + c->fx_vcur;
-    fx_vmax_kernel<<<(int)g, 256, 0, c->stream>>>(MODE == STAGE_ADJOINT ? a.lp : a.lq, n, c->fx_vmax + c->fx_vcur,
-                                                 c->fx_vmax + (1 - c->fx_vcur));
+    const int64_t g = std::min<int64_t>((c->N + 255) / 256, c->nsm);
+    a.vrange = c->fx_vrange + c->fx_vcur;
+    fx_vrange_kernel<<<(int)g, 256, 0, c->stream>>>(MODE == STAGE_ADJOINT ? a.lp : a.lq, c->N, c->fx_vrange + c->fx_vcur,
+                                                   c->fx_vrange + (1 - c->fx_vcur));
     MD_LAUNCHED(c);
     c->fx_vcur = 1 - c->fx_vcur;
   }
