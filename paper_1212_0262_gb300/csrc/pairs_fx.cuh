@@ -23,6 +23,7 @@ namespace {
 constexpr int kFxFlush = 16;        // units between moves of the row sums into doubles
 // What stage() finds in a 16-byte chunk of a tile, and load() in a thread's rows (State::flags)
 constexpr int kFxWild = 1;    // out of the fixed-point range
+constexpr int kFxNarrow = 2;  // so small that the fixed-point form has fewer bits than a double
 
 // Row sums of a thread in shared memory: [value][thread]
 template <int V>
@@ -181,7 +182,7 @@ struct FxGrav {
     fx64::Acc96 acc[R][NACC];
     FxRowSums<R * NACC> rows;
     int units;     // since the last flush
-    int flags;     // kFxWild, of the rows of this thread
+    int flags;     // kFxWild, kFxNarrow: of the rows of this thread
   };
   // floor(log2(eps) / 2)
   __device__ static int half_exp(const PairArgs &a) { return ((int)(fx64::hi_word(a.epsd) >> 20) - 1023) >> 1; }
@@ -320,6 +321,11 @@ using FxGrav3D = FxGrav<3, R, TJ>;
 // turned into integers once per unit, by the thread that loaded them.  137 instructions per
 // pair; one force at N = 49,152: 36.3 ms with RingF64, 7.11 here (bound by the integer pipe,
 // 51%, and by dependent instructions at 4 warps per scheduler).
+// The sine of a difference has an error of some 2^-59 here, a product of two doubles' one of
+// 2^-53 of the larger sine: less where both angles lie within 2^-6 of 0 (or of pi).  One such
+// pair beside N others does not matter to a particle's sum, a system or cluster of such angles
+// does (extent 1e-6: forces to 1e-12): a unit with narrow rows and a quarter or more of its
+// columns narrow runs RingF64's tile.
 // eps of the fixed-point form: shifts of 0 .. 31 bits, sums below 2^95
 inline bool fx_ring_applies(double eps) { return eps >= 0x1p-17 && eps <= 4.0; }
 
@@ -335,6 +341,7 @@ struct RingFx {
   static constexpr int FMT = 0;
   static constexpr int COL_BYTES = (NT / 32) * TJ * NACC * (int)sizeof(uint4);
   static constexpr int STAGE_BYTES = TJ * JB;
+  static constexpr int NARROW = TJ / 4;  // narrow columns from which a unit with narrow rows runs in FP64
   __device__ static int row_of(int r) { return r * NT + (int)threadIdx.x; }
   struct State {
     fx64::Limbs s[R], c[R], a[R], g[R];
@@ -352,6 +359,10 @@ struct RingFx {
   }
   __device__ static int lsb(const PairArgs &a) { return top(a) - 83; }
   __device__ static bool out_of_range(double v) { return (fx64::hi_word(v) & 0x7fffffffu) > 0x3ff00000u; }
+  // |sin theta| below 2^-6 (a padding record's cosine is zero)
+  __device__ static bool narrow(double s, double c) {
+    return (fx64::hi_word(s) & 0x7fffffffu) < (1017u << 20) && c != 0.0;
+  }
   __device__ static void load(State &st, const void *mirror, int64_t i0, const PairArgs &a, double *rowsm) {
     st.flags = 0;
     fx_clear<State, R, NACC>(st, rowsm);
@@ -359,6 +370,7 @@ struct RingFx {
     for (int r = 0; r < R; r++) {
       const double *m = (const double *)mirror + (i0 + row_of(r)) * 4;
       if (out_of_range(m[0]) || out_of_range(m[1]) || out_of_range(m[2]) || out_of_range(m[3])) st.flags |= kFxWild;
+      if (narrow(m[0], m[1])) st.flags |= kFxNarrow;
       st.s[r] = fx64::limbs_of(m[0]);
       st.c[r] = fx64::limbs_of(m[1]);
       st.a[r] = fx64::limbs_of(m[2]);
@@ -372,7 +384,7 @@ struct RingFx {
     const double2 v = ((const double2 *)tile)[ch];
     const fx64::Limbs x = fx64::limbs_of(-v.x), y = fx64::limbs_of(v.y);
     ((int4 *)out)[ch] = make_int4(x.h, x.l, y.h, y.l);
-    return out_of_range(v.x) || out_of_range(v.y) ? kFxWild : 0;
+    return (out_of_range(v.x) || out_of_range(v.y) ? kFxWild : 0) | ((ch & 1) == 0 && narrow(v.x, v.y) ? kFxNarrow : 0);
   }
   template <bool COL>
   __device__ static void unit(State &st, const unsigned char *, const unsigned char *staged, const PairArgs &a,

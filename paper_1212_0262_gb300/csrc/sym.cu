@@ -67,6 +67,11 @@ template <class P, class = void>
 struct IsFx : std::false_type {};
 template <class P>
 struct IsFx<P, std::void_t<decltype(P::FX)>> : std::true_type {};
+// and with a rule on narrow records
+template <class P, class = void>
+struct HasNarrow : std::false_type {};
+template <class P>
+struct HasNarrow<P, std::void_t<decltype(P::NARROW)>> : std::true_type {};
 
 // Shared-memory bytes of a unit's column sums.
 template <class Pol>
@@ -140,9 +145,19 @@ __global__ void __launch_bounds__(Pol::THREADS, Pol::MINB) sym_pairs_kernel(Pair
       }
       bool wild = false;  // FX: a coordinate of the unit lies out of the fixed-point range
       if constexpr (FX) {
-        int flags = st.flags;
-        for (int ch = threadIdx.x; ch < CHUNKS; ch += THR) flags |= Pol::stage(sbuf[buf], ch, staged, a);
-        wild = __syncthreads_or(flags & kFxWild);
+        int flags = 0, narrow = 0;
+        for (int ch = threadIdx.x; ch < CHUNKS; ch += THR) {
+          const int f = Pol::stage(sbuf[buf], ch, staged, a);
+          flags |= f;
+          narrow += (f & kFxNarrow) != 0;
+        }
+        wild = __syncthreads_or((flags | st.flags) & kFxWild);
+        if constexpr (HasNarrow<Pol>::value) {
+          static_assert(CHUNKS <= 2 * THR, "at most two chunks per thread");
+          int n = __syncthreads_count(narrow > 0);
+          if (CHUNKS > THR) n += __syncthreads_count(narrow > 1);
+          if (n >= Pol::NARROW && __syncthreads_or(st.flags & kFxNarrow)) wild = true;
+        }
       } else {
         __syncthreads();
       }
