@@ -18,7 +18,7 @@
 // triangular (system, i-tile, j-tile) units of its systems stream-K style and
 // writing row and column partials (diagonal units too: their above-diagonal
 // blocks are evaluated once, with column sums), then one finish launch with a CTA
-// per (system, block of 256 outputs, chunk of 128 row segments or column-partial rows)
+// per (system, block of 256 particles, chunk of 128 row segments or column-partial rows)
 // that sums them in a fixed order and runs the epilogue.  (The one-sided form shares one launch
 // between the parts, split by md_batch_set_tuning's `split`.)
 #include <algorithm>
@@ -45,6 +45,16 @@ struct SysDesc {
   double epsd, dt;
 };
 
+// What a finish CTA does (symmetric form): chunk c of the nch of block `block` (of its part) in tile
+// `tile` of system `sys`, whose row's segments are those of the ranges cf .. cl.
+struct __align__(16) FinTask {
+  int sys, tile, sub;      // sub: the block's place in its tile
+  int block;
+  int c, nchc, nch;        // nchc chunks of column-partial rows, then the segments'
+  int cf, cl, cf_first;    // cf_first: range cf begins inside the row
+  int pad[2];
+};
+
 struct PartArgs {
   const SysDesc *sys;
   int nsys;
@@ -58,11 +68,11 @@ struct PartArgs {
   int waves;         // virtual CTAs per physical CTA: P = waves x grid
   unsigned *next;    // next virtual CTA to take (the finish kernel sets it back to 0)
   int m;             // TI / TJ of the part
-  int64_t nblk;      // finish blocks of the part
-  int nc;            // chunks per finish block, at most
+  const FinTask *fin;  // finish CTAs of the part
+  int nfin;
   double *rowfull;   // [rows][NACC][TI]
   float *colslot;    // [U][TJ][NACC]
-  double *chunks;    // [nblk][nc][kFinishThreadsB]
+  double *chunks;    // [nfin][kFinishThreadsB][NACC]
 };
 
 // index of the system whose unit range holds u (binary search on ubeg)
@@ -232,18 +242,19 @@ __global__ void __launch_bounds__(NT) batch_kernel(PartArgs ring, PartArgs grav)
 
 // ------------------------------------------------- Newton's-third-law form --
 
-// Finish phase as in sym.cu, in blocks of 256 outputs (256 Ring or 128 2D particles) and
-// chunks of kChunkB column-partial rows or row segments (ranges that cover part of the row).
-// A tile per CTA took 145 us of a stage of 4 systems (pair phase 557 us); a stage of 4, 8, 24
-// systems 770, 974, 2855 us, now 573, 896, 2825 (chunks of 32 rows: 582, 910, 2870: more CTAs
-// with nothing to sum).
+// Finish phase as in sym.cu, in blocks of 256 particles, one per thread, and chunks of kChunkB
+// column-partial rows or row segments (ranges that cover part of the row).  The CTAs' tasks are
+// listed on the host: no searches or divisions in the kernel, and no CTA with nothing to sum.
+// In ensembles of many systems nearly every row is one range's, so up to kDirectB segments are
+// read by the CTA that finishes the block instead of having a CTA and a ticket of their own.
+// Microseconds of a stage of 4, 8, 24, 64, 256 systems: with a tile per CTA 636, 1107, 2818,
+// 8490, 29180; blocks of 256 outputs with the largest system's chunks everywhere, each CTA
+// searching for its block, 524, 1049, 2811, 8580, 29720; here 525, 1028, 2761, 8420, 29090 (the
+// launch's arguments by reference to a function that was not inlined cost 64 KB of local
+// stores per CTA in both).
 constexpr int kFinishThreadsB = 256;
 constexpr int kChunkB = 128;
-
-template <class Pol>
-constexpr int finish_block() {
-  return kFinishThreadsB / Pol::NACC;
-}
+constexpr int kDirectB = 4;
 
 // (system, local row) of part-local unit u in the triangular layout
 __device__ __forceinline__ void sym_locate(const PartArgs &A, int64_t u, int &s, int64_t &it, int64_t &jt) {
@@ -343,84 +354,87 @@ __device__ __forceinline__ void batch_sym_pairs(const PartArgs &A, int64_t cta, 
   }
 }
 
-// index of the system whose finish blocks hold block b (binary search on bbeg)
-__device__ __forceinline__ int sys_of_block(const PartArgs &A, int64_t b) {
-  int lo = 0, hi = A.nsys - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (A.sys[mid].bbeg <= b) lo = mid;
-    else hi = mid - 1;
-  }
-  return lo;
-}
-
-// Finish phase of one part, CTA f: chunk c of block b (of tile T of a system).
+// Finish phase of one part, CTA f: a particle per thread.
 template <class Pol, int MODEL, int MODE>
-__device__ __noinline__ void batch_sym_finish(const PartArgs &A, int64_t f) {
-  constexpr int NACC = Pol::NACC, TJ = Pol::TJ, FB = finish_block<Pol>();
+__device__ __forceinline__ void batch_sym_finish(const PartArgs &A, int f) {
+  constexpr int NACC = Pol::NACC, TJ = Pol::TJ;
   constexpr int64_t TI = (int64_t)NT * Pol::R;
-  static_assert(TI % FB == 0, "whole blocks per tile");
+  static_assert(TI % kFinishThreadsB == 0, "whole blocks per tile");
   __shared__ bool s_last;
-  const int64_t b = f / A.nc;
-  const int c = (int)(f % A.nc);
-  const SysDesc &S = A.sys[sys_of_block(A, b)];
-  const int64_t lb = b - S.bbeg, T = lb / (TI / FB);
-  const int m = A.m;
-  const RowChunks rc = row_chunks(A.U, A.P, S.ubeg, S.n_jt, m, T, T + 1, kChunkB);
-  const int64_t cf = rc.cf, cl = rc.cl;
-  const int nchc = rc.cols, nch = nchc + rc.segs;
-  if (c >= nch) return;
-  double *chunk = A.chunks + b * A.nc * kFinishThreadsB;
-  const int lr = (int)((lb % (TI / FB)) * FB) + threadIdx.x / NACC, d = threadIdx.x % NACC;
-  double v = 0.0;
+  const FinTask t = A.fin[f];
+  const SysDesc &S = A.sys[t.sys];
+  const int64_t T = t.tile;
+  const int c = t.c, nchc = t.nchc, nch = t.nch, cf = t.cf, cl = t.cl, m = A.m;
+  const int lr = t.sub * kFinishThreadsB + threadIdx.x;
+  // component e of the particle's row from range c2.  c2 > cf begins inside the row: its first
+  // slot; cf may begin before it
+  auto segment = [&](int c2, int e) {
+    return __ldcg(cf == cl ? A.rowfull + ((S.rbeg + T) * NACC + e) * TI + lr
+                           : A.slots + (((int64_t)c2 * 2 + (c2 > cf || t.cf_first ? 0 : 1)) * NACC + e) * TI + lr);
+  };
+  double v[NACC] = {};
   if (c < nchc) {  // column partials of the rows I_lo .. (the diagonal units' included)
     const int64_t I_lo = (int64_t)c * kChunkB, I_hi = min(T + 1, I_lo + kChunkB);
-    const int jsub = lr / TJ, rest = (lr % TJ) * NACC + d;
-    CompSum cs{0.f, 0.f};
+    const int jsub = lr / TJ, rest = (lr % TJ) * NACC;
+    CompSum cs[NACC] = {};
     // unit (I2, T m + jsub) advances by n_jt - m (I2 + 1) from I2 to I2 + 1
     int64_t off = (S.ubeg + sym_rowstart(I_lo, S.n_jt, m) + (T * m + jsub - (int64_t)m * I_lo)) * (TJ * NACC) + rest;
     int64_t step = (S.n_jt - (int64_t)m * (I_lo + 1)) * (TJ * NACC);
     const int64_t dstep = (int64_t)m * (TJ * NACC);
 #pragma unroll 8
     for (int64_t I2 = I_lo; I2 < I_hi; I2++) {
-      csum_add(cs, __ldcg(A.colslot + off));
+      if constexpr (NACC == 2) {
+        const float2 x = __ldcg((const float2 *)(A.colslot + off));
+        csum_add(cs[0], x.x);
+        csum_add(cs[1], x.y);
+      } else {
+        csum_add(cs[0], __ldcg(A.colslot + off));
+      }
       off += step;
       step -= dstep;
     }
-    v = -csum_total(cs);
-  } else if (cf == cl) {
-    v = __ldcg(A.rowfull + ((S.rbeg + T) * NACC + d) * TI + lr);
-  } else {
-    // virtual CTA c2 > cf begins inside the row: its first slot; cf may begin before it
-    const int64_t lo = cf + (int64_t)(c - nchc) * kChunkB, hi = min(cl + 1, lo + kChunkB);
-    const bool cf_first = unit_begin(A.U, A.P, cf) >= rc.ubeg;
-    const double *src = A.slots + d * TI + lr;
-#pragma unroll 8
-    for (int64_t c2 = lo; c2 < hi; c2++)
-      v += __ldcg(src + (c2 * 2 + (c2 > cf || cf_first ? 0 : 1)) * (NACC * TI));
-  }
-  chunk[c * kFinishThreadsB + threadIdx.x] = v;
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(&A.tickets[b], 1u) + 1u == (unsigned)nch;
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  const int64_t i = lb * FB + threadIdx.x;
-  if (threadIdx.x < FB && i < S.N) {
-    double tot[NACC];
 #pragma unroll
-    for (int e = 0; e < NACC; e++) tot[e] = 0.0;
-    const double *mine = chunk + threadIdx.x * NACC;
+    for (int e = 0; e < NACC; e++) v[e] = -csum_total(cs[e]);
+  } else {
+    const int lo = cf + (c - nchc) * kChunkB, hi = min(cl + 1, lo + kChunkB);
+#pragma unroll 8
+    for (int c2 = lo; c2 < hi; c2++)
+#pragma unroll
+      for (int e = 0; e < NACC; e++) v[e] += segment(c2, e);
+  }
+  double *chunk = A.chunks + ((int64_t)(f - c) * kFinishThreadsB + threadIdx.x) * NACC;
+  constexpr int CHUNK = kFinishThreadsB * NACC;
+  if (nch > 1) {
+#pragma unroll
+    for (int e = 0; e < NACC; e++) chunk[c * CHUNK + e] = v[e];
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(&A.tickets[t.block], 1u) + 1u == (unsigned)nch;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    if (threadIdx.x == 0) A.tickets[t.block] = 0u;
+  }
+  const int64_t i = T * TI + lr;
+  if (i >= S.N) return;
+  double tot[NACC] = {};
+  if (nch == nchc)
+#pragma unroll 4
+    for (int c2 = cf; c2 <= cl; c2++)
+#pragma unroll
+      for (int e = 0; e < NACC; e++) tot[e] += segment(c2, e);
+  if (nch == 1) {
+#pragma unroll
+    for (int e = 0; e < NACC; e++) tot[e] += v[e];
+  } else {
 #pragma unroll 2
     for (int k = 0; k < nch; k++) {  // segments, then columns
-      const int at = (k < nch - nchc ? nchc + k : k - (nch - nchc)) * kFinishThreadsB;
+      const int at = (k < nch - nchc ? nchc + k : k - (nch - nchc)) * CHUNK;
 #pragma unroll
-      for (int e = 0; e < NACC; e++) tot[e] += __ldcg(mine + at + e);
+      for (int e = 0; e < NACC; e++) tot[e] += __ldcg(chunk + at + e);
     }
-    finish<Pol, MODEL, true, MODE>(view(A, S), i, tot);
   }
-  if (threadIdx.x == 0) A.tickets[b] = 0u;
+  finish<Pol, MODEL, true, MODE>(view(A, S), i, tot);
 }
 
 template <class Pol>
@@ -453,11 +467,10 @@ __global__ void __launch_bounds__(NT, Pol::MINB) batch_sym_pairs_kernel(PartArgs
 template <class PolR, class PolG, int MODE>
 __global__ void __launch_bounds__(kFinishThreadsB) batch_sym_finish_kernel(PartArgs ring, PartArgs grav) {
   if (blockIdx.x == 0 && threadIdx.x == 0) *ring.next = *grav.next = 0u;  // the pair kernels have ended
-  const int64_t nr = ring.nblk * ring.nc;
-  if ((int64_t)blockIdx.x < nr)
+  if ((int)blockIdx.x < ring.nfin)
     batch_sym_finish<PolR, MD_RING, MODE>(ring, blockIdx.x);
   else
-    batch_sym_finish<PolG, MD_GRAV2D, MODE>(grav, (int64_t)blockIdx.x - nr);
+    batch_sym_finish<PolG, MD_GRAV2D, MODE>(grav, (int)blockIdx.x - ring.nfin);
 }
 
 struct Config {
@@ -492,6 +505,12 @@ struct md_batch {
   int64_t Ur = 0, Ug = 0, rows_r = 0, rows_g = 0, blk_r = 0, blk_g = 0;
   int64_t rec_bytes_r = 0, rec_bytes_g = 0;  // forward-record bytes of each part's systems
   int nr = 0;
+  std::vector<SysDesc> hs;  // the descriptors in d_sys
+  // symmetric form: finish CTAs (Ring, then 2D), for these numbers of ranges
+  FinTask *fin = nullptr;
+  size_t fin_bytes = 0;
+  int64_t fin_P[2] = {-1, -1};
+  int nfin_r = 0, nfin_g = 0;
   int mirror_sym = -1;  // form the mirrors were written for (Ring records differ)
   double *rowfull = nullptr;  // Newton's-third-law form: row partials, column partials, chunk sums
   size_t rowfull_bytes = 0;
@@ -543,7 +562,7 @@ int build_layout(md_batch *b, const int64_t TI[2], const int64_t TJ[2], const in
     for (int s = 0; s < b->nsys; s++) {
       if (b->model[s] != want) continue;
       md_ctx *c = b->ctx[s];
-      SysDesc d;
+      SysDesc d{};
       d.q = c->q;
       d.p = c->p;
       d.f = c->f;
@@ -562,7 +581,7 @@ int build_layout(md_batch *b, const int64_t TI[2], const int64_t TJ[2], const in
       d.bbeg = blk;
       U += sym ? sym_rowstart(d.n_it, d.n_jt, (int)m) : d.n_it * d.n_jt;
       rows += d.n_it;
-      blk += sym ? d.n_it * (ti * nacc[pass] / kFinishThreadsB) : d.n_it;
+      blk += sym ? d.n_it * (ti / kFinishThreadsB) : d.n_it;
       // forward records: Ring tensor-core fragments (symmetric form) or interleaved FP32
       (pass == 0 ? b->rec_bytes_r : b->rec_bytes_g) += c->N * (pass == 0 ? (sym ? 64 : 16) : 8);
       hs.push_back(d);
@@ -578,8 +597,10 @@ int build_layout(md_batch *b, const int64_t TI[2], const int64_t TJ[2], const in
 int ensure_layout(md_batch *b, const int64_t TI[2], const int64_t TJ[2], const int nacc[2], bool sym) {
   const int64_t key[7] = {TI[0], TJ[0], TI[1], TJ[1], sym ? 1 : 0, nacc[0], nacc[1]};
   if (std::equal(key, key + 7, b->layout_key)) return MD_OK;
-  std::vector<SysDesc> hs;
+  std::vector<SysDesc> &hs = b->hs;
   build_layout(b, TI, TJ, nacc, sym, hs);
+  b->fin_P[0] = b->fin_P[1] = -1;
+  std::fill(b->layout_key, b->layout_key + 7, -1);  // until the descriptors are uploaded
   if (hs.size() > b->d_sys_count) {
     dev_free(b->d_sys);
     b->d_sys = (SysDesc *)dev_alloc(hs.size() * sizeof(SysDesc));
@@ -599,6 +620,37 @@ int grow(md_batch *b, T *&ptr, size_t &have, size_t need, const char *what) {
   ptr = (T *)dev_alloc(need);
   have = ptr ? need : 0;
   return ptr ? MD_OK : berr(b, MD_ENOMEM, "%s", what);
+}
+
+// Finish CTAs for Pr and Pg ranges of the two parts (symmetric form; not inside a capture, like
+// ensure_layout).  TI, m: rows and j-tiles of the parts' tiles.
+int ensure_finish(md_batch *b, int64_t Pr, int64_t Pg, const int64_t TI[2], const int m[2]) {
+  if (b->fin_P[0] == Pr && b->fin_P[1] == Pg) return MD_OK;
+  b->fin_P[0] = b->fin_P[1] = -1;
+  std::vector<FinTask> tasks;
+  for (int s = 0; s < (int)b->hs.size(); s++) {
+    const SysDesc &d = b->hs[s];
+    const int part = s < b->nr ? 0 : 1, per_tile = (int)(TI[part] / kFinishThreadsB);
+    const int64_t U = part == 0 ? b->Ur : b->Ug, P = part == 0 ? Pr : Pg;
+    if (s == b->nr) b->nfin_r = (int)tasks.size();
+    for (int T = 0; T < (int)d.n_it; T++) {
+      const RowChunks rc = row_chunks(U, (int)P, d.ubeg, d.n_jt, m[part], T, T + 1, kChunkB, kDirectB);
+      const int first = unit_begin(U, (int)P, rc.cf) >= rc.ubeg ? 1 : 0;
+      for (int sub = 0; sub < per_tile; sub++)
+        for (int c = 0; c < rc.cols + rc.segs; c++)
+          tasks.push_back(FinTask{part == 0 ? s : s - b->nr, T, sub, (int)d.bbeg + T * per_tile + sub, c, rc.cols,
+                                  rc.cols + rc.segs, (int)rc.cf, (int)rc.cl, first, {0, 0}});
+    }
+  }
+  if (b->nr == (int)b->hs.size()) b->nfin_r = (int)tasks.size();
+  b->nfin_g = (int)tasks.size() - b->nfin_r;
+  B_CUDA(b, cudaStreamSynchronize(b->stream));  // no launch may still read the old tasks
+  int rc = grow(b, b->fin, b->fin_bytes, tasks.size() * sizeof(FinTask), "batch finish tasks");
+  if (rc) return rc;
+  B_CUDA(b, cudaMemcpy(b->fin, tasks.data(), tasks.size() * sizeof(FinTask), cudaMemcpyHostToDevice));
+  b->fin_P[0] = Pr;
+  b->fin_P[1] = Pg;
+  return MD_OK;
 }
 
 int ensure_tickets(md_batch *b) {
@@ -674,21 +726,9 @@ int launch_batch_sym(md_batch *b, double bc, double dc) {
   const size_t slot_r = (size_t)Pr * 2 * NAr * TIr, slot_g = (size_t)Pg * 2 * NAg * TIg;
   const size_t row_r = (size_t)b->rows_r * NAr * TIr, row_g = (size_t)b->rows_g * NAg * TIg;
   const size_t col_r = (size_t)b->Ur * PolR::TJ * NAr, col_g = (size_t)b->Ug * PolG::TJ * NAg;
-  // chunks per finish block: those of the tile with the most
-  auto chunks_of = [&](int model, int64_t ti, int64_t tj, int64_t P, int64_t U) {
-    int nc = 1;
-    int64_t ubeg = 0;
-    for (int s = 0; s < b->nsys; s++) {
-      if (b->model[s] != model) continue;
-      const int64_t m = ti / tj, n_it = (b->ctx[s]->N + ti - 1) / ti;
-      nc = std::max(nc, most_chunks(U, (int)P, ubeg, n_it, (int)m, true, kChunkB));
-      ubeg += sym_rowstart(n_it, m * n_it, (int)m);
-    }
-    return nc;
-  };
-  const int nc_r = b->Ur > 0 ? chunks_of(MD_RING, TIr, PolR::TJ, Pr, b->Ur) : 1;
-  const int nc_g = b->Ug > 0 ? chunks_of(MD_GRAV2D, TIg, PolG::TJ, Pg, b->Ug) : 1;
-  const size_t ch_r = (size_t)b->blk_r * nc_r * kFinishThreadsB, ch_g = (size_t)b->blk_g * nc_g * kFinishThreadsB;
+  const int m[2] = {(int)(TIr / PolR::TJ), (int)(TIg / PolG::TJ)};
+  if ((rc = ensure_finish(b, Pr, Pg, TI, m))) return rc;
+  const size_t ch_r = (size_t)b->nfin_r * kFinishThreadsB * NAr, ch_g = (size_t)b->nfin_g * kFinishThreadsB * NAg;
   if ((rc = grow(b, b->slots, b->slots_bytes, (slot_r + slot_g) * sizeof(double), "batch slots")) ||
       (rc = grow(b, b->rowfull, b->rowfull_bytes, (row_r + row_g) * sizeof(double), "batch row partials")) ||
       (rc = grow(b, b->colslot, b->colslot_bytes, (col_r + col_g) * sizeof(float), "batch column partials")) ||
@@ -702,9 +742,9 @@ int launch_batch_sym(md_batch *b, double bc, double dc) {
   ar.P = (int)Pr;
   ar.waves = Wr;
   ar.next = b->tickets + b->blk_r + b->blk_g;
-  ar.m = (int)(TIr / PolR::TJ);
-  ar.nblk = b->blk_r;
-  ar.nc = nc_r;
+  ar.m = m[0];
+  ar.fin = b->fin;
+  ar.nfin = b->nfin_r;
   ar.slots = b->slots;
   ar.rowfull = b->rowfull;
   ar.colslot = b->colslot;
@@ -716,9 +756,9 @@ int launch_batch_sym(md_batch *b, double bc, double dc) {
   ag.P = (int)Pg;
   ag.waves = Wg;
   ag.next = ar.next + 1;
-  ag.m = (int)(TIg / PolG::TJ);
-  ag.nblk = b->blk_g;
-  ag.nc = nc_g;
+  ag.m = m[1];
+  ag.fin = b->fin + b->nfin_r;
+  ag.nfin = b->nfin_g;
   ag.slots = b->slots + slot_r;
   ag.rowfull = b->rowfull + row_r;
   ag.colslot = b->colslot + col_r;
@@ -735,7 +775,7 @@ int launch_batch_sym(md_batch *b, double bc, double dc) {
     kern_g<<<(int)Gg, NT, 0, b->stream>>>(ag);
     b->launches++;
   }
-  batch_sym_finish_kernel<PolR, PolG, MODE><<<(unsigned)(b->blk_r * nc_r + b->blk_g * nc_g), kFinishThreadsB, 0, b->stream>>>(ar, ag);
+  batch_sym_finish_kernel<PolR, PolG, MODE><<<(unsigned)(b->nfin_r + b->nfin_g), kFinishThreadsB, 0, b->stream>>>(ar, ag);
   b->launches++;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return berr(b, MD_ECUDA, "batch launch: %s", cudaGetErrorString(e));
@@ -896,6 +936,7 @@ void md_batch_free(md_batch *b) {
   dev_free(b->d_sys);
   dev_free(b->slots);
   dev_free(b->tickets);
+  dev_free(b->fin);
   dev_free(b->rowfull);
   dev_free(b->colslot);
   dev_free(b->chunks);

@@ -21,27 +21,29 @@ SK_FN int64_t sym_rowstart(int64_t I, int64_t n_jt, int m) { return I * n_jt - (
 
 // What the finish phase adds up for tile T of a system whose first unit is ubeg: `rows` rows of
 // column partials and the row's segments, those of the ranges cf .. cl, each in chunks of at
-// most ch.
+// most ch.  Up to `direct` segments need no chunk: the CTA that finishes the tile reads them.
 struct RowChunks {
   int64_t ubeg, cf, cl;  // the row's first unit, and the ranges that hold units of it
   int cols, segs;        // chunks of column-partial rows and of segments
 };
-SK_FN RowChunks row_chunks(int64_t U, int P, int64_t ubeg, int64_t n_jt, int m, int64_t T, int64_t rows, int ch) {
+SK_FN RowChunks row_chunks(int64_t U, int P, int64_t ubeg, int64_t n_jt, int m, int64_t T, int64_t rows, int ch,
+                           int direct) {
   RowChunks r;
   r.ubeg = ubeg + sym_rowstart(T, n_jt, m);
   r.cf = cta_of_unit(U, P, r.ubeg);
   r.cl = cta_of_unit(U, P, ubeg + sym_rowstart(T + 1, n_jt, m) - 1);
   r.cols = (int)((rows + ch - 1) / ch);
-  r.segs = (int)((r.cl - r.cf + ch) / ch);
+  r.segs = r.cl - r.cf < direct ? 0 : (int)((r.cl - r.cf + ch) / ch);
   return r;
 }
 
 // The largest number of chunks over a system's tiles, which sizes the finish grid.  A sum of two
 // rounded-up quotients, one rising and one falling with T: its maximum can be anywhere.
-static inline int most_chunks(int64_t U, int P, int64_t ubeg, int64_t n_it, int m, bool diag, int ch) {
+static inline int most_chunks(int64_t U, int P, int64_t ubeg, int64_t n_it, int m, bool diag, int ch,
+                              int direct) {
   int most = 1;
   for (int64_t T = 0; T < n_it; T++) {
-    const RowChunks r = row_chunks(U, P, ubeg, m * n_it, m, T, T + (diag ? 1 : 0), ch);
+    const RowChunks r = row_chunks(U, P, ubeg, m * n_it, m, T, T + (diag ? 1 : 0), ch, direct);
     most = r.cols + r.segs > most ? r.cols + r.segs : most;
   }
   return most;

@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(kFinishBlock * Pol::NACC) sym_finish_kernel(Pa
   const int c = (int)(blockIdx.x % s.nc), sb = (int)(b % SB);
   const int m = s.m;
   const int64_t rows = T + (HasDiagSym<Pol>::value ? 1 : 0);  // column-partial rows I of tile T
-  const RowChunks rc = row_chunks(a.U, a.P, 0, a.n_jt, m, T, rows, s.ch);
+  const RowChunks rc = row_chunks(a.U, a.P, 0, a.n_jt, m, T, rows, s.ch, 0);
   const int64_t cf = rc.cf, cl = rc.cl;
   const int nchc = rc.cols, nch = nchc + rc.segs;
   if (c >= nch) return;
@@ -340,7 +340,7 @@ int launch_sym(md_ctx *c, PairArgs a) {
   // Longer chunks where the column partials are many and narrow (Ring FP32: the chunk sums
   // would cost an eighth of their traffic).
   s.ch = Pol::NACC == 1 && a.n_it >= 256 ? 64 : 16;
-  s.nc = most_chunks(a.U, a.P, 0, a.n_it, s.m, HasDiagSym<Pol>::value, s.ch);
+  s.nc = most_chunks(a.U, a.P, 0, a.n_it, s.m, HasDiagSym<Pol>::value, s.ch, 0);
   const int64_t blocks = a.n_it * (TI / kFinishBlock);
   const size_t need_row = (size_t)a.n_it * NACC * TI * sizeof(double);
   const size_t need_col = (size_t)a.U * TJ * NACC * sizeof(typename Pol::ColT);

@@ -14,10 +14,10 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
 SRC = r"""
 #include "streamk.cuh"
 extern "C" {
-int most(int64_t U, int P, int64_t ubeg, int64_t n_it, int m, int diag, int ch) { return most_chunks(U, P, ubeg, n_it, m, diag, ch); }
+int most(int64_t U, int P, int64_t ubeg, int64_t n_it, int m, int diag, int ch, int direct) { return most_chunks(U, P, ubeg, n_it, m, diag, ch, direct); }
 int64_t units(int64_t n_it, int m) { return sym_rowstart(n_it, m * n_it, m); }
-void row(int64_t U, int P, int64_t ubeg, int64_t n_it, int m, int64_t T, int64_t rows, int ch, int64_t *o) {
-  const RowChunks r = row_chunks(U, P, ubeg, m * n_it, m, T, rows, ch);
+void row(int64_t U, int P, int64_t ubeg, int64_t n_it, int m, int64_t T, int64_t rows, int ch, int direct, int64_t *o) {
+  const RowChunks r = row_chunks(U, P, ubeg, m * n_it, m, T, rows, ch, direct);
   o[0] = r.cf; o[1] = r.cl; o[2] = r.cols; o[3] = r.segs; o[4] = r.ubeg; o[5] = unit_begin(U, P, r.cf); o[6] = unit_begin(U, P, r.cl + 1);
 }
 }
@@ -34,25 +34,26 @@ def lib(tmp_path_factory):
     subprocess.run([cxx, "-O1", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, "-o", str(d / "t.so"), str(d / "t.cpp")], check=True)
     so = ctypes.CDLL(str(d / "t.so"))
     i64, i32 = ctypes.c_int64, ctypes.c_int
-    so.most.argtypes = [i64, i32, i64, i64, i32, i32, i32]
+    so.most.argtypes = [i64, i32, i64, i64, i32, i32, i32, i32]
     so.units.argtypes, so.units.restype = [i64, i32], i64
-    so.row.argtypes = [i64, i32, i64, i64, i32, i64, i64, i32, ctypes.c_void_p]
+    so.row.argtypes = [i64, i32, i64, i64, i32, i64, i64, i32, i32, ctypes.c_void_p]
     return so
 
 
-def _check(lib, U, P, ubeg, n_it, m, diag, ch):
-    nc, at = lib.most(U, P, ubeg, n_it, m, diag, ch), []
+def _check(lib, U, P, ubeg, n_it, m, diag, ch, direct=0):
+    nc, at = lib.most(U, P, ubeg, n_it, m, diag, ch, direct), []
     o = (ctypes.c_int64 * 7)()
     first = ubeg
     for T in range(n_it):
         rows = T + diag
-        lib.row(U, P, ubeg, n_it, m, T, rows, ch, o)
+        lib.row(U, P, ubeg, n_it, m, T, rows, ch, direct, o)
         cf, cl, cols, segs, u0, lo, hi = o
         assert u0 == first and lo <= first  # the row's units are those of the ranges cf .. cl
         first += m * (n_it - T)
-        assert hi >= first and (cols - 1) * ch < rows <= cols * ch and (segs - 1) * ch < cl - cf + 1 <= segs * ch
+        assert hi >= first and (cols - 1) * ch < rows <= cols * ch
+        assert segs == 0 if cl - cf < direct else (segs - 1) * ch < cl - cf + 1 <= segs * ch
         at.append(cols + segs)
-    assert max(at) == nc
+    assert max(1, *at) == nc
     return at
 
 
@@ -76,5 +77,5 @@ def test_systems_of_an_ensemble(lib):
     for P in (608, 1216, 3648, U):
         ubeg = 0
         for n in tiles:
-            _check(lib, U, P, ubeg, n, 1, 1, 128)
+            _check(lib, U, P, ubeg, n, 1, 1, 128, 4)
             ubeg += lib.units(n, 1)
