@@ -100,16 +100,26 @@ __device__ __forceinline__ int4 angle_fx(double th, const scfx::Entry *tab, long
   return make_int4(c.h, c.l, s.h, s.l);
 }
 
-// The FP64 stages' magnetization: as limbs (My, -Mx) for the integer force
+// The FP64 stages' magnetization: (My, -Mx) 2^e as limbs for the integer force, the larger of
+// them in [1/2, 1), so that a force has the bits of a double relative to |M|, however small.
 struct HmfM {
   fx64::Limbs my, nmx;
+  int e;
   bool fx;  // finite and of ordinary size
 };
+// high word of the larger of |Mx|, |My|: from 2^-600 to 1.5 the integer form takes them
+__device__ __forceinline__ unsigned hmf_top(double mx, double my) {
+  return max(fx64::hi_word(mx) & 0x7fffffffu, fx64::hi_word(my) & 0x7fffffffu);
+}
+constexpr unsigned kTopMin = (1023u - 600u) << 20, kTopMax = 0x3ff80000u;
 __device__ __forceinline__ HmfM hmf_m_of(double mx, double my) {
   HmfM m;
-  m.fx = fabs(mx) < 1.5 && fabs(my) < 1.5;
-  m.my = fx64::limbs_of(m.fx ? my : 0.0);
-  m.nmx = fx64::limbs_of(m.fx ? -mx : 0.0);
+  const unsigned top = hmf_top(mx, my);
+  m.fx = top >= kTopMin && top < kTopMax;
+  m.e = 1022 - (int)(top >> 20);
+  const double scale = __hiloint2double(m.fx ? (1023 + 62 + m.e) << 20 : 0, 0);  // 2^(62 + e)
+  m.my = scfx::split(__double2ll_rn(my * scale));
+  m.nmx = scfx::split(__double2ll_rn(-mx * scale));
   return m;
 }
 
@@ -167,7 +177,7 @@ __device__ __forceinline__ void hmf_particle_fp64(double &th, double &pp, int4 &
                                                   double mx, double my, long long &aci, long long &asi, int64_t i,
                                                   const scfx::Entry *tab) {
   const fx64::Limbs c{cs.x, cs.y}, s{cs.z, cs.w};
-  double f = scfx::to_double60(fx64::dot2(c, s, m.my, m.nmx));  // cos My - sin Mx
+  double f = scfx::to_double60(fx64::dot2(c, s, m.my, m.nmx), m.e);  // cos My - sin Mx
   if (!m.fx) f = hmf_force_fp64((double)scfx::join(c.h, c.l) * 0x1p-62, (double)scfx::join(s.h, s.l) * 0x1p-62, mx, my, a.invN);
   if (cs.x == kNoAngle) f = __longlong_as_double(0x7ff8000000000000LL);
   if (a.invN == 1.0) f = 0.0;  // a lone particle's self-term
