@@ -64,7 +64,8 @@ __device__ __forceinline__ void load_sincos_tab(double2 *sm) {
 // operations (12 with the sine and cosine of sincos_fp64.cuh and an FP64 force, which bound
 // the stage).  Per stage at N = 5e7: 1149 -> 582 us, 3.2 GB at 81% of the copy rate; the
 // integer pipe is half busy, the next pair's loads run ahead of the arithmetic (604 us without).
-// A non-finite angle is marked by kNoAngle: its force is NaN, and so are the sums.
+// A non-finite angle is marked by kNoAngle: its force is NaN, and so are the sums.  Cold systems
+// hold doubles instead (hmf_sweep64).
 __device__ scfx::Entry g_sincos_fx[kTabN];
 constexpr int kNoAngle = (int)0x80000000;
 
@@ -81,7 +82,14 @@ __device__ __forceinline__ void load_sincos_fx(scfx::Entry *sm) {
   __syncthreads();
 }
 
-// (cos, sin) of th as stored (cos.h, cos.l, sin.h, sin.l), and their sums in units of 2^-54.
+// (cos, sin) as stored: (cos.h, cos.l, sin.h, sin.l)
+__device__ __forceinline__ int4 angle_fx_of(double s, double c) {
+  if (!(fabs(s) <= 1.0)) return make_int4(kNoAngle, 0, 0, 0);
+  const fx64::Limbs lc = fx64::limbs_of(c), ls = fx64::limbs_of(s);
+  return make_int4(lc.h, lc.l, ls.h, ls.l);
+}
+
+// (cos, sin) of th as stored, and their sums in units of 2^-54.
 __device__ __forceinline__ int4 angle_fx(double th, const scfx::Entry *tab, long long &aci, long long &asi) {
   fx64::i64 s62, c62;
   if (!scfx::sincos_fx(th, tab, s62, c62)) {
@@ -134,6 +142,7 @@ struct HmfArgs {
   unsigned *ticket;
   double *fout;  // STAGE_FORCE_ONLY output
   int4 *cs;      // FP64 path: (cos, sin) of the current angles, rewritten by drifts
+  unsigned *fmt; // FP64 path: whether cs holds doubles (hmf_sweep64)
   int rev;       // sweep the particles from the top end down
   int nsum;      // row shard: m_in holds nsum (sum cos, sum sin) pairs, one per rank
 };
@@ -192,8 +201,9 @@ __device__ __forceinline__ void hmf_particle_fp64(double &th, double &pp, int4 &
   }
 }
 
-// Grid finish: write this CTA's partial; the last CTA sums all partials in order.
-__device__ __forceinline__ void grid_finish(double sc, double ss, double *partials, double *m_out,
+// Grid finish: write this CTA's partial; the last CTA sums all partials in order
+// (true in that one).
+__device__ __forceinline__ bool grid_finish(double sc, double ss, double *partials, double *m_out,
                                             unsigned *ticket) {
   __shared__ double2 red[NT / 32];
   __shared__ bool last;
@@ -206,7 +216,7 @@ __device__ __forceinline__ void grid_finish(double sc, double ss, double *partia
     last = (t == gridDim.x - 1);
   }
   __syncthreads();
-  if (!last) return;
+  if (!last) return false;
   __threadfence();
   double c0 = 0.0, c1 = 0.0;
   for (int j = threadIdx.x; j < (int)gridDim.x; j += NT) {
@@ -220,6 +230,100 @@ __device__ __forceinline__ void grid_finish(double sc, double ss, double *partia
     m_out[1] = t.y;
     *ticket = 0u;
   }
+  return true;
+}
+
+// Cold systems, whose angles all lie near 0, pi / 2, pi or 3 pi / 2 (|Mx| or |My| above 1 - 2^-11:
+// within some 2^-5): the forces are differences of sines (cosines) and a magnetization component
+// that are small themselves, where doubles have more bits than fixed-point numbers.  Their
+// stages are all FP64: (cos, sin) kept as doubles (*HmfArgs::fmt = 1), the table-driven sines and
+// cosines of sincos_fp64.cuh, FP64 sums; 12 FP64 operations per particle-stage, 8.0 us at
+// N = 10,007, 1.31 ms at N = 5e7.  A stage whose predecessor's M was cold reads doubles, one whose own M is cold
+// writes them.
+__device__ __forceinline__ bool hmf_cold(double mx, double my) {
+  const unsigned top = hmf_top(mx, my);
+  return top > 0x3feffc00u && top < kTopMax;
+}
+template <int MODE, bool CG>
+__device__ __noinline__ double2 hmf_sweep64(double *q, double *p, int4 *cs, double *fout, int64_t N, double invN,
+                                            double kick, double drift, double mx, double my, const double2 *tab,
+                                            int in64, int out64) {
+  auto load = [](const auto *ptr) {
+    if constexpr (CG) return __ldcg(ptr);
+    else return *ptr;
+  };
+  double2 sum = make_double2(0.0, 0.0);
+  auto particle = [&](double &th, double &pp, int4 &w, int64_t i) {
+    double c, s;
+    if (in64) {
+      c = __hiloint2double(w.y, w.x);
+      s = __hiloint2double(w.w, w.z);
+    } else {
+      c = (double)scfx::join(w.x, w.y) * 0x1p-62;
+      s = (double)scfx::join(w.z, w.w) * 0x1p-62;
+    }
+    const double f = hmf_force_fp64(c, s, mx, my, invN);
+    if (MODE == STAGE_FORCE_ONLY) {
+      fout[i] = f;
+      return;
+    }
+    pp = fma(kick, f, pp);
+    if (MODE == STAGE_KICK_DRIFT) {
+      th = fma(drift, pp, th);
+      sincos_tab(th, tab, &s, &c);
+      sum.x += c;
+      sum.y += s;
+      w = out64 ? make_int4(__double2loint(c), __double2hiint(c), __double2loint(s), __double2hiint(s)) : angle_fx_of(s, c);
+    }
+  };
+  constexpr int UN = CG ? 1 : UNROLL;  // the cluster kernel has no registers for two pairs
+  const int64_t G = (int64_t)gridDim.x * NT, npairs = N >> 1;
+  const int64_t t0 = (int64_t)blockIdx.x * NT + threadIdx.x;
+  for (int64_t k = t0; k < npairs; k += UN * G) {
+    double2 qv[UN], pv[UN];
+    int4 w[UN][2];
+#pragma unroll
+    for (int u = 0; u < UN; u++)
+      if (k + u * G < npairs) {
+        const int64_t ix = k + u * G;
+        qv[u] = load((const double2 *)q + ix);
+        pv[u] = load((const double2 *)p + ix);
+        w[u][0] = load(cs + 2 * ix);
+        w[u][1] = load(cs + 2 * ix + 1);
+      }
+#pragma unroll
+    for (int u = 0; u < UN; u++)
+      if (k + u * G < npairs) {
+        const int64_t ix = k + u * G;
+        particle(qv[u].x, pv[u].x, w[u][0], 2 * ix);
+        particle(qv[u].y, pv[u].y, w[u][1], 2 * ix + 1);
+        if (MODE != STAGE_FORCE_ONLY) ((double2 *)p)[ix] = pv[u];
+        if (MODE == STAGE_KICK_DRIFT) {
+          ((double2 *)q)[ix] = qv[u];
+          cs[2 * ix] = w[u][0];
+          cs[2 * ix + 1] = w[u][1];
+        }
+      }
+  }
+  if ((N & 1) && t0 == 0) {
+    double th = load(q + N - 1), pp = load(p + N - 1);
+    int4 w = load(cs + N - 1);
+    particle(th, pp, w, N - 1);
+    if (MODE != STAGE_FORCE_ONLY) p[N - 1] = pp;
+    if (MODE == STAGE_KICK_DRIFT) {
+      q[N - 1] = th;
+      cs[N - 1] = w;
+    }
+  }
+  return sum;
+}
+template <int MODE, bool CG>
+__device__ __forceinline__ void hmf_sweep64(const HmfArgs &a, double mx, double my, const void *tab, bool in64, bool out64,
+                                            double &acd, double &asd) {
+  const double2 sum = hmf_sweep64<MODE, CG>(a.q, a.p, a.cs, a.fout, a.N, a.invN, a.kick, a.drift, mx, my,
+                                            (const double2 *)tab, in64, out64);
+  acd = sum.x;
+  asd = sum.y;
 }
 
 // One sweep over the particles: the stage's work of this thread, its sums of the new angles'
@@ -345,10 +449,20 @@ __global__ void __launch_bounds__(NT, MODE != STAGE_KICK_DRIFT ? 1 : MIXED ? 4 :
       sy += a.m_in[2 * r + 1];
     }
   const double mx = sx * a.invN, my = sy * a.invN;
-  extern __shared__ __align__(16) unsigned char tabraw[];  // FP64 kick-drift stages: the sine/cosine table (kTabBytes)
+  extern __shared__ __align__(16) unsigned char tabraw[];  // FP64 kick-drift stages: a sine/cosine table (kTabBytes)
   scfx::Entry *tab = (scfx::Entry *)tabraw;
-  if constexpr (!MIXED && MODE == STAGE_KICK_DRIFT) load_sincos_fx(tab);
   double acd = 0.0, asd = 0.0;
+  if constexpr (!MIXED) {
+    const bool in64 = *a.fmt != 0u, out64 = MODE == STAGE_KICK_DRIFT && hmf_cold(mx, my);
+    if (in64 || out64) {
+      if (MODE == STAGE_KICK_DRIFT) load_sincos_tab((double2 *)tabraw);
+      hmf_sweep64<MODE, false>(a, mx, my, tabraw, in64, out64, acd, asd);
+      // the last CTA to finish: every other has read *a.fmt
+      if (MODE == STAGE_KICK_DRIFT && grid_finish(acd, asd, a.partials, a.m_out, a.ticket) && threadIdx.x == 0) *a.fmt = out64;
+      return;
+    }
+    if (MODE == STAGE_KICK_DRIFT) load_sincos_fx(tab);
+  }
   hmf_sweep<MIXED, MODE, false>(a, mx, my, tab, acd, asd);
   if (MODE == STAGE_KICK_DRIFT) grid_finish(acd, asd, a.partials, a.m_out, a.ticket);
 }
@@ -383,7 +497,8 @@ __global__ void __launch_bounds__(NT, 3) hmf_run_fp64_kernel(HmfArgs a, HmfRun r
   scfx::Entry *tab = (scfx::Entry *)tabraw;
   __shared__ double2 part[2], msum;
   __shared__ double2 red[NT / 32];
-  load_sincos_fx(tab);
+  int table = -1;  // the one in shared memory: of hmf_sweep (0) or hmf_sweep64 (1)
+  bool in64 = *a.fmt != 0u;
   const int rev0 = a.rev;
   double2 s = make_double2(a.m_in[0], a.m_in[1]);
   for (int64_t st = r.begin; st < r.end; st++) {
@@ -392,7 +507,17 @@ __global__ void __launch_bounds__(NT, 3) hmf_run_fp64_kernel(HmfArgs a, HmfRun r
     a.drift = ph == 1 ? r.d1 : r.d0;
     a.rev = r.rev(st, rev0);
     double acd = 0.0, asd = 0.0;
-    hmf_sweep<false, STAGE_KICK_DRIFT, true>(a, s.x * a.invN, s.y * a.invN, tab, acd, asd);
+    const double mx = s.x * a.invN, my = s.y * a.invN;
+    const bool out64 = hmf_cold(mx, my);
+    const int want = in64 || out64;
+    if (table != want) {  // every thread is past its last look-up: it has been at the cluster barrier since
+      if (want) load_sincos_tab((double2 *)tabraw);
+      else load_sincos_fx(tab);
+      table = want;
+    }
+    if (want) hmf_sweep64<STAGE_KICK_DRIFT, true>(a, mx, my, tabraw, in64, out64, acd, asd);
+    else hmf_sweep<false, STAGE_KICK_DRIFT, true>(a, mx, my, tab, acd, asd);
+    in64 = out64;
     const double2 b = block_sum2<NT>(acd, asd, red);
     if (threadIdx.x == 0) part[st & 1] = b;
     cluster.sync();  // the partial sums and the state of every CTA are visible
@@ -412,6 +537,7 @@ __global__ void __launch_bounds__(NT, 3) hmf_run_fp64_kernel(HmfArgs a, HmfRun r
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     a.m_out[0] = s.x;
     a.m_out[1] = s.y;
+    *a.fmt = in64;
   }
   cluster.sync();  // no CTA leaves while another reads its partial sums
 }
@@ -555,6 +681,29 @@ __global__ void __launch_bounds__(NT) hmf_prime_fp64_kernel(const double *__rest
   grid_finish(acd, asd, partials, m_out, ticket);
 }
 
+// After it: a cold system's (cos, sin) once more as doubles, and their FP64 sums (others leave at
+// once; the whole grid decides alike, as the last CTA alone writes m_out and fmt).
+__global__ void __launch_bounds__(NT) hmf_prime_cold_kernel(const double *__restrict__ q, int64_t N, double *partials,
+                                                            double *m_out, unsigned *ticket, int4 *__restrict__ cs,
+                                                            unsigned *fmt) {
+  const double inv = 1.0 / (double)N;
+  const bool cold = hmf_cold(m_out[0] * inv, m_out[1] * inv);
+  if (!cold) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *fmt = 0u;
+    return;
+  }
+  double acd = 0.0, asd = 0.0;
+  const int64_t G = (int64_t)gridDim.x * NT;
+  for (int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x; i < N; i += G) {
+    double s, c;
+    sincos(q[i], &s, &c);
+    acd += c;
+    asd += s;
+    cs[i] = make_int4(__double2loint(c), __double2hiint(c), __double2loint(s), __double2hiint(s));
+  }
+  if (grid_finish(acd, asd, partials, m_out, ticket) && threadIdx.x == 0) *fmt = 1u;
+}
+
 // (sum cos, sum sin) of the given angles.  MIXED: FP32 sine/cosine after FP64
 // range reduction, FP32 per-thread sums; otherwise FP64 throughout.
 // FP64: use_tab selects the table-driven sine and cosine of the FP64 stages (the table
@@ -612,6 +761,9 @@ int grid_for(md_ctx *c, const void *kern, int64_t work_items, int cap = 0, size_
   return (int)g;
 }
 
+// The word that says how hmf_cs holds (cos, sin).
+unsigned *hmf_fmt(md_ctx *c) { return (unsigned *)(c->hmf_m + 4); }
+
 template <bool MIXED, int MODE>
 int launch_stage(md_ctx *c, double kick, double drift, double *fout) {
   HmfArgs a;
@@ -627,6 +779,7 @@ int launch_stage(md_ctx *c, double kick, double drift, double *fout) {
   a.ticket = c->hmf_ticket;
   a.fout = fout;
   a.cs = (int4 *)c->hmf_cs;
+  a.fmt = hmf_fmt(c);
   // Consecutive stages sweep the state in opposite directions, so a stage starts on
   // the lines the previous one wrote last, which are still in L2 (dirty lines that
   // are overwritten before eviction are never written back either).
@@ -734,6 +887,9 @@ int hmf_prime(md_ctx *c) {
     hmf_prime_fp64_kernel<<<g, NT, kTabBytes, c->stream>>>(c->q, c->N, c->hmf_partials, out, c->hmf_ticket,
                                                            (int4 *)c->hmf_cs);
     MD_LAUNCHED(c);
+    hmf_prime_cold_kernel<<<g, NT, 0, c->stream>>>(c->q, c->N, c->hmf_partials, out, c->hmf_ticket, (int4 *)c->hmf_cs,
+                                                   hmf_fmt(c));
+    MD_LAUNCHED(c);
   }
   c->hmf_m_valid = true;
   c->hmf_m_prec = c->prec;
@@ -772,6 +928,9 @@ int hmf_shard_prime(md_ctx *c) {
     int g = grid_for(c, (const void *)hmf_prime_fp64_kernel, c->N, 0, kTabBytes);
     hmf_prime_fp64_kernel<<<g, NT, kTabBytes, c->stream>>>(c->q, c->N, c->hmf_partials, out, c->hmf_ticket,
                                                            (int4 *)c->hmf_cs);
+    MD_LAUNCHED(c);
+    hmf_prime_cold_kernel<<<g, NT, 0, c->stream>>>(c->q, c->N, c->hmf_partials, out, c->hmf_ticket, (int4 *)c->hmf_cs,
+                                                   hmf_fmt(c));
   }
   MD_LAUNCHED(c);
   c->hmf_m_valid = false;  // md_step's own sums are not kept on a shard
@@ -796,6 +955,7 @@ int launch_shard_stage(md_ctx *c, double kick, double drift, double *fout) {
   a.ticket = c->hmf_ticket;
   a.fout = fout;
   a.cs = (int4 *)c->hmf_cs;
+  a.fmt = hmf_fmt(c);
   a.rev = c->hmf_rev;
   c->hmf_rev ^= 1;
   auto kern = hmf_stage_kernel<MIXED, MODE, true>;
@@ -857,6 +1017,7 @@ int hmf_run(md_ctx *c, int64_t nsteps, int64_t block_steps, const double *k4, do
   a.N = c->N;
   a.invN = 1.0 / (double)c->N;
   a.cs = (int4 *)c->hmf_cs;
+  a.fmt = hmf_fmt(c);
   a.m_in = c->hmf_m + 2 * c->hmf_cur;
   a.rev = c->hmf_rev;
   // launched stages alternate the direction, replayed blocks keep the one they were captured with

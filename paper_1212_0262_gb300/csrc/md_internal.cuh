@@ -60,13 +60,13 @@ struct md_ctx {
 
   // HMF: per-CTA partial sums, magnetization double buffer, finish ticket
   double *hmf_partials = nullptr;  // 2 * hmf_grid_max
-  double *hmf_m = nullptr;         // [2][2]: (sum cos, sum sin) of the current / next angles
+  double *hmf_m = nullptr;         // [2][2]: (sum cos, sum sin) of the current / next angles; [4]: format of hmf_cs; [8..]: scalars
   unsigned *hmf_ticket = nullptr;
   int hmf_grid_max = 0;
   int hmf_cur = 0;
   int hmf_rev = 0;                    // sweep direction of the next stage (alternates)
   bool hmf_m_valid = false;           // FP64: the (cos, sin) buffer is valid with the sums
-  double *hmf_cs = nullptr;           // FP64 path: (cos, sin) of the current angles, N int4 (fixed point)
+  double *hmf_cs = nullptr;           // FP64 path: (cos, sin) of the current angles, N int4 (fixed point) or double2
   size_t hmf_cs_bytes = 0;
   int hmf_m_prec = -1;
 

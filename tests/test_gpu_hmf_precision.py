@@ -31,3 +31,46 @@ def test_forces_keep_their_bits_with_a_small_magnetization(size, kick):
     size = float(np.hypot(*m.astype(float)))
     assert size > 0
     assert float(np.abs(A @ m - f).max()) <= 5 * 2.0**-53 * size
+
+
+@pytest.mark.parametrize("steps", [0, 1, 9])
+@pytest.mark.parametrize("extent", [1e-12, 1e-6, 1e-3, 0.02])
+@pytest.mark.parametrize("N", [2, 3, 1000, 50_000])
+def test_forces_of_cold_systems(N, extent, steps):
+    """All angles near 0, where doubles have more bits than fixed-point numbers: forces at the
+    given state and after steps (in one launch for the smaller N) against long double, within 76
+    roundings (12 of a term, 64 of the sums) of |cos t_i| mean|sin| + |sin t_i| mean|cos|.  The
+    stages' table-driven sine rounds its term r^3 / 6 to FP32, |r| the smaller of the angle and half
+    a table step: 2^-23 of it for the particle's sine and for the mean's."""
+    g = np.random.default_rng(N)
+    with System(0, N, 0.0, 0.1, 1, precision="fp64") as s:
+        s.set_state(extent * (2 * g.random(N) - 1), np.zeros(N))
+        s.step(steps)
+        q = s.get_state()[0]
+        f = s.force()
+    t = q.astype(np.longdouble)
+    sn, cs = np.sin(t), np.cos(t)
+    want = cs * sn.mean() - sn * cs.mean()
+    scale = (np.abs(cs) * np.abs(sn).mean() + np.abs(sn) * np.abs(cs).mean()).astype(np.float64)
+    r = min(float(np.abs(t).max()), np.pi / 4096)
+    assert np.all(np.abs((f - want).astype(np.float64)) <= 76 * 2.0**-53 * scale + (steps > 0) * 2 * 2.0**-23 * r**3 / 6)
+
+
+def test_a_system_that_becomes_cold_and_warm_again():
+    """Angles that their momenta draw together and apart again: the stages change between the two
+    forms, launched and in one launch alike (the same bits), and the forces stay within 1e-13 of
+    long double."""
+    N = 3000
+    q = 0.5 * (2 * np.random.default_rng(1).random(N) - 1)
+    for n in range(0, 10, 3):
+        out = []
+        for graphs in (1, 0):
+            with System(0, N, 0.0, 1.0, 1, precision="fp64") as s:
+                s.set_tuning("step_graphs", graphs)
+                s.set_state(q, -0.25 * q)
+                s.step(n)
+                out.append((s.get_state()[0], s.force()))
+        assert all(np.array_equal(a, b) for a, b in zip(*out))
+        t = out[0][0].astype(np.longdouble)
+        sn, cs = np.sin(t), np.cos(t)
+        assert np.all(np.abs(out[0][1] - (cs * sn.mean() - sn * cs.mean())) <= 1e-13)
