@@ -403,6 +403,7 @@ StepGraphKey step_key_of(const md_ctx *c, double h) {
   key.pt = c->pt;
   key.ht = c->ht;
   key.mirror_fmt = c->mirror_fmt;
+  key.wide_units = c->fx_wide_units;
   const void *b[14] = {c->q,           c->p,          c->mirror[0],    c->mirror[1], c->sk_slots,
                        c->sk_tickets,  c->sym_rowfull, c->sym_colslot, c->sym_chunks, c->hmf_partials,
                        c->hmf_m,       c->hmf_ticket, c->f,            c->hmf_cs};

@@ -42,6 +42,7 @@ struct StepGraphKey {
   PairTuning pt;
   HmfTuning ht;
   int mirror_fmt;
+  int wide_units;  // md_ctx::fx_wide_units
   const void *bufs[14];
 };
 

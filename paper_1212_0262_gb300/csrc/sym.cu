@@ -403,17 +403,20 @@ size_t column_bytes(int64_t N, int64_t TI, int64_t TJ, int nacc, int col) {
   return (size_t)sym_rowstart(n_it, m * n_it, (int)m) * TJ * nacc * col;
 }
 
-// The context's column buffer made this large; false if the memory is not to be had.  Inside a
-// caller's capture, where nothing can be allocated, the stage itself reports what is missing.
+// The context's column buffer made this large; false if the memory is not to be had, the old
+// buffer then kept (other stages, and graphs of them, use it).  Inside a caller's capture, where
+// nothing can be allocated, the stage itself reports what is missing.
 bool reserve_columns(md_ctx *c, size_t need) {
   if (need <= c->sym_colslot_bytes) return true;
   cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(c->stream, &st) != cudaSuccess) cudaGetLastError();
   else if (st != cudaStreamCaptureStatusNone) return true;
+  void *buf = dev_alloc(need);
+  if (!buf) return false;
   dev_free(c->sym_colslot);
-  c->sym_colslot = dev_alloc(need);
-  c->sym_colslot_bytes = c->sym_colslot ? need : 0;
-  return c->sym_colslot != nullptr;
+  c->sym_colslot = buf;
+  c->sym_colslot_bytes = need;
+  return true;
 }
 
 // FP64 stages with integer pair arithmetic: Fx<rows per thread, j-tile>.  A unit is one
