@@ -123,8 +123,9 @@ __device__ __forceinline__ void fx_add(unsigned sg, unsigned w2, unsigned w1, un
 // pair, 57% of the integer pipe and of the FP64 pipe (4 warps per scheduler; dependent
 // instructions are what is left).  One 2D force at N = 49,152: 28.1 ms with GravF64, 9.74 with
 // s on the FP64 pipe, 7.25 as it stands.
-// eps of the fixed-point form (below, the unit 2^lsb of the sums would grow too large)
-inline bool fx_grav_applies(double eps) { return eps >= 0x1p-28; }
+// eps of the fixed-point form: below, the unit 2^lsb of the sums would grow too large; far above,
+// it would lie below the smallest double, and the terms of padding above it
+inline bool fx_grav_applies(double eps) { return eps >= 0x1p-28 && eps <= 0x1p600; }
 
 template <int D>
 struct FxGravTraits;
@@ -486,9 +487,10 @@ struct FxGrav2DAdj {
   // divided by its s must vanish)
   __device__ static int vexp(const PairArgs &a) { return *a.vrange == 0u ? 299 : (int)(*a.vrange >> 20) - 1021; }
   // the v too large (or not finite) or, not all equal, too close for the exponents used here
+  // (the unit of j from 2^-1022 on)
   __device__ static bool v_wild(const PairArgs &a) {
     const unsigned m = *a.vrange;
-    return m >= (1322u << 20) || (m != 0u && m < (223u << 20));
+    return m >= (1322u << 20) || (m != 0u && m < (unsigned)max(223, 2 * Fwd::half_exp(a) + 83) << 20);
   }
   // units of the sums of f, j, e: |f| <= 2^(-half - 1), |j| <= 2^(vexp + 1/2 - 2 half),
   // |e| <= 0.325 eps^(-3/2) <= 2^(-3 half - 1), each 2^83 units at most
