@@ -248,10 +248,11 @@ FX_FN void add96_carry(Acc96 &a, u32 w2, u32 w1, u32 w0, u32 c) {
 
 // A lane's column sum (|sum| < 2^85) as limbs of 27, 27 and 27 bits and a sign, each of which
 // adds over 32 lanes without overflow (the top one below 2^31: 0.77 2^85 is the largest sum of
-// the policies).  The low 5 bits are rounded to nearest: but for half a unit (ties go up) that
-// error has no sign, so it does not grow with the number of sums like a truncation's.
-FX_FN void column_limbs(Acc96 a, u32 &l0, u32 &l1, int &l2) {
-  add96(a, 0u, 0u, 16u);
+// the policies).  The low 5 bits are rounded to nearest, by starting the sum at half of 2^5: but
+// for half a unit (ties go up) that error has no sign, so it does not grow with the number of
+// sums like a truncation's.
+FX_FN Acc96 column_start() { return Acc96{16u, 0u, 0u}; }
+FX_FN void column_limbs(const Acc96 &a, u32 &l0, u32 &l1, int &l2) {
   l0 = a.w0 >> 5;
   l1 = a.w1 & 0x07ffffffu;
   l2 = (int)shf_r(a.w1, a.w2, 27);

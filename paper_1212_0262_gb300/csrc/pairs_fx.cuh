@@ -32,8 +32,8 @@ struct FxRowSums {
   __device__ double &at(int v) const { return p[v * NT]; }
 };
 
-// Warp total of a 96-bit sum (|sum| < 2^85 per lane) to the nearest 2^5: three limbs, each
-// added over the 32 lanes without overflow.
+// Warp total of 96-bit sums from column_start() (|sum| < 2^85 per lane) to the nearest 2^5: three
+// limbs, each added over the 32 lanes without overflow.
 __device__ __forceinline__ uint4 fx_warp_sum(const fx64::Acc96 &a) {
   unsigned l0, l1;
   int l2;
@@ -229,7 +229,7 @@ struct FxGrav {
       const Vec o = sm[j];
       fx64::Acc96 col[D];
 #pragma unroll
-      for (int c = 0; c < D; c++) col[c] = fx64::Acc96{0u, 0u, 0u};
+      for (int c = 0; c < D; c++) col[c] = fx64::column_start();
       unsigned h[R][D], yh[R][D], yl[R][D];
       unsigned long long pw[R];
       int k[R][D];
@@ -399,7 +399,7 @@ struct RingFx {
     for (int j = 0; j < TJ; j++) {
       const int4 p = sm[2 * j], q = sm[2 * j + 1];
       const fx64::Limbs ns{p.x, p.y}, c{p.z, p.w}, na{q.x, q.y}, g{q.z, q.w};
-      fx64::Acc96 col{0u, 0u, 0u};
+      fx64::Acc96 col = fx64::column_start();
 #pragma unroll
       for (int r = 0; r < R; r++) {
         const long long S = fx64::dot2(st.s[r], st.c[r], c, ns);     // sin(theta_i - theta_j) 2^60

@@ -21,7 +21,9 @@ extern "C" void warp(const u32 *w, u32 *o0, u32 *o1, int *o2) {
   u32 t0 = 0, t1 = 0, t2 = 0;
   for (int i = 0; i < 32; i++) {
     u32 l0, l1; int l2;
-    column_limbs(Acc96{w[3 * i], w[3 * i + 1], w[3 * i + 2]}, l0, l1, l2);
+    Acc96 a = column_start();
+    add96(a, w[3 * i + 2], w[3 * i + 1], w[3 * i]);
+    column_limbs(a, l0, l1, l2);
     t0 += l0; t1 += l1; t2 += (u32)l2;
   }
   *o0 = t0; *o1 = t1; *o2 = (int)t2;
