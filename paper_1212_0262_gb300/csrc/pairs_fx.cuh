@@ -9,7 +9,9 @@
 // A unit that touches a coordinate beyond RANGE, 2^26 sqrt(eps) (3D: 2^15), or a non-finite one
 // runs the FP64 policy's tile instead: at twice that distance in every component a 2D term is
 // still 2^54 units long and a 3D term 2^50, so that half a unit per term stays below the
-// rounding of FP64 sums.  Error against 64 bits of 1,024 particles in a disk or ball of radius
+// rounding of FP64 sums.  So does a unit all of whose particles lie within 2^-24 sqrt(eps) (CLOSE)
+// of its first row, whose terms, about d / eps, are as small: that is a system, or a group in one,
+// whose extent is nothing against its softening length.  Error against 64 bits of 1,024 particles in a disk or ball of radius
 // R, rms over the particles of |error| / sum of |terms|, column sums truncated to 2^11 units,
 // rounded to 2^5, and all in FP64: 2D R = 1000, eps = 1e-8 1.7e-15, 3.8e-17, 4.3e-16;
 // 3D R = 30, eps = 1e-6 2.7e-14, 4.6e-17, 4.2e-16.  The CTA decides per unit with one vote,
@@ -23,7 +25,8 @@ namespace {
 constexpr int kFxFlush = 16;        // units between moves of the row sums into doubles
 // What stage() finds in a 16-byte chunk of a tile, and load() in a thread's rows (State::flags)
 constexpr int kFxWild = 1;    // out of the fixed-point range
-constexpr int kFxNarrow = 2;  // so small that the fixed-point form has fewer bits than a double
+constexpr int kFxNarrow = 2;  // Ring: so small that the fixed-point form has fewer bits than a double
+constexpr int kFxBroad = 4;   // 2D, 3D: far enough from the unit's first row for the fixed-point form
 
 // Row sums of a thread in shared memory: [value][thread]
 template <int V>
@@ -183,7 +186,7 @@ struct FxGrav {
     fx64::Acc96 acc[R][NACC];
     FxRowSums<R * NACC> rows;
     int units;     // since the last flush
-    int flags;     // kFxWild, kFxNarrow: of the rows of this thread
+    int flags;     // kFxWild, kFxBroad: of the rows of this thread
   };
   // floor(log2(eps) / 2)
   __device__ static int half_exp(const PairArgs &a) { return ((int)(fx64::hi_word(a.epsd) >> 20) - 1023) >> 1; }
@@ -192,8 +195,15 @@ struct FxGrav {
     const unsigned h = fx64::hi_word(v) & 0x7fffffffu;
     return h >= ((unsigned)(1023 + range + half) << 20) && h != (fx64::hi_word(1.0e150));  // padding: its terms vanish
   }
+  // v farther from the reference coordinate than CLOSE (padding is not)
+  static constexpr int CLOSE = 24;
+  __device__ static bool broad(double v, double ref, int half) {
+    return (fx64::hi_word(v - ref) & 0x7fffffffu) >= ((unsigned)(1023 - CLOSE + half) << 20) &&
+           (fx64::hi_word(v) & 0x7fffffffu) != fx64::hi_word(1.0e150);
+  }
   __device__ static void load(State &st, const void *mirror, int64_t i0, const PairArgs &a, double *rowsm) {
     const int half = half_exp(a);
+    const Vec ref = ((const Vec *)mirror)[i0];
     st.flags = 0;
     fx_clear<State, R, NACC>(st, rowsm);
 #pragma unroll
@@ -202,7 +212,8 @@ struct FxGrav {
 #pragma unroll
       for (int d = 0; d < D; d++) {
         st.x[r][d] = fx_coord(m, d);
-        if (out_of_range(st.x[r][d], half)) st.flags = kFxWild;
+        if (out_of_range(st.x[r][d], half)) st.flags |= kFxWild;
+        if (broad(st.x[r][d], fx_coord(ref, d), half)) st.flags |= kFxBroad;
       }
     }
   }
@@ -211,11 +222,14 @@ struct FxGrav {
 #pragma unroll
     for (int d = 0; d < NACC; d++) out[d] = st.rows.at(r * NACC + d);
   }
-  // a 16-byte chunk of the tile: whether it is out of range (3D: (x, y) or (z, 0))
-  __device__ static int stage(const unsigned char *tile, int ch, unsigned char *, const PairArgs &a) {
-    const double2 v = ((const double2 *)tile)[ch];
+  // a 16-byte chunk of the tile, all or half of a record (3D: (x, y) or (z, 0)), and the same of the
+  // unit's first row
+  __device__ static int stage(const unsigned char *tile, int ch, unsigned char *, const PairArgs &a, int64_t i0) {
+    constexpr int PER = JB / 16;
+    const double2 v = ((const double2 *)tile)[ch], ref = ((const double2 *)a.mirror_in)[i0 * PER + ch % PER];
     const int half = half_exp(a);
-    return out_of_range(v.x, half) || out_of_range(v.y, half) ? kFxWild : 0;
+    return (out_of_range(v.x, half) || out_of_range(v.y, half) ? kFxWild : 0) |
+           (broad(v.x, ref.x, half) || broad(v.y, ref.y, half) ? kFxBroad : 0);
   }
   template <bool COL>
   __device__ static void unit(State &st, const unsigned char *smb, const unsigned char *, const PairArgs &a,
@@ -381,7 +395,7 @@ struct RingFx {
   __device__ static void flush(State &st, const PairArgs &a) { fx_flush<State, R, NACC>(st, lsb(a)); }
   __device__ static void total(const State &st, int r, double *out) { out[0] = st.rows.at(r); }
   // half a record, (s, c) or (a, g): as (-s, c) or (-a, g) limbs
-  __device__ static int stage(const unsigned char *tile, int ch, unsigned char *out, const PairArgs &) {
+  __device__ static int stage(const unsigned char *tile, int ch, unsigned char *out, const PairArgs &, int64_t) {
     const double2 v = ((const double2 *)tile)[ch];
     const fx64::Limbs x = fx64::limbs_of(-v.x), y = fx64::limbs_of(v.y);
     ((int4 *)out)[ch] = make_int4(x.h, x.l, y.h, y.l);
@@ -482,6 +496,7 @@ struct FxGrav2DAdj {
     int flags;
   };
   static constexpr int RANGE = 9;
+  static constexpr int CLOSE = Fwd::CLOSE;
   __device__ static bool out_of_range(double v, int half) { return Fwd::out_of_range(v, half, RANGE); }
   // |w_d| <= 2 W < 2^vexp.  All v equal: any exponent will do (the w of padding, up to 2^299,
   // divided by its s must vanish)
@@ -500,6 +515,7 @@ struct FxGrav2DAdj {
   __device__ static int lsb(const PairArgs &a, int d) { return lsb_of(d >> 1, Fwd::half_exp(a), vexp(a)); }
   __device__ static void load(State &st, const void *mirror, int64_t i0, const PairArgs &a, double *rowsm) {
     const int half = Fwd::half_exp(a);
+    const double2 ref = *(const double2 *)((const double4_16a *)mirror + i0);
     st.flags = v_wild(a) ? kFxWild : 0;
     fx_clear<State, R, NACC>(st, rowsm);
 #pragma unroll
@@ -509,7 +525,8 @@ struct FxGrav2DAdj {
       st.x[r][1] = m.y;
       st.v[r][0] = m.z;
       st.v[r][1] = m.w;
-      if (out_of_range(m.x, half) || out_of_range(m.y, half)) st.flags = kFxWild;
+      if (out_of_range(m.x, half) || out_of_range(m.y, half)) st.flags |= kFxWild;
+      if (Fwd::broad(m.x, ref.x, half) || Fwd::broad(m.y, ref.y, half)) st.flags |= kFxBroad;
     }
   }
   __device__ static void flush(State &st, const PairArgs &a) {
@@ -527,10 +544,12 @@ struct FxGrav2DAdj {
     for (int d = 0; d < NACC; d++) out[d] = st.rows.at(r * NACC + d);
   }
   // half a record, (x, y) or (vx, vy)
-  __device__ static int stage(const unsigned char *tile, int ch, unsigned char *, const PairArgs &a) {
-    const double2 m = ((const double2 *)tile)[ch];
+  __device__ static int stage(const unsigned char *tile, int ch, unsigned char *, const PairArgs &a, int64_t i0) {
+    if (ch & 1) return 0;
+    const double2 m = ((const double2 *)tile)[ch], ref = ((const double2 *)a.mirror_in)[2 * i0];
     const int half = Fwd::half_exp(a);
-    return (ch & 1) == 0 && (out_of_range(m.x, half) || out_of_range(m.y, half)) ? kFxWild : 0;
+    return (out_of_range(m.x, half) || out_of_range(m.y, half) ? kFxWild : 0) |
+           (Fwd::broad(m.x, ref.x, half) || Fwd::broad(m.y, ref.y, half) ? kFxBroad : 0);
   }
   template <bool COL>
   __device__ static void unit(State &st, const unsigned char *smb, const unsigned char *, const PairArgs &a,

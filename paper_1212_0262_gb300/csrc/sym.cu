@@ -67,7 +67,11 @@ template <class P, class = void>
 struct IsFx : std::false_type {};
 template <class P>
 struct IsFx<P, std::void_t<decltype(P::FX)>> : std::true_type {};
-// and with a rule on narrow records
+// and with a rule on units of close particles, or on narrow records
+template <class P, class = void>
+struct HasClose : std::false_type {};
+template <class P>
+struct HasClose<P, std::void_t<decltype(P::CLOSE)>> : std::true_type {};
 template <class P, class = void>
 struct HasNarrow : std::false_type {};
 template <class P>
@@ -147,11 +151,16 @@ __global__ void __launch_bounds__(Pol::THREADS, Pol::MINB) sym_pairs_kernel(Pair
       if constexpr (FX) {
         int flags = 0, narrow = 0;
         for (int ch = threadIdx.x; ch < CHUNKS; ch += THR) {
-          const int f = Pol::stage(sbuf[buf], ch, staged, a);
+          const int f = Pol::stage(sbuf[buf], ch, staged, a, i0);
           flags |= f;
           narrow += (f & kFxNarrow) != 0;
         }
         wild = __syncthreads_or((flags | st.flags) & kFxWild);
+        if constexpr (HasClose<Pol>::value) {
+          const bool broad = __syncthreads_or((flags | st.flags) & kFxBroad);
+          const int64_t rows = a.N - i0, cols = a.N - jt * TJ;  // particles, padding follows
+          if (!broad && cols > 0 && !(rows == 1 && cols == 1)) wild = true;
+        }
         if constexpr (HasNarrow<Pol>::value) {
           static_assert(CHUNKS <= 2 * THR, "at most two chunks per thread");
           int n = __syncthreads_count(narrow > 0);
