@@ -233,16 +233,21 @@ __device__ __forceinline__ bool grid_finish(double sc, double ss, double *partia
   return true;
 }
 
-// Cold systems, whose angles all lie near 0, pi / 2, pi or 3 pi / 2 (|Mx| or |My| above 1 - 2^-11:
-// within some 2^-5): the forces are differences of sines (cosines) and a magnetization component
+// Cold systems, whose angles all lie near 0, pi / 2, pi or 3 pi / 2 (|Mx| or |My| above 1 - 2^-24:
+// within some 3e-4): the forces are differences of sines (cosines) and a magnetization component
 // that are small themselves, where doubles have more bits than fixed-point numbers.  Their
 // stages are all FP64: (cos, sin) kept as doubles (*HmfArgs::fmt = 1), the table-driven sines and
 // cosines of sincos_fp64.cuh, FP64 sums; 12 FP64 operations per particle-stage, 8.0 us at
-// N = 10,007, 1.31 ms at N = 5e7.  A stage whose predecessor's M was cold reads doubles, one whose own M is cold
-// writes them.
+// N = 10,007, 1.31 ms at N = 5e7.  Wider systems are more exact in fixed point (N = 50,000, angles
+// up to 1e-3, rms of |error| / scale of a force 9e-16 against 2.8e-15, whose table sine rounds r^3 / 6
+// to FP32), narrower ones as doubles (up to 1e-6 7e-13 against 7e-17).  A stage whose
+// predecessor's M was cold reads doubles, one whose own M is cold writes them.
+__device__ __forceinline__ bool hmf_near_one(double m) {
+  const unsigned h = fx64::hi_word(m) & 0x7fffffffu;
+  return h >= 0x3fefffffu && h < kTopMax && (h > 0x3fefffffu || fx64::lo_word(m) > 0xe0000000u);
+}
 __device__ __forceinline__ bool hmf_cold(double mx, double my) {
-  const unsigned top = hmf_top(mx, my);
-  return top > 0x3feffc00u && top < kTopMax;
+  return (hmf_near_one(mx) && hmf_top(0.0, my) < kTopMax) || (hmf_near_one(my) && hmf_top(mx, 0.0) < kTopMax);
 }
 template <int MODE, bool CG>
 __device__ __noinline__ double2 hmf_sweep64(double *q, double *p, int4 *cs, double *fout, int64_t N, double invN,
