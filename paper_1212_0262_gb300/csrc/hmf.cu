@@ -562,7 +562,9 @@ __device__ __forceinline__ long long fix38(float v) {
 // cluster barrier every warp adds them for itself.  A drift of some 2^23 and more in one stage
 // leaves the FP32 reduction's range: its cosine can be of any size, infinite or NaN.  A warp
 // that holds one puts kWildSum in place of its total, every CTA sees it in the sum, and the
-// stage's sums are added in FP64, as the launched stages do.
+// stage's sums are added in FP64, as the launched stages do.  So they are where a sum is below
+// 2^-13 per group (all sines or cosines small, or as many of either sign): there the groups'
+// 2^-39 could reach M's FP32.
 constexpr long long kWildSum = 1ll << 54;  // the particles' own sums stay below 2^53, 128 of these below 2^62
 __global__ void __launch_bounds__(NT, 1) hmf_run_mixed_kernel(HmfArgs a, HmfRun r) {
   namespace cg = cooperative_groups;
@@ -630,7 +632,7 @@ __global__ void __launch_bounds__(NT, 1) hmf_run_mixed_kernel(HmfArgs a, HmfRun 
     }
     sx = (double)v.x * 0x1p-38;
     sy = (double)v.y * 0x1p-38;
-    if (v.x > kWildSum / 2) {  // the same in every thread of the cluster
+    if (v.x > kWildSum / 2 || llabs(v.x) < G << 25 || llabs(v.y) < G << 25) {  // the same in every thread of the cluster
       const double2 b = block_sum2<NT>((double)ac + (double)co, (double)as + (double)so, red);
       if (threadIdx.x == 0) wide = b;
       cluster.sync();
