@@ -62,10 +62,10 @@ __device__ __forceinline__ void load_sincos_tab(double2 *sm) {
 // (sincos_fx.cuh), 16 bytes per particle, so that the stage's force, its sine and cosine and
 // the magnetization sums are integer arithmetic; the kick and the drift are its FP64
 // operations (12 with the sine and cosine of sincos_fp64.cuh and an FP64 force, which bound
-// the stage).  Per stage at N = 5e7: 1149 -> 582 us, 3.2 GB at 81% of the copy rate; the
+// the stage).  Per stage at N = 5e7: 1149 -> 556 us, 3.2 GB at 85% of the copy rate; the
 // integer pipe is half busy, the next pair's loads run ahead of the arithmetic (604 us without).
-// A non-finite angle is marked by kNoAngle: its force is NaN, and so are the sums.  Cold systems
-// hold doubles instead (hmf_sweep64).
+// A non-finite angle is marked by kNoAngle and makes the sums NaN, and with them every force.
+// Cold systems hold doubles instead (hmf_sweep64).
 __device__ scfx::Entry g_sincos_fx[kTabN];
 constexpr int kNoAngle = (int)0x80000000;
 
@@ -109,23 +109,28 @@ __device__ __forceinline__ int4 angle_fx(double th, const scfx::Entry *tab, long
 }
 
 // The FP64 stages' magnetization: (My, -Mx) 2^e as limbs for the integer force, the larger of
-// them in [1/2, 1), so that a force has the bits of a double relative to |M|, however small.
+// them in [1/2, 1), so that a force has the bits of a double relative to |M|, however small.  The
+// kicks' coefficient takes the 2^-e.
 struct HmfM {
   fx64::Limbs my, nmx;
-  int e;
-  bool fx;  // finite and of ordinary size
+  double unit;  // 2^-e
 };
-// high word of the larger of |Mx|, |My|: from 2^-600 to 1.5 the integer form takes them
+// high word of the larger of |Mx|, |My|
 __device__ __forceinline__ unsigned hmf_top(double mx, double my) {
   return max(fx64::hi_word(mx) & 0x7fffffffu, fx64::hi_word(my) & 0x7fffffffu);
 }
-constexpr unsigned kTopMin = (1023u - 600u) << 20, kTopMax = 0x3ff80000u;
-__device__ __forceinline__ HmfM hmf_m_of(double mx, double my) {
-  HmfM m;
+constexpr unsigned kTopMin = (1023u - 200u) << 20, kTopMax = 0x3ff80000u;  // 2^-200, 1.5
+// M that the integer force takes: not those that are not finite (some angle is not), or too small.
+__device__ __forceinline__ bool hmf_ordinary(double mx, double my) {
   const unsigned top = hmf_top(mx, my);
-  m.fx = top >= kTopMin && top < kTopMax;
-  m.e = 1022 - (int)(top >> 20);
-  const double scale = __hiloint2double(m.fx ? (1023 + 62 + m.e) << 20 : 0, 0);  // 2^(62 + e)
+  return top >= kTopMin && top < kTopMax;
+}
+// of an ordinary M; lone: N = 1, whose particle's force, its self-term, is exactly zero
+__device__ __forceinline__ HmfM hmf_m_of(double mx, double my, bool lone) {
+  HmfM m;
+  const int e = 1022 - (int)(hmf_top(mx, my) >> 20);
+  const double scale = __hiloint2double(lone ? 0 : (1023 + 62 + e) << 20, 0);
+  m.unit = __hiloint2double((1023 - e) << 20, 0);
   m.my = scfx::split(__double2ll_rn(my * scale));
   m.nmx = scfx::split(__double2ll_rn(-mx * scale));
   return m;
@@ -180,21 +185,18 @@ __device__ __forceinline__ void hmf_particle_mixed(double &th, double &pp, const
   }
 }
 
-// One particle of an FP64 stage; cs: its (cos, sin), rewritten by a drift.
+// One particle of an FP64 stage; cs: its (cos, sin), rewritten by a drift; kick: a.kick m.unit.
 template <int MODE>
 __device__ __forceinline__ void hmf_particle_fp64(double &th, double &pp, int4 &cs, const HmfArgs &a, const HmfM &m,
-                                                  double mx, double my, long long &aci, long long &asi, int64_t i,
+                                                  double kick, long long &aci, long long &asi, int64_t i,
                                                   const scfx::Entry *tab) {
   const fx64::Limbs c{cs.x, cs.y}, s{cs.z, cs.w};
-  double f = scfx::to_double60(fx64::dot2(c, s, m.my, m.nmx), m.e);  // cos My - sin Mx
-  if (!m.fx) f = hmf_force_fp64((double)scfx::join(c.h, c.l) * 0x1p-62, (double)scfx::join(s.h, s.l) * 0x1p-62, mx, my, a.invN);
-  if (cs.x == kNoAngle) f = __longlong_as_double(0x7ff8000000000000LL);
-  if (a.invN == 1.0) f = 0.0;  // a lone particle's self-term
+  const double f = scfx::to_double60(fx64::dot2(c, s, m.my, m.nmx));  // (cos My - sin Mx) 2^e
   if (MODE == STAGE_FORCE_ONLY) {
-    a.fout[i] = f;
+    a.fout[i] = f * m.unit;
     return;
   }
-  pp = fma(a.kick, f, pp);
+  pp = fma(kick, f, pp);
   if (MODE == STAGE_KICK_DRIFT) {
     th = fma(a.drift, pp, th);
     cs = angle_fx(th, tab, aci, asi);
@@ -238,7 +240,7 @@ __device__ __forceinline__ bool grid_finish(double sc, double ss, double *partia
 // that are small themselves, where doubles have more bits than fixed-point numbers.  Their
 // stages are all FP64: (cos, sin) kept as doubles (*HmfArgs::fmt = 1), the table-driven sines and
 // cosines of sincos_fp64.cuh, FP64 sums; 12 FP64 operations per particle-stage, 8.0 us at
-// N = 10,007, 1.31 ms at N = 5e7.  Wider systems are more exact in fixed point (N = 50,000, angles
+// N = 10,007, 1.31 ms at N = 5e7.  So are stages whose M is not finite, or below 2^-200.  Wider systems are more exact in fixed point (N = 50,000, angles
 // up to 1e-3, rms of |error| / scale of a force 9e-16 against 2.8e-15, whose table sine rounds r^3 / 6
 // to FP32), narrower ones as doubles (up to 1e-6 7e-13 against 7e-17).  A stage whose
 // predecessor's M was cold reads doubles, one whose own M is cold writes them.
@@ -341,7 +343,8 @@ __device__ __forceinline__ void hmf_sweep(const HmfArgs &a, double mx, double my
     if constexpr (CG) return __ldcg(ptr);
     else return *ptr;
   };
-  const HmfM m = hmf_m_of(mx, my);
+  const HmfM m = hmf_m_of(mx, my, a.invN == 1.0);
+  const double kick = a.kick * m.unit;
   const float mxf = (float)mx, myf = (float)my, dtf = (float)a.drift;
   float acf = 0.f, asf = 0.f;
   long long aci = 0, asi = 0;
@@ -395,8 +398,8 @@ __device__ __forceinline__ void hmf_sweep(const HmfArgs &a, double mx, double my
         an = load(a.cs + 2 * nx);
         bn = load(a.cs + 2 * nx + 1);
       }
-      hmf_particle_fp64<MODE>(qv.x, pv.x, ca, a, m, mx, my, aci, asi, 2 * ix, tab);
-      hmf_particle_fp64<MODE>(qv.y, pv.y, cb, a, m, mx, my, aci, asi, 2 * ix + 1, tab);
+      hmf_particle_fp64<MODE>(qv.x, pv.x, ca, a, m, kick, aci, asi, 2 * ix, tab);
+      hmf_particle_fp64<MODE>(qv.y, pv.y, cb, a, m, kick, aci, asi, 2 * ix + 1, tab);
       if (MODE == STAGE_KICK_DRIFT) {
         a.cs[2 * ix] = ca;
         a.cs[2 * ix + 1] = cb;
@@ -423,7 +426,7 @@ __device__ __forceinline__ void hmf_sweep(const HmfArgs &a, double mx, double my
       hmf_particle_mixed<MODE>(th, pp, a, mxf, myf, dtf, acf, asf, i);
     } else {
       int4 c = load(a.cs + i);
-      hmf_particle_fp64<MODE>(th, pp, c, a, m, mx, my, aci, asi, i, tab);
+      hmf_particle_fp64<MODE>(th, pp, c, a, m, kick, aci, asi, i, tab);
       if (MODE == STAGE_KICK_DRIFT) a.cs[i] = c;
     }
     if (MODE == STAGE_KICK_DRIFT) a.q[i] = th;
@@ -459,7 +462,7 @@ __global__ void __launch_bounds__(NT, MODE != STAGE_KICK_DRIFT ? 1 : MIXED ? 4 :
   double acd = 0.0, asd = 0.0;
   if constexpr (!MIXED) {
     const bool in64 = *a.fmt != 0u, out64 = MODE == STAGE_KICK_DRIFT && hmf_cold(mx, my);
-    if (in64 || out64) {
+    if (in64 || out64 || !hmf_ordinary(mx, my)) {
       if (MODE == STAGE_KICK_DRIFT) load_sincos_tab((double2 *)tabraw);
       hmf_sweep64<MODE, false>(a, mx, my, tabraw, in64, out64, acd, asd);
       // the last CTA to finish: every other has read *a.fmt
@@ -514,7 +517,7 @@ __global__ void __launch_bounds__(NT, 3) hmf_run_fp64_kernel(HmfArgs a, HmfRun r
     double acd = 0.0, asd = 0.0;
     const double mx = s.x * a.invN, my = s.y * a.invN;
     const bool out64 = hmf_cold(mx, my);
-    const int want = in64 || out64;
+    const int want = in64 || out64 || !hmf_ordinary(mx, my);
     if (table != want) {  // every thread is past its last look-up: it has been at the cluster barrier since
       if (want) load_sincos_tab((double2 *)tabraw);
       else load_sincos_fx(tab);

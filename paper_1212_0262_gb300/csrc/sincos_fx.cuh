@@ -79,8 +79,8 @@ FX_FN bool sincos_fx(double th, const Entry *tab, i64 &s62, i64 &c62) {
   return true;
 }
 
-// v 2^(-60 - e) as a double (rounded to nearest), |v| < 2^62, -300 <= e <= 900
-FX_FN double to_double60(i64 v, int e = 0) {
+// v 2^-60 as a double (rounded to nearest), |v| < 2^62
+FX_FN double to_double60(i64 v) {
   const u32 sg = (u32)((int)(u32)((u64)v >> 32) >> 31);
   const u64 a = (u64)(v < 0 ? -v : v);
   u32 h = (u32)(a >> 32), l = (u32)a;
@@ -93,8 +93,8 @@ FX_FN double to_double60(i64 v, int e = 0) {
   }
   const int lz = sc64::clz32(h);  // normalise to bit 63
   const u32 nh = fx64::shf_l(l, h, lz & 31), nl = l << lz;
-  // value = (nh:nl) 2^-(60 + e + z + lz): exponent of bit 63 is 3 - e - z - lz
-  const u32 oh = (sg & 0x80000000u) | ((u32)(1023 + 3 - e - z - lz - 1) << 20);
+  // value = (nh:nl) 2^-(60 + z + lz): exponent of bit 63 is 3 - z - lz
+  const u32 oh = (sg & 0x80000000u) | ((u32)(1023 + 3 - z - lz - 1) << 20);
   const u64 m = (((((u64)nh << 32) | nl) >> 10) + 1) >> 1;  // 53 bits; the leading one adds 1 to the exponent
   return sc64::bitsd(((u64)oh << 32) + m);
 }
