@@ -466,14 +466,14 @@ struct RingFx {
 // unit of j also follows from the v: from W, the largest |v_k - v_0| (found before the stage).
 // Every particle has a partner whose w is at least W / 2, however the other w are spread, so
 // the sum of its |j| is at least 2^58 units within RANGE; terms of j are rounded to
-// nearest and column sums are exact, so that N small terms beside that one add no bias.  Error
+// nearest and its column sums are exact, so that N small terms beside that one add no bias.  Error
 // against 64 bits of 1,024 particles in a disk of radius R, rms of |error| / sum of |terms|,
 // one-sided in FP64 and here: R = 1, eps = 1e-3 (2^5 sqrt(eps)) j 1.1e-16, 4.7e-17, e 1.5e-16,
 // 9.5e-17; eps = 4e-6 (2^9) j 2.1e-16, 9.3e-17, e 2.9e-16, 1.5e-16; eps = 1e-8 (FP64 units here)
 // j 2.2e-16, 1.4e-16, e 2.9e-16, 2.1e-16.
 //
 // Bound by the FP64 pipe (78% at N = 16,384).  A stage of N = 1,000, 8,192 and 16,385: one-sided in
-// FP64 165, 2290, 8070 us, here 61, 526, 2160; all units out of range, as in GravF64Adj but with
+// FP64 165, 2290, 8070 us, here 61, 522, 2160; all units out of range, as in GravF64Adj but with
 // columns, 92, 1930, 7160.
 template <int R_, int TJ_>
 struct FxGrav2DAdj {
@@ -565,7 +565,7 @@ struct FxGrav2DAdj {
       const double4_16a o = sm[j];
       fx64::Acc96 col[NACC];
 #pragma unroll
-      for (int c = 0; c < NACC; c++) col[c] = fx64::Acc96{0u, 0u, 0u};
+      for (int c = 0; c < NACC; c++) col[c] = c >> 1 == 1 ? fx64::Acc96{0u, 0u, 0u} : fx64::column_start();
 #pragma unroll
       for (int r = 0; r < R; r++) {
         const double d[2] = {st.x[r][0] - o.x, st.x[r][1] - o.y}, v[2] = {st.v[r][0] - o.z, st.v[r][1] - o.w};
@@ -625,7 +625,7 @@ struct FxGrav2DAdj {
       if (COL) {
 #pragma unroll
         for (int c = 0; c < NACC; c++) {
-          const uint4 s = fx_warp_sum_exact(col[c]);
+          const uint4 s = c >> 1 == 1 ? fx_warp_sum_exact(col[c]) : fx_warp_sum(col[c]);
           if (lane == 0) colsm[NACC * j + c] = s;
         }
       }
