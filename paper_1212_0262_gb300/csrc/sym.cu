@@ -117,9 +117,11 @@ __global__ void __launch_bounds__(Pol::THREADS, Pol::MINB) sym_pairs_kernel(Pair
     for (int ch = threadIdx.x; ch < CHUNKS; ch += THR) cp_async16(&sbuf[buf][ch * 16], src + ch * 16);
     cp_async_commit();
   };
+  bool rows_broad = true;  // FX: some row is broad, whatever the columns are
   auto load_rows = [&](typename Pol::State &st, int64_t i0) {
     if constexpr (FX) Pol::load(st, a.mirror_in, i0, a, rowsm);
     else Pol::load(st, a.mirror_in, i0);
+    if constexpr (HasClose<Pol>::value) rows_broad = __syncthreads_or(st.flags & kFxBroad);
   };
 
   for (;;) {
@@ -157,9 +159,10 @@ __global__ void __launch_bounds__(Pol::THREADS, Pol::MINB) sym_pairs_kernel(Pair
         }
         wild = __syncthreads_or((flags | st.flags) & kFxWild);
         if constexpr (HasClose<Pol>::value) {
-          const bool broad = __syncthreads_or((flags | st.flags) & kFxBroad);
-          const int64_t rows = a.N - i0, cols = a.N - jt * TJ;  // particles, padding follows
-          if (!broad && cols > 0 && !(rows == 1 && cols == 1)) wild = true;
+          if (!rows_broad && !__syncthreads_or(flags & kFxBroad)) {
+            const int64_t rows = a.N - i0, cols = a.N - jt * TJ;  // particles, padding follows
+            if (cols > 0 && !(rows == 1 && cols == 1)) wild = true;
+          }
         }
         if constexpr (HasNarrow<Pol>::value) {
           static_assert(CHUNKS <= 2 * THR, "at most two chunks per thread");
