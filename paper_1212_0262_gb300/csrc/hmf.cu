@@ -63,7 +63,7 @@ __device__ __forceinline__ void load_sincos_tab(double2 *sm) {
 // the magnetization sums are integer arithmetic; the kick and the drift are its FP64
 // operations (12 with the sine and cosine of sincos_fp64.cuh and an FP64 force, which bound
 // the stage).  Per stage at N = 5e7: 1149 -> 556 us, 3.2 GB at 85% of the copy rate; the
-// integer pipe is half busy, the next pair's loads run ahead of the arithmetic (604 us without).
+// integer pipe is half busy, the next pair's loads run ahead of the arithmetic (22 us more without).
 // A non-finite angle is marked by kNoAngle and makes the sums NaN, and with them every force.
 // Cold systems hold doubles instead (hmf_sweep64).
 __device__ scfx::Entry g_sincos_fx[kTabN];
@@ -479,7 +479,7 @@ __global__ void __launch_bounds__(NT, MODE != STAGE_KICK_DRIFT ? 1 : MIXED ? 4 :
 // these sizes is all latency, so the stages follow one another behind a cluster barrier instead
 // of a kernel boundary, with the grid, the sweep directions and the groupings of the launched
 // stages, and so with their results.  Microseconds per stage at N = 300, 3,000, 10,007:
-// mixed 5.9, 6.7, 7.8 launched, 1.5, 2.0, 2.1 here; FP64 7.9, 10.8, 12.3 and 4.5, 6.2, 6.9 (the
+// mixed 5.9, 6.7, 7.8 launched, 1.7, 2.0, 2.2 here; FP64 7.9, 10.8, 12.3 and 4.2, 5.9, 6.2 (the
 // state through L2: 4.5 us in mixed, too).
 constexpr int kRunCtas = 16;  // CTAs of the largest cluster
 
@@ -635,7 +635,9 @@ __global__ void __launch_bounds__(NT, 1) hmf_run_mixed_kernel(HmfArgs a, HmfRun 
     }
     sx = (double)v.x * 0x1p-38;
     sy = (double)v.y * 0x1p-38;
-    if (v.x > kWildSum / 2 || llabs(v.x) < G << 25 || llabs(v.y) < G << 25) {  // the same in every thread of the cluster
+    // kWildSum, or a total below G 2^25 (t in the high word); the same in every thread of the cluster
+    const int hx = (int)(v.x >> 32), hy = (int)(v.y >> 32), t = (int)(G >> 7);
+    if (hx > (int)(kWildSum >> 33) || (unsigned)(hx + t) < 2u * t || (unsigned)(hy + t) < 2u * t) {
       const double2 b = block_sum2<NT>((double)ac + (double)co, (double)as + (double)so, red);
       if (threadIdx.x == 0) wide = b;
       cluster.sync();
