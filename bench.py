@@ -94,12 +94,13 @@ PAIR_KERNELS_FP64 = {
     (3, 1): ("streamk_kernel<Grav3DF64<2,128>>", 16, False),
 }
 # The symmetric FP64 kernels run the pair arithmetic on the integer pipe: name and
-# instructions issued per unordered pair (ncu, N = 49,152; 3D from its share of the 2D rate),
-# against 128 lanes per SM and clock
+# instructions issued per unordered pair (ncu smsp__inst_executed at N = 16,384 x 32 lanes /
+# unordered pairs, each kernel's own), against 128 lanes per SM and clock: the fraction says how
+# full the issue slots are, not how far the kernel is from a floor.
 PAIR_KERNELS_INT = {
-    (1, 6): ("sym_pairs_kernel<RingFx>", 137),
-    (2, 6): ("sym_pairs_kernel<FxGrav<2>>", 147),
-    (3, 6): ("sym_pairs_kernel<FxGrav<3>>", 235),
+    (1, 6): ("sym_pairs_kernel<RingFx>", 132),
+    (2, 6): ("sym_pairs_kernel<FxGrav<2>>", 137),
+    (3, 6): ("sym_pairs_kernel<FxGrav<3>>", 213),
 }
 
 

@@ -148,9 +148,13 @@ int md_set_eps(md_ctx *ctx, double eps);
  *                      one-sided kernel runs.  Sheets at eps = 0 count ranks in sorted
  *                      tiles instead (the same whole numbers, no such storage).  FP64 2D
  *                      md_grad / md_tangent_step stages take this form too (3 N^2 / 16
- *                      bytes up to N = 10,000, 3 N^2 / 32 above).
+ *                      bytes up to N = 10,000, 3 N^2 / 32 above).  The storage is kept
+ *                      until md_free; where it is refused, larger units or the one-sided
+ *                      kernel run from then on.
  *   "step_graphs"      md_step replays its steps after the first from captured CUDA
- *                      graphs of 8 steps (1, default) or launches every stage (0).
+ *                      graphs of 8 steps, or, for HMF systems of up to about 16,000
+ *                      particles, runs all its stages in one launch (1, default; the same
+ *                      results), or launches every stage (0).
  * MD_EINVAL for an unknown key or value. */
 int md_set_tuning(md_ctx *ctx, const char *key, int64_t value);
 

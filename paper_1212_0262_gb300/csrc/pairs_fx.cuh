@@ -122,10 +122,10 @@ __device__ __forceinline__ void fx_add(unsigned sg, unsigned w2, unsigned w1, un
 // ------------------------------------------------------------ forward 2D and 3D
 // Terms d / s (2D) and d s^(-3/2) (3D), s = |d|^2 + eps.  Per pair only the coordinate
 // differences are FP64 operations (2 instead of 14, 3 instead of 23.4); the squared distance,
-// its inverse power, the products and the sums are integers: about 147 instructions per 2D
-// pair, 57% of the integer pipe and of the FP64 pipe (4 warps per scheduler; dependent
+// its inverse power, the products and the sums are integers: 137 instructions per 2D pair and
+// 213 per 3D pair, 57% of the integer pipe and of the FP64 pipe (4 warps per scheduler; dependent
 // instructions are what is left).  One 2D force at N = 49,152: 28.1 ms with GravF64, 9.74 with
-// s on the FP64 pipe, 7.25 as it stands.
+// s on the FP64 pipe, 6.07 as it stands; 3D 49.6 and 9.7.
 // eps of the fixed-point form: below, the unit 2^lsb of the sums would grow too large; far above,
 // it would lie below the smallest double, and the terms of padding above it
 inline bool fx_grav_applies(double eps) { return eps >= 0x1p-28 && eps <= 0x1p600; }
@@ -333,8 +333,8 @@ using FxGrav3D = FxGrav<3, R, TJ>;
 // Sines and cosines are numbers of at most 1, so the whole pair term is fixed-point: S and
 // sin(d/2) as 62-bit dot products, sin^2 + eps/2 in 96 bits, its power -3/2 from an FP32 seed
 // and one third-order step, no FP64 operation (15.5 in RingF64).  The tile's records are
-// turned into integers once per unit, by the thread that loaded them.  137 instructions per
-// pair; one force at N = 49,152: 36.3 ms with RingF64, 7.11 here (bound by the integer pipe,
+// turned into integers once per unit, by the thread that loaded them.  132 instructions per
+// pair; one force at N = 49,152: 36.3 ms with RingF64, 6.08 here (bound by the integer pipe,
 // 51%, and by dependent instructions at 4 warps per scheduler).
 // The sine of a difference has an error of some 2^-59 here, a product of two doubles' one of
 // 2^-53 of the larger sine: less where both angles lie within 2^-6 of 0 (or of pi).  One such

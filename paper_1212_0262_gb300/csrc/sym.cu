@@ -342,8 +342,10 @@ int launch_sym(md_ctx *c, PairArgs a) {
   // single values, 4 for these two among them): 8 for the Ring tensor-core kernel, 3 for
   // the FP64 3D kernel, 4 for the others
   int kv = c->pt.vcta > 0 ? c->pt.vcta : Pol::FMT == 1 ? 8 : (MODEL == MD_GRAV3D && !MIXED) ? 3 : 4;
-  // integer policies: units are long; below 16 per CTA one range each is best (N = 16,385,
-  // Ring: 983 us, 1079 / 1031 / 994 with 2 / 3 / 4 ranges)
+  // integer policies, whose units are long: below 16 per CTA one range each.  Neither is best
+  // throughout; microseconds per force with one range and with four at N = 4,096, 8,192, 12,000,
+  // 16,385: Ring 85, 82; 245, 249; 435, 429; 785, 794; 2D 84, 79; 238, 251; 422, 412; 780, 780;
+  // 3D 122, 113; 366, 386; 683, 663; 1260, 1251.
   if (IsFx<Pol>::value && c->pt.vcta == 0 && a.U < 16 * G) kv = 1;
   a.P = (int)vcta_count(G, a.U, kv, IsFx<Pol>::value ? 1 : 16);
   int rc = ensure_pair_buffers(c, (int)TI, a.P, NACC);
@@ -436,7 +438,7 @@ bool reserve_columns(md_ctx *c, size_t need) {
 // cycles of latency, so small systems want small units (N = 1,000, microseconds per force,
 // 2D: 45 with <1, 64>, 58 with <2, 64>, 147 with <4, 128>), larger ones more rows to share
 // the column reductions (N = 16,385: 967, 915, 1020; N = 8,192: 264, 281, 343).  <4, 128> needs
-// half the column storage of <2, 64> and is 2-5% slower (N = 49,152: 7.17 against 7.07 ms).
+// half the column storage of <2, 64> and is 2-5% slower.
 constexpr int64_t kFxSmall = 10000, kFxLarge = 262144;
 // Where it does not fit (the caller's allocator may be bounded), <4, 128> runs at every size.
 template <template <int, int> class Fx, int MODEL, int MODE>
