@@ -62,7 +62,7 @@ __device__ __forceinline__ void load_sincos_tab(double2 *sm) {
 // (sincos_fx.cuh), 16 bytes per particle, so that the stage's force, its sine and cosine and
 // the magnetization sums are integer arithmetic; the kick and the drift are its FP64
 // operations (12 with the sine and cosine of sincos_fp64.cuh and an FP64 force, which bound
-// the stage).  Per stage at N = 5e7: 1149 -> 556 us, 3.2 GB at 85% of the copy rate; the
+// the stage).  Per stage at N = 5e7: 1149 -> 565 us, 3.2 GB at 84% of the copy rate; the
 // integer pipe is half busy, the next pair's loads run ahead of the arithmetic (22 us more without).
 // A non-finite angle is marked by kNoAngle and makes the sums NaN, and with them every force.
 // Cold systems hold doubles instead (hmf_sweep64).

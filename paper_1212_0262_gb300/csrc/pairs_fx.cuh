@@ -125,7 +125,7 @@ __device__ __forceinline__ void fx_add(unsigned sg, unsigned w2, unsigned w1, un
 // its inverse power, the products and the sums are integers: 137 instructions per 2D pair and
 // 213 per 3D pair, 57% of the integer pipe and of the FP64 pipe (4 warps per scheduler; dependent
 // instructions are what is left).  One 2D force at N = 49,152: 28.1 ms with GravF64, 9.74 with
-// s on the FP64 pipe, 6.07 as it stands; 3D 49.6 and 9.7.
+// s on the FP64 pipe, 7.07 as it stands; 3D 49.6 and 11.3.
 // eps of the fixed-point form: below, the unit 2^lsb of the sums would grow too large; far above,
 // it would lie below the smallest double, and the terms of padding above it
 inline bool fx_grav_applies(double eps) { return eps >= 0x1p-28 && eps <= 0x1p600; }
@@ -334,7 +334,7 @@ using FxGrav3D = FxGrav<3, R, TJ>;
 // sin(d/2) as 62-bit dot products, sin^2 + eps/2 in 96 bits, its power -3/2 from an FP32 seed
 // and one third-order step, no FP64 operation (15.5 in RingF64).  The tile's records are
 // turned into integers once per unit, by the thread that loaded them.  132 instructions per
-// pair; one force at N = 49,152: 36.3 ms with RingF64, 6.08 here (bound by the integer pipe,
+// pair; one force at N = 49,152: 36.3 ms with RingF64, 7.10 here (bound by the integer pipe,
 // 51%, and by dependent instructions at 4 warps per scheduler).
 // The sine of a difference has an error of some 2^-59 here, a product of two doubles' one of
 // 2^-53 of the larger sine: less where both angles lie within 2^-6 of 0 (or of pi).  One such
@@ -473,8 +473,8 @@ struct RingFx {
 // j 2.2e-16, 1.4e-16, e 2.9e-16, 2.1e-16.
 //
 // Bound by the FP64 pipe (78% at N = 16,384).  A stage of N = 1,000, 8,192 and 16,385: one-sided in
-// FP64 165, 2290, 8070 us, here 61, 522, 2160; all units out of range, as in GravF64Adj but with
-// columns, 92, 1930, 7160.
+// FP64 220, 3040, 10750 us, here 81, 696, 2880; all units out of range, as in GravF64Adj but with
+// columns, 123, 2580, 9550.
 template <int R_, int TJ_>
 struct FxGrav2DAdj {
   using Fwd = FxGrav<2, R_, TJ_>;

@@ -344,8 +344,8 @@ int launch_sym(md_ctx *c, PairArgs a) {
   int kv = c->pt.vcta > 0 ? c->pt.vcta : Pol::FMT == 1 ? 8 : (MODEL == MD_GRAV3D && !MIXED) ? 3 : 4;
   // integer policies, whose units are long: below 16 per CTA one range each.  Neither is best
   // throughout; microseconds per force with one range and with four at N = 4,096, 8,192, 12,000,
-  // 16,385: Ring 85, 82; 245, 249; 435, 429; 785, 794; 2D 84, 79; 238, 251; 422, 412; 780, 780;
-  // 3D 122, 113; 366, 386; 683, 663; 1260, 1251.
+  // 16,385: Ring 86, 83; 261, 266; 508, 501; 916, 926; 2D 85, 80; 254, 268; 492, 481; 910, 911;
+  // 3D 124, 115; 390, 412; 797, 774; 1470, 1459.
   if (IsFx<Pol>::value && c->pt.vcta == 0 && a.U < 16 * G) kv = 1;
   a.P = (int)vcta_count(G, a.U, kv, IsFx<Pol>::value ? 1 : 16);
   int rc = ensure_pair_buffers(c, (int)TI, a.P, NACC);
