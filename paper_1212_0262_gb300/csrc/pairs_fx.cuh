@@ -6,16 +6,18 @@
 // units; column sums are added over the warp with redux.sync on 27-bit limbs (rounded to 2^5
 // units), over the warps as integers, and stored as doubles.
 //
-// A unit that touches a coordinate beyond RANGE, 2^26 sqrt(eps) (3D: 2^15), or a non-finite one
-// runs the FP64 policy's tile instead: at twice that distance in every component a 2D term is
-// still 2^54 units long and a 3D term 2^50, so that half a unit per term stays below the
-// rounding of FP64 sums.  So does a unit all of whose particles lie within 2^-24 sqrt(eps) (CLOSE)
-// of its first row, whose terms, about d / eps, are as small: that is a system, or a group in one,
-// whose extent is nothing against its softening length.  Error against 64 bits of 1,024 particles in a disk or ball of radius
-// R, rms over the particles of |error| / sum of |terms|, column sums truncated to 2^11 units,
-// rounded to 2^5, and all in FP64: 2D R = 1000, eps = 1e-8 1.7e-15, 3.8e-17, 4.3e-16;
-// 3D R = 30, eps = 1e-6 2.7e-14, 4.6e-17, 4.2e-16.  The CTA decides per unit with one vote,
-// which replaces the barrier after the tile's load.
+// A unit with a particle beyond RANGE, 2^26 sqrt(eps) (3D: 2^15), of its first row in some
+// coordinate, or with a non-finite one runs the FP64 policy's tile instead: at twice that
+// distance in every component a 2D term is still 2^54 units long and a 3D term 2^50, so that
+// half a unit per term stays below the rounding of FP64 sums.  So does a unit all of whose
+// particles lie within 2^-24 sqrt(eps) (CLOSE) of its first row, whose terms, about d / eps, are
+// as small: that is a system, or a group in one, whose extent is nothing against its softening
+// length.  The CTA decides per unit with one vote, which replaces the barrier after the
+// tile's load, and with a second one where its rows are close to each other.
+// Error against 64 bits of 1,024 particles in a disk or ball of radius R, rms over the particles
+// of |error| / sum of |terms|, column sums truncated to 2^11 units, rounded to 2^5, and all in
+// FP64: 2D R = 1000, eps = 1e-8 1.7e-15, 3.8e-17, 4.3e-16; 3D R = 30, eps = 1e-6 2.7e-14, 4.6e-17,
+// 4.2e-16.
 #pragma once
 #include "fx64.cuh"
 #include "pairs_impl.cuh"
@@ -135,7 +137,7 @@ struct FxGravTraits;
 template <>
 struct FxGravTraits<2> {
   static constexpr int MODEL = MD_GRAV2D, MINB = 4;
-  static constexpr int RANGE = 26;  // coordinates below 2^RANGE sqrt(eps)
+  static constexpr int RANGE = 26;  // coordinates within 2^RANGE sqrt(eps) of the first row's
   template <int R, int TJ>
   using Wild = GravF64<R, TJ, STAGE_KICK_DRIFT>;
   using Vec = double2;
@@ -191,15 +193,14 @@ struct FxGrav {
   // floor(log2(eps) / 2)
   __device__ static int half_exp(const PairArgs &a) { return ((int)(fx64::hi_word(a.epsd) >> 20) - 1023) >> 1; }
   __device__ static int lsb(const PairArgs &a) { return Tr::lsb(half_exp(a)); }
-  __device__ static bool out_of_range(double v, int half, int range = Tr::RANGE) {
-    const unsigned h = fx64::hi_word(v) & 0x7fffffffu;
-    return h >= ((unsigned)(1023 + range + half) << 20) && h != (fx64::hi_word(1.0e150));  // padding: its terms vanish
-  }
-  // v farther from the reference coordinate than CLOSE (padding is not)
+  // Where a coordinate lies from the unit's first row's: kFxWild from 2^range sqrt(eps) on (or
+  // not finite), kFxBroad from 2^-CLOSE on.  Padding's terms vanish.
   static constexpr int CLOSE = 24;
-  __device__ static bool broad(double v, double ref, int half) {
-    return (fx64::hi_word(v - ref) & 0x7fffffffu) >= ((unsigned)(1023 - CLOSE + half) << 20) &&
-           (fx64::hi_word(v) & 0x7fffffffu) != fx64::hi_word(1.0e150);
+  __device__ static int place(double v, double ref, int half, int range = Tr::RANGE) {
+    const unsigned h = fx64::hi_word(v - ref) & 0x7fffffffu;
+    if ((fx64::hi_word(v) & 0x7fffffffu) == fx64::hi_word(1.0e150)) return 0;
+    return (h >= ((unsigned)(1023 + range + half) << 20) ? kFxWild : 0) |
+           (h >= ((unsigned)(1023 - CLOSE + half) << 20) ? kFxBroad : 0);
   }
   __device__ static void load(State &st, const void *mirror, int64_t i0, const PairArgs &a, double *rowsm) {
     const int half = half_exp(a);
@@ -212,8 +213,7 @@ struct FxGrav {
 #pragma unroll
       for (int d = 0; d < D; d++) {
         st.x[r][d] = fx_coord(m, d);
-        if (out_of_range(st.x[r][d], half)) st.flags |= kFxWild;
-        if (broad(st.x[r][d], fx_coord(ref, d), half)) st.flags |= kFxBroad;
+        st.flags |= place(st.x[r][d], fx_coord(ref, d), half);
       }
     }
   }
@@ -228,8 +228,7 @@ struct FxGrav {
     constexpr int PER = JB / 16;
     const double2 v = ((const double2 *)tile)[ch], ref = ((const double2 *)a.mirror_in)[i0 * PER + ch % PER];
     const int half = half_exp(a);
-    return (out_of_range(v.x, half) || out_of_range(v.y, half) ? kFxWild : 0) |
-           (broad(v.x, ref.x, half) || broad(v.y, ref.y, half) ? kFxBroad : 0);
+    return place(v.x, ref.x, half) | place(v.y, ref.y, half);
   }
   template <bool COL>
   __device__ static void unit(State &st, const unsigned char *smb, const unsigned char *, const PairArgs &a,
@@ -462,7 +461,7 @@ struct RingFx {
 //
 // f falls as 1 / r, j as 1 / r^2, e as 1 / r^3, each against a unit that its largest term,
 // at r = sqrt(eps), sets: RANGE is where a term of e is still 2^52 units long (coordinates
-// below 2^9 sqrt(eps); farther apart e at 2^26, the forward range, would be 2^5 units).  The
+// within 2^9 sqrt(eps) of the first row's; e at 2^26, the forward range, would be 2^5 units).  The
 // unit of j also follows from the v: from W, the largest |v_k - v_0| (found before the stage).
 // Every particle has a partner whose w is at least W / 2, however the other w are spread, so
 // the sum of its |j| is at least 2^58 units within RANGE; terms of j are rounded to
@@ -497,7 +496,6 @@ struct FxGrav2DAdj {
   };
   static constexpr int RANGE = 9;
   static constexpr int CLOSE = Fwd::CLOSE;
-  __device__ static bool out_of_range(double v, int half) { return Fwd::out_of_range(v, half, RANGE); }
   // |w_d| <= 2 W < 2^vexp.  All v equal: any exponent will do (the w of padding, up to 2^299,
   // divided by its s must vanish)
   __device__ static int vexp(const PairArgs &a) { return *a.vrange == 0u ? 299 : (int)(*a.vrange >> 20) - 1021; }
@@ -525,8 +523,7 @@ struct FxGrav2DAdj {
       st.x[r][1] = m.y;
       st.v[r][0] = m.z;
       st.v[r][1] = m.w;
-      if (out_of_range(m.x, half) || out_of_range(m.y, half)) st.flags |= kFxWild;
-      if (Fwd::broad(m.x, ref.x, half) || Fwd::broad(m.y, ref.y, half)) st.flags |= kFxBroad;
+      st.flags |= Fwd::place(m.x, ref.x, half, RANGE) | Fwd::place(m.y, ref.y, half, RANGE);
     }
   }
   __device__ static void flush(State &st, const PairArgs &a) {
@@ -548,8 +545,7 @@ struct FxGrav2DAdj {
     if (ch & 1) return 0;
     const double2 m = ((const double2 *)tile)[ch], ref = ((const double2 *)a.mirror_in)[2 * i0];
     const int half = Fwd::half_exp(a);
-    return (out_of_range(m.x, half) || out_of_range(m.y, half) ? kFxWild : 0) |
-           (Fwd::broad(m.x, ref.x, half) || Fwd::broad(m.y, ref.y, half) ? kFxBroad : 0);
+    return Fwd::place(m.x, ref.x, half, RANGE) | Fwd::place(m.y, ref.y, half, RANGE);
   }
   template <bool COL>
   __device__ static void unit(State &st, const unsigned char *smb, const unsigned char *, const PairArgs &a,
