@@ -22,6 +22,7 @@
 // that sums them in a fixed order and runs the epilogue.  (The one-sided form shares one launch
 // between the parts, split by md_batch_set_tuning's `split`.)
 #include <algorithm>
+#include <new>
 #include <vector>
 
 #include "pairs_impl.cuh"
@@ -628,19 +629,23 @@ int ensure_finish(md_batch *b, int64_t Pr, int64_t Pg, const int64_t TI[2], cons
   if (b->fin_P[0] == Pr && b->fin_P[1] == Pg) return MD_OK;
   b->fin_P[0] = b->fin_P[1] = -1;
   std::vector<FinTask> tasks;
-  for (int s = 0; s < (int)b->hs.size(); s++) {
-    const SysDesc &d = b->hs[s];
-    const int part = s < b->nr ? 0 : 1, per_tile = (int)(TI[part] / kFinishThreadsB);
-    const int64_t U = part == 0 ? b->Ur : b->Ug, P = part == 0 ? Pr : Pg;
-    if (s == b->nr) b->nfin_r = (int)tasks.size();
-    for (int T = 0; T < (int)d.n_it; T++) {
-      const RowChunks rc = row_chunks(U, (int)P, d.ubeg, d.n_jt, m[part], T, T + 1, kChunkB, kDirectB);
-      const int first = unit_begin(U, (int)P, rc.cf) >= rc.ubeg ? 1 : 0;
-      for (int sub = 0; sub < per_tile; sub++)
-        for (int c = 0; c < rc.cols + rc.segs; c++)
-          tasks.push_back(FinTask{part == 0 ? s : s - b->nr, T, sub, (int)d.bbeg + T * per_tile + sub, c, rc.cols,
-                                  rc.cols + rc.segs, (int)rc.cf, (int)rc.cl, first, {0, 0}});
+  try {
+    for (int s = 0; s < (int)b->hs.size(); s++) {
+      const SysDesc &d = b->hs[s];
+      const int part = s < b->nr ? 0 : 1, per_tile = (int)(TI[part] / kFinishThreadsB);
+      const int64_t U = part == 0 ? b->Ur : b->Ug, P = part == 0 ? Pr : Pg;
+      if (s == b->nr) b->nfin_r = (int)tasks.size();
+      for (int T = 0; T < (int)d.n_it; T++) {
+        const RowChunks rc = row_chunks(U, (int)P, d.ubeg, d.n_jt, m[part], T, T + 1, kChunkB, kDirectB);
+        const int first = unit_begin(U, (int)P, rc.cf) >= rc.ubeg ? 1 : 0;
+        for (int sub = 0; sub < per_tile; sub++)
+          for (int c = 0; c < rc.cols + rc.segs; c++)
+            tasks.push_back(FinTask{part == 0 ? s : s - b->nr, T, sub, (int)d.bbeg + T * per_tile + sub, c, rc.cols,
+                                    rc.cols + rc.segs, (int)rc.cf, (int)rc.cl, first, {0, 0}});
+      }
     }
+  } catch (const std::bad_alloc &) {
+    return berr(b, MD_ENOMEM, "%s", "batch finish tasks (host)");
   }
   if (b->nr == (int)b->hs.size()) b->nfin_r = (int)tasks.size();
   b->nfin_g = (int)tasks.size() - b->nfin_r;

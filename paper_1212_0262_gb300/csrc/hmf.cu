@@ -240,10 +240,11 @@ __device__ __forceinline__ bool grid_finish(double sc, double ss, double *partia
 // that are small themselves, where doubles have more bits than fixed-point numbers.  Their
 // stages are all FP64: (cos, sin) kept as doubles (*HmfArgs::fmt = 1), the table-driven sines and
 // cosines of sincos_fp64.cuh, FP64 sums; 12 FP64 operations per particle-stage, 8.0 us at
-// N = 10,007, 1.31 ms at N = 5e7.  So are stages whose M is not finite, or below 2^-200.  Wider systems are more exact in fixed point (N = 50,000, angles
-// up to 1e-3, rms of |error| / scale of a force 9e-16 against 2.8e-15, whose table sine rounds r^3 / 6
-// to FP32), narrower ones as doubles (up to 1e-6 7e-13 against 7e-17).  A stage whose
-// predecessor's M was cold reads doubles, one whose own M is cold writes them.
+// N = 10,007, 1.31 ms at N = 5e7.  So are stages whose M is not finite, or below 2^-200.
+// Wider systems are more exact in fixed point (N = 50,000, angles up to 1e-3, rms of |error| /
+// scale of a force 9e-16 against 2.8e-15, whose table sine rounds r^3 / 6 to FP32), narrower ones
+// as doubles (up to 1e-6 7e-13 against 7e-17).  A stage whose predecessor's M was cold reads
+// doubles, one whose own M is cold writes them.
 __device__ __forceinline__ bool hmf_near_one(double m) {
   const unsigned h = fx64::hi_word(m) & 0x7fffffffu;
   return h >= 0x3fefffffu && h < kTopMax && (h > 0x3fefffffu || fx64::lo_word(m) > 0xe0000000u);
